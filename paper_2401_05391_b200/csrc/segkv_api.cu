@@ -399,6 +399,32 @@ int stream_splits(const segkv* h) {
     return best;
 }
 
+// Which handles take the wide kernel (tcgen05, up to 32 query columns): those the tiled kernel has no form for.
+bool use_wide(const segkv* h) { return !tiled_supported(h->d); }
+
+// Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA, where a
+// round of items costs its tiles plus about two tiles' time to start and finish an item, and meeting in the
+// workspace costs about two more.
+int wide_splits(const segkv* h) {
+    const Dims& d = h->d;
+    const long long slabs = (long long)d.batch * d.kv_heads;
+    const int keys = wide_tile_keys(d);
+    const long long ntp = ((h->prompt_len > 0 ? h->prompt_len : 0) + keys - 1) / keys;
+    const long long ntr = (h->steps + 2 * d.beams + keys - 1) / keys;      // estimate, rows are mostly shared
+    if (h->splits_forced > 0) return h->splits_forced;
+    int best = 1;
+    long long best_cost = 0;
+    for (int s = 1; s <= h->ws_splits && s <= kMaxSplits && s <= ntp + ntr; ++s) {
+        const long long rounds = (slabs * s + h->sm_count - 1) / h->sm_count;
+        const long long cost = rounds * ((ntp + s - 1) / s + (ntr + s - 1) / s + 2) + (s > 1 ? 2 : 0);
+        if (s == 1 || cost < best_cost) {
+            best = s;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 // Does the separate attention call run in the persistent form?
 bool use_stream(const segkv* h) {
     if (h->persist_mode == 0 || !stream_supported(h->d) || h->tile_forced != 0 || h->combine_forced == 2) return false;
@@ -781,15 +807,18 @@ int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_sl
     if (h->prompt_len < 0) return SEGKV_ESTATE;
     if (h->prompt_len + h->steps <= 0) return SEGKV_ESTATE;
     if (h->leader && h->leader->steps != h->steps) return SEGKV_ESTATE;   // the shared tables describe another step
-    if (!tiled_supported(h->d)) {
-        SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, 1);
-        SEGKV_CUDA(launch_sdpa_rowwise(h->d, a, (cudaStream_t)stream));
-        count_launch(h, (cudaStream_t)stream);
-        return SEGKV_OK;
-    }
     {
         int rc = ensure_lists(h, (cudaStream_t)stream);
         if (rc != SEGKV_OK) return rc;
+    }
+    if (use_wide(h)) {
+        SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, wide_splits(h));
+        a.pdl = h->overlap;
+        h->dbg_wait_ns = 0;
+        h->dbg_skip = false;
+        SEGKV_CUDA(launch_sdpa_wide(h->d, a, h->tm_kp, h->tm_vp, h->sm_count, (cudaStream_t)stream));
+        count_launch(h, (cudaStream_t)stream);
+        return SEGKV_OK;
     }
     if (use_stream(h)) {
         const int sp = stream_splits(h);
@@ -872,8 +901,8 @@ int segkv_decode_step(segkv_t h, int step, const int32_t* beam_parent, const voi
     if (h->prompt_len < 0) return SEGKV_ESTATE;
     if (step != h->steps) return SEGKV_ESTATE;
     if (step >= h->d.max_steps) return SEGKV_ECAPACITY;
-    if (!tiled_supported(h->d) || h->leader) {
-        // shapes the tiled kernel does not take, and handles that use another handle's tables
+    if (use_wide(h) || h->leader) {
+        // the wide kernel has no fused form, and handles that use another handle's tables
         // (nothing to update in the attention kernel): the two separate launches
         int rc = segkv_append(h, step, beam_parent, k_new, v_new, stream);
         if (rc != SEGKV_OK) return rc;
@@ -1177,6 +1206,7 @@ int segkv_truncate_last(segkv_t h) {
     if (h->steps <= 0 || h->truncated) return SEGKV_ESTATE;
     h->steps -= 1;
     h->truncated = true;
+    h->lists_valid = false;              // they describe the dropped step; the table of the step before is kept
     return SEGKV_OK;
 }
 
@@ -1252,7 +1282,7 @@ int segkv_set_tuning(segkv_t h, int splits, int stages, int combine) {
 
 int segkv_get_splits(segkv_t h) {
     if (!h) return SEGKV_EINVAL;
-    if (!tiled_supported(h->d)) return 1;
+    if (use_wide(h)) return wide_splits(h);
     return choose_tiling(h, false).splits;
 }
 

@@ -184,8 +184,7 @@ struct SdpaArgs {
     int32_t* parent_row;
 };
 
-// Plain gather kernel: one CTA per (beam slot, head), fp32 ALU; kept for shapes
-// the tiled kernel does not cover and as an in-library cross-check.
+// Plain gather kernel: one CTA per (beam slot, head), fp32 ALU; kept as an in-library cross-check.
 cudaError_t launch_sdpa_rowwise(const Dims& d, const SdpaArgs& a, cudaStream_t st);
 
 // Tiled split-KV kernel (TMA-staged prompt tiles, gathered response rows, tensor-core tiles).
@@ -203,7 +202,13 @@ cudaError_t launch_sdpa_stream(const Dims& d, const SdpaArgs& a, const CUtensorM
 cudaError_t launch_sdpa_tiled(const Dims& d, const SdpaArgs& a, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                               int stages, cudaStream_t st);
 
-// Same kernel with its split workspace in a fixed device array of the module (no allocation).
+// Work groups of more query columns than the tiled kernel takes (segkv_sdpa_wide.cu, tcgen05): a resident grid
+// walks the (work group, split) items; a.splits items per work group, merged through the workspace.
+int wide_tile_keys(const Dims& d);
+cudaError_t launch_sdpa_wide(const Dims& d, const SdpaArgs& a, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
+                             int sm_count, cudaStream_t st);
+
+// The tiled kernel with its split workspace in a fixed device array of the module (no allocation).
 size_t tiled_static_scratch_bytes();
 cudaError_t launch_sdpa_tiled_static(const Dims& d, SdpaArgs a, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                                      int stages, cudaStream_t st, int* too_big);

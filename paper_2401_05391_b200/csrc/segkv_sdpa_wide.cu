@@ -1,0 +1,708 @@
+// Decode attention for work groups of many query columns (beams * query heads per kv head from 9 to 32) on the
+// fifth-generation tensor cores (tcgen05 + tensor memory), head_dim 64, 128 or 256.  Same contract as the
+// tiled kernel's separate form (paper Sections 3.2, 3.3): the prompt segment is read once for all columns of
+// a (request, kv head), the response rows through the request's list of distinct rows, one softmax over both.
+//
+// What bounds it: HBM, once the columns share every key.  The tiled kernel keeps O^T of all columns in one
+// warp's registers (mma.sync), which ends at 16 columns (8 at head_dim 256); beyond that the only kernel
+// was the row-wise one, which reads the prompt once per beam and query head.
+//
+//  * one persistent CTA per SM walks the items (work group, split) round-robin;
+//  * S[128 rows, KEYS] = Q.K^T with M = 128: the at most 32 query columns are the rows, REPEATED FOUR TIMES, so
+//    that each of the four softmax warps finds all columns in its own tensor-memory lanes and takes a
+//    quarter of the tile's keys (one column per lane, KEYS/4 keys per thread: no shuffles).  The repeated
+//    rows cost MMA time the tensor pipe has to spare: 8 + 4 MMAs per 32 KB of keys and values, about 900
+//    clocks, against about 1300 clocks for an SM's share of HBM bandwidth;
+//  * the four warps agree on a column's maximum through shared memory (one barrier per tile, which also
+//    carries the "a wait ran out" flag, so that all warps leave together) and write the weights P, rounded
+//    to the 16-bit type, into ONE shared-memory tile of 32 rows: the A operand of O[128, D] += P.V, whose rows
+//    past the real ones are never read.  bf16 weights go in two parts (p = hi + lo, 16 significant bits):
+//    hi in rows 0..31, lo in rows 32..63 of the same MMA, added up in the epilogue, at no extra MMA;
+//  * O stays in tensor memory and is rescaled only when a column's maximum has grown by more than 2^8 over
+//    the reference in use (sum and weights use the same reference, so the result is exact);
+//  * prompt tiles arrive by TMA in one ring; response tiles are gathered row by row (cp.async into the same
+//    128-byte-swizzled layout) by two groups of two warps, one stage each, so that two gathers are in
+//    flight; the gather warps also place the query block;
+//  * splits of a work group meet in the global workspace: the last CTA to arrive folds them (as in the tiled
+//    kernel).
+// Every mbarrier is waited on phase by phase and every wait is bounded; on expiry the kernel flags
+// SEGKV_DEV_WAIT_LIMIT, leaves the output alone and still releases its tensor memory and its tickets.
+#include "segkv_internal.h"
+#include "segkv_ptx.cuh"
+#include "segkv_tc5.cuh"
+
+namespace segkv_impl {
+
+namespace {
+
+using namespace ptx;
+
+constexpr int kTicketAbortedW = 1 << 16;     // same marker as the tiled kernel's
+constexpr int kCols = kMaxCols;              // query columns of a work group, padded: one tensor-memory lane each
+
+// AND of a predicate over the threads that meet at a named barrier
+__device__ __forceinline__ bool bar_and(int id, int threads, bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "barrier.cta.red.and.pred p, %2, %3, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r) : "r"((uint32_t)ok), "r"(id), "r"(threads) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void bar_sync_n(int id, int threads) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// Registers written by a tcgen05.ld may be used from here on (after the wait): keeps their uses behind it.
+template <int N>
+__device__ __forceinline__ void pin(uint32_t* r) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
+
+struct WideParams {
+    const void* q;
+    void* out;
+    const float* slopes;
+    const char* kr;                // response K (V row = K row + vdelta)
+    const char* const* k_chunks;   // growing capacity: chunk base pointers, chunk_steps steps each
+    long long vdelta;
+    const URow* ulist;
+    const int32_t* ucount;
+    const int32_t* plens;
+    float* ws_o;                   // [item][ncols][D] un-normalised partial outputs
+    float* ws_ml;                  // [item][ncols][2] reference maximum (base-2 domain) and sum
+    int* tickets;
+    int* err_word;
+    int P, steps, S, W, G, H, Hkv, rows, max_steps, ncols, chunk_steps, quota, items;
+    int early_prompt, dbg_skip;
+    unsigned long long wait_ns;
+    float scale2;
+    uint32_t idesc_qk, idesc_pv;
+};
+
+template <int D_>
+struct WideLayout {
+    static constexpr int D = D_;
+    static constexpr int KEYS = D == 256 ? 32 : 64;              // keys of a tile: one box of the prompt's tensor map
+    static constexpr int KW = KEYS / 4;                          // keys of a softmax warp
+    static constexpr int kDBoxes = D / 64;                       // 128-byte column blocks of a row
+    static constexpr int kColTile = KEYS * 128;
+    static constexpr int kTile = kDBoxes * kColTile;             // bytes of a K (or a V) tile
+    static constexpr int kStage = 2 * kTile;
+    static constexpr int SP = D == 64 ? 7 : (D == 128 ? 3 : 2);  // prompt stages
+    static constexpr int SR = 2;                                 // response stages: one per gather group
+    static constexpr int kQ = kDBoxes * 128 * 128;               // the query block, four times
+    static constexpr int kP = 64 * 128;                          // one buffer of weights: 32 rows hi, 32 rows lo
+    static constexpr int kMeta = SR * KEYS * (int)sizeof(URow);
+    static constexpr int kPtr = SR * KEYS * 8;
+    static constexpr int kMax = 2 * 4 * kCols * 4, kSum = 4 * kCols * 4;
+    static constexpr int kBars = 2 * SP + 2 * SR + 2 + 6 + 1;    // rings, query full/empty, S/P/O x 2, wind-down
+    static constexpr size_t kBytes = 1024 + (size_t)kQ + 2 * kP + (SP + SR) * kStage + kMeta + kPtr + kMax + kSum + 8 * kBars + 64;
+    static constexpr int kColO = 2 * KEYS;                       // tensor memory: two S buffers, then O
+    static constexpr int kTmemCols = kColO + D <= 256 ? 256 : 512;
+    static constexpr int kThreads = 320;                         // 4 softmax warps, TMA, MMA, 2 x 2 gather warps
+    static_assert(kColO + D <= kTmemCols, "tensor memory");
+    static_assert(kBytes <= 232448, "shared memory");
+};
+
+template <typename T, int D>
+__global__ void __launch_bounds__(320, 1)
+sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const WideParams p) {
+    using L = WideLayout<D>;
+    constexpr int KEYS = L::KEYS, KW = L::KW, SP = L::SP, SR = L::SR;
+    constexpr bool kTwoPart = !Mma<T>::kWeights11Bits;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* q_smem = smem;                                       // per column block [4 x 32 rows][128 bytes]
+    uint8_t* p_smem = q_smem + L::kQ;                             // two buffers; their A operands reach into the ring behind
+    uint8_t* p_ring = p_smem + 2 * L::kP;
+    uint8_t* r_ring = p_ring + (size_t)SP * L::kStage;
+    URow* meta = reinterpret_cast<URow*>(r_ring + (size_t)SR * L::kStage);
+    const char** gk = reinterpret_cast<const char**>(meta + SR * KEYS);
+    float* s_max = reinterpret_cast<float*>(gk + SR * KEYS);      // [2][4 warps][kCols]
+    float* s_sum = s_max + 2 * 4 * kCols;                         // [4 warps][kCols]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s_sum + 4 * kCols);
+    const uint32_t pfull = smem_u32(bars), pempty = pfull + 8 * SP, rfull = pempty + 8 * SP, rempty = rfull + 8 * SR;
+    const uint32_t qfull = rempty + 8 * SR, qempty = qfull + 8;
+    const uint32_t bar_s = qempty + 8, bar_p = bar_s + 16, bar_o = bar_p + 16;     // two each: tile parity
+    const uint32_t bar_end = bar_o + 16;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
+    __shared__ int s_abort, s_ticket;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    // One item: the split's share of a work group (prompt tiles, and a range of the request's distinct rows)
+    struct Item { int slab, split, b, kvh, P, pt0, npt; };
+    auto item_of = [&](int it) {
+        Item x;
+        x.slab = it / p.S;
+        x.split = it - x.slab * p.S;
+        x.b = x.slab / p.Hkv;
+        x.kvh = x.slab - x.b * p.Hkv;
+        x.P = p.plens ? __ldg(p.plens + x.b) : p.P;
+        const int ntp = (x.P + KEYS - 1) / KEYS;
+        x.pt0 = (int)((long long)x.split * ntp / p.S);
+        x.npt = (int)((long long)(x.split + 1) * ntp / p.S) - x.pt0;
+        return x;
+    };
+    auto rows_of = [&](const Item& x, int& e0, int& e1) {
+        const int n_b = p.steps > 0 ? p.ucount[x.b] : 0;
+        e0 = min(x.split * p.quota, n_b);
+        e1 = x.split == p.S - 1 ? n_b : min((x.split + 1) * p.quota, n_b);
+    };
+    auto issue_prompt = [&](const Item& x, int k, uint32_t pos) {
+        const uint32_t st = pos % SP, full = pfull + 8 * st;
+        const uint32_t k_dst = smem_u32(p_ring) + st * (uint32_t)L::kStage, v_dst = k_dst + L::kTile;
+        mbar_arrive_expect_tx(full, (uint32_t)L::kStage);
+        const int y = (x.pt0 + k) * KEYS;
+#pragma unroll
+        for (int bx = 0; bx < L::kDBoxes; ++bx) tma_load_4d(k_dst + bx * L::kColTile, &tm_k, bx * 64, x.kvh, y, x.b, full);
+#pragma unroll
+        for (int bx = 0; bx < L::kDBoxes; ++bx) tma_load_4d(v_dst + bx * L::kColTile, &tm_v, bx * 64, x.kvh, y, x.b, full);
+    };
+
+    // Set-up by the TMA warp, which then starts the first prompt tiles before the CTA has synchronised (and,
+    // when nothing can still be writing the prompt, before the previous kernel has finished).
+    int first = 0;                       // prompt tiles of the CTA's first item already requested
+    if (warp == 4 && lane == 0) {
+        for (int s = 0; s < SP; ++s) {
+            mbar_init(pfull + 8 * s, 1);
+            mbar_init(pempty + 8 * s, 1);
+        }
+        for (int s = 0; s < SR; ++s) {
+            mbar_init(rfull + 8 * s, 1);
+            mbar_init(rempty + 8 * s, 1);
+        }
+        mbar_init(qfull, 2);
+        mbar_init(qempty, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar_s + 8 * i, 1);
+            mbar_init(bar_p + 8 * i, 128);
+            mbar_init(bar_o + 8 * i, 1);
+        }
+        mbar_init(bar_end, 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async();
+        if (!p.early_prompt) asm volatile("griddepcontrol.wait;" ::: "memory");
+        const Item x = item_of((int)blockIdx.x);
+        first = min(x.npt, SP);
+        for (int k = 0; k < first; ++k) issue_prompt(x, k, (uint32_t)k);
+    }
+    if (warp == 5) {                     // this warp owns the tensor memory
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "n"(L::kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    if (warp != 4) {
+        // everything but the prompt tiles follows the previous kernel; its successors are let go only after that
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+
+    if (warp == 4) {
+        // ------------------------------- prompt tiles (TMA) -------------------------------
+        if (lane == 0) {
+            uint32_t pos = 0;
+            bool ok = true;
+            for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
+                const Item x = item_of(it);
+                int k = 0;
+                if (it == (int)blockIdx.x) pos = (uint32_t)(k = first);
+                for (; k < x.npt; ++k, ++pos) {
+                    ok = mbar_wait(pempty + 8 * (pos % SP), ((pos / SP) & 1) ^ 1, p.wait_ns);
+                    if (!ok) break;
+                    issue_prompt(x, k, pos);
+                }
+            }
+            if (!ok) {
+                s_abort = 1;
+                for (uint32_t k = pos > (uint32_t)SP ? pos - SP : 0; k < pos; ++k)       // copies in flight land first
+                    (void)mbar_wait(pfull + 8 * (k % SP), (k / SP) & 1, p.wait_ns);
+            }
+        }
+    } else if (warp == 5) {
+        // -------------------------------- MMA issuer --------------------------------
+        if (lane == 0) {
+            uint32_t n = 0, pos = 0, rn = 0, qi = 0;              // tiles, prompt tiles, response tiles, items so far
+            const uint64_t q_desc = smem_desc(smem_u32(q_smem), 16, 1024);
+            const uint64_t p_desc = smem_desc(smem_u32(p_smem), 16, 1024);
+            bool ok = true;
+            for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
+                const Item x = item_of(it);
+                int e0, e1;
+                rows_of(x, e0, e1);
+                const int tiles = x.npt + (e1 - e0 + KEYS - 1) / KEYS;
+                if (tiles == 0) continue;
+                auto stage_addr = [&](int t) -> uint32_t {        // prompt tiles first, then response tiles
+                    return t < x.npt ? smem_u32(p_ring) + ((pos + t) % SP) * (uint32_t)L::kStage
+                                     : smem_u32(r_ring) + ((rn + t - x.npt) % SR) * (uint32_t)L::kStage;
+                };
+                auto wait_tile = [&](int t) -> bool {
+                    bool r;
+                    if (t < x.npt) r = mbar_wait_hot(pfull + 8 * ((pos + t) % SP), ((pos + t) / SP) & 1, p.wait_ns);
+                    else r = mbar_wait_hot(rfull + 8 * ((rn + t - x.npt) % SR), ((rn + t - x.npt) / SR) & 1, p.wait_ns);
+                    tc_fence_after();
+                    return r;
+                };
+                auto issue_qk = [&](int t) {
+                    const uint32_t buf = (n + (uint32_t)t) & 1;
+                    const uint64_t kd = smem_desc(stage_addr(t), 16, 1024);
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks)
+                        tc_mma_ss(tmem + buf * KEYS, q_desc + (uint64_t)(((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4),
+                                  kd + (uint64_t)(((ks >> 2) * L::kColTile + (ks & 3) * 32) >> 4), p.idesc_qk, ks > 0);
+                    tc_commit(bar_s + 8 * buf);
+                    if (t == tiles - 1) tc_commit(qempty);        // the query block may be replaced
+                };
+                ok = mbar_wait_hot(qfull, qi++ & 1, p.wait_ns) && wait_tile(0);
+                if (!ok) break;
+                issue_qk(0);
+                for (int t = 0; t < tiles; ++t) {
+                    if (t + 1 < tiles) {                          // the next scores run under this tile's softmax
+                        ok = wait_tile(t + 1);
+                        if (!ok) break;
+                        issue_qk(t + 1);
+                    }
+                    const uint32_t m = n + (uint32_t)t, buf = m & 1;
+                    ok = mbar_wait_hot(bar_p + 8 * buf, (m >> 1) & 1, p.wait_ns);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t pd = p_desc + (uint64_t)((buf * (uint32_t)L::kP) >> 4);
+                    const uint64_t vd = smem_desc(stage_addr(t) + L::kTile, L::kColTile, 1024);
+#pragma unroll
+                    for (int kk = 0; kk < KEYS / 16; ++kk)        // O += P[:, 16 keys] . V[16 keys, :]
+                        tc_mma_ss(tmem + L::kColO, pd + (uint64_t)((kk * 32) >> 4), vd + (uint64_t)((kk * 2048) >> 4),
+                                  p.idesc_pv, t > 0 || kk > 0);
+                    tc_commit(bar_o + 8 * buf);
+                    tc_commit(t < x.npt ? pempty + 8 * ((pos + t) % SP) : rempty + 8 * ((rn + t - x.npt) % SR));
+                }
+                if (!ok) break;
+                n += (uint32_t)tiles;
+                pos += (uint32_t)x.npt;
+                rn += (uint32_t)(tiles - x.npt);
+            }
+            if (!ok) s_abort = 1;
+        }
+    } else if (warp >= 6) {
+        // ------------------- the query block, and response tiles: index select fused into the load -------------------
+        const int grp = (warp - 6) >> 1, gt = tid - 192 - grp * 64, bid = 2 + grp;
+        constexpr int CPR = D / 8;                                // 16-byte chunks per row
+        constexpr int RPI = 64 / CPR;                             // rows the group's threads cover at once
+        const size_t slab_bytes = (size_t)p.rows * p.Hkv * (size_t)(D * 2);
+        uint8_t* stage = r_ring + (size_t)grp * L::kStage;        // the group's stage
+        URow* meta_g = meta + grp * KEYS;
+        const char** gk_g = gk + grp * KEYS;
+        uint32_t rn = 0, qi = 0;
+        bool ok = true;
+        for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
+            const Item x = item_of(it);
+            int e0, e1;
+            rows_of(x, e0, e1);
+            const int nrt = (e1 - e0 + KEYS - 1) / KEYS;
+            if (x.npt + nrt == 0) continue;
+            // the group's half of the query rows, into all four copies; rows past the last column are zeros
+            uint4 v[16 / RPI];
+#pragma unroll
+            for (int i = 0; i < 16 / RPI; ++i) {
+                const int col = grp * 16 + i * RPI + gt / CPR, c = gt % CPR;
+                v[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (col < p.ncols)
+                    v[i] = *reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p.q) +
+                               ((size_t)(x.b * p.W + col / p.G) * p.H + x.kvh * p.G + col % p.G) * D + c * 8);
+            }
+            ok = mbar_wait(qempty, (qi & 1) ^ 1, p.wait_ns);
+            ok = bar_and(bid, 64, ok);
+            if (!ok) break;
+            ++qi;
+#pragma unroll
+            for (int i = 0; i < 16 / RPI; ++i) {
+                const int col = grp * 16 + i * RPI + gt / CPR, c = gt % CPR;
+                uint8_t* dst = q_smem + (size_t)(c >> 3) * (128 * 128) + col * 128 + (((c & 7) ^ (col & 7)) << 4);
+#pragma unroll
+                for (int rep = 0; rep < 4; ++rep) *reinterpret_cast<uint4*>(dst + rep * 32 * 128) = v[i];
+            }
+            fence_proxy_async();
+            bar_sync_n(bid, 64);
+            if (gt == 0) mbar_arrive(qfull);
+            const URow* list = p.ulist + (size_t)x.b * p.W * p.max_steps;
+            for (int r = 0; r < nrt; ++r) {
+                const uint32_t pos = rn + (uint32_t)r;
+                if ((pos & 1) != (uint32_t)grp) continue;         // the other group's tile
+                const int eb = e0 + r * KEYS, cnt = min(KEYS, e1 - eb);
+                URow u = {0, 0u};
+                if (gt < cnt) u = list[eb + gt];
+                ok = mbar_wait(rempty + 8 * grp, ((pos >> 1) & 1) ^ 1, p.wait_ns);
+                ok = bar_and(bid, 64, ok);
+                if (!ok) break;
+                if (gt < KEYS) {
+                    const int s = u.row / p.rows;
+                    const char* base = p.chunk_steps == 0 ? p.kr + (size_t)s * slab_bytes
+                                                          : p.k_chunks[s / p.chunk_steps] + (size_t)(s % p.chunk_steps) * slab_bytes;
+                    gk_g[gt] = base + ((size_t)(u.row - s * p.rows) * p.Hkv + x.kvh) * (size_t)(D * 2);
+                    u.row = s;                                    // the softmax threads need the step only
+                    meta_g[gt] = u;                               // (no beam reads the padding of the last tile)
+                }
+                bar_sync_n(bid, 64);
+                const int c = gt % CPR;
+                uint8_t* dst0 = stage + (size_t)(c >> 3) * L::kColTile;
+#pragma unroll 4
+                for (int i = 0; i < KEYS / RPI; ++i) {
+                    const int key = i * RPI + gt / CPR;
+                    uint8_t* dst = dst0 + key * 128 + (((c & 7) ^ (key & 7)) << 4);
+                    if (key < cnt) {
+                        const char* src = gk_g[key] + c * 16;
+                        cp_async_16(smem_u32(dst), src);
+                        cp_async_16(smem_u32(dst + L::kTile), src + p.vdelta);
+                    } else {                                      // a weight of zero times whatever was here need not be zero
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4*>(dst + L::kTile) = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                }
+                cp_async_wait_all();
+                fence_proxy_async();
+                bar_sync_n(bid, 64);
+                if (gt == 0) mbar_arrive(rfull + 8 * grp);
+            }
+            rn += (uint32_t)nrt;
+        }
+        if (!ok && gt == 0) s_abort = 1;
+    } else {
+        // ---------------------- softmax warps: one column per lane, a quarter of the keys per warp ----------------------
+        const uint32_t tm_lane = tmem + ((uint32_t)(warp * 32) << 16);
+        const uint32_t tm_o = tm_lane + (uint32_t)L::kColO;
+        const bool owns_o = warp == 0 || (kTwoPart && warp == 1);    // rows 0..31 of O, and 32..63 for the low parts
+        const bool real = lane < p.ncols;
+        const int beam = real ? lane / p.G : 0, hg = real ? lane % p.G : 0;
+        const uint32_t beambit = real ? 1u << beam : 0u;
+        uint32_t n = 0, rn = 0;                                   // tiles and response tiles so far
+        bool ok = true, gone = false;                             // a wait of this thread ran out; the four warps have agreed to leave
+        int it = blockIdx.x;
+        for (; it < p.items; it += gridDim.x) {
+            const Item x = item_of(it);
+            int e0, e1;
+            rows_of(x, e0, e1);
+            const int nrt = (e1 - e0 + KEYS - 1) / KEYS, tiles = x.npt + nrt;
+            const float slope2 = (p.slopes && real) ? p.slopes[x.kvh * p.G + hg] * 1.4426950408889634f : 0.f;
+            const int qpos = x.P + (p.steps > 0 ? p.steps - 1 : -1);
+            float m_ref = -INFINITY, l_run = 0.f;
+            for (int t = 0; t < tiles; ++t, ++n) {
+                const uint32_t buf = n & 1;
+                const bool resp = t >= x.npt;
+                const uint32_t rpos = rn + (uint32_t)(t - x.npt);
+                if (ok && resp) ok = mbar_wait_hot(rfull + 8 * (rpos % SR), (rpos / SR) & 1, p.wait_ns);   // the tile's records
+                if (ok) ok = mbar_wait_hot(bar_s + 8 * buf, (n >> 1) & 1, p.wait_ns);
+                ok = __all_sync(0xffffffffu, ok);
+                float v[KW];
+                float tmax = -INFINITY;
+                if (ok) {
+                    tc_fence_after();
+                    uint32_t sr[KW];
+                    if (KW == 16) tc_ld16(tm_lane + buf * KEYS + warp * KW, sr);
+                    else tc_ld8(tm_lane + buf * KEYS + warp * KW, sr);
+                    tc_wait_ld();
+                    pin<KW>(sr);
+                    if (!resp) {
+                        const int key0 = (x.pt0 + t) * KEYS + warp * KW, left = x.P - key0;      // keys past the prompt are masked
+                        const float bias0 = slope2 * (float)(key0 - qpos);
+#pragma unroll
+                        for (int i = 0; i < KW; ++i) {
+                            v[i] = fmaf(__uint_as_float(sr[i]), p.scale2, fmaf(slope2, (float)i, bias0));
+                            if (i >= left) v[i] = -INFINITY;
+                        }
+                    } else {
+                        const URow* mt = meta + (rpos % SR) * KEYS + warp * KW;
+#pragma unroll
+                        for (int i = 0; i < KW; ++i) {
+                            const int2 u = *reinterpret_cast<const int2*>(mt + i);                  // {step, beams that read the row}
+                            v[i] = fmaf(__uint_as_float(sr[i]), p.scale2, slope2 * (float)(x.P + u.x - qpos));
+                            if (!((uint32_t)u.y & beambit)) v[i] = -INFINITY;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < KW; ++i) tmax = fmaxf(tmax, v[i]);
+                }
+                s_max[(buf * 4 + warp) * kCols + lane] = tmax;
+                ok = bar_and(1, 128, ok);                         // everybody's maxima are there, or everybody leaves
+                gone = !ok;
+                if (gone) break;
+#pragma unroll
+                for (int w = 0; w < 4; ++w) tmax = fmaxf(tmax, s_max[(buf * 4 + w) * kCols + lane]);
+                const bool need = tmax > m_ref + 8.f;
+                float alpha = 1.f;
+                if (need) {
+                    alpha = exp2f(m_ref - tmax);                  // 0 on the first keys
+                    m_ref = tmax;
+                }
+                const float m_use = m_ref == -INFINITY ? 0.f : m_ref;       // no key of this column so far
+                float ls[2] = {0.f, 0.f};
+                uint32_t hi[KW / 2], lo[KW / 2];
+#pragma unroll
+                for (int i = 0; i < KW; i += 2) {
+                    const float a = exp2f(v[i] - m_use), c = exp2f(v[i + 1] - m_use);
+                    ls[(i >> 1) & 1] += a + c;
+                    hi[i >> 1] = Mma<T>::pack(a, c);
+                    if (kTwoPart) {
+                        const uint32_t h = hi[i >> 1];
+                        lo[i >> 1] = Mma<T>::pack(a - __uint_as_float(h << 16), c - __uint_as_float(h & 0xFFFF0000u));
+                    }
+                }
+                l_run = l_run * alpha + (ls[0] + ls[1]);
+                // the weights' buffer is free once P.V of the tile before last is done
+                if (n >= 2) ok = mbar_wait_hot(bar_o + 8 * buf, ((n - 2) >> 1) & 1, p.wait_ns);
+                if (t > 0 && owns_o && __any_sync(0xffffffffu, need)) {
+                    ok = mbar_wait_hot(bar_o + 8 * (buf ^ 1), ((n - 1) >> 1) & 1, p.wait_ns) && ok;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (ok) {
+                        tc_fence_after();
+#pragma unroll 1
+                        for (int c = 0; c < D / 32; ++c) {
+                            uint32_t o[32];
+                            tc_ld32(tm_o + c * 32, o);
+                            tc_wait_ld();
+                            pin<32>(o);
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            tc_st32(tm_o + c * 32, o);
+                        }
+                        tc_wait_st();
+                    }
+                }
+                if (ok) {
+                    uint8_t* dst = p_smem + buf * L::kP + lane * 128;
+#pragma unroll
+                    for (int c = 0; c < KW / 8; ++c) {
+                        const int ch = ((warp * (KW / 8) + c) ^ (lane & 7)) << 4;
+                        *reinterpret_cast<uint4*>(dst + ch) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
+                        if (kTwoPart)
+                            *reinterpret_cast<uint4*>(dst + 32 * 128 + ch) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
+                    }
+                    fence_proxy_async();
+                    tc_fence_before();
+                    if (!(p.dbg_skip && tid == 0 && n == 0)) mbar_arrive(bar_p + 8 * buf);
+                }
+            }
+            if (gone) break;
+            // ---- the item's result: sums over the warps, O once its last P.V is done ----
+            s_sum[warp * kCols + lane] = l_run;
+            if (tiles > 0 && ok) ok = mbar_wait_hot(bar_o + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1, p.wait_ns);
+            ok = bar_and(1, 128, ok);
+            gone = !ok;
+            if (gone) break;
+            tc_fence_after();
+            float l = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) l += s_sum[w * kCols + lane];
+            const float scale = p.S == 1 ? 1.f / l : 1.f;
+            if (owns_o) {
+                float* xch = reinterpret_cast<float*>(p_smem);    // [128 of D][32 columns]: the weights have been consumed
+                constexpr int XC = D < 128 ? D : 128;
+                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(x.b * p.W + beam) * p.H + x.kvh * p.G + hg) * D;
+                float* wrow = p.ws_o + ((size_t)it * p.ncols + lane) * D;
+#pragma unroll 1
+                for (int d0 = 0; d0 < D; d0 += XC) {
+                    if (kTwoPart) {
+                        if (warp == 1) {
+#pragma unroll 1
+                            for (int c = 0; c < XC; c += 32) {
+                                uint32_t o[32];
+                                tc_ld32(tm_o + d0 + c, o);
+                                tc_wait_ld();
+                                pin<32>(o);
+#pragma unroll
+                                for (int i = 0; i < 32; ++i) xch[(c + i) * 32 + lane] = __uint_as_float(o[i]);
+                            }
+                        }
+                        bar_sync_n(4, 64);
+                    }
+                    if (warp == 0) {
+#pragma unroll 1
+                        for (int c = 0; c < XC; c += 32) {
+                            uint32_t o[32];
+                            tc_ld32(tm_o + d0 + c, o);
+                            tc_wait_ld();
+                            pin<32>(o);
+                            float f[32];
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) {
+                                f[i] = __uint_as_float(o[i]);
+                                if (kTwoPart) f[i] += xch[(c + i) * 32 + lane];
+                                f[i] = tiles > 0 ? f[i] * scale : 0.f;     // (a split without keys has no O)
+                            }
+                            if (real) {
+                                if (p.S == 1) {
+#pragma unroll
+                                    for (int i = 0; i < 32; i += 8)
+                                        *reinterpret_cast<uint4*>(orow + d0 + c + i) =
+                                            make_uint4(Mma<T>::pack(f[i], f[i + 1]), Mma<T>::pack(f[i + 2], f[i + 3]),
+                                                       Mma<T>::pack(f[i + 4], f[i + 5]), Mma<T>::pack(f[i + 6], f[i + 7]));
+                                } else {
+#pragma unroll
+                                    for (int i = 0; i < 32; i += 4)
+                                        *reinterpret_cast<float4*>(wrow + d0 + c + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+                                }
+                            }
+                        }
+                    }
+                    if (kTwoPart) bar_sync_n(4, 64);
+                }
+                if (p.S > 1 && warp == 0 && real)
+                    *reinterpret_cast<float2*>(p.ws_ml + ((size_t)it * p.ncols + lane) * 2) = make_float2(m_ref, l);
+            }
+            rn += (uint32_t)nrt;
+            if (p.S == 1) continue;
+            // ---- split merge: the last CTA of the work group to arrive folds all partials ----
+            if (warp == 0) __syncwarp();
+            if (tid == 0) {
+                // (the partials are warp 0's own stores, ordered before by the warp barrier; acq_rel publishes them)
+                int ticket;
+                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(ticket) : "l"(p.tickets + x.slab) : "memory");
+                const bool last = (ticket & (kTicketAbortedW - 1)) == p.S - 1;
+                s_ticket = last ? 1 + (ticket >= kTicketAbortedW ? 1 : 0) : 0;
+                if (last) p.tickets[x.slab] = 0;              // everybody has arrived: ready for the next launch
+            }
+            bar_sync_n(1, 128);
+            const int verdict = s_ticket;
+            bar_sync_n(1, 128);
+            if (verdict != 1) continue;                       // not the last, or a CTA of the group gave up: no merge
+            const int it0 = it - x.split;
+            const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * p.ncols * 2);
+            const float* o0 = p.ws_o + (size_t)it0 * p.ncols * D;
+            constexpr int D4 = D / 4;
+            for (int e = tid; e < p.ncols * D4; e += 128) {
+                const int col = e / D4, d = (e % D4) * 4;
+                float mm = -INFINITY, ll = 0.f;
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int s0 = 0; s0 < p.S; s0 += 4) {
+                    float2 ml[4];
+                    float4 w[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const bool in = s0 + u < p.S;
+                        ml[u] = in ? __ldcg(ml0 + (size_t)(s0 + u) * p.ncols + col) : make_float2(-INFINITY, 0.f);
+                        w[u] = in ? __ldcg(reinterpret_cast<const float4*>(o0 + ((size_t)(s0 + u) * p.ncols + col) * D + d))
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    float bm = mm;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) bm = fmaxf(bm, ml[u].x);
+                    const float fo = mm == -INFINITY ? 0.f : exp2f(mm - bm);
+                    ll *= fo; o.x *= fo; o.y *= fo; o.z *= fo; o.w *= fo;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float f = ml[u].x == -INFINITY ? 0.f : exp2f(ml[u].x - bm);
+                        ll += ml[u].y * f;
+                        o.x += w[u].x * f; o.y += w[u].y * f; o.z += w[u].z * f; o.w += w[u].w * f;
+                    }
+                    mm = bm;
+                }
+                const float inv = 1.f / ll;
+                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(x.b * p.W + col / p.G) * p.H + x.kvh * p.G + col % p.G) * D + d;
+                *reinterpret_cast<uint2*>(orow) = make_uint2(Mma<T>::pack(o.x * inv, o.y * inv), Mma<T>::pack(o.z * inv, o.w * inv));
+            }
+        }
+        if (gone) {
+            if (tid == 0) {
+                s_abort = 1;
+                // the arrival counters must still come back to zero: marked tickets for what this CTA leaves undone
+                for (; it < p.items && p.S > 1; it += gridDim.x) {
+                    int* tk = p.tickets + it / p.S;
+                    int ticket;
+                    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(ticket) : "l"(tk), "r"(kTicketAbortedW + 1) : "memory");
+                    if ((ticket & (kTicketAbortedW - 1)) == p.S - 1) *tk = 0;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 5) {
+        if (s_abort) {
+            // MMAs may still be in flight: let them finish (bounded) before the tensor memory goes back
+            if (lane == 0) {
+                tc_commit(bar_end);
+                (void)mbar_wait(bar_end, 0, p.wait_ns);
+                atomicOr(p.err_word, SEGKV_DEV_WAIT_LIMIT);
+            }
+            __syncwarp();
+        }
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(L::kTmemCols) : "memory");
+    }
+}
+
+template <typename T, int D>
+cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
+    using L = WideLayout<D>;
+    // never two CTAs on one SM: the second would wait for tensor memory inside its allocation
+    constexpr size_t smem = L::kBytes > 120 * 1024 ? L::kBytes : 120 * 1024;
+    auto kern = sdpa_wide_kernel<T, D>;
+    static bool configured[64] = {false};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !configured[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    WideParams p;
+    p.q = a.q; p.out = a.out; p.slopes = a.slopes;
+    p.kr = (const char*)a.kr; p.k_chunks = (const char* const*)a.k_chunks; p.vdelta = a.vdelta; p.chunk_steps = d.chunk_steps;
+    p.ulist = a.ulist; p.ucount = a.ucount; p.plens = a.plens;
+    p.tickets = a.tickets; p.err_word = a.err_word;
+    p.P = a.prompt_len; p.steps = a.steps; p.S = a.splits; p.W = d.beams; p.G = d.group; p.H = d.heads; p.Hkv = d.kv_heads;
+    p.rows = d.rows; p.max_steps = d.max_steps; p.ncols = d.beams * d.group;
+    p.quota = (a.steps + 2 * d.beams + a.splits - 1) / a.splits;
+    p.items = d.batch * d.kv_heads * a.splits;
+    p.ws_o = a.ws;
+    p.ws_ml = a.ws + (size_t)p.items * p.ncols * D;
+    p.early_prompt = (a.pdl && a.prompt_immutable) ? 1 : 0;
+    p.dbg_skip = a.dbg_skip ? 1 : 0;
+    p.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
+    p.scale2 = 1.4426950408889634f / sqrtf((float)D);
+    // instruction descriptors: fp32 accumulate, A/B format, N >> 3, M = 128; V is the MN-major operand
+    const uint32_t fmt = d.dtype == SEGKV_BF16 ? 1u : 0u;
+    const uint32_t common = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(128 >> 4) << 24);
+    p.idesc_qk = common | ((uint32_t)(L::KEYS >> 3) << 17);
+    p.idesc_pv = common | (1u << 16) | ((uint32_t)(D >> 3) << 17);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.items < sms ? p.items : sms), 1, 1);
+    cfg.blockDim = dim3(L::kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    if (a.pdl) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, tmk, tmv, p);
+}
+
+template <typename T>
+cudaError_t dispatch(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
+    switch (d.head_dim) {
+        case 64: return launch_one<T, 64>(d, a, tmk, tmv, sms, st);
+        case 128: return launch_one<T, 128>(d, a, tmk, tmv, sms, st);
+        case 256: return launch_one<T, 256>(d, a, tmk, tmv, sms, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+int wide_tile_keys(const Dims& d) { return d.head_dim == 256 ? WideLayout<256>::KEYS : WideLayout<128>::KEYS; }
+
+cudaError_t launch_sdpa_wide(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
+    if (a.splits < 1 || a.splits > kMaxSplits || d.beams * d.group > kCols) return cudaErrorInvalidValue;
+    return d.dtype == SEGKV_BF16 ? dispatch<__nv_bfloat16>(d, a, tmk, tmv, sms, st) : dispatch<__half>(d, a, tmk, tmv, sms, st);
+}
+
+}  // namespace segkv_impl

@@ -1,0 +1,83 @@
+"""Decode attention for work groups of many query columns (the tcgen05 kernel): beams x query heads per kv
+head beyond what the tiled kernel takes, against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2401_05391_b200 import segkv as sk
+from paper_2401_05391_b200 import workloads as wl
+
+from _harness import Run, all_pairs, sampled_pairs
+from test_gpu_parity import run_workload, run_workload_fused
+
+pytestmark = pytest.mark.gpu
+
+
+def _w(name, batch, beams, group, hkv, D, P, steps, dtype="f16", parents="uniform", alibi=False, seed=0):
+    return wl.Workload(name, batch, beams, hkv * group, hkv, D, P, steps, dtype, parents, alibi, 300 + seed)
+
+
+# prompts at the edges of a key tile (64 keys; 32 at head_dim 256), responses of none, one and several tiles,
+# column counts from the smallest to the full 32, one and several splits
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,beams,group,P,splits", [
+    (64, 4, 8, 63, 0), (64, 32, 1, 129, 3), (64, 3, 7, 1, 1),
+    (128, 4, 8, 64, 0), (128, 8, 4, 200, 3), (128, 17, 1, 65, 1), (128, 5, 5, 520, 0),
+    (256, 4, 8, 33, 0), (256, 9, 1, 31, 1), (256, 4, 4, 150, 3)])
+def test_wide_small_shapes(dtype, D, beams, group, P, splits):
+    w = _w("wide", 2, beams, group, 2, D, P, 40, dtype, alibi=group == 4, seed=D + beams)
+    run_workload(w, all_pairs, check_steps=(0, 1, 15, 39), splits=splits, every_step_ancestry=False)
+
+
+@pytest.mark.parametrize("D,dtype", [(64, "bf16"), (128, "f16"), (256, "bf16")])
+def test_wide_many_items_per_cta(D, dtype):
+    # more work groups than SMs: every CTA walks several items, with rings and phases carried across them
+    w = _w("many", 50, 4, 5, 8, D, 70, 9, dtype, alibi=True, seed=1)
+    run_workload(w, sampled_pairs, check_steps=(0, 8), every_step_ancestry=False)
+    run_workload(w, sampled_pairs, check_steps=(8,), splits=2, every_step_ancestry=False)
+
+
+@pytest.mark.parametrize("layout", [None, "token_major", "seq_first"])
+def test_wide_ragged_prompts_growing_cache_and_layouts(layout):
+    for D, dtype in ((64, "f16"), (128, "bf16"), (256, "f16")):
+        w = _w("ragged", 4, 6, 3, 2, D, 140, 21, dtype, seed=2)
+        run_workload(w, all_pairs, check_steps=(0, 16, 20), prompt_lens=[140, 1, 64, 97], chunk_steps=8,
+                     prompt_layout=layout, every_step_ancestry=False)
+
+
+def test_wide_no_prompt_fused_call_and_redone_step():
+    run_workload(_w("none", 2, 8, 4, 2, 128, 0, 30, seed=3), all_pairs, check_steps=(0, 1, 29))
+    w = _w("fused", 1, 4, 8, 2, 128, 100, 12, "bf16", seed=4)
+    run_workload_fused(w, all_pairs, check_steps=(0, 5, 11))
+    r = Run(w)
+    try:
+        r.advance_to(6)
+        for t in (6, 5):                           # the step before the dropped one is attended to again
+            q = r.q_steps[t]
+            out, _ = r.decode(q)
+            r.check(out, q, t, all_pairs(w))
+            r.h.truncate_last() if t == 6 else None
+    finally:
+        r.close()
+
+
+@pytest.mark.parametrize("splits", [1, 3])
+def test_wide_wait_runs_out_and_the_handle_recovers(splits):
+    w = _w("wait", 2, 4, 8, 2, 128, 200, 6, "bf16", seed=5)
+    r = Run(w, splits=splits)
+    try:
+        r.advance_to(3)
+        q = r.q_steps[-1]
+        out = torch.full((w.rows, w.heads, w.head_dim), float("nan"), dtype=w.torch_dtype, device="cuda")
+        r.h.debug_inject(1_000_000, True)
+        r.h.decode_sdpa(q, out)
+        torch.cuda.synchronize()
+        assert r.h.get_error() & sk.SEGKV_DEV_WAIT_LIMIT
+        assert torch.isnan(out.float()).all()
+        for _ in range(2):
+            out2, q2 = r.decode()
+            r.check(out2, q2, 3, all_pairs(w))
+        assert r.h.get_error() == 0
+        assert np.array_equal(r.h.get_ancestry(), r.oracle_ancestry(3))
+    finally:
+        r.close()
