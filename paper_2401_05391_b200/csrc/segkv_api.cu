@@ -230,6 +230,7 @@ int alloc_workspace(segkv* h, int splits) {
     const Dims& d = h->d;
     size_t cols = (size_t)d.beams * d.group;
     size_t bytes = (size_t)d.batch * d.kv_heads * splits * cols * (d.head_dim + 2) * sizeof(float);
+    if (!tiled_supported(d)) bytes *= wide_parts(d);
     if (h->ws) {
         cudaFree(h->ws);
         h->ws = nullptr;

@@ -54,13 +54,6 @@ __device__ __forceinline__ bool bar_and(int id, int threads, bool ok) {
 __device__ __forceinline__ void bar_sync_n(int id, int threads) {
     asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-// Registers written by a tcgen05.ld may be used from here on (after the wait): keeps their uses behind it.
-template <int N>
-__device__ __forceinline__ void pin(uint32_t* r) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
-}
-
 struct WideParams {
     const void* q;
     void* out;
@@ -71,8 +64,8 @@ struct WideParams {
     const URow* ulist;
     const int32_t* ucount;
     const int32_t* plens;
-    float* ws_o;                   // [item][ncols][D] un-normalised partial outputs
-    float* ws_ml;                  // [item][ncols][2] reference maximum (base-2 domain) and sum
+    float* ws_o;                   // [item][part][ncols][D] un-normalised partial outputs (bf16: high and low parts)
+    float* ws_ml;                  // [item][part][ncols][2] reference maximum (base-2 domain) and sum
     int* tickets;
     int* err_word;
     int P, steps, S, W, G, H, Hkv, rows, max_steps, ncols, chunk_steps, quota, items;
@@ -91,19 +84,23 @@ struct WideLayout {
     static constexpr int kColTile = KEYS * 128;
     static constexpr int kTile = kDBoxes * kColTile;             // bytes of a K (or a V) tile
     static constexpr int kStage = 2 * kTile;
-    static constexpr int SP = D == 64 ? 7 : (D == 128 ? 3 : 2);  // prompt stages
+    static constexpr int SP = D == 64 ? 8 : 4;                   // prompt stages
     static constexpr int SR = 2;                                 // response stages: one per gather group
-    static constexpr int kQ = kDBoxes * 128 * 128;               // the query block, four times
-    static constexpr int kP = 64 * 128;                          // one buffer of weights: 32 rows hi, 32 rows lo
+    static constexpr int kPRows = 64 * 128;                      // weights of a tile: 32 rows hi, 32 rows lo, 128 bytes each
+    // two buffers of weights: tiles of 32 keys fill half a row each, and the other half is the other buffer
+    static constexpr int kPBuf = KEYS == 32 ? 64 : kPRows;
+    static constexpr int kP = KEYS == 32 ? kPRows : 2 * kPRows;
+    static constexpr int kQ = kCols * D * 2;                     // the next query block, on its way to tensor memory
     static constexpr int kMeta = SR * KEYS * (int)sizeof(URow);
     static constexpr int kPtr = SR * KEYS * 8;
     static constexpr int kMax = 2 * 4 * kCols * 4, kSum = 4 * kCols * 4;
-    static constexpr int kBars = 2 * SP + 2 * SR + 2 + 6 + 1;    // rings, query full/empty, S/P/O x 2, wind-down
-    static constexpr size_t kBytes = 1024 + (size_t)kQ + 2 * kP + (SP + SR) * kStage + kMeta + kPtr + kMax + kSum + 8 * kBars + 64;
-    static constexpr int kColO = 2 * KEYS;                       // tensor memory: two S buffers, then O
-    static constexpr int kTmemCols = kColO + D <= 256 ? 256 : 512;
+    static constexpr int kBars = 3 * SP + 2 * SR + 3 + 6 + 1;    // rings, query, S/P/O x 2, wind-down
+    static constexpr size_t kBytes = 1024 + (size_t)kP + kQ + (SP + SR) * kStage + kMeta + kPtr + kMax + kSum + 8 * kBars + 64;
+    // tensor memory: two S buffers, O, and the query block (16-bit, two elements per column)
+    static constexpr int kColO = 2 * KEYS, kColQ = kColO + D, kColEnd = kColQ + D / 2;
+    static constexpr int kTmemCols = kColEnd <= 256 ? 256 : 512;
     static constexpr int kThreads = 320;                         // 4 softmax warps, TMA, MMA, 2 x 2 gather warps
-    static_assert(kColO + D <= kTmemCols, "tensor memory");
+    static_assert(kColEnd <= kTmemCols, "tensor memory");
     static_assert(kBytes <= 232448, "shared memory");
 };
 
@@ -113,20 +110,22 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     using L = WideLayout<D>;
     constexpr int KEYS = L::KEYS, KW = L::KW, SP = L::SP, SR = L::SR;
     constexpr bool kTwoPart = !Mma<T>::kWeights11Bits;
+    constexpr int kParts = kTwoPart ? 2 : 1;                      // partial outputs of an item in the split workspace
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* q_smem = smem;                                       // per column block [4 x 32 rows][128 bytes]
-    uint8_t* p_smem = q_smem + L::kQ;                             // two buffers; their A operands reach into the ring behind
-    uint8_t* p_ring = p_smem + 2 * L::kP;
+    uint8_t* p_smem = smem;                                       // two buffers; their A operands reach into the ring behind
+    uint8_t* p_ring = p_smem + L::kP;
     uint8_t* r_ring = p_ring + (size_t)SP * L::kStage;
-    URow* meta = reinterpret_cast<URow*>(r_ring + (size_t)SR * L::kStage);
+    uint8_t* q_smem = r_ring + (size_t)SR * L::kStage;            // [32 rows][D], 16-byte chunks XOR-swizzled by the row
+    URow* meta = reinterpret_cast<URow*>(q_smem + L::kQ);
     const char** gk = reinterpret_cast<const char**>(meta + SR * KEYS);
     float* s_max = reinterpret_cast<float*>(gk + SR * KEYS);      // [2][4 warps][kCols]
     float* s_sum = s_max + 2 * 4 * kCols;                         // [4 warps][kCols]
     uint64_t* bars = reinterpret_cast<uint64_t*>(s_sum + 4 * kCols);
-    const uint32_t pfull = smem_u32(bars), pempty = pfull + 8 * SP, rfull = pempty + 8 * SP, rempty = rfull + 8 * SR;
-    const uint32_t qfull = rempty + 8 * SR, qempty = qfull + 8;
-    const uint32_t bar_s = qempty + 8, bar_p = bar_s + 16, bar_o = bar_p + 16;     // two each: tile parity
+    const uint32_t pfull = smem_u32(bars), kempty = pfull + 8 * SP, vempty = kempty + 8 * SP;
+    const uint32_t rfull = vempty + 8 * SP, rempty = rfull + 8 * SR, qfull = rempty + 8 * SR;
+    const uint32_t sfull = qfull + 8, sempty = sfull + 8;         // the query block in shared memory
+    const uint32_t bar_s = sempty + 8, bar_p = bar_s + 16, bar_o = bar_p + 16;     // two each: tile parity
     const uint32_t bar_end = bar_o + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
     __shared__ int s_abort, s_ticket;
@@ -147,59 +146,59 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         x.npt = (int)((long long)(x.split + 1) * ntp / p.S) - x.pt0;
         return x;
     };
-    auto rows_of = [&](const Item& x, int& e0, int& e1) {
-        const int n_b = p.steps > 0 ? p.ucount[x.b] : 0;
+    // the distinct rows of an item's request; asked for one item ahead
+    auto count_of = [&](int it) { return p.steps > 0 && it < p.items ? p.ucount[it / p.S / p.Hkv] : 0; };
+    auto rows_of = [&](const Item& x, int n_b, int& e0, int& e1) {
         e0 = min(x.split * p.quota, n_b);
         e1 = x.split == p.S - 1 ? n_b : min((x.split + 1) * p.quota, n_b);
     };
-    auto issue_prompt = [&](const Item& x, int k, uint32_t pos) {
-        const uint32_t st = pos % SP, full = pfull + 8 * st;
-        const uint32_t k_dst = smem_u32(p_ring) + st * (uint32_t)L::kStage, v_dst = k_dst + L::kTile;
-        mbar_arrive_expect_tx(full, (uint32_t)L::kStage);
-        const int y = (x.pt0 + k) * KEYS;
+    // the K (or V) part of the item's prompt tile k
+    auto issue_part = [&](const CUtensorMap* tm, const Item& x, int k, uint32_t dst, uint32_t full) {
+        mbar_arrive_expect_tx(full, (uint32_t)L::kTile);
 #pragma unroll
-        for (int bx = 0; bx < L::kDBoxes; ++bx) tma_load_4d(k_dst + bx * L::kColTile, &tm_k, bx * 64, x.kvh, y, x.b, full);
-#pragma unroll
-        for (int bx = 0; bx < L::kDBoxes; ++bx) tma_load_4d(v_dst + bx * L::kColTile, &tm_v, bx * 64, x.kvh, y, x.b, full);
+        for (int bx = 0; bx < L::kDBoxes; ++bx) tma_load_4d(dst + bx * L::kColTile, tm, bx * 64, x.kvh, (x.pt0 + k) * KEYS, x.b, full);
     };
+    const uint32_t p_ring_u = smem_u32(p_ring), r_ring_u = smem_u32(r_ring);
 
-    // Set-up by the TMA warp, which then starts the first prompt tiles before the CTA has synchronised (and,
-    // when nothing can still be writing the prompt, before the previous kernel has finished).
-    int first = 0;                       // prompt tiles of the CTA's first item already requested
-    if (warp == 4 && lane == 0) {
-        for (int s = 0; s < SP; ++s) {
-            mbar_init(pfull + 8 * s, 1);
-            mbar_init(pempty + 8 * s, 1);
+    // Set-up by the TMA warp, which then goes straight to its prompt tiles (when nothing can still be writing the
+    // prompt, before the previous kernel has finished).
+    if (warp == 4) {
+        if (lane == 0) {
+            for (int s = 0; s < SP; ++s) {
+                mbar_init(pfull + 8 * s, 2);                      // the K part and the V part
+                mbar_init(kempty + 8 * s, 1);
+                mbar_init(vempty + 8 * s, 1);
+            }
+            for (int s = 0; s < SR; ++s) {
+                mbar_init(rfull + 8 * s, 1);
+                mbar_init(rempty + 8 * s, 1);
+            }
+            mbar_init(qfull, 128);
+            mbar_init(sfull, 128);
+            mbar_init(sempty, 128);
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(bar_s + 8 * i, 1);
+                mbar_init(bar_p + 8 * i, 128);
+                mbar_init(bar_o + 8 * i, 1);
+            }
+            mbar_init(bar_end, 1);
+            s_abort = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_proxy_async();
         }
-        for (int s = 0; s < SR; ++s) {
-            mbar_init(rfull + 8 * s, 1);
-            mbar_init(rempty + 8 * s, 1);
+        __syncwarp();
+        asm volatile("barrier.cta.arrive 5, %0;" ::"n"(L::kThreads) : "memory");    // the others go on; this warp needs nothing of theirs
+    } else {
+        if (warp == 5) {                 // this warp owns the tensor memory
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                         ::"r"(smem_u32(tmem_slot)), "n"(L::kTmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
-        mbar_init(qfull, 2);
-        mbar_init(qempty, 1);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(bar_s + 8 * i, 1);
-            mbar_init(bar_p + 8 * i, 128);
-            mbar_init(bar_o + 8 * i, 1);
-        }
-        mbar_init(bar_end, 1);
-        s_abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_proxy_async();
-        if (!p.early_prompt) asm volatile("griddepcontrol.wait;" ::: "memory");
-        const Item x = item_of((int)blockIdx.x);
-        first = min(x.npt, SP);
-        for (int k = 0; k < first; ++k) issue_prompt(x, k, (uint32_t)k);
+        tc_fence_before();
+        bar_sync_n(5, L::kThreads);
+        tc_fence_after();
     }
-    if (warp == 5) {                     // this warp owns the tensor memory
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(tmem_slot)), "n"(L::kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp == 4 ? 0u : *tmem_slot;
     if (warp != 4) {
         // everything but the prompt tiles follows the previous kernel; its successors are let go only after that
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -211,85 +210,91 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         if (lane == 0) {
             uint32_t pos = 0;
             bool ok = true;
+            if (!p.early_prompt) asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
                 const Item x = item_of(it);
-                int k = 0;
-                if (it == (int)blockIdx.x) pos = (uint32_t)(k = first);
-                for (; k < x.npt; ++k, ++pos) {
-                    ok = mbar_wait(pempty + 8 * (pos % SP), ((pos / SP) & 1) ^ 1, p.wait_ns);
+                for (int k = 0; k < x.npt; ++k, ++pos) {
+                    const uint32_t st = pos % SP, ph = ((pos / SP) & 1) ^ 1, dst = p_ring_u + st * (uint32_t)L::kStage;
+                    ok = mbar_wait(kempty + 8 * st, ph, p.wait_ns);
                     if (!ok) break;
-                    issue_prompt(x, k, pos);
+                    issue_part(&tm_k, x, k, dst, pfull + 8 * st);
+                    ok = mbar_wait(vempty + 8 * st, ph, p.wait_ns);
+                    if (!ok) break;
+                    issue_part(&tm_v, x, k, dst + L::kTile, pfull + 8 * st);
                 }
             }
             if (!ok) {
                 s_abort = 1;
-                for (uint32_t k = pos > (uint32_t)SP ? pos - SP : 0; k < pos; ++k)       // copies in flight land first
+                // copies in flight land first (or the limit runs out: a K part may have been asked for without its V part)
+                for (uint32_t k = pos > (uint32_t)SP ? pos - SP : 0; k <= pos; ++k)
                     (void)mbar_wait(pfull + 8 * (k % SP), (k / SP) & 1, p.wait_ns);
             }
         }
     } else if (warp == 5) {
         // -------------------------------- MMA issuer --------------------------------
-        if (lane == 0) {
-            uint32_t n = 0, pos = 0, rn = 0, qi = 0;              // tiles, prompt tiles, response tiles, items so far
-            const uint64_t q_desc = smem_desc(smem_u32(q_smem), 16, 1024);
-            const uint64_t p_desc = smem_desc(smem_u32(p_smem), 16, 1024);
-            bool ok = true;
-            for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
-                const Item x = item_of(it);
-                int e0, e1;
-                rows_of(x, e0, e1);
-                const int tiles = x.npt + (e1 - e0 + KEYS - 1) / KEYS;
-                if (tiles == 0) continue;
-                auto stage_addr = [&](int t) -> uint32_t {        // prompt tiles first, then response tiles
-                    return t < x.npt ? smem_u32(p_ring) + ((pos + t) % SP) * (uint32_t)L::kStage
-                                     : smem_u32(r_ring) + ((rn + t - x.npt) % SR) * (uint32_t)L::kStage;
-                };
-                auto wait_tile = [&](int t) -> bool {
-                    bool r;
-                    if (t < x.npt) r = mbar_wait_hot(pfull + 8 * ((pos + t) % SP), ((pos + t) / SP) & 1, p.wait_ns);
-                    else r = mbar_wait_hot(rfull + 8 * ((rn + t - x.npt) % SR), ((rn + t - x.npt) / SR) & 1, p.wait_ns);
-                    tc_fence_after();
-                    return r;
-                };
-                auto issue_qk = [&](int t) {
-                    const uint32_t buf = (n + (uint32_t)t) & 1;
-                    const uint64_t kd = smem_desc(stage_addr(t), 16, 1024);
+        // (the whole warp runs this, converged: see tc_mma_ss_if.  What decides the control flow is made uniform by
+        // a warp reduction or vote.)
+        const uint32_t lead = elect_one();
+        const uint32_t p_lo = (smem_u32(p_smem) & 0x3FFFFu) >> 4, ring_lo = (p_ring_u & 0x3FFFFu) >> 4, resp_lo = (r_ring_u & 0x3FFFFu) >> 4;
+        const uint64_t dk = smem_desc(0, 16, 1024), dv = smem_desc(0, L::kColTile, 1024);     // descriptors without an address
+        uint32_t n = 0, qi = 0, ps = 0, pph = 0, rs = 0, rph = 0;   // tiles, items; prompt / response stage and phase of the next tile
+        bool ok = true;
+        auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+            return __all_sync(0xffffffffu, mbar_wait_hot(bar, parity, p.wait_ns));
+        };
+        int n_next = count_of((int)blockIdx.x);
+        for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
+            const Item x = item_of(it);
+            int e0, e1;
+            rows_of(x, n_next, e0, e1);
+            n_next = count_of(it + (int)gridDim.x);
+            const int npt = (int)__reduce_max_sync(0xffffffffu, (unsigned)x.npt);
+            const int tiles = npt + (int)__reduce_max_sync(0xffffffffu, (unsigned)((e1 - e0 + KEYS - 1) / KEYS));
+            if (tiles == 0) continue;
+            uint32_t v_lo = 0, v_empty = 0;                       // the V part of the tile whose scores were issued last
+            auto issue_qk = [&](int t, uint32_t buf) -> bool {
+                const bool prompt = t < npt;
+                const uint32_t lo = prompt ? ring_lo + ps * (uint32_t)(L::kStage >> 4) : resp_lo + rs * (uint32_t)(L::kStage >> 4);
+                const uint32_t full = prompt ? pfull + 8 * ps : rfull + 8 * rs, par = prompt ? pph : rph;
+                v_lo = lo + (uint32_t)(L::kTile >> 4);
+                v_empty = prompt ? vempty + 8 * ps : rempty + 8 * rs;
+                if (!wait(full, par)) return false;
+                tc_fence_after();
+                const uint64_t kd = dk + lo;
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks)
-                        tc_mma_ss(tmem + buf * KEYS, q_desc + (uint64_t)(((ks >> 2) * (128 * 128) + (ks & 3) * 32) >> 4),
-                                  kd + (uint64_t)(((ks >> 2) * L::kColTile + (ks & 3) * 32) >> 4), p.idesc_qk, ks > 0);
-                    tc_commit(bar_s + 8 * buf);
-                    if (t == tiles - 1) tc_commit(qempty);        // the query block may be replaced
-                };
-                ok = mbar_wait_hot(qfull, qi++ & 1, p.wait_ns) && wait_tile(0);
-                if (!ok) break;
-                issue_qk(0);
-                for (int t = 0; t < tiles; ++t) {
-                    if (t + 1 < tiles) {                          // the next scores run under this tile's softmax
-                        ok = wait_tile(t + 1);
-                        if (!ok) break;
-                        issue_qk(t + 1);
-                    }
-                    const uint32_t m = n + (uint32_t)t, buf = m & 1;
-                    ok = mbar_wait_hot(bar_p + 8 * buf, (m >> 1) & 1, p.wait_ns);
+                for (int ks = 0; ks < D / 16; ++ks)
+                    tc_mma_ts_if(lead, tmem + buf * KEYS, tmem + L::kColQ + ks * 8,
+                                 kd + (uint64_t)(((ks >> 2) * L::kColTile + (ks & 3) * 32) >> 4), p.idesc_qk, ks > 0);
+                tc_commit_if(lead, bar_s + 8 * buf);
+                if (prompt) {
+                    tc_commit_if(lead, kempty + 8 * ps);
+                    if (++ps == SP) { ps = 0; pph ^= 1u; }
+                } else if (++rs == SR) { rs = 0; rph ^= 1u; }
+                return true;
+            };
+            ok = wait(qfull, qi & 1);
+            ++qi;
+            if (ok) ok = issue_qk(0, n & 1);
+            if (!ok) break;
+            for (int t = 0; t < tiles; ++t, ++n) {
+                const uint32_t buf = n & 1, lo = v_lo, empty = v_empty;
+                if (t + 1 < tiles) {                              // the next scores run under this tile's softmax
+                    ok = issue_qk(t + 1, buf ^ 1);
                     if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t pd = p_desc + (uint64_t)((buf * (uint32_t)L::kP) >> 4);
-                    const uint64_t vd = smem_desc(stage_addr(t) + L::kTile, L::kColTile, 1024);
-#pragma unroll
-                    for (int kk = 0; kk < KEYS / 16; ++kk)        // O += P[:, 16 keys] . V[16 keys, :]
-                        tc_mma_ss(tmem + L::kColO, pd + (uint64_t)((kk * 32) >> 4), vd + (uint64_t)((kk * 2048) >> 4),
-                                  p.idesc_pv, t > 0 || kk > 0);
-                    tc_commit(bar_o + 8 * buf);
-                    tc_commit(t < x.npt ? pempty + 8 * ((pos + t) % SP) : rempty + 8 * ((rn + t - x.npt) % SR));
                 }
+                ok = wait(bar_p + 8 * buf, (n >> 1) & 1);
                 if (!ok) break;
-                n += (uint32_t)tiles;
-                pos += (uint32_t)x.npt;
-                rn += (uint32_t)(tiles - x.npt);
+                tc_fence_after();
+                const uint64_t pd = dk + (p_lo + buf * (uint32_t)(L::kPBuf >> 4)), vd = dv + lo;
+#pragma unroll
+                for (int kk = 0; kk < KEYS / 16; ++kk)            // O += P[:, 16 keys] . V[16 keys, :]
+                    tc_mma_ss_if(lead, tmem + L::kColO, pd + (uint64_t)((kk * 32) >> 4), vd + (uint64_t)((kk * 2048) >> 4),
+                                 p.idesc_pv, t > 0 || kk > 0);
+                tc_commit_if(lead, bar_o + 8 * buf);
+                tc_commit_if(lead, empty);
             }
-            if (!ok) s_abort = 1;
         }
+        if (!ok && lane == 0) s_abort = 1;
     } else if (warp >= 6) {
         // ------------------- the query block, and response tiles: index select fused into the load -------------------
         const int grp = (warp - 6) >> 1, gt = tid - 192 - grp * 64, bid = 2 + grp;
@@ -303,34 +308,31 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         bool ok = true;
         for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
             const Item x = item_of(it);
-            int e0, e1;
-            rows_of(x, e0, e1);
-            const int nrt = (e1 - e0 + KEYS - 1) / KEYS;
-            if (x.npt + nrt == 0) continue;
-            // the group's half of the query rows, into all four copies; rows past the last column are zeros
-            uint4 v[16 / RPI];
+            const int n_b = count_of(it);
+            // this thread's share of the query block: whole rows side by side; rows past the last column are zeros
+            constexpr int QI = kCols * CPR / 128;
+            uint4 w[QI];
 #pragma unroll
-            for (int i = 0; i < 16 / RPI; ++i) {
-                const int col = grp * 16 + i * RPI + gt / CPR, c = gt % CPR;
-                v[i] = make_uint4(0u, 0u, 0u, 0u);
+            for (int i = 0; i < QI; ++i) {
+                const int col = (i * 128 + tid - 192) / CPR, c = (tid - 192) % CPR;
+                w[i] = make_uint4(0u, 0u, 0u, 0u);
                 if (col < p.ncols)
-                    v[i] = *reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p.q) +
+                    w[i] = *reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p.q) +
                                ((size_t)(x.b * p.W + col / p.G) * p.H + x.kvh * p.G + col % p.G) * D + c * 8);
             }
-            ok = mbar_wait(qempty, (qi & 1) ^ 1, p.wait_ns);
+            ok = mbar_wait(sempty, (qi & 1) ^ 1, p.wait_ns);
             ok = bar_and(bid, 64, ok);
             if (!ok) break;
             ++qi;
 #pragma unroll
-            for (int i = 0; i < 16 / RPI; ++i) {
-                const int col = grp * 16 + i * RPI + gt / CPR, c = gt % CPR;
-                uint8_t* dst = q_smem + (size_t)(c >> 3) * (128 * 128) + col * 128 + (((c & 7) ^ (col & 7)) << 4);
-#pragma unroll
-                for (int rep = 0; rep < 4; ++rep) *reinterpret_cast<uint4*>(dst + rep * 32 * 128) = v[i];
+            for (int i = 0; i < QI; ++i) {
+                const int col = (i * 128 + tid - 192) / CPR, c = (tid - 192) % CPR;
+                *reinterpret_cast<uint4*>(q_smem + (size_t)col * (D * 2) + ((c ^ (col & 7)) << 4)) = w[i];
             }
-            fence_proxy_async();
-            bar_sync_n(bid, 64);
-            if (gt == 0) mbar_arrive(qfull);
+            mbar_arrive(sfull);
+            int e0, e1;
+            rows_of(x, n_b, e0, e1);
+            const int nrt = (e1 - e0 + KEYS - 1) / KEYS;
             const URow* list = p.ulist + (size_t)x.b * p.W * p.max_steps;
             for (int r = 0; r < nrt; ++r) {
                 const uint32_t pos = rn + (uint32_t)r;
@@ -381,14 +383,44 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         const bool real = lane < p.ncols;
         const int beam = real ? lane / p.G : 0, hg = real ? lane % p.G : 0;
         const uint32_t beambit = real ? 1u << beam : 0u;
-        uint32_t n = 0, rn = 0;                                   // tiles and response tiles so far
-        bool ok = true, gone = false;                             // a wait of this thread ran out; the four warps have agreed to leave
-        int it = blockIdx.x;
-        for (; it < p.items; it += gridDim.x) {
-            const Item x = item_of(it);
+        uint32_t n = 0, rn = 0, qi = 0;                           // tiles, response tiles and items so far
+        // The next item's query block, from shared memory into this warp's lanes of tensor memory (one column's row per
+        // lane).  An item without any tile (a split beyond a request's keys) uses none.
+        auto place_query = [&](bool used) -> bool {
+            bool got = mbar_wait_hot(sfull, qi & 1, p.wait_ns);
+            got = __all_sync(0xffffffffu, got);
+            if (!got) return false;
+            ++qi;
+            if (used) {
+#pragma unroll 1
+                for (int c0 = 0; c0 < D / 8; c0 += 8) {           // 8 chunks of 16 bytes (32 columns) at a time
+                    uint4 w[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        w[i] = *reinterpret_cast<const uint4*>(q_smem + (size_t)lane * (D * 2) + (((c0 + i) ^ (lane & 7)) << 4));
+                    tc_st32(tm_lane + L::kColQ + c0 * 4, reinterpret_cast<const uint32_t*>(w));
+                }
+                tc_wait_st();
+                tc_fence_before();
+                mbar_arrive(qfull);
+            }
+            mbar_arrive(sempty);
+            return true;
+        };
+        auto share_of = [&](int i, int n_b, Item& x) {            // item i and its response tiles
+            x = item_of(i);
             int e0, e1;
-            rows_of(x, e0, e1);
-            const int nrt = (e1 - e0 + KEYS - 1) / KEYS, tiles = x.npt + nrt;
+            rows_of(x, n_b, e0, e1);
+            return (e1 - e0 + KEYS - 1) / KEYS;
+        };
+        bool gone = false;                                        // the four warps have agreed to leave: a wait ran out
+        int it = blockIdx.x;
+        Item x;
+        int nrt = share_of(it, count_of(it), x);
+        bool ok = place_query(x.npt + nrt > 0);
+        while (it < p.items) {
+            const int tiles = x.npt + nrt, it_next = it + (int)gridDim.x;
+            const int n_next = count_of(it_next);
             const float slope2 = (p.slopes && real) ? p.slopes[x.kvh * p.G + hg] * 1.4426950408889634f : 0.f;
             const int qpos = x.P + (p.steps > 0 ? p.steps - 1 : -1);
             float m_ref = -INFINITY, l_run = 0.f;
@@ -425,39 +457,50 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                             if (!((uint32_t)u.y & beambit)) v[i] = -INFINITY;
                         }
                     }
+                    float tm[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-                    for (int i = 0; i < KW; ++i) tmax = fmaxf(tmax, v[i]);
+                    for (int i = 4; i < KW; ++i) tm[i & 3] = fmaxf(tm[i & 3], v[i]);
+                    tmax = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3]));
                 }
-                s_max[(buf * 4 + warp) * kCols + lane] = tmax;
-                ok = bar_and(1, 128, ok);                         // everybody's maxima are there, or everybody leaves
-                gone = !ok;
-                if (gone) break;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) tmax = fmaxf(tmax, s_max[(buf * 4 + w) * kCols + lane]);
-                const bool need = tmax > m_ref + 8.f;
-                float alpha = 1.f;
-                if (need) {
-                    alpha = exp2f(m_ref - tmax);                  // 0 on the first keys
-                    m_ref = tmax;
-                }
-                const float m_use = m_ref == -INFINITY ? 0.f : m_ref;       // no key of this column so far
-                float ls[2] = {0.f, 0.f};
+                // The reference in use nearly always stands, so the weights are worked out with it before the warps
+                // meet; that one of them needs a new one is found at the meeting.
+                float ls[2];
                 uint32_t hi[KW / 2], lo[KW / 2];
+                auto weigh = [&]() {
+                    const float m_use = m_ref == -INFINITY ? 0.f : m_ref;       // no key of this column so far
+                    ls[0] = ls[1] = 0.f;
 #pragma unroll
-                for (int i = 0; i < KW; i += 2) {
-                    const float a = exp2f(v[i] - m_use), c = exp2f(v[i + 1] - m_use);
-                    ls[(i >> 1) & 1] += a + c;
-                    hi[i >> 1] = Mma<T>::pack(a, c);
-                    if (kTwoPart) {
-                        const uint32_t h = hi[i >> 1];
-                        lo[i >> 1] = Mma<T>::pack(a - __uint_as_float(h << 16), c - __uint_as_float(h & 0xFFFF0000u));
+                    for (int i = 0; i < KW; i += 2) {
+                        const float a = exp2f(v[i] - m_use), c = exp2f(v[i + 1] - m_use);
+                        ls[(i >> 1) & 1] += a + c;
+                        hi[i >> 1] = Mma<T>::pack(a, c);
+                        if (kTwoPart) {
+                            const uint32_t h = hi[i >> 1];
+                            lo[i >> 1] = Mma<T>::pack(a - __uint_as_float(h << 16), c - __uint_as_float(h & 0xFFFF0000u));
+                        }
                     }
+                };
+                if (ok) weigh();
+                bool need = tmax > m_ref + 8.f;
+                float alpha = 1.f;
+                if (!bar_and(1, 128, ok && !need)) {
+                    s_max[(buf * 4 + warp) * kCols + lane] = tmax;
+                    ok = bar_and(1, 128, ok);                     // everybody's maxima are there, or everybody leaves
+                    gone = !ok;
+                    if (gone) break;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) tmax = fmaxf(tmax, s_max[(buf * 4 + w) * kCols + lane]);
+                    need = tmax > m_ref + 8.f;
+                    if (need) {
+                        alpha = exp2f(m_ref - tmax);              // 0 on the first keys
+                        m_ref = tmax;
+                    }
+                    weigh();
                 }
                 l_run = l_run * alpha + (ls[0] + ls[1]);
-                // the weights' buffer is free once P.V of the tile before last is done
-                if (n >= 2) ok = mbar_wait_hot(bar_o + 8 * buf, ((n - 2) >> 1) & 1, p.wait_ns);
+                // (The buffer the weights go to is free: these scores were issued behind P.V of the tile before last.)
                 if (t > 0 && owns_o && __any_sync(0xffffffffu, need)) {
-                    ok = mbar_wait_hot(bar_o + 8 * (buf ^ 1), ((n - 1) >> 1) & 1, p.wait_ns) && ok;
+                    ok = mbar_wait_hot(bar_o + 8 * (buf ^ 1), ((n - 1) >> 1) & 1, p.wait_ns);
                     ok = __all_sync(0xffffffffu, ok);
                     if (ok) {
                         tc_fence_after();
@@ -475,10 +518,10 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                     }
                 }
                 if (ok) {
-                    uint8_t* dst = p_smem + buf * L::kP + lane * 128;
+                    uint8_t* dst = p_smem + (KEYS == 32 ? 0 : buf * L::kPBuf) + lane * 128;
 #pragma unroll
                     for (int c = 0; c < KW / 8; ++c) {
-                        const int ch = ((warp * (KW / 8) + c) ^ (lane & 7)) << 4;
+                        const int ch = (((KEYS == 32 ? 4 * (int)buf : 0) + warp * (KW / 8) + c) ^ (lane & 7)) << 4;
                         *reinterpret_cast<uint4*>(dst + ch) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
                         if (kTwoPart)
                             *reinterpret_cast<uint4*>(dst + 32 * 128 + ch) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
@@ -489,6 +532,14 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 }
             }
             if (gone) break;
+            // the next item's query, whose first scores then run under this item's epilogue (this item's scores are all done)
+            ok = __all_sync(0xffffffffu, ok);
+            const Item done = x;
+            const int done_nrt = nrt;
+            if (it_next < p.items) {
+                nrt = share_of(it_next, n_next, x);
+                if (ok) ok = place_query(x.npt + nrt > 0);
+            }
             // ---- the item's result: sums over the warps, O once its last P.V is done ----
             s_sum[warp * kCols + lane] = l_run;
             if (tiles > 0 && ok) ok = mbar_wait_hot(bar_o + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1, p.wait_ns);
@@ -499,28 +550,46 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             float l = 0.f;
 #pragma unroll
             for (int w = 0; w < 4; ++w) l += s_sum[w * kCols + lane];
-            const float scale = p.S == 1 ? 1.f / l : 1.f;
-            if (owns_o) {
-                float* xch = reinterpret_cast<float*>(p_smem);    // [128 of D][32 columns]: the weights have been consumed
-                constexpr int XC = D < 128 ? D : 128;
-                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(x.b * p.W + beam) * p.H + x.kvh * p.G + hg) * D;
-                float* wrow = p.ws_o + ((size_t)it * p.ncols + lane) * D;
+            rn += (uint32_t)done_nrt;
+            if (p.S > 1) {
+                // a split's partial: one row per lane; the low parts are a partial of their own, with no weight in the sum
+                if (owns_o) {
+                    const size_t part = (size_t)it * kParts + warp;
+                    if (real) *reinterpret_cast<float2*>(p.ws_ml + (part * p.ncols + lane) * 2) = make_float2(m_ref, warp == 0 ? l : 0.f);
+                    float* wrow = p.ws_o + (part * p.ncols + lane) * D;
+#pragma unroll 1
+                    for (int d0 = 0; d0 < D; d0 += 32) {
+                        uint32_t o[32];
+                        tc_ld32(tm_o + d0, o);
+                        tc_wait_ld();
+                        pin<32>(o);
+                        if (real) {
+#pragma unroll
+                            for (int i = 0; i < 32; i += 4)       // (a split without keys has no O)
+                                *reinterpret_cast<uint4*>(wrow + d0 + i) = tiles > 0 ? make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]) : make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                }
+            } else if (owns_o) {
+                // the output rows; low parts come over through shared memory, where the weights have been consumed
+                constexpr int XC = KEYS == 32 ? 64 : (D < 128 ? D : 128);
+                float* xch = reinterpret_cast<float*>(p_smem);    // [XC of D][32 columns]
+                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + beam) * p.H + done.kvh * p.G + hg) * D;
+                const float inv = 1.f / l;
 #pragma unroll 1
                 for (int d0 = 0; d0 < D; d0 += XC) {
-                    if (kTwoPart) {
-                        if (warp == 1) {
+                    if (kTwoPart && warp == 1) {
 #pragma unroll 1
-                            for (int c = 0; c < XC; c += 32) {
-                                uint32_t o[32];
-                                tc_ld32(tm_o + d0 + c, o);
-                                tc_wait_ld();
-                                pin<32>(o);
+                        for (int c = 0; c < XC; c += 32) {
+                            uint32_t o[32];
+                            tc_ld32(tm_o + d0 + c, o);
+                            tc_wait_ld();
+                            pin<32>(o);
 #pragma unroll
-                                for (int i = 0; i < 32; ++i) xch[(c + i) * 32 + lane] = __uint_as_float(o[i]);
-                            }
+                            for (int i = 0; i < 32; ++i) xch[(c + i) * 32 + lane] = __uint_as_float(o[i]);
                         }
-                        bar_sync_n(4, 64);
                     }
+                    if (kTwoPart) bar_sync_n(4, 64);
                     if (warp == 0) {
 #pragma unroll 1
                         for (int c = 0; c < XC; c += 32) {
@@ -530,72 +599,62 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                             pin<32>(o);
                             float f[32];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                f[i] = __uint_as_float(o[i]);
-                                if (kTwoPart) f[i] += xch[(c + i) * 32 + lane];
-                                f[i] = tiles > 0 ? f[i] * scale : 0.f;     // (a split without keys has no O)
-                            }
+                            for (int i = 0; i < 32; ++i) f[i] = (__uint_as_float(o[i]) + (kTwoPart ? xch[(c + i) * 32 + lane] : 0.f)) * inv;
                             if (real) {
-                                if (p.S == 1) {
 #pragma unroll
-                                    for (int i = 0; i < 32; i += 8)
-                                        *reinterpret_cast<uint4*>(orow + d0 + c + i) =
-                                            make_uint4(Mma<T>::pack(f[i], f[i + 1]), Mma<T>::pack(f[i + 2], f[i + 3]),
-                                                       Mma<T>::pack(f[i + 4], f[i + 5]), Mma<T>::pack(f[i + 6], f[i + 7]));
-                                } else {
-#pragma unroll
-                                    for (int i = 0; i < 32; i += 4)
-                                        *reinterpret_cast<float4*>(wrow + d0 + c + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
-                                }
+                                for (int i = 0; i < 32; i += 8)
+                                    *reinterpret_cast<uint4*>(orow + d0 + c + i) =
+                                        make_uint4(Mma<T>::pack(f[i], f[i + 1]), Mma<T>::pack(f[i + 2], f[i + 3]),
+                                                   Mma<T>::pack(f[i + 4], f[i + 5]), Mma<T>::pack(f[i + 6], f[i + 7]));
                             }
                         }
                     }
                     if (kTwoPart) bar_sync_n(4, 64);
                 }
-                if (p.S > 1 && warp == 0 && real)
-                    *reinterpret_cast<float2*>(p.ws_ml + ((size_t)it * p.ncols + lane) * 2) = make_float2(m_ref, l);
             }
-            rn += (uint32_t)nrt;
+            const int it_done = it;
+            it = it_next;
             if (p.S == 1) continue;
             // ---- split merge: the last CTA of the work group to arrive folds all partials ----
-            if (warp == 0) __syncwarp();
+            bar_sync_n(1, 128);
             if (tid == 0) {
-                // (the partials are warp 0's own stores, ordered before by the warp barrier; acq_rel publishes them)
+                // (the partials are ordered before by the barrier; acq_rel publishes them)
                 int ticket;
-                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(ticket) : "l"(p.tickets + x.slab) : "memory");
+                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(ticket) : "l"(p.tickets + done.slab) : "memory");
                 const bool last = (ticket & (kTicketAbortedW - 1)) == p.S - 1;
                 s_ticket = last ? 1 + (ticket >= kTicketAbortedW ? 1 : 0) : 0;
-                if (last) p.tickets[x.slab] = 0;              // everybody has arrived: ready for the next launch
+                if (last) p.tickets[done.slab] = 0;              // everybody has arrived: ready for the next launch
             }
             bar_sync_n(1, 128);
             const int verdict = s_ticket;
             bar_sync_n(1, 128);
             if (verdict != 1) continue;                       // not the last, or a CTA of the group gave up: no merge
-            const int it0 = it - x.split;
-            const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * p.ncols * 2);
-            const float* o0 = p.ws_o + (size_t)it0 * p.ncols * D;
+            const int it0 = it_done - done.split;
+            const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * kParts * p.ncols * 2);
+            const float* o0 = p.ws_o + (size_t)it0 * kParts * p.ncols * D;
+            const int parts = p.S * kParts;
             constexpr int D4 = D / 4;
             for (int e = tid; e < p.ncols * D4; e += 128) {
                 const int col = e / D4, d = (e % D4) * 4;
                 float mm = -INFINITY, ll = 0.f;
                 float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int s0 = 0; s0 < p.S; s0 += 4) {
-                    float2 ml[4];
-                    float4 w[4];
+                for (int s0 = 0; s0 < parts; s0 += 8) {
+                    float2 ml[8];
+                    float4 w[8];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const bool in = s0 + u < p.S;
+                    for (int u = 0; u < 8; ++u) {
+                        const bool in = s0 + u < parts;
                         ml[u] = in ? __ldcg(ml0 + (size_t)(s0 + u) * p.ncols + col) : make_float2(-INFINITY, 0.f);
                         w[u] = in ? __ldcg(reinterpret_cast<const float4*>(o0 + ((size_t)(s0 + u) * p.ncols + col) * D + d))
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
                     float bm = mm;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) bm = fmaxf(bm, ml[u].x);
+                    for (int u = 0; u < 8; ++u) bm = fmaxf(bm, ml[u].x);
                     const float fo = mm == -INFINITY ? 0.f : exp2f(mm - bm);
                     ll *= fo; o.x *= fo; o.y *= fo; o.z *= fo; o.w *= fo;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
+                    for (int u = 0; u < 8; ++u) {
                         const float f = ml[u].x == -INFINITY ? 0.f : exp2f(ml[u].x - bm);
                         ll += ml[u].y * f;
                         o.x += w[u].x * f; o.y += w[u].y * f; o.z += w[u].z * f; o.w += w[u].w * f;
@@ -603,7 +662,7 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                     mm = bm;
                 }
                 const float inv = 1.f / ll;
-                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(x.b * p.W + col / p.G) * p.H + x.kvh * p.G + col % p.G) * D + d;
+                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + col / p.G) * p.H + done.kvh * p.G + col % p.G) * D + d;
                 *reinterpret_cast<uint2*>(orow) = make_uint2(Mma<T>::pack(o.x * inv, o.y * inv), Mma<T>::pack(o.z * inv, o.w * inv));
             }
         }
@@ -661,7 +720,7 @@ cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk,
     p.quota = (a.steps + 2 * d.beams + a.splits - 1) / a.splits;
     p.items = d.batch * d.kv_heads * a.splits;
     p.ws_o = a.ws;
-    p.ws_ml = a.ws + (size_t)p.items * p.ncols * D;
+    p.ws_ml = a.ws + (size_t)p.items * wide_parts(d) * p.ncols * D;
     p.early_prompt = (a.pdl && a.prompt_immutable) ? 1 : 0;
     p.dbg_skip = a.dbg_skip ? 1 : 0;
     p.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
@@ -697,6 +756,8 @@ cudaError_t dispatch(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, c
 }
 
 }  // namespace
+
+int wide_parts(const Dims& d) { return d.dtype == SEGKV_BF16 ? 2 : 1; }
 
 int wide_tile_keys(const Dims& d) { return d.head_dim == 256 ? WideLayout<256>::KEYS : WideLayout<128>::KEYS; }
 
