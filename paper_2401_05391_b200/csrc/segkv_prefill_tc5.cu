@@ -5,25 +5,33 @@
 //
 //   * one persistent CTA per SM walks a static list of work items (one or two groups of 128
 //     query rows of one (request, head)), longest first; a group's rows are one per TMEM lane and
-//     per softmax thread;
+//     per TWO softmax threads, which take one half of a tile's keys each;
 //   * Q of each group arrives by TMA (a per-call tensor map over [B, N, H, D]) in the
 //     128-byte-swizzled K-major layout; K and V tiles (128 keys; 64 at head_dim 256) arrive by TMA
 //     in the same layout through separate rings: a K tile is needed one step before the V tile
 //     of the same keys.  They come from the prompt segment, or (fused prefill) from the caller's
 //     arrays, and are then also stored on into the segment, each tile by one CTA;
-//   * one elected thread issues the MMAs: S = Q.K^T (M 128, N = keys of a tile, K-steps of 16)
+//   * one warp, converged, issues one lane's MMAs: S = Q.K^T (M 128, N = keys of a tile, K-steps of 16)
 //     into a TMEM buffer and O += P.V (M 128, N = head_dim) into a TMEM accumulator.  P never
-//     touches shared memory: the softmax threads write it, rounded to the 16-bit type, over the
-//     first half of the columns of the S buffer it came from, and the MMA takes its A operand
-//     from tensor memory.  V is consumed as an MN-major B operand straight from its row-major
-//     tile;
+//     touches shared memory: the softmax threads write it, rounded to the 16-bit type, over
+//     the scores it came from (32 keys' weights over the first half of their columns), and the MMA
+//     takes its A operand from tensor memory.  V is consumed as an MN-major B operand straight from
+//     its row-major tile;
 //   * the softmax threads read S with tcgen05.ld (no shuffles for the row max / sum) and
 //     rescale O in tensor memory only when a row's maximum has grown by more than 2^8 since the
-//     reference it is using (the sum uses the same reference, so the result is exact);
+//     reference it is using (the sum uses the same reference, so the result is exact).  fp16 weights are
+//     worked out with the reference in use in one pass over the scores, and the maximum of that pass decides
+//     whether they stand;
 //   * with two groups per CTA each has one S buffer and the tensor cores work for one group
 //     while the other is in its softmax; with one group S is double-buffered so that Q.K^T of
 //     tile j+1 runs under the softmax of tile j.  The tail of one item overlaps the head of the
 //     next (loads, and the first Q.K^T while the previous output is stored).
+//
+// What bounds it (64 requests x 56 heads x 2048 tokens, D 128, fp16: 4.09 ms, 942 TFLOP/s, 0.59 of the cuBLAS burst rate;
+// it was 4.41 ms): a group's chain softmax (1700 clocks a tile of 128 keys, 1024 of them the special-function
+// unit's) -> P.V -> Q.K^T (1024 clocks of MMAs and about 500 of barriers and pipeline), which the
+// other group's overlaps only in part.  Putting a share of the exponentials on the FMA pipes as a polynomial
+// was measured slower (4.42 ms): the issue slots it costs are on the same chain.
 //
 // Tensor memory (all 512 columns are allocated): S buffers first, then one O accumulator per
 // group.  Every mbarrier is waited on phase by phase (a parity wait cannot tell phases two
@@ -58,7 +66,6 @@ struct Tc5Params {
     unsigned long long wait_ns;   // limit of every bounded wait
 };
 
-template <bool B> struct BoolC { static constexpr bool value = B; };
 template <typename T> struct SplitP { typedef char yes; static constexpr bool value = false; };
 template <> struct SplitP<__nv_bfloat16> { typedef char yes; static constexpr bool value = true; };
 
@@ -82,7 +89,8 @@ template <int D_, int KEYS_, int NG_>
 struct Tc5Layout {
     static constexpr int D = D_, KEYS = KEYS_, NG = NG_;
     static constexpr int NB = NG == 1 ? 2 : 1;                   // S buffers per group
-    static constexpr int kThreads = 32 * (4 * NG + 2);
+    static constexpr int kSoftWarps = 8 * NG;                    // two softmax threads per query row
+    static constexpr int kThreads = 32 * (kSoftWarps + 2);
     static constexpr int kDBoxes = D / 64;                       // 64-element (128-byte) column blocks of a row
     static constexpr int kBoxRows = D == 256 ? 32 : 64;          // rows of one TMA box of the prompt segment's tensor map
     static constexpr int kBoxBytes = kBoxRows * 128;
@@ -95,26 +103,23 @@ struct Tc5Layout {
     static constexpr int kQGroup = kDBoxes * kBoxQ;              // bytes of one group's Q
     static constexpr int kQ = NG * kQGroup;
     static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 6 * NG;   // K full/empty, V full/empty, per group: S0 S1 P O Qfull Qempty
-    static constexpr size_t kBytes = 1024 + (size_t)kRingK + kRingV + kQ + 8 * kBars + 64;
+    static constexpr size_t kBytes = 1024 + (size_t)kRingK + kRingV + kQ + 8 * kBars + NG * kRows * 4 + 64;
     // tensor memory: S buffers of KEYS columns first, then one O accumulator of D columns per group
     static constexpr int kColO = NG * NB * KEYS;
     static_assert(kColO + NG * D <= kTmemCols, "tensor memory");
     static_assert(kBytes <= 232448, "shared memory");
 };
 
-// Row maximum of one tile's scores.  BIAS: sv[i] <- sv[i] * scale2 + slope2 * (key_i - row), the
-// maximum is in log2 units; otherwise sv keeps the raw dot products and the maximum is raw.
-// MASK: keys above the row (i > lim) are set to -inf first.
-template <int KEYS, bool BIAS, bool MASK>
-__device__ __forceinline__ float score_max(float* sv, float scale2, float slope2, float bias0, int lim) {
+// Maximum of 32 scores of a row, in log2 units with BIAS (s * scale2 + bias0 + slope2 * i), else raw dot products;
+// MASK: keys above the row (i > lim) do not count.
+template <bool BIAS, bool MASK>
+__device__ __forceinline__ float max32(const uint32_t* sr, float scale2, float slope2, float bias0, int lim) {
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int i = 0; i < KEYS; ++i) {
-        float v = sv[i];
+    for (int i = 0; i < 32; ++i) {
+        float v = __uint_as_float(sr[i]);
         if (BIAS) v = fmaf(v, scale2, fmaf(slope2, (float)i, bias0));
-        if (MASK) v = i > lim ? -INFINITY : v;
-        if (BIAS || MASK) sv[i] = v;
-        mx[i & 3] = fmaxf(mx[i & 3], v);
+        mx[i & 3] = fmaxf(mx[i & 3], MASK && i > lim ? -INFINITY : v);
     }
     return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
@@ -130,9 +135,61 @@ __device__ __forceinline__ float score_max(float* sv, float scale2, float slope2
 constexpr float kSplitSlope = 0.0625f;   // weights fall by e^-slope per key: below this, dozens of keys share a row's weight
 constexpr int kSplitWindow = 64;
 // Do the `nkeys` keys from `key0` on get two-part weights, for the group whose first row is row0?
-__device__ __forceinline__ bool split_p_keys(int row0, int key0, int nkeys, float slope) {
+__device__ __forceinline__ bool split_p_keys(int row0, int key0, int nkeys, bool steep) {
     if (row0 == 0 && key0 < kRows) return true;
-    return slope >= kSplitSlope && key0 + nkeys - 1 >= row0 - kSplitWindow;
+    return steep && key0 + nkeys - 1 >= row0 - kSplitWindow;
+}
+
+// Two fp32 values in one 64-bit register pair, for the packed fp32 instructions.
+__device__ __forceinline__ uint64_t f2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float f2_lo(uint64_t v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float f2_hi(uint64_t v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return b;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Weights of 32 keys of a row from their scores: 2^(s * scale2 + c0 + slope2 * i), c0 = bias minus the row's reference;
+// packed in 16 bits (SPLIT: a second set of 16 words with the low parts), their sum added to ls.  Returns the largest exponent.
+template <typename T, bool BIAS, bool MASK, bool SPLIT>
+__device__ __forceinline__ float weigh32(const uint32_t* sr, float scale2, float slope2, float c0, int lim, uint64_t* ls, uint32_t* hi, uint32_t* lo) {
+    const uint64_t sc = f2(scale2, scale2), sl = f2(slope2, slope2), cc = f2(c0, c0);
+    float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const uint64_t x = f2_fma(f2(__uint_as_float(sr[2 * k]), __uint_as_float(sr[2 * k + 1])), sc,
+                                  BIAS ? f2_fma(sl, f2((float)(2 * k), (float)(2 * k + 1)), cc) : cc);
+        const float xa = MASK && 2 * k > lim ? -INFINITY : f2_lo(x), xb = MASK && 2 * k + 1 > lim ? -INFINITY : f2_hi(x);
+        asm("max.f32 %0, %0, %1, %2;" : "+f"(mx[k & 1]) : "f"(xa), "f"(xb));
+        const float ea = exp2f(xa), eb = exp2f(xb);
+        ls[k & 1] = f2_add(ls[k & 1], f2(ea, eb));
+        if (!SPLIT) {
+            hi[k] = Mma<T>::pack(ea, eb);
+        } else {
+            const uint32_t b0 = __float_as_uint(ea), b1 = __float_as_uint(eb);
+            hi[k] = __byte_perm(b0, b1, 0x7632);
+            lo[k] = Mma<T>::pack(ea - __uint_as_float(b0 & 0xFFFF0000u), eb - __uint_as_float(b1 & 0xFFFF0000u));
+        }
+    }
+    return fmaxf(mx[0], mx[1]);
 }
 
 // One CTA per SM walks a static list of work items (128*NG query rows of one (request, head)),
@@ -160,8 +217,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     uint64_t* bars = reinterpret_cast<uint64_t*>(q_smem + L::kQ);
     const uint32_t kfull0 = smem_u32(bars), kempty0 = kfull0 + 8 * SK;
     const uint32_t vfull0 = kempty0 + 8 * SK, vempty0 = vfull0 + 8 * SV;
-    const uint32_t gbar0 = vempty0 + 8 * SV;                      // group g: +48 g; S buffer 0, S buffer 1, P, O, Q full, Q empty
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
+    const uint32_t gbar0 = vempty0 + 8 * SV;                      // group g: + kGB g; S buffer 0, S buffer 1, P, O, Q full, Q empty
+    constexpr uint32_t kGB = 48;
+    float* s_row = reinterpret_cast<float*>(bars + L::kBars);     // one value per query row, between its two threads
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_row + NG * kRows);
     __shared__ int s_abort;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -213,18 +272,18 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             mbar_init(vempty0 + 8 * s, STORE ? 2 : 1);
         }
         for (int g = 0; g < NG; ++g) {
-            mbar_init(gbar0 + 48 * g, 1);
-            mbar_init(gbar0 + 48 * g + 8, 1);
-            mbar_init(gbar0 + 48 * g + 16, 128);
-            mbar_init(gbar0 + 48 * g + 24, 1);
-            mbar_init(gbar0 + 48 * g + 32, 1);
-            mbar_init(gbar0 + 48 * g + 40, 1);
+            mbar_init(gbar0 + kGB * g, 1);
+            mbar_init(gbar0 + kGB * g + 8, 1);
+            mbar_init(gbar0 + kGB * g + 16, 256);                 // both threads of every row
+            mbar_init(gbar0 + kGB * g + 24, 1);
+            mbar_init(gbar0 + kGB * g + 32, 1);
+            mbar_init(gbar0 + kGB * g + 40, 1);
         }
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
     }
-    if (warp == 4 * NG + 1) {                                     // this warp owns the tensor memory
+    if (warp == L::kSoftWarps + 1) {                                     // this warp owns the tensor memory
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "n"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -234,7 +293,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 4 * NG) {
+    if (warp == L::kSoftWarps) {
         // ------------------------------- TMA producer -------------------------------
         if (lane == 0) {
             prefetch_tmap(&tm_q);
@@ -267,10 +326,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     nkt = max(nkt, gt);
                     if (gt == 0) continue;
                     // the group's Q rows (past the prompt: zeros), once its previous Q is no longer read
-                    ok = mbar_wait(gbar0 + 48 * g + 40, (qi[g] & 1) ^ 1, p.wait_ns);
+                    ok = mbar_wait(gbar0 + kGB * g + 40, (qi[g] & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
                     ++qi[g];
-                    const uint32_t qfull = gbar0 + 48 * g + 32;
+                    const uint32_t qfull = gbar0 + kGB * g + 32;
                     const uint32_t dst = smem_u32(q_smem) + (uint32_t)g * L::kQGroup;
                     mbar_arrive_expect_tx(qfull, (uint32_t)L::kQGroup);
 #pragma unroll
@@ -334,23 +393,52 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             bulk_wait_all();                                      // the stores themselves, before the CTA may exit
             if (!ok) s_abort = 1;
         }
-    } else if (warp == 4 * NG + 1) {
+    } else if (warp == L::kSoftWarps + 1) {
         // -------------------------------- MMA issuer --------------------------------
-        if (lane == 0) {
-            uint32_t tp = 0;                                       // ring position of the item's first K/V tile
-            const uint64_t q_desc0 = smem_desc(smem_u32(q_smem), 16, 1024);
-            const uint64_t k_desc0 = smem_desc(smem_u32(k_ring), 16, 1024);
-            const uint64_t v_desc0 = smem_desc(smem_u32(v_ring), kColTile, 1024);
+        // (the whole warp runs this, converged, and one lane's MMAs are issued: see tc_mma_ss_if.  What decides the
+        // control flow is made uniform by a warp reduction or vote.)
+        {
+            // Ring positions are counted, not computed with remainders, so that descriptors stay in uniform
+            // registers: MMAs follow each other at 64 clocks then, and at about 108 with remainders.
+            const uint32_t lead = elect_one();
+            auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+                return __all_sync(0xffffffffu, mbar_wait_hot(bar, parity, p.wait_ns));
+            };
+            const uint32_t q_lo = (smem_u32(q_smem) & 0x3FFFFu) >> 4, k_lo0 = (smem_u32(k_ring) & 0x3FFFFu) >> 4;
+            const uint32_t v_lo0 = (smem_u32(v_ring) & 0x3FFFFu) >> 4;
+            const uint64_t dk = smem_desc(0, 16, 1024), dv = smem_desc(0, kColTile, 1024);   // descriptors without an address
+            uint32_t kst = 0, kph = 0, vst = 0, vph = 0;          // stage and phase of the next K and V tile
             uint32_t n[NG], qi[NG];                               // tiles / items of group g so far: barrier phases
 #pragma unroll
             for (int g = 0; g < NG; ++g) n[g] = qi[g] = 0;
             bool ok = true;
+            // S_g[buf] = Q_g . K^T for the K tile of stage kst; after the group's last one its Q may be replaced
+            auto issue_qk = [&](int g, uint32_t buf, bool last) {
+                const uint64_t qd = dk + (q_lo + (uint32_t)g * (uint32_t)(L::kQGroup >> 4));
+                const uint64_t kd = dk + (k_lo0 + kst * (uint32_t)(kTileKV >> 4));
+                const uint32_t d_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + buf);
+#pragma unroll
+                for (int ks = 0; ks < kD / 16; ++ks)
+                    tc_mma_ss_if(lead, d_tmem, qd + (uint64_t)(((ks >> 2) * kBoxQ + (ks & 3) * 32) >> 4),
+                                 kd + (uint64_t)(((ks >> 2) * kColTile + (ks & 3) * 32) >> 4), p.idesc_qk, ks > 0);
+                tc_commit_if(lead, gbar0 + kGB * g + 8 * buf);
+                if (last) tc_commit_if(lead, gbar0 + kGB * g + 40);
+            };
+            auto wait_k = [&]() -> bool {
+                const bool r = wait(kfull0 + 8 * kst, kph);
+                tc_fence_after();
+                return r;
+            };
+            auto release_k = [&]() {                              // K stage free once these MMAs are done
+                tc_commit_if(lead, kempty0 + 8 * kst);
+                if (++kst == SK) { kst = 0; kph ^= 1u; }
+            };
             for (int j = 0; j < p.rounds && ok; ++j) {
                 const int w = round_item(j);
                 if (w >= n_items) continue;
-                const int qt = item_qt(w), nb = request_len((w % hb_count) / p.H);
-                // requested here, used after the first waits of the item
-                const float slope = (kSplitP && p.slopes) ? __ldg(p.slopes + (w % hb_count) % p.H) : 0.f;
+                const int qt = item_qt(w), nb = RAGGED ? (int)__reduce_max_sync(0xffffffffu, (unsigned)request_len((w % hb_count) / p.H)) : p.N;
+                // is the head's slope one of those whose weights go in two parts next to the diagonal?
+                const bool steep = kSplitP && p.slopes && __any_sync(0xffffffffu, __ldg(p.slopes + (w % hb_count) % p.H) >= kSplitSlope);
                 int gt[NG], nkt = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
@@ -358,107 +446,86 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     nkt = max(nkt, gt[g]);
                 }
                 if (nkt == 0) continue;                           // the request ends before this item's rows
-                // S_g[buf] = Q_g . K^T for the group's tile kt; after its last one the group's Q may be replaced
-                auto issue_qk = [&](int g, int kt, int buf) {
-                    // One descriptor per operand and tile; a K-step only moves the start address, which
-                    // sits in the descriptor's low bits in units of 16 bytes: the issuing thread is a
-                    // single lane, and every instruction it spends per MMA is time the tensor pipe waits.
-                    const uint64_t qd = q_desc0 + (uint64_t)(((uint32_t)g * L::kQGroup) >> 4);
-                    const uint64_t kd = k_desc0 + (uint64_t)((((tp + kt) % SK) * (uint32_t)kTileKV) >> 4);
-                    const uint32_t d_tmem = tmem + (uint32_t)(kKeys * (g * NB + buf));
-#pragma unroll
-                    for (int ks = 0; ks < kD / 16; ++ks)
-                        tc_mma_ss(d_tmem, qd + (uint64_t)(((ks >> 2) * kBoxQ + (ks & 3) * 32) >> 4),
-                                  kd + (uint64_t)(((ks >> 2) * kColTile + (ks & 3) * 32) >> 4), p.idesc_qk, ks > 0);
-                    tc_commit(gbar0 + 48 * g + 8 * buf);
-                    if (kt + 1 == gt[g]) tc_commit(gbar0 + 48 * g + 40);
-                };
-                auto wait_k = [&](int kt) -> bool {
-                    const bool r = mbar_wait_hot(kfull0 + 8 * ((tp + kt) % SK), ((tp + kt) / SK) & 1, p.wait_ns);
-                    tc_fence_after();
-                    return r;
-                };
+                // (each group's query is waited for when its own scores are due: the second group's arrives later, as its
+                // last tile of the item before runs after the first group's)
+                ok = wait_k();
 #pragma unroll
                 for (int g = 0; g < NG; ++g)
-                    if (gt[g] > 0 && ok) ok = mbar_wait_hot(gbar0 + 48 * g + 32, qi[g]++ & 1, p.wait_ns);   // Q_g landed
-                if (ok) ok = wait_k(0);
+                    if (gt[g] > 0 && ok) {
+                        ok = wait(gbar0 + kGB * g + 32, qi[g]++ & 1);   // Q_g landed
+                        if (ok) issue_qk(g, NB == 2 ? n[g] & 1 : 0u, gt[g] == 1);
+                    }
                 if (!ok) break;
-#pragma unroll
-                for (int g = 0; g < NG; ++g)
-                    if (gt[g] > 0) issue_qk(g, 0, NB == 2 ? (int)(n[g] & 1) : 0);
-                tc_commit(kempty0 + 8 * (tp % SK));                // K stage free once these MMAs are done
+                release_k();
                 for (int kt = 0; kt < nkt && ok; ++kt) {
                     TC5_STAMP(2, kt, 0);
                     if (NB == 2 && kt + 1 < nkt) {                // next tile's scores run under this tile's softmax
-                        ok = wait_k(kt + 1);
+                        ok = wait_k();
                         if (!ok) break;
 #pragma unroll
                         for (int g = 0; g < NG; ++g)
-                            if (kt + 1 < gt[g]) issue_qk(g, kt + 1, (int)((n[g] + 1) & 1));
-                        tc_commit(kempty0 + 8 * ((tp + kt + 1) % SK));
+                            if (kt + 1 < gt[g]) issue_qk(g, (n[g] + 1) & 1, kt + 2 == gt[g]);
+                        release_k();
                     }
-                    const uint32_t sv = (tp + kt) % SV;
-                    const uint64_t vd = v_desc0 + (uint64_t)((sv * (uint32_t)kTileKV) >> 4);
-                    ok = mbar_wait_hot(vfull0 + 8 * sv, ((tp + kt) / SV) & 1, p.wait_ns);
+                    const uint64_t vd = dv + (v_lo0 + vst * (uint32_t)(kTileKV >> 4));
+                    ok = wait(vfull0 + 8 * vst, vph);
                     if (!ok) break;
                     bool k_next = false;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
                         if (kt >= gt[g]) continue;
-                        ok = mbar_wait_hot(gbar0 + 48 * g + 16, n[g] & 1, p.wait_ns);   // P_g written over its S buffer
+                        ok = wait(gbar0 + kGB * g + 16, n[g] & 1);   // P_g written over its S buffer
                         if (!ok) break;
                         TC5_STAMP(2, kt, 1 + 3 * g);
                         tc_fence_after();
-                        const uint32_t p_tmem = tmem + (uint32_t)(kKeys * (g * NB + (NB == 2 ? (int)(n[g] & 1) : 0)));
+                        const uint32_t p_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + (NB == 2 ? n[g] & 1 : 0u));
 #pragma unroll
                         for (int kk = 0; kk < kKeys / 16; ++kk)   // O_g += P_g[:, 16 keys] . V[16 keys, :]
-                            tc_mma_ts(tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 8,
-                                      vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (kt > 0 || kk > 0));
-                        if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, slope)) {
+                            tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + (kk >> 1) * 32 + (kk & 1) * 8,
+                                         vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (kt > 0 || kk > 0));
+                        if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, steep)) {
 #pragma unroll
                             for (int kk = 0; kk < kKeys / 16; ++kk)   // ... and the low parts of the weights that have one
-                                if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, slope))
-                                    tc_mma_ts(tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kKeys / 2 + kk * 8,
-                                              vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
+                                if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, steep))
+                                    tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + (kk >> 1) * 32 + 16 + (kk & 1) * 8,
+                                                 vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
                         }
-                        tc_commit(gbar0 + 48 * g + 24);
-#if defined(SEGKV_TC5_TIMELINE) && SEGKV_TC5_TIMELINE == 3
-                        mbar_wait_hot(gbar0 + 48 * g + 24, n[g] & 1, p.wait_ns);   // measurement only: serialise on P.V
-                        TC5_STAMP(2, kt, 2 + 3 * g);
-#endif
+                        tc_commit_if(lead, gbar0 + kGB * g + 24);
                         ++n[g];
                         if (NB == 1 && kt + 1 < gt[g]) {          // the group's next scores, behind its P.V in the pipe
                             if (!k_next) {
-                                ok = wait_k(kt + 1);
+                                ok = wait_k();
                                 if (!ok) break;
                                 k_next = true;
                             }
-                            issue_qk(g, kt + 1, 0);
-#if defined(SEGKV_TC5_TIMELINE) && SEGKV_TC5_TIMELINE == 3
-                            mbar_wait_hot(gbar0 + 48 * g, n[g] & 1, p.wait_ns);    // measurement only: serialise on Q.K^T
-                            TC5_STAMP(2, kt, 3 + 3 * g);
-#endif
+                            issue_qk(g, 0u, kt + 2 == gt[g]);
                         }
                     }
                     if (!ok) break;
-                    tc_commit(vempty0 + 8 * sv);                  // stages free once every MMA so far is done
-                    if (NB == 1 && kt + 1 < nkt) tc_commit(kempty0 + 8 * ((tp + kt + 1) % SK));
+                    tc_commit_if(lead, vempty0 + 8 * vst);        // stage free once every MMA so far is done
+                    if (++vst == SV) { vst = 0; vph ^= 1u; }
+                    if (NB == 1 && kt + 1 < nkt) release_k();
                 }
-                tp += (uint32_t)nkt;
             }
-            if (!ok) s_abort = 1;
+            if (!ok && lane == 0) s_abort = 1;
         }
     } else {
-        // ------------------------------ softmax warps: one row per thread ------------------------------
-        const int g = warp >> 2, r = tid & (kRows - 1);
-        const uint32_t bar_s0 = gbar0 + 48 * g, bar_p = bar_s0 + 16, bar_o = bar_s0 + 24;
+        // ------------------------------ softmax warps: two threads per row ------------------------------
+        // Each takes one half of a tile's keys, and at the end of an item one half of the output row.  (One thread per row
+        // spent 2200 clocks on a tile of 128 keys, of which 1170 are hidden behind the other group's MMAs: the
+        // chain softmax -> P.V -> next Q.K^T bound the kernel.  Twice the warps hide each other's latencies.)
+        constexpr int KH = kKeys / 2, DH = kD / 2;
+        const int g = warp >> 3, half = (warp >> 2) & 1, r = (warp & 3) * 32 + lane;
+        const int pair = 1 + g * 4 + (warp & 3);                  // barrier of the two warps that share these rows
+        const uint32_t bar_s0 = gbar0 + kGB * g, bar_p = bar_s0 + 16, bar_o = bar_s0 + 24;
         const uint32_t tm_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);     // this warp's TMEM lanes
-        const uint32_t tm_o = tm_lane + (uint32_t)(L::kColO + kD * g);
-        const bool stamp = lane == 0 && (warp & 3) == 0;
+        const uint32_t tm_o = tm_lane + (uint32_t)(L::kColO + kD * g + DH * half);
+        float* xrow = s_row + g * kRows + r;
+        const bool stamp = lane == 0 && (warp & 7) == 0;
         const size_t qstride = (size_t)p.H * kD;
         uint32_t n = 0;                                           // tiles of this group so far: barrier phases
-        bool ok = true;
-        for (int j = 0; j < p.rounds && ok; ++j) {
+        bool ok = true, gone = false;                             // a wait of this thread ran out; the pair of warps has agreed to leave
+        for (int j = 0; j < p.rounds && !gone; ++j) {
             const int w = round_item(j);
             if (w >= n_items) continue;
             const int qt = item_qt(w), hb = w % hb_count, h = hb % p.H, b = hb / p.H;
@@ -467,147 +534,222 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const int row0 = (qt * NG + g) * kRows, row = row0 + r;
             const float slope_nat = p.slopes ? p.slopes[h] : 0.f;
             const float slope2 = slope_nat * 1.4426950408889634f;
+            const bool biased = p.slopes != nullptr;
             float m_ref = -INFINITY, l_run = 0.f;
             for (int kt = 0; kt < my_tiles; ++kt, ++n) {
                 const int buf = NB == 2 ? (int)(n & 1) : 0;
                 const uint32_t tm_s = tm_lane + (uint32_t)(kKeys * (g * NB + buf));
-                ok = mbar_wait_hot(bar_s0 + 8 * buf, (NB == 2 ? (n >> 1) : n) & 1, p.wait_ns);
+                if (ok) ok = mbar_wait_hot(bar_s0 + 8 * buf, (NB == 2 ? (n >> 1) : n) & 1, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
                 if (stamp) TC5_STAMP(g, kt, 0);
-                // One tile of the group, from the scores in tensor memory to the weights handed to the
-                // MMA thread.  Two instances (weights in one part / in two parts) rather than a branch
-                // in the middle: the 128 scores live in registers, and a fork with all of them live
-                // costs the two-group shape hundreds of bytes of spills.
-                auto tile = [&](auto two_parts) -> bool {
-                    constexpr bool split = decltype(two_parts)::value;
-                    tc_fence_after();
-                    uint32_t sr[kKeys];
-#pragma unroll
-                    for (int c = 0; c < kKeys / 32; ++c) tc_ld32(tm_s + 32 * c, sr + 32 * c);
-                    tc_wait_ld();
-                    if (stamp) TC5_STAMP(g, kt, 1);
-                    float* sv = reinterpret_cast<float*>(sr);
-                    const int key0 = kt * kKeys;
-                    const bool diag = key0 + kKeys - 1 > row0;         // a tile that reaches past the group's first row
-                    // scores in log2 units: s * scale2 (+ ALiBi bias); the scale is folded into the exponent's
-                    // FMA unless a bias has to be added first; keys above the row (diagonal tile) become -inf
-                    const bool biased = p.slopes != nullptr;
-                    const int lim = row - key0;                        // key index i of this tile is visible iff i <= lim
-                    const float bias0 = slope2 * (float)(key0 - row);
-                    float tmax;
-                    if (biased) tmax = diag ? score_max<kKeys, true, true>(sv, p.scale2, slope2, bias0, lim)
-                                            : score_max<kKeys, true, false>(sv, p.scale2, slope2, bias0, lim);
-                    else tmax = (diag ? score_max<kKeys, false, true>(sv, p.scale2, slope2, bias0, lim)
-                                      : score_max<kKeys, false, false>(sv, p.scale2, slope2, bias0, lim)) * p.scale2;
-                    // a new reference only when the maximum has grown by more than 2^8: exponentials stay
-                    // below 2^8 of the reference, the sum and O use the same reference
-                    const bool need = tmax > m_ref + 8.f;
-                    float alpha = 1.f;
-                    if (need) {
-                        alpha = exp2f(m_ref - tmax);                   // 0 on the first tile
-                        m_ref = tmax;
-                    }
-                    float ls[4] = {0.f, 0.f, 0.f, 0.f};
-                    uint32_t pk[kKeys / 2];
-                    const float sc = biased ? 1.f : p.scale2, nm = -m_ref;
-                    if (!split) {
-#pragma unroll
-                        for (int i = 0; i < kKeys; i += 2) {
-                            const float e0 = exp2f(fmaf(sv[i], sc, nm)), e1 = exp2f(fmaf(sv[i + 1], sc, nm));
-                            ls[(i >> 1) & 3] += e0 + e1;
-                            pk[i >> 1] = Mma<T>::pack(e0, e1);
-                        }
-                    } else {
-                        // weights as two bf16 parts: the high parts over the first half of the S buffer's
-                        // columns, the low parts over the second half, 32 keys at a time (S is in registers
-                        // and the MMAs that read the buffer's previous contents have completed)
-#pragma unroll
-                        for (int c = 0; c < kKeys / 32; ++c) {
-                            uint32_t ph[16], pl[16];
-#pragma unroll
-                            for (int i = 0; i < 32; i += 2) {
-                                const float e0 = exp2f(fmaf(sv[32 * c + i], sc, nm)), e1 = exp2f(fmaf(sv[32 * c + i + 1], sc, nm));
-                                ls[(i >> 1) & 3] += e0 + e1;
-                                const uint32_t b0 = __float_as_uint(e0), b1 = __float_as_uint(e1);
-                                ph[i >> 1] = __byte_perm(b0, b1, 0x7632);
-                                pl[i >> 1] = Mma<T>::pack(e0 - __uint_as_float(b0 & 0xFFFF0000u), e1 - __uint_as_float(b1 & 0xFFFF0000u));
-                            }
-                            tc_st16(tm_s + 16 * c, ph);
-                            tc_st16(tm_s + kKeys / 2 + 16 * c, pl);
-                        }
-                    }
-                    l_run = l_run * alpha + ((ls[0] + ls[1]) + (ls[2] + ls[3]));
-                    if (stamp) TC5_STAMP(g, kt, 2);
-                    // O may be touched once P.V of the previous tile is done.  A parity wait is only
-                    // meaningful on the barrier's current or previous phase, so with two S buffers,
-                    // where nothing else ties this thread to the P.V before last, every phase of the O
-                    // barrier is waited for in turn (with one S buffer the scores of this tile were
-                    // produced behind that P.V in the pipe, and waiting here is only needed to rescale).
-                    const bool rescale = kt > 0 && __any_sync(0xffffffffu, need);
-                    if (kt > 0 && (NB == 2 || rescale)) {
-                        bool arrived = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
-                        arrived = __all_sync(0xffffffffu, arrived);
-                        if (!arrived) return false;
+                // One tile of the group, from the scores in tensor memory to the weights handed to the MMA thread.
+                // P goes in place of the scores: 32 keys' weights, two to a column, over the first half of those
+                // keys' columns, low parts (bf16, where the weights go in two parts) over the second half.
+                const int key0 = kt * kKeys + half * KH;
+                const bool diag = key0 + KH - 1 > row0;            // keys that reach past the group's first row
+                const int lim = row - key0;                        // key index i is visible iff i <= lim
+                const float bias0 = slope2 * (float)(key0 - row);
+                const uint32_t tm_sh = tm_s + KH * half;
+                const bool two = kSplitP && split_p_keys(row0, kt * kKeys, kKeys, slope_nat >= kSplitSlope);
+                float alpha = 1.f;
+                uint64_t ls[2] = {0ull, 0ull};
+                // The reference in use nearly always stands after the first tile: the weights are worked out with it
+                // in one pass over the scores that notes their maximum on the way, and stored when both threads of
+                // the row know that it stands.  (Not under a slope that lifts the maximum
+                // by 2^4 and more from tile to tile; nor in bf16, whose two kinds of weights leave no registers for it:
+                // 2.61 against 1.92 ms at 32 x 112 heads x 1024 with ALiBi.)
+                bool stands = !kSplitP && kt > 0 && slope2 * (float)kKeys < 4.f;
+                if (stands) {
+                    float mx = -INFINITY;
+                    uint32_t pk[KH / 2];
+                    if (ok) {
                         tc_fence_after();
-                    }
-                    if (rescale) {
 #pragma unroll
-                        for (int c = 0; c < kD / 32; ++c) {
-                            uint32_t orr[32];
-                            tc_ld32(tm_o + c * 32, orr);
+                        for (int c = 0; c < KH; c += 32) {
+                            uint32_t sr[32];
+                            tc_ld32(tm_sh + c, sr);
                             tc_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
-                            tc_st32(tm_o + c * 32, orr);
+                            pin<32>(sr);
+                            if (c == 0 && stamp) TC5_STAMP(g, kt, 1);
+                            const float c0 = (biased ? bias0 + slope2 * (float)c : 0.f) - m_ref;
+                            if (biased) {
+                                if (diag) mx = fmaxf(mx, weigh32<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
+                                else mx = fmaxf(mx, weigh32<T, true, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
+                            } else {
+                                if (diag) mx = fmaxf(mx, weigh32<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
+                                else mx = fmaxf(mx, weigh32<T, false, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
+                            }
                         }
-                        if (stamp) TC5_STAMP(g, kt, 3);
                     }
-                    // P over the first 64 columns of the S buffer: two 16-bit weights per column, the A
-                    // operand layout of the MMA that follows.  S has been read completely above.
-                    if (!split) {
+                    stands = bar_and(pair, 64, ok && !(mx > 8.f));
+                    if (stands) {
 #pragma unroll
-                        for (int c = 0; c < kKeys / 32; ++c) tc_st16(tm_s + 16 * c, pk + 16 * c);
+                        for (int c = 0; c < KH; c += 32) tc_st16(tm_sh + c, pk + c / 2);
                     }
-                    tc_wait_st();
-                    tc_fence_before();
-                    if (!(p.dbg_skip && tid == 0 && n == 0)) mbar_arrive(bar_p);
-                    if (stamp) TC5_STAMP(g, kt, 4);
-                    return true;
-                };
-                ok = (kSplitP && split_p_keys(row0, kt * kKeys, kKeys, slope_nat)) ? tile(BoolC<kSplitP>{}) : tile(BoolC<false>{});
-                if (!ok) break;
+                }
+                if (!stands) {
+                    // A new reference, if the maximum has grown by more than 2^8: exponentials stay below 2^8 of the
+                    // reference, the sum and O use the same reference, so the result is exact.
+                    float tmax = -INFINITY;
+                    if (ok) {
+                        tc_fence_after();
+#pragma unroll 1
+                        for (int c = 0; c < KH; c += 32) {
+                            uint32_t sr[32];
+                            tc_ld32(tm_sh + c, sr);
+                            tc_wait_ld();
+                            pin<32>(sr);
+                            // in log2 units; without a bias the scale is folded into the exponent's FMA
+                            float m;
+                            if (biased) m = diag ? max32<true, true>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c)
+                                                 : max32<true, false>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c);
+                            else m = (diag ? max32<false, true>(sr, p.scale2, slope2, bias0, lim - c)
+                                           : max32<false, false>(sr, p.scale2, slope2, bias0, lim - c)) * p.scale2;
+                            tmax = fmaxf(tmax, m);
+                        }
+                    }
+                    bool need = tmax > m_ref + 8.f;
+                    if (!bar_and(pair, 64, ok && !need)) {            // the two threads of a row compare notes only then
+                        if (half == 0) *xrow = tmax;
+                        ok = bar_and(pair, 64, ok);
+                        gone = !ok;
+                        if (gone) break;
+                        if (half == 1) {
+                            tmax = fmaxf(tmax, *xrow);
+                            *xrow = tmax;
+                        }
+                        bar_sync_n(pair, 64);
+                        if (half == 0) tmax = *xrow;
+                        need = tmax > m_ref + 8.f;
+                        if (need) {
+                            alpha = exp2f(m_ref - tmax);               // 0 on the first tile
+                            m_ref = tmax;
+                        }
+                        // O is rescaled (half a row per thread) before any weight of this tile is handed over, once P.V of the
+                        // previous tile is done
+                        if (kt > 0 && __any_sync(0xffffffffu, need)) {
+                            ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
+                            ok = __all_sync(0xffffffffu, ok);
+                            if (ok) {
+                                tc_fence_after();
+#pragma unroll 1
+                                for (int c = 0; c < DH / 16; ++c) {
+                                    uint32_t orr[16];
+                                    tc_ld16(tm_o + c * 16, orr);
+                                    tc_wait_ld();
+                                    pin<16>(orr);
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
+                                    tc_st16(tm_o + c * 16, orr);
+                                }
+                                tc_wait_st();
+                                tc_fence_before();
+                            }
+                            ok = bar_and(pair, 64, ok);                // both halves are
+                            gone = !ok;
+                            if (gone) break;
+                            tc_fence_after();
+                            if (stamp) TC5_STAMP(g, kt, 3);
+                        }
+                    }
+                    ls[0] = ls[1] = 0ull;
+#pragma unroll 1
+                    for (int c = 0; c < KH; c += 32) {
+                        uint32_t sr[32], hi[16], lo[16];
+                        tc_ld32(tm_sh + c, sr);
+                        tc_wait_ld();
+                        pin<32>(sr);
+                        const float c0 = (biased ? bias0 + slope2 * (float)c : 0.f) - m_ref;
+                        if (kSplitP && two) {
+                            if (biased) (void)weigh32<T, true, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                            else (void)weigh32<T, false, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                            tc_st16(tm_sh + c + 16, lo);
+                        } else {
+                            if (biased) {
+                                if (diag) (void)weigh32<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                                else (void)weigh32<T, true, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                            } else {
+                                if (diag) (void)weigh32<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                                else (void)weigh32<T, false, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                            }
+                        }
+                        tc_st16(tm_sh + c, hi);
+                    }
+                }
+                const uint64_t lt = f2_add(ls[0], ls[1]);
+                l_run = l_run * alpha + (f2_lo(lt) + f2_hi(lt));
+                if (stamp) TC5_STAMP(g, kt, 2);
+                // With one S buffer these scores were issued behind P.V of the previous tile, which keeps the O and P
+                // barriers at the phases waited for; with two, where a thread could run two phases ahead of the
+                // MMA thread, every phase of the O barrier is waited for in turn.
+                if (NB == 2 && kt > 0) {
+                    ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
+                    ok = __all_sync(0xffffffffu, ok);
+                }
+                tc_wait_st();
+                tc_fence_before();
+                if (ok && !(p.dbg_skip && tid == 0 && n == 0)) mbar_arrive(bar_p);
+                if (stamp) TC5_STAMP(g, kt, 4);
             }
-            if (!ok) break;
+            if (gone) break;
             // the item's output: O / l, once the last P.V has landed.  The next item's first P.V
             // cannot overwrite O before these loads: it waits for this thread's next P arrival.
-            ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
+            if (ok) ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
             ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
+            ok = bar_and(pair, 64, ok);
+            gone = !ok;
+            if (gone) break;
             tc_fence_after();
+            if (half == 0) *xrow = l_run;
+            bar_sync_n(pair, 64);
+            if (half == 1) {
+                l_run += *xrow;
+                *xrow = l_run;
+            }
+            bar_sync_n(pair, 64);
+            if (half == 0) l_run = *xrow;
             const float inv = 1.f / l_run;
-            T* orow = reinterpret_cast<T*>(p.out) + ((size_t)b * p.N * p.H + h) * kD + (size_t)row * qstride;
-#pragma unroll
-            for (int c = 0; c < kD / 32; ++c) {
+            // Four lanes trade 16-byte pieces of their rows, so that a store instruction writes 64 bytes of each of 8 rows
+            // instead of 16 of 32: with one row per lane the stores of an item took 3400 clocks (6500 at head_dim 256).
+            const int len = request_len(b), q4 = lane & 3, rowq = row0 + (r & ~3);
+            T* oq = reinterpret_cast<T*>(p.out) + ((size_t)b * p.N * p.H + h) * kD + (size_t)rowq * qstride + DH * half + q4 * 8;
+#pragma unroll 1
+            for (int c = 0; c < DH / 32; ++c) {
                 uint32_t orr[32];
                 tc_ld32(tm_o + c * 32, orr);
                 tc_wait_ld();
-                if (row < request_len(b)) {
+                pin<32>(orr);
+                uint32_t v[4][4];                                 // [piece][word]
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        *reinterpret_cast<uint4*>(orow + c * 32 + i * 8) = make_uint4(
-                            Mma<T>::pack(__uint_as_float(orr[8 * i]) * inv, __uint_as_float(orr[8 * i + 1]) * inv),
-                            Mma<T>::pack(__uint_as_float(orr[8 * i + 2]) * inv, __uint_as_float(orr[8 * i + 3]) * inv),
-                            Mma<T>::pack(__uint_as_float(orr[8 * i + 4]) * inv, __uint_as_float(orr[8 * i + 5]) * inv),
-                            Mma<T>::pack(__uint_as_float(orr[8 * i + 6]) * inv, __uint_as_float(orr[8 * i + 7]) * inv));
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        v[i][u] = Mma<T>::pack(__uint_as_float(orr[8 * i + 2 * u]) * inv, __uint_as_float(orr[8 * i + 2 * u + 1]) * inv);
+#pragma unroll
+                for (int x = 1; x <= 2; x <<= 1) {                // a 4 x 4 transposition in two exchanges
+                    const bool up = (lane & x) != 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (i & x) continue;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint32_t t = __shfl_xor_sync(0xffffffffu, up ? v[i][u] : v[i | x][u], x);
+                            if (up) v[i][u] = t;
+                            else v[i | x][u] = t;
+                        }
+                    }
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (rowq + i < len)
+                        *reinterpret_cast<uint4*>(oq + (size_t)i * qstride + c * 32) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
             }
         }
         if (!ok && lane == 0) s_abort = 1;
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 4 * NG + 1) {
+    if (warp == L::kSoftWarps + 1) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
         if (lane == 0 && s_abort) atomicOr(p.err_word, SEGKV_DEV_WAIT_LIMIT);

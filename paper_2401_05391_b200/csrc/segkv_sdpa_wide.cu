@@ -40,20 +40,6 @@ using namespace ptx;
 constexpr int kTicketAbortedW = 1 << 16;     // same marker as the tiled kernel's
 constexpr int kCols = kMaxCols;              // query columns of a work group, padded: one tensor-memory lane each
 
-// AND of a predicate over the threads that meet at a named barrier
-__device__ __forceinline__ bool bar_and(int id, int threads, bool ok) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "barrier.cta.red.and.pred p, %2, %3, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(r) : "r"((uint32_t)ok), "r"(id), "r"(threads) : "memory");
-    return r != 0;
-}
-__device__ __forceinline__ void bar_sync_n(int id, int threads) {
-    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 struct WideParams {
     const void* q;
     void* out;

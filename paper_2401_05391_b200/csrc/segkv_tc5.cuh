@@ -127,6 +127,20 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
     return ((uint64_t)hi << 32) | lo;
 }
 
+// AND of a predicate over the threads that meet at a named barrier
+__device__ __forceinline__ bool bar_and(int id, int threads, bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "barrier.cta.red.and.pred p, %2, %3, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r) : "r"((uint32_t)ok), "r"(id), "r"(threads) : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void bar_sync_n(int id, int threads) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 // Critical-path wait: poll without sleeping first (the hardware suspends the thread inside
 // try_wait for a while), then fall back to the bounded, sleeping wait.
 __device__ __forceinline__ bool mbar_wait_hot(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
