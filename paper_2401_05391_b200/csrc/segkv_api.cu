@@ -135,12 +135,19 @@ int make_prompt_map(const segkv* h, void* base, int prompt_len, int box_tokens, 
 
 // The handle's maps of its prompt segment: boxes of one regular tile (which the prefill kernel
 // shares) and boxes of 32 tokens for the small-CTA form of the decode kernel.
+// They depend on the handle's own memory, the layout and the length, so prompts of the length before keep them.
 int make_prompt_maps(segkv* h, int prompt_len) {
+    if (h->tm_len == prompt_len && h->tm_layout == h->d.prompt_layout) return SEGKV_OK;
+    h->tm_len = -1;
     const int box = tiled_tile_keys(h->d.head_dim, false);
     int rc = make_prompt_map(h, h->kp, prompt_len, box, &h->tm_kp);
     if (rc == SEGKV_OK) rc = make_prompt_map(h, h->vp, prompt_len, box, &h->tm_vp);
     if (rc == SEGKV_OK) rc = make_prompt_map(h, h->kp, prompt_len, 32, &h->tm_kp32);
     if (rc == SEGKV_OK) rc = make_prompt_map(h, h->vp, prompt_len, 32, &h->tm_vp32);
+    if (rc == SEGKV_OK) {
+        h->tm_len = prompt_len;
+        h->tm_layout = h->d.prompt_layout;
+    }
     return rc;
 }
 
@@ -458,6 +465,10 @@ bool rows_settled(const segkv* h, cudaStream_t st, bool lists_too) {
     return settled(&index_of(h)->lists_mark, st);
 }
 
+// May an attention launch start before its predecessor in the stream has finished?  Not before the first step: the
+// predecessor may then be the prompt store, whose prompt lengths the kernels read ahead of their wait.
+bool may_overlap(const segkv* h) { return h->overlap && h->steps > 0; }
+
 SdpaArgs sdpa_args(const segkv* h, const void* q, void* out, const float* slopes, int splits) {
     SdpaArgs a;
     a.q = q;
@@ -553,6 +564,7 @@ int segkv_create_growing(segkv_t* out, int batch, int beams, int heads, int kv_h
     d.group = heads / kv_heads; d.max_prompt = max_prompt; d.max_steps = max_steps;
     d.rows = batch * beams; d.dtype = dtype; d.chunk_steps = chunk_steps;
     h->prompt_len = -1;
+    h->tm_len = -1;
     h->overlap = true;
     h->persist_mode = -1;
     h->prefill_groups = 0;
@@ -632,12 +644,12 @@ int segkv_destroy(segkv_t h) {
     return SEGKV_OK;
 }
 
-static int prefill_write_impl(segkv_t h, const void* k, const void* v, int prompt_len, const int32_t* plens_dev,
-                              void* stream);
+static int prefill_write_impl(segkv_t h, const void* k, const void* v, int prompt_len, int32_t* plens_dev,
+                              const int32_t* lens_host, void* stream);
 
 int segkv_prefill_write(segkv_t h, const void* k, const void* v, int prompt_len, void* stream) {
     if (!h) return SEGKV_EINVAL;
-    int rc = prefill_write_impl(h, k, v, prompt_len, nullptr, stream);
+    int rc = prefill_write_impl(h, k, v, prompt_len, nullptr, nullptr, stream);
     if (rc == SEGKV_OK) h->ragged = false;
     return rc;
 }
@@ -648,24 +660,27 @@ int segkv_prefill_write_ragged(segkv_t h, const void* k, const void* v, int padd
     if (padded_len > h->d.max_prompt) return SEGKV_ECAPACITY;
     for (int b = 0; b < h->d.batch; ++b)
         if (prompt_lens[b] < 1 || prompt_lens[b] > padded_len) return SEGKV_EINVAL;
-    // the lengths travel on the caller's stream, ahead of the kernel that reads them; the source
-    // is pageable host memory, so the copy has been staged by the time the call returns
-    SEGKV_CUDA(cudaMemcpyAsync(h->plens, prompt_lens, (size_t)h->d.batch * sizeof(int32_t), cudaMemcpyHostToDevice,
-                               (cudaStream_t)stream));
-    int rc = prefill_write_impl(h, k, v, padded_len, h->plens, stream);
+    // the lengths of up to kMaxLensByValue requests travel as an argument of the kernel that zeroes the padding,
+    // which leaves them in h->plens for the kernels after it; more are copied ahead of it on the caller's stream (the
+    // source is pageable host memory, so the copy has been staged by the time the call returns)
+    const bool by_value = h->d.batch <= kMaxLensByValue;
+    if (!by_value)
+        SEGKV_CUDA(cudaMemcpyAsync(h->plens, prompt_lens, (size_t)h->d.batch * sizeof(int32_t), cudaMemcpyHostToDevice,
+                                   (cudaStream_t)stream));
+    int rc = prefill_write_impl(h, k, v, padded_len, h->plens, by_value ? prompt_lens : nullptr, stream);
     if (rc == SEGKV_OK) h->ragged = true;
     return rc;
 }
 
-static int prefill_write_impl(segkv_t h, const void* k, const void* v, int prompt_len, const int32_t* plens_dev,
-                              void* stream) {
+static int prefill_write_impl(segkv_t h, const void* k, const void* v, int prompt_len, int32_t* plens_dev,
+                              const int32_t* lens_host, void* stream) {
     if (!h || prompt_len < 0) return SEGKV_EINVAL;
     if (prompt_len > h->d.max_prompt) return SEGKV_ECAPACITY;
     if (prompt_len > 0 && (!k || !v || !aligned16(k) || !aligned16(v))) return SEGKV_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     h->tm_valid = false;
     if (prompt_len > 0) {
-        SEGKV_CUDA(launch_prefill_transpose(h->d, k, v, h->kp, h->vp, plens_dev, prompt_len, h->sm_count, st));
+        SEGKV_CUDA(launch_prefill_transpose(h->d, k, v, h->kp, h->vp, plens_dev, lens_host, prompt_len, h->sm_count, st));
         count_launch(h, st);
         int rc = make_prompt_maps(h, prompt_len);
         if (rc != SEGKV_OK) return rc;
@@ -814,7 +829,7 @@ int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_sl
     }
     if (use_wide(h)) {
         SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, wide_splits(h));
-        a.pdl = h->overlap;
+        a.pdl = may_overlap(h);
         h->dbg_wait_ns = 0;
         h->dbg_skip = false;
         SEGKV_CUDA(launch_sdpa_wide(h->d, a, h->tm_kp, h->tm_vp, h->sm_count, (cudaStream_t)stream));
@@ -829,7 +844,7 @@ int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_sl
             if (rc != SEGKV_OK) return rc;
         }
         SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, sp);
-        a.pdl = h->overlap;
+        a.pdl = may_overlap(h);
         h->dbg_wait_ns = 0;
         h->dbg_skip = false;
         SEGKV_CUDA(launch_sdpa_stream(h->d, a, h->tm_kp, h->tm_vp, h->sm_count, (cudaStream_t)stream));
@@ -851,7 +866,7 @@ int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_sl
     a.one_wave = tl.one_wave;
     a.tail_groups = tl.tail_groups;
     a.tail_splits = tl.tail_splits;
-    a.pdl = h->overlap;
+    a.pdl = may_overlap(h);
     a.rows_immutable = rows_settled(h, (cudaStream_t)stream, true);
     h->dbg_wait_ns = 0;                  // an injected fault applies to one launch
     h->dbg_skip = false;
@@ -875,7 +890,7 @@ int segkv_decode_sdpa_static(segkv_t h, const void* q, void* out, const float* a
     const Tiling tl = choose_tiling(h, false);
     const int splits = tl.splits;
     SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, splits);
-    a.pdl = h->overlap;
+    a.pdl = may_overlap(h);
     a.small = tl.small;
     a.one_wave = tl.one_wave;
     int too_big = 0;

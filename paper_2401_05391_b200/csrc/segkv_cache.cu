@@ -15,11 +15,18 @@ namespace segkv_impl {
 // One thread moves one 16-byte chunk; consecutive threads read consecutive
 // chunks of the source.
 // ---------------------------------------------------------------------------
+struct Lens {
+    int n;                                   // 0: none by value
+    int32_t len[kMaxLensByValue];
+};
+
 __global__ void prefill_transpose_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v,
                                          uint4* __restrict__ kp, uint4* __restrict__ vp, int B, int P,
                                          int Hkv, int chunks /* D*2/16 */, long long sb, long long sh,
                                          long long sp /* strides in 16-byte chunks */,
-                                         const int32_t* __restrict__ plens) {
+                                         int32_t* __restrict__ plens, const __grid_constant__ Lens lens) {
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < lens.n; i += blockDim.x) plens[i] = lens.len[i];
     const long long total = (long long)B * P * Hkv * chunks;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -32,14 +39,14 @@ __global__ void prefill_transpose_kernel(const uint4* __restrict__ k, const uint
         long long dst = b * sb + h * sh + p * sp + c;
         // ragged prompts: the padding of a shorter request is stored as zeros, so that a masked
         // key can never put a NaN or an infinity into a weighted sum
-        const bool pad = plens && p >= plens[b];
+        const bool pad = plens && p >= (lens.n ? lens.len[b] : plens[b]);
         kp[dst] = pad ? make_uint4(0u, 0u, 0u, 0u) : k[i];
         vp[dst] = pad ? make_uint4(0u, 0u, 0u, 0u) : v[i];
     }
 }
 
-cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, const int32_t* plens,
-                                     int prompt_len, int sm_count, cudaStream_t st) {
+cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, int32_t* plens,
+                                     const int32_t* lens, int prompt_len, int sm_count, cudaStream_t st) {
     const int chunks = d.head_dim * 2 / 16;
     const PromptStrides ps = prompt_strides(d);
     long long total = (long long)d.batch * prompt_len * d.kv_heads * chunks;
@@ -47,9 +54,12 @@ cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v
     int threads = 256;
     long long blocks = (total + threads - 1) / threads;
     if (blocks > (long long)sm_count * 32) blocks = (long long)sm_count * 32;
+    Lens by_value;
+    by_value.n = lens ? d.batch : 0;
+    for (int b = 0; b < by_value.n; ++b) by_value.len[b] = lens[b];
     prefill_transpose_kernel<<<(unsigned)blocks, threads, 0, st>>>(
         (const uint4*)k, (const uint4*)v, (uint4*)kp, (uint4*)vp, d.batch, prompt_len, d.kv_heads, chunks,
-        ps.b / 8, ps.h / 8, ps.p / 8, plens);
+        ps.b / 8, ps.h / 8, ps.p / 8, plens, by_value);
     return cudaGetLastError();
 }
 

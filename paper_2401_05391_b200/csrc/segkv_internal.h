@@ -110,6 +110,7 @@ struct segkv {
     CUtensorMap tm_kp, tm_vp;
     CUtensorMap tm_kp32, tm_vp32;   // the same arrays in boxes of 32 tokens, for the small-CTA form of the decode kernel
     bool tm_valid;
+    int tm_len, tm_layout;          // prompt length and layout the maps were made for (length -1: none)
 };
 
 namespace segkv_impl {
@@ -125,9 +126,11 @@ struct RopeArgs {
     int head_dim, kv_heads, bf16;
 };
 
-// plens (device, [batch]) or NULL: tokens at or past a request's own length are stored as zeros
-cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, const int32_t* plens,
-                                     int prompt_len, int sm_count, cudaStream_t st);
+// plens (device, [batch]) or NULL: tokens at or past a request's own length are stored as zeros.  lens (host) or NULL: the
+// lengths to use, passed by value and written to plens by the kernel (at most kMaxLensByValue requests).
+constexpr int kMaxLensByValue = 256;
+cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, int32_t* plens,
+                                     const int32_t* lens, int prompt_len, int sm_count, cudaStream_t st);
 
 cudaError_t launch_append(const Dims& d, int step, const int32_t* beam_parent, const void* k_new,
                           const void* v_new, void* kr_slab, void* vr_slab, int32_t* parent_tab,

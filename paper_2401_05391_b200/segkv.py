@@ -121,8 +121,14 @@ def _check(code: int, where: str) -> None:
         raise SegKVError(code, where)
 
 
+# the current stream's handle without a Stream object around it (about 1 us of a call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -130,6 +136,8 @@ def _stream_ptr(stream) -> int:
 def _dev(t: Optional[torch.Tensor], shape, dtype, name: str) -> Optional[int]:
     if t is None:
         return None
+    if t.dtype is dtype and t.shape == shape and t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA tensor")
     if t.dtype != dtype or tuple(t.shape) != tuple(shape):
@@ -174,6 +182,9 @@ class SegKV:
         self.head_dim, self.max_prompt, self.max_steps = head_dim, max_prompt, max_steps
         self.dtype = dtype
         self.rows = batch * beams
+        # what the calls of the decode loop check their tensors against
+        self._kv_shape, self._q_shape = (self.rows, kv_heads, head_dim), (self.rows, heads, head_dim)
+        self._parent_shape, self._slopes_shape = (self.rows,), (heads,)
         code = {torch.float16: SEGKV_F16, torch.bfloat16: SEGKV_BF16}.get(dtype, -1)
         self._h = _vp()
         if chunk_steps:
@@ -245,10 +256,12 @@ class SegKV:
 
     def append(self, step: int, beam_parent: Optional[torch.Tensor], k_new: torch.Tensor, v_new: torch.Tensor,
                stream=None) -> None:
-        shape = (self.rows, self.kv_heads, self.head_dim)
-        _check(lib().segkv_append(self._h, step, _dev(beam_parent, (self.rows,), torch.int32, "beam_parent"),
-                                  _dev(k_new, shape, self.dtype, "k_new"), _dev(v_new, shape, self.dtype, "v_new"),
-                                  _stream_ptr(stream)), "segkv_append")
+        dt = self.dtype
+        code = lib().segkv_append(self._h, step, _dev(beam_parent, self._parent_shape, torch.int32, "beam_parent"),
+                                  _dev(k_new, self._kv_shape, dt, "k_new"), _dev(v_new, self._kv_shape, dt, "v_new"),
+                                  _stream_ptr(stream))
+        if code:
+            _check(code, "segkv_append")
 
     ROPE_STYLES = {"half": 1, "interleaved": 2}
 
@@ -256,38 +269,41 @@ class SegKV:
                     rope_cos: torch.Tensor, rope_sin: torch.Tensor, style="half", stream=None) -> None:
         """append() with the rotary embedding applied to the new K rows; rope_cos / rope_sin are
         device fp32 [positions, head_dim/2]."""
-        shape = (self.rows, self.kv_heads, self.head_dim)
-        n = int(rope_cos.shape[0])
+        dt, n = self.dtype, rope_cos.shape[0]
         tshape = (n, self.head_dim // 2)
-        code = self.ROPE_STYLES[style] if isinstance(style, str) else int(style)
-        _check(lib().segkv_append_rope(self._h, step, _dev(beam_parent, (self.rows,), torch.int32, "beam_parent"),
-                                       _dev(k_new, shape, self.dtype, "k_new"), _dev(v_new, shape, self.dtype, "v_new"),
+        style = self.ROPE_STYLES[style] if isinstance(style, str) else int(style)
+        code = lib().segkv_append_rope(self._h, step, _dev(beam_parent, self._parent_shape, torch.int32, "beam_parent"),
+                                       _dev(k_new, self._kv_shape, dt, "k_new"), _dev(v_new, self._kv_shape, dt, "v_new"),
                                        _dev(rope_cos, tshape, torch.float32, "rope_cos"),
-                                       _dev(rope_sin, tshape, torch.float32, "rope_sin"), n, code,
-                                       _stream_ptr(stream)), "segkv_append_rope")
+                                       _dev(rope_sin, tshape, torch.float32, "rope_sin"), n, style, _stream_ptr(stream))
+        if code:
+            _check(code, "segkv_append_rope")
 
     def decode_sdpa(self, q: torch.Tensor, out: Optional[torch.Tensor] = None,
                     alibi_slopes: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-        shape = (self.rows, self.heads, self.head_dim)
         if out is None:
-            out = torch.empty(shape, dtype=self.dtype, device=q.device)
-        _check(lib().segkv_decode_sdpa(self._h, _dev(q, shape, self.dtype, "q"), _dev(out, shape, self.dtype, "out"),
-                                       _dev(alibi_slopes, (self.heads,), torch.float32, "alibi_slopes"),
-                                       _stream_ptr(stream)), "segkv_decode_sdpa")
+            out = torch.empty(self._q_shape, dtype=self.dtype, device=q.device)
+        dt = self.dtype
+        code = lib().segkv_decode_sdpa(self._h, _dev(q, self._q_shape, dt, "q"), _dev(out, self._q_shape, dt, "out"),
+                                       _dev(alibi_slopes, self._slopes_shape, torch.float32, "alibi_slopes"),
+                                       _stream_ptr(stream))
+        if code:
+            _check(code, "segkv_decode_sdpa")
         return out
 
     def decode_step(self, step: int, beam_parent: Optional[torch.Tensor], k_new: torch.Tensor, v_new: torch.Tensor,
                     q: torch.Tensor, out: Optional[torch.Tensor] = None,
                     alibi_slopes: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-        kv = (self.rows, self.kv_heads, self.head_dim)
-        qs = (self.rows, self.heads, self.head_dim)
         if out is None:
-            out = torch.empty(qs, dtype=self.dtype, device=q.device)
-        _check(lib().segkv_decode_step(self._h, step, _dev(beam_parent, (self.rows,), torch.int32, "beam_parent"),
-                                       _dev(k_new, kv, self.dtype, "k_new"), _dev(v_new, kv, self.dtype, "v_new"),
-                                       _dev(q, qs, self.dtype, "q"), _dev(out, qs, self.dtype, "out"),
-                                       _dev(alibi_slopes, (self.heads,), torch.float32, "alibi_slopes"),
-                                       _stream_ptr(stream)), "segkv_decode_step")
+            out = torch.empty(self._q_shape, dtype=self.dtype, device=q.device)
+        dt, kv, qs = self.dtype, self._kv_shape, self._q_shape
+        code = lib().segkv_decode_step(self._h, step, _dev(beam_parent, self._parent_shape, torch.int32, "beam_parent"),
+                                       _dev(k_new, kv, dt, "k_new"), _dev(v_new, kv, dt, "v_new"),
+                                       _dev(q, qs, dt, "q"), _dev(out, qs, dt, "out"),
+                                       _dev(alibi_slopes, self._slopes_shape, torch.float32, "alibi_slopes"),
+                                       _stream_ptr(stream))
+        if code:
+            _check(code, "segkv_decode_step")
         return out
 
     def decode_sdpa_static(self, q: torch.Tensor, out: torch.Tensor,
@@ -344,15 +360,17 @@ class SegKV:
         _check(lib().segkv_reset(self._h, int(keep_prompt)), "segkv_reset")
 
     def truncate_last(self) -> None:
-        _check(lib().segkv_truncate_last(self._h), "segkv_truncate_last")
+        code = lib().segkv_truncate_last(self._h)
+        if code:
+            _check(code, "segkv_truncate_last")
 
     @property
     def steps(self) -> int:
-        return int(lib().segkv_steps(self._h))
+        return lib().segkv_steps(self._h)
 
     @property
     def prompt_len(self) -> int:
-        return int(lib().segkv_prompt_len(self._h))
+        return lib().segkv_prompt_len(self._h)
 
     def get_ancestry(self, stream=None) -> np.ndarray:
         out = np.empty((self.rows, self.steps), dtype=np.int32)
