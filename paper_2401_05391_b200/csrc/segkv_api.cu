@@ -233,11 +233,13 @@ cudaError_t dmalloc(T** p, size_t bytes) {
     return cudaMalloc((void**)p, bytes ? bytes : 16);
 }
 
+bool wide_possible(const Dims& d);
+
 int alloc_workspace(segkv* h, int splits) {
     const Dims& d = h->d;
     size_t cols = (size_t)d.beams * d.group;
     size_t bytes = (size_t)d.batch * d.kv_heads * splits * cols * (d.head_dim + 2) * sizeof(float);
-    if (!tiled_supported(d)) bytes *= wide_parts(d);
+    if (wide_possible(d)) bytes *= wide_parts(d);
     if (h->ws) {
         cudaFree(h->ws);
         h->ws = nullptr;
@@ -407,24 +409,40 @@ int stream_splits(const segkv* h) {
     return best;
 }
 
-// Which handles take the wide kernel (tcgen05, up to 32 query columns): those the tiled kernel has no form for.
-bool use_wide(const segkv* h) { return !tiled_supported(h->d); }
+// Can the wide kernel (tcgen05, up to 32 query columns) serve this shape at some length?
+bool wide_possible(const Dims& d) { return !tiled_supported(d) || (d.head_dim == 128 && d.beams * d.group > 8); }
 
-// Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA, where a
-// round of items costs its tiles plus about two tiles' time to start and finish an item, and meeting in the
-// workspace costs about two more.
+// Does it serve this call?  Always where the tiled kernel has no form.  Nine to 16 columns at head_dim 128 run on
+// either: the wide kernel needs a few microseconds more to start, finish and (with an append of its own) fuse
+// nothing, and gets keys through faster.  Measured step, tiled / wide in us, at work groups x prompt = 8 K: 14.1 / 21.2
+// (4 x 2048), 9.8 / 14.0 (16 x 512); at 16 K: 28.8 / 21.8 (4 x 4096), 19.3 / 14.7 (16 x 1024), 18.5 / 14.7 (32 x 512),
+// 21.3 / 11.3 (128 x 128); at 128 K 31 / 21 (128 x 1024).  (At head_dim 64 the tiled kernel stays ahead: 11.6 / 20.8 at
+// 240 x 634.)  A handle whose launch shape has been set by hand keeps the kernel that the setting is for.
+bool use_wide(const segkv* h) {
+    if (!tiled_supported(h->d)) return true;
+    return wide_possible(h->d) && h->splits_forced == 0 && h->stages_forced == 0 && h->combine_forced == 0 && h->tile_forced == 0 &&
+           h->overlap && (long long)h->d.batch * h->d.kv_heads * (h->prompt_len > 0 ? h->prompt_len : 0) >= 16384;
+}
+
+// Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA.  In units of a tile
+// (0.65 us): a round of items costs its tiles plus about two to start and finish an item; meeting in the
+// workspace costs about four (a partial's stores, the arrival, one trip for the factors) plus one per 16 loads of
+// the last CTA's threads.
 int wide_splits(const segkv* h) {
     const Dims& d = h->d;
+    const int most = wide_max_splits(d) < h->ws_splits ? wide_max_splits(d) : h->ws_splits;
+    if (h->splits_forced > 0) return h->splits_forced < most ? h->splits_forced : most;
     const long long slabs = (long long)d.batch * d.kv_heads;
     const int keys = wide_tile_keys(d);
     const long long ntp = ((h->prompt_len > 0 ? h->prompt_len : 0) + keys - 1) / keys;
     const long long ntr = (h->steps + 2 * d.beams + keys - 1) / keys;      // estimate, rows are mostly shared
-    if (h->splits_forced > 0) return h->splits_forced;
+    const long long passes = ((long long)d.beams * d.group * d.head_dim + 2047) / 2048;
     int best = 1;
     long long best_cost = 0;
-    for (int s = 1; s <= h->ws_splits && s <= kMaxSplits && s <= ntp + ntr; ++s) {
+    for (int s = 1; s <= most && s <= ntp + ntr; ++s) {
         const long long rounds = (slabs * s + h->sm_count - 1) / h->sm_count;
-        const long long cost = rounds * ((ntp + s - 1) / s + (ntr + s - 1) / s + 2) + (s > 1 ? 2 : 0);
+        const long long merge = s > 1 ? 4 + passes * ((s * wide_parts(d) + 3) / 4) : 0;
+        const long long cost = rounds * ((ntp + s - 1) / s + (ntr + s - 1) / s + 2) + merge;
         if (s == 1 || cost < best_cost) {
             best = s;
             best_cost = cost;

@@ -40,6 +40,18 @@ using namespace ptx;
 constexpr int kTicketAbortedW = 1 << 16;     // same marker as the tiled kernel's
 constexpr int kCols = kMaxCols;              // query columns of a work group, padded: one tensor-memory lane each
 
+// Loads of the split merge, from the L2 (other SMs wrote the data), issued in program order.
+__device__ __forceinline__ float4 ldcg4(const float4* a) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(a));
+    return v;
+}
+__device__ __forceinline__ float2 ldcg2(const float2* a) {
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(a));
+    return v;
+}
+
 struct WideParams {
     const void* q;
     void* out;
@@ -619,38 +631,69 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * kParts * p.ncols * 2);
             const float* o0 = p.ws_o + (size_t)it0 * kParts * p.ncols * D;
             const int parts = p.S * kParts;
-            constexpr int D4 = D / 4;
-            for (int e = tid; e < p.ncols * D4; e += 128) {
-                const int col = e / D4, d = (e % D4) * 4;
+            // Two passes: each part's factor per column, then 16 loads in flight per thread.  (One float4 of one column at
+            // a time, its parts' loads ordered by the use of each, cost most of the about 7 us that merging four splits took.)
+            float* fac = reinterpret_cast<float*>(p_smem);        // [part][32 columns]: 2^(m_part - m) / sum
+            if (warp == 0 && real) {
                 float mm = -INFINITY, ll = 0.f;
-                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
                 for (int s0 = 0; s0 < parts; s0 += 8) {
                     float2 ml[8];
-                    float4 w[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const bool in = s0 + u < parts;
-                        ml[u] = in ? __ldcg(ml0 + (size_t)(s0 + u) * p.ncols + col) : make_float2(-INFINITY, 0.f);
-                        w[u] = in ? __ldcg(reinterpret_cast<const float4*>(o0 + ((size_t)(s0 + u) * p.ncols + col) * D + d))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
                     float bm = mm;
 #pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        ml[u] = ldcg2(ml0 + (size_t)min(s0 + u, parts - 1) * p.ncols + lane);
+                        if (s0 + u >= parts) ml[u] = make_float2(-INFINITY, 0.f);
+                    }
+#pragma unroll
                     for (int u = 0; u < 8; ++u) bm = fmaxf(bm, ml[u].x);
-                    const float fo = mm == -INFINITY ? 0.f : exp2f(mm - bm);
-                    ll *= fo; o.x *= fo; o.y *= fo; o.z *= fo; o.w *= fo;
+                    ll *= mm == -INFINITY ? 0.f : exp2f(mm - bm);
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        const float f = ml[u].x == -INFINITY ? 0.f : exp2f(ml[u].x - bm);
-                        ll += ml[u].y * f;
-                        o.x += w[u].x * f; o.y += w[u].y * f; o.z += w[u].z * f; o.w += w[u].w * f;
+                        ll += ml[u].x == -INFINITY ? 0.f : ml[u].y * exp2f(ml[u].x - bm);
+                        if (s0 + u < parts) fac[(s0 + u) * kCols + lane] = ml[u].x;
                     }
                     mm = bm;
                 }
                 const float inv = 1.f / ll;
-                T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + col / p.G) * p.H + done.kvh * p.G + col % p.G) * D + d;
-                *reinterpret_cast<uint2*>(orow) = make_uint2(Mma<T>::pack(o.x * inv, o.y * inv), Mma<T>::pack(o.z * inv, o.w * inv));
+                for (int u = 0; u < parts; ++u) {
+                    const float m = fac[u * kCols + lane];
+                    fac[u * kCols + lane] = m == -INFINITY ? 0.f : exp2f(m - mm) * inv;
+                }
             }
+            bar_sync_n(1, 128);
+            constexpr int D4 = D / 4, NE = 4;
+            const int n4 = p.ncols * D4;
+            for (int e0 = tid; e0 < n4; e0 += 128 * NE) {
+                float4 o[NE];
+#pragma unroll
+                for (int i = 0; i < NE; ++i) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                for (int s0 = 0; s0 < parts; s0 += 4) {
+                    float4 w[NE][4];
+#pragma unroll
+                    for (int i = 0; i < NE; ++i)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            w[i][u] = ldcg4(reinterpret_cast<const float4*>(o0) + (size_t)min(s0 + u, parts - 1) * n4 + min(e0 + 128 * i, n4 - 1));
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (s0 + u >= parts) break;
+#pragma unroll
+                        for (int i = 0; i < NE; ++i) {
+                            const float f = fac[(s0 + u) * kCols + min(e0 + 128 * i, n4 - 1) / D4];
+                            o[i].x += w[i][u].x * f; o[i].y += w[i][u].y * f; o[i].z += w[i][u].z * f; o[i].w += w[i][u].w * f;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < NE; ++i) {
+                    const int e = e0 + 128 * i, col = e / D4, d = (e % D4) * 4;
+                    if (e >= n4) break;
+                    T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + col / p.G) * p.H + done.kvh * p.G + col % p.G) * D + d;
+                    *reinterpret_cast<uint2*>(orow) = make_uint2(Mma<T>::pack(o[i].x, o[i].y), Mma<T>::pack(o[i].z, o[i].w));
+                }
+            }
+            bar_sync_n(1, 128);                                   // the factors' place takes weights again
         }
         if (gone) {
             if (tid == 0) {
@@ -745,10 +788,16 @@ cudaError_t dispatch(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, c
 
 int wide_parts(const Dims& d) { return d.dtype == SEGKV_BF16 ? 2 : 1; }
 
+// the split merge keeps one factor per part and column where the weights were
+int wide_max_splits(const Dims& d) {
+    const int n = (d.head_dim == 256 ? WideLayout<256>::kP : WideLayout<128>::kP) / (kCols * 4 * wide_parts(d));
+    return n < kMaxSplits ? n : kMaxSplits;
+}
+
 int wide_tile_keys(const Dims& d) { return d.head_dim == 256 ? WideLayout<256>::KEYS : WideLayout<128>::KEYS; }
 
 cudaError_t launch_sdpa_wide(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
-    if (a.splits < 1 || a.splits > kMaxSplits || d.beams * d.group > kCols) return cudaErrorInvalidValue;
+    if (a.splits < 1 || a.splits > wide_max_splits(d) || d.beams * d.group > kCols) return cudaErrorInvalidValue;
     return d.dtype == SEGKV_BF16 ? dispatch<__nv_bfloat16>(d, a, tmk, tmv, sms, st) : dispatch<__half>(d, a, tmk, tmv, sms, st);
 }
 

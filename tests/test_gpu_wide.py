@@ -81,3 +81,24 @@ def test_wide_wait_runs_out_and_the_handle_recovers(splits):
         assert np.array_equal(r.h.get_ancestry(), r.oracle_ancestry(3))
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("dtype,beams,group", [("f16", 3, 3), ("bf16", 4, 4)])
+def test_nine_to_sixteen_columns_on_both_sides_of_the_dispatch(dtype, beams, group):
+    # head_dim 128: from 16384 prompt keys over all work groups on, these columns run on the wide kernel
+    for P, wide in ((511, False), (512, True)):
+        w = _w("nt2", 4, beams, group, 8, 128, P, 20, dtype, alibi=group == 4, seed=6)
+        run_workload(w, sampled_pairs, check_steps=(0, 19), every_step_ancestry=False)
+        run_workload_fused(w, sampled_pairs, check_steps=(0, 7, 19))
+
+
+def test_more_forced_splits_than_the_merge_has_room_for():
+    w = _w("cap", 1, 4, 8, 1, 256, 100, 4, "bf16", seed=7)
+    r = Run(w, splits=64)
+    try:
+        r.advance_to(3)
+        assert r.h.get_splits() == 32                  # two partials (high and low parts) per split
+        out, q = r.decode()
+        r.check(out, q, 3, all_pairs(w))
+    finally:
+        r.close()
