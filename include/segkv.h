@@ -200,7 +200,8 @@ SEGKV_API int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float
  * following steps.  Saves a launch and a dependent memory round trip per layer.
  * Arguments, layouts and errors are those of the two calls.  The library runs
  * the step as the two launches instead where that is the faster form or the only
- * one: shapes with more than 16 query columns per kv head, handles that share
+ * one: shapes with many query columns per kv head (more than 16, or more than 8
+ * at head_dim 256 or over long prompts at head_dim 128), handles that share
  * another handle's tables, launches whose work groups fill the GPU without being
  * split, and launches whose CTAs would each have many steps' rows or many prompt
  * tiles to go through.  Both forms give the same beam-index tables bit by bit and
@@ -383,8 +384,8 @@ SEGKV_API int segkv_get_splits(segkv_t h);
 /*
  * The same attention as segkv_decode_sdpa computed by the plain per-beam kernel
  * (each beam walks its own rows through the beam-index table, Section 3.3's
- * formulation taken literally; the prompt is re-read per beam).  Used for
- * shapes with more than 16 query columns per kv head, and as a cross-check.
+ * formulation taken literally; the prompt is re-read per beam).  A
+ * cross-check; no other entry point uses it.
  * Arguments and errors as segkv_decode_sdpa.
  */
 SEGKV_API int segkv_decode_sdpa_rowwise(segkv_t h, const void* q, void* out, const float* alibi_slopes,
