@@ -558,7 +558,8 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // the row know that it stands.  (Not under a slope that lifts the maximum
                 // by 2^4 and more from tile to tile; nor in bf16, whose two kinds of weights leave no registers for it:
                 // 2.61 against 1.92 ms at 32 x 112 heads x 1024 with ALiBi.)
-                bool stands = !kSplitP && kt > 0 && slope2 * (float)kKeys < 4.f;
+                const int steady = slope2 * (float)kKeys < 4.f;
+                bool stands = !kSplitP && kt > 0 && steady;
                 if (stands) {
                     float mx = -INFINITY;
                     uint32_t pk[KH / 2];
@@ -609,7 +610,8 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         }
                     }
                     bool need = tmax > m_ref + 8.f;
-                    if (!bar_and(pair, 64, ok && !need)) {            // the two threads of a row compare notes only then
+                    // the two threads of a row compare notes only then (at once where a new reference is expected)
+                    if (kt == 0 || steady < 1 || !bar_and(pair, 64, ok && !need)) {
                         if (half == 0) *xrow = tmax;
                         ok = bar_and(pair, 64, ok);
                         gone = !ok;
@@ -624,32 +626,6 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         if (need) {
                             alpha = exp2f(m_ref - tmax);               // 0 on the first tile
                             m_ref = tmax;
-                        }
-                        // O is rescaled (half a row per thread) before any weight of this tile is handed over, once P.V of the
-                        // previous tile is done
-                        if (kt > 0 && __any_sync(0xffffffffu, need)) {
-                            ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
-                            ok = __all_sync(0xffffffffu, ok);
-                            if (ok) {
-                                tc_fence_after();
-#pragma unroll 1
-                                for (int c = 0; c < DH / 16; ++c) {
-                                    uint32_t orr[16];
-                                    tc_ld16(tm_o + c * 16, orr);
-                                    tc_wait_ld();
-                                    pin<16>(orr);
-#pragma unroll
-                                    for (int i = 0; i < 16; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
-                                    tc_st16(tm_o + c * 16, orr);
-                                }
-                                tc_wait_st();
-                                tc_fence_before();
-                            }
-                            ok = bar_and(pair, 64, ok);                // both halves are
-                            gone = !ok;
-                            if (gone) break;
-                            tc_fence_after();
-                            if (stamp) TC5_STAMP(g, kt, 3);
                         }
                     }
                     ls[0] = ls[1] = 0ull;
@@ -674,6 +650,26 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                             }
                         }
                         tc_st16(tm_sh + c, hi);
+                    }
+                    // O is rescaled, half a row per thread, before this thread hands over its weights (the MMA thread waits for both
+                    // threads'), once P.V of the previous tile is done: after the weights, under which that P.V runs
+                    if (kt > 0 && __any_sync(0xffffffffu, need)) {
+                        ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (ok) {
+                            tc_fence_after();
+#pragma unroll 1
+                            for (int c = 0; c < DH / 16; ++c) {
+                                uint32_t orr[16];
+                                tc_ld16(tm_o + c * 16, orr);
+                                tc_wait_ld();
+                                pin<16>(orr);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) orr[i] = __float_as_uint(__uint_as_float(orr[i]) * alpha);
+                                tc_st16(tm_o + c * 16, orr);
+                            }
+                        }
+                        if (stamp) TC5_STAMP(g, kt, 3);
                     }
                 }
                 const uint64_t lt = f2_add(ls[0], ls[1]);

@@ -3,8 +3,7 @@
 // direct transcription of the paper's per-beam formulation (Section 3.3): loop
 // over the prompt rows, then over the index-selected response rows, one online
 // softmax across both.  It re-reads the prompt once per beam, so it is not the
-// fast path; the library uses it for shapes the tiled kernel does not take and
-// exposes it as a cross-check.
+// fast path; the library exposes it as a cross-check.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
