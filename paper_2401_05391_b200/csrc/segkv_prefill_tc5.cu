@@ -556,10 +556,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // The reference in use nearly always stands after the first tile: the weights are worked out with it
                 // in one pass over the scores that notes their maximum on the way, and stored when both threads of
                 // the row know that it stands.  (Not under a slope that lifts the maximum
-                // by 2^4 and more from tile to tile; nor in bf16, whose two kinds of weights leave no registers for it:
+                // by 2^4 and more from tile to tile; nor in bf16 with two groups, whose two kinds of weights leave no registers for it, or with ALiBi, 30.2 against 26.7 us at 1 x 32 x 1024:
                 // 2.61 against 1.92 ms at 32 x 112 heads x 1024 with ALiBi.)
-                const int steady = slope2 * (float)kKeys < 4.f;
-                bool stands = !kSplitP && kt > 0 && steady;
+                const bool steady = slope2 * (float)kKeys < 4.f;
+                bool stands = (!kSplitP || (NG == 1 && !biased)) && kt > 0 && !two && steady;
                 if (stands) {
                     float mx = -INFINITY;
                     uint32_t pk[KH / 2];
@@ -611,7 +611,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     }
                     bool need = tmax > m_ref + 8.f;
                     // the two threads of a row compare notes only then (at once where a new reference is expected)
-                    if (kt == 0 || steady < 1 || !bar_and(pair, 64, ok && !need)) {
+                    if (kt == 0 || !steady || !bar_and(pair, 64, ok && !need)) {
                         if (half == 0) *xrow = tmax;
                         ok = bar_and(pair, 64, ok);
                         gone = !ok;
@@ -678,7 +678,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // With one S buffer these scores were issued behind P.V of the previous tile, which keeps the O and P
                 // barriers at the phases waited for; with two, where a thread could run two phases ahead of the
                 // MMA thread, every phase of the O barrier is waited for in turn.
-                if (NB == 2 && kt > 0) {
+                if (NB == 2 && kt > 0 && ok) {
                     ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
                     ok = __all_sync(0xffffffffu, ok);
                 }
