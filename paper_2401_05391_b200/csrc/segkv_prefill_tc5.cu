@@ -555,9 +555,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 uint64_t ls[2] = {0ull, 0ull};
                 // The reference in use nearly always stands after the first tile: the weights are worked out with it
                 // in one pass over the scores that notes their maximum on the way, and stored when both threads of
-                // the row know that it stands.  (Not under a slope that lifts the maximum
-                // by 2^4 and more from tile to tile; nor in bf16 with two groups, whose two kinds of weights leave no registers for it, or with ALiBi, 30.2 against 26.7 us at 1 x 32 x 1024:
-                // 2.61 against 1.92 ms at 32 x 112 heads x 1024 with ALiBi.)
+                // the row know that it stands.  (Not under a slope that lifts the maximum by 2^4 and more from tile to
+                // tile; nor in bf16 with two groups, whose two kinds of weights leave no registers for it, 2.61 against
+                // 1.92 ms at 32 x 112 heads x 1024 with ALiBi, or with a bias, 30.2 against 26.7 us at 1 x 32 x 1024.)
                 const bool steady = slope2 * (float)kKeys < 4.f;
                 bool stands = (!kSplitP || (NG == 1 && !biased)) && kt > 0 && !two && steady;
                 if (stands) {
