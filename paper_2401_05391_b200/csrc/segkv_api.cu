@@ -233,13 +233,10 @@ cudaError_t dmalloc(T** p, size_t bytes) {
     return cudaMalloc((void**)p, bytes ? bytes : 16);
 }
 
-bool wide_possible(const Dims& d);
-
 int alloc_workspace(segkv* h, int splits) {
     const Dims& d = h->d;
     size_t cols = (size_t)d.beams * d.group;
     size_t bytes = (size_t)d.batch * d.kv_heads * splits * cols * (d.head_dim + 2) * sizeof(float);
-    if (wide_possible(d)) bytes *= wide_parts(d);
     if (h->ws) {
         cudaFree(h->ws);
         h->ws = nullptr;
@@ -441,7 +438,7 @@ int wide_splits(const segkv* h) {
     long long best_cost = 0;
     for (int s = 1; s <= most && s <= ntp + ntr; ++s) {
         const long long rounds = (slabs * s + h->sm_count - 1) / h->sm_count;
-        const long long merge = s > 1 ? 4 + passes * ((s * wide_parts(d) + 3) / 4) : 0;
+        const long long merge = s > 1 ? 4 + passes * ((s + 3) / 4) : 0;
         const long long cost = rounds * ((ntp + s - 1) / s + (ntr + s - 1) / s + 2) + merge;
         if (s == 1 || cost < best_cost) {
             best = s;

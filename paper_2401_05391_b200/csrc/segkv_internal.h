@@ -209,7 +209,6 @@ cudaError_t launch_sdpa_tiled(const Dims& d, const SdpaArgs& a, const CUtensorMa
 // walks the (work group, split) items; a.splits items per work group, merged through the workspace.
 int wide_tile_keys(const Dims& d);
 int wide_max_splits(const Dims& d);
-int wide_parts(const Dims& d);                           // partial outputs an item leaves in the workspace
 cudaError_t launch_sdpa_wide(const Dims& d, const SdpaArgs& a, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                              int sm_count, cudaStream_t st);
 

@@ -14,17 +14,19 @@
 //    rows cost MMA time the tensor pipe has to spare: 8 + 4 MMAs per 32 KB of keys and values, about 900
 //    clocks, against about 1300 clocks for an SM's share of HBM bandwidth;
 //  * the four warps agree on a column's maximum through shared memory (one barrier per tile, which also
-//    carries the "a wait ran out" flag, so that all warps leave together) and write the weights P, rounded
-//    to the 16-bit type, into ONE shared-memory tile of 32 rows: the A operand of O[128, D] += P.V, whose rows
-//    past the real ones are never read.  bf16 weights go in two parts (p = hi + lo, 16 significant bits):
-//    hi in rows 0..31, lo in rows 32..63 of the same MMA, added up in the epilogue, at no extra MMA;
+//    carries the "a wait ran out" flag, so that all warps leave together) and write the weights P into ONE
+//    shared-memory tile, the A operand of O[128, D] += P.V.  The weights keep what fp32 has of them: they go as the
+//    sum of two fp16 or three bf16 parts, each part 32 rows of the same MMA, which has rows to spare, and the
+//    parts of O are added up in the epilogue.  (One fp16 part: error against 64 bits 2.9e-4 of the result instead
+//    of the 2.1e-4 that rounding the output takes; two bf16 parts: 1.65e-3, which is that rounding, but five times
+//    as many outputs are not the nearest number, 0.25 %.)  Rows past the parts' are never read;
 //  * O stays in tensor memory and is rescaled only when a column's maximum has grown by more than 2^8 over
 //    the reference in use (sum and weights use the same reference, so the result is exact);
 //  * prompt tiles arrive by TMA in one ring; response tiles are gathered row by row (cp.async into the same
 //    128-byte-swizzled layout) by two groups of two warps, one stage each, so that two gathers are in
 //    flight; the gather warps also place the query block;
-//  * splits of a work group meet in the global workspace: the last CTA to arrive folds them (as in the tiled
-//    kernel).
+//  * splits of a work group meet in the global workspace, the parts of each added up: the last CTA to arrive folds
+//    them (as in the tiled kernel).
 // Every mbarrier is waited on phase by phase and every wait is bounded; on expiry the kernel flags
 // SEGKV_DEV_WAIT_LIMIT, leaves the output alone and still releases its tensor memory and its tickets.
 #include "segkv_internal.h"
@@ -62,8 +64,8 @@ struct WideParams {
     const URow* ulist;
     const int32_t* ucount;
     const int32_t* plens;
-    float* ws_o;                   // [item][part][ncols][D] un-normalised partial outputs (bf16: high and low parts)
-    float* ws_ml;                  // [item][part][ncols][2] reference maximum (base-2 domain) and sum
+    float* ws_o;                   // [item][ncols][D] un-normalised partial outputs
+    float* ws_ml;                  // [item][ncols][2] reference maximum (base-2 domain) and sum
     int* tickets;
     int* err_word;
     int P, steps, S, W, G, H, Hkv, rows, max_steps, ncols, chunk_steps, quota, items;
@@ -73,9 +75,39 @@ struct WideParams {
     uint32_t idesc_qk, idesc_pv;
 };
 
-template <int D_>
+// A softmax weight as a sum of 16-bit parts for the tensor cores, with what fp32 has of it: fp16 in two (22 bits), bf16
+// in three cut off one behind the other (8 bits each: all 24).  fp16 weights carry a factor of 2^7 (the sum does
+// too), so that parts below fp16's smallest number are 2^-31 of the largest weight and not 2^-24.
+template <typename T> struct Parts;
+template <> struct Parts<__half> {
+    static constexpr int kNum = 2;
+    static constexpr float kShift = 7.f;              // the largest weight is 2^8 times this factor: 2^15
+    static __device__ __forceinline__ void split(float a, float c, uint32_t* w) {
+        const __half2 h = __floats2half2_rn(a, c);
+        const float2 f = __half22float2(h);
+        w[0] = *reinterpret_cast<const uint32_t*>(&h);
+        w[1] = ptx::Mma<__half>::pack(a - f.x, c - f.y);
+    }
+};
+template <> struct Parts<__nv_bfloat16> {
+    static constexpr int kNum = 3;
+    static constexpr float kShift = 0.f;
+    static __device__ __forceinline__ void split(float a, float c, uint32_t* w) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t x = __float_as_uint(a), y = __float_as_uint(c);
+            w[i] = __byte_perm(x, y, 0x7632);
+            a -= __uint_as_float(x & 0xFFFF0000u);
+            c -= __uint_as_float(y & 0xFFFF0000u);
+        }
+        w[2] = ptx::Mma<__nv_bfloat16>::pack(a, c);
+    }
+};
+
+template <typename T, int D_>
 struct WideLayout {
     static constexpr int D = D_;
+    static constexpr int kParts = Parts<T>::kNum;
     static constexpr int KEYS = D == 256 ? 32 : 64;              // keys of a tile: one box of the prompt's tensor map
     static constexpr int KW = KEYS / 4;                          // keys of a softmax warp
     static constexpr int kDBoxes = D / 64;                       // 128-byte column blocks of a row
@@ -84,16 +116,21 @@ struct WideLayout {
     static constexpr int kStage = 2 * kTile;
     static constexpr int SP = D == 64 ? 8 : 4;                   // prompt stages
     static constexpr int SR = 2;                                 // response stages: one per gather group
-    static constexpr int kPRows = 64 * 128;                      // weights of a tile: 32 rows hi, 32 rows lo, 128 bytes each
+    static constexpr int kPRows = kParts * 32 * 128;             // weights of a tile: 32 rows of each part, 128 bytes each
     // two buffers of weights: tiles of 32 keys fill half a row each, and the other half is the other buffer
     static constexpr int kPBuf = KEYS == 32 ? 64 : kPRows;
     static constexpr int kP = KEYS == 32 ? kPRows : 2 * kPRows;
     static constexpr int kQ = kCols * D * 2;                     // the next query block, on its way to tensor memory
     static constexpr int kMeta = SR * KEYS * (int)sizeof(URow);
-    static constexpr int kPtr = SR * KEYS * 8;
     static constexpr int kMax = 2 * 4 * kCols * 4, kSum = 4 * kCols * 4;
     static constexpr int kBars = 3 * SP + 2 * SR + 3 + 6 + 1;    // rings, query, S/P/O x 2, wind-down
-    static constexpr size_t kBytes = 1024 + (size_t)kP + kQ + (SP + SR) * kStage + kMeta + kPtr + kMax + kSum + 8 * kBars + 64;
+    // the small arrays first, then, on a swizzle atom's boundary, weights, rings and the query block
+    static constexpr int kSmall = (kMeta + kMax + kSum + 8 * kBars + 16 + 1023) & ~1023;
+    static constexpr size_t kBytes = (size_t)kSmall + kP + (SP + SR) * kStage + kQ;
+    // the parts of O meet in shared memory, where the weights were, XC of D at a time in two buffers in turn
+    static constexpr int kXch = (kParts - 1) * kCols * 4;        // bytes of one of D
+    static constexpr int XC = kP >= 64 * kXch ? 32 : 16;
+    static_assert(2 * XC * kXch <= kP, "exchange of the parts");
     // tensor memory: two S buffers, O, and the query block (16-bit, two elements per column)
     static constexpr int kColO = 2 * KEYS, kColQ = kColO + D, kColEnd = kColQ + D / 2;
     static constexpr int kTmemCols = kColEnd <= 256 ? 256 : 512;
@@ -105,28 +142,26 @@ struct WideLayout {
 template <typename T, int D>
 __global__ void __launch_bounds__(320, 1)
 sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const WideParams p) {
-    using L = WideLayout<D>;
+    using L = WideLayout<T, D>;
     constexpr int KEYS = L::KEYS, KW = L::KW, SP = L::SP, SR = L::SR;
-    constexpr bool kTwoPart = !Mma<T>::kWeights11Bits;
-    constexpr int kParts = kTwoPart ? 2 : 1;                      // partial outputs of an item in the split workspace
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* p_smem = smem;                                       // two buffers; their A operands reach into the ring behind
+    constexpr int kParts = L::kParts;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    URow* meta = reinterpret_cast<URow*>(smem);
+    float* s_max = reinterpret_cast<float*>(meta + SR * KEYS);    // [2][4 warps][kCols]
+    float* s_sum = s_max + 2 * 4 * kCols;                         // [4 warps][kCols]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(s_sum + 4 * kCols);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
+    volatile int* s_flags = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int &s_abort = s_flags[0], &s_ticket = s_flags[1];
+    uint8_t* p_smem = smem + L::kSmall;                           // two buffers; their A operands reach into the ring behind
     uint8_t* p_ring = p_smem + L::kP;
     uint8_t* r_ring = p_ring + (size_t)SP * L::kStage;
     uint8_t* q_smem = r_ring + (size_t)SR * L::kStage;            // [32 rows][D], 16-byte chunks XOR-swizzled by the row
-    URow* meta = reinterpret_cast<URow*>(q_smem + L::kQ);
-    const char** gk = reinterpret_cast<const char**>(meta + SR * KEYS);
-    float* s_max = reinterpret_cast<float*>(gk + SR * KEYS);      // [2][4 warps][kCols]
-    float* s_sum = s_max + 2 * 4 * kCols;                         // [4 warps][kCols]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(s_sum + 4 * kCols);
     const uint32_t pfull = smem_u32(bars), kempty = pfull + 8 * SP, vempty = kempty + 8 * SP;
     const uint32_t rfull = vempty + 8 * SP, rempty = rfull + 8 * SR, qfull = rempty + 8 * SR;
     const uint32_t sfull = qfull + 8, sempty = sfull + 8;         // the query block in shared memory
     const uint32_t bar_s = sempty + 8, bar_p = bar_s + 16, bar_o = bar_p + 16;     // two each: tile parity
     const uint32_t bar_end = bar_o + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
-    __shared__ int s_abort, s_ticket;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -297,11 +332,11 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         // ------------------- the query block, and response tiles: index select fused into the load -------------------
         const int grp = (warp - 6) >> 1, gt = tid - 192 - grp * 64, bid = 2 + grp;
         constexpr int CPR = D / 8;                                // 16-byte chunks per row
-        constexpr int RPI = 64 / CPR;                             // rows the group's threads cover at once
+        constexpr int RW = KEYS / 2, RPI = 32 / CPR;              // rows of a tile that a warp fetches, and how many at once
         const size_t slab_bytes = (size_t)p.rows * p.Hkv * (size_t)(D * 2);
         uint8_t* stage = r_ring + (size_t)grp * L::kStage;        // the group's stage
+        const int wrow = (gt >> 5) * RW;                          // the warp's first row
         URow* meta_g = meta + grp * KEYS;
-        const char** gk_g = gk + grp * KEYS;
         uint32_t rn = 0, qi = 0;
         bool ok = true;
         for (int it = blockIdx.x; it < p.items && ok; it += gridDim.x) {
@@ -336,28 +371,28 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 const uint32_t pos = rn + (uint32_t)r;
                 if ((pos & 1) != (uint32_t)grp) continue;         // the other group's tile
                 const int eb = e0 + r * KEYS, cnt = min(KEYS, e1 - eb);
-                URow u = {0, 0u};
-                if (gt < cnt) u = list[eb + gt];
+                URow u = {0, 0u};                                 // lane i < RW: the warp's row i
+                if (lane < RW && wrow + lane < cnt) u = list[eb + wrow + lane];
                 ok = mbar_wait(rempty + 8 * grp, ((pos >> 1) & 1) ^ 1, p.wait_ns);
                 ok = bar_and(bid, 64, ok);
                 if (!ok) break;
-                if (gt < KEYS) {
+                unsigned long long row_at;
+                {
                     const int s = u.row / p.rows;
                     const char* base = p.chunk_steps == 0 ? p.kr + (size_t)s * slab_bytes
                                                           : p.k_chunks[s / p.chunk_steps] + (size_t)(s % p.chunk_steps) * slab_bytes;
-                    gk_g[gt] = base + ((size_t)(u.row - s * p.rows) * p.Hkv + x.kvh) * (size_t)(D * 2);
+                    row_at = (unsigned long long)(base + ((size_t)(u.row - s * p.rows) * p.Hkv + x.kvh) * (size_t)(D * 2));
                     u.row = s;                                    // the softmax threads need the step only
-                    meta_g[gt] = u;                               // (no beam reads the padding of the last tile)
+                    if (lane < RW) meta_g[wrow + lane] = u;       // (no beam reads the padding of the last tile)
                 }
-                bar_sync_n(bid, 64);
-                const int c = gt % CPR;
+                const int c = lane % CPR;
                 uint8_t* dst0 = stage + (size_t)(c >> 3) * L::kColTile;
 #pragma unroll 4
-                for (int i = 0; i < KEYS / RPI; ++i) {
-                    const int key = i * RPI + gt / CPR;
+                for (int i = 0; i < RW / RPI; ++i) {
+                    const int row = i * RPI + lane / CPR, key = wrow + row;
+                    const char* src = reinterpret_cast<const char*>(__shfl_sync(0xffffffffu, row_at, row)) + c * 16;
                     uint8_t* dst = dst0 + key * 128 + (((c & 7) ^ (key & 7)) << 4);
                     if (key < cnt) {
-                        const char* src = gk_g[key] + c * 16;
                         cp_async_16(smem_u32(dst), src);
                         cp_async_16(smem_u32(dst + L::kTile), src + p.vdelta);
                     } else {                                      // a weight of zero times whatever was here need not be zero
@@ -377,7 +412,7 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         // ---------------------- softmax warps: one column per lane, a quarter of the keys per warp ----------------------
         const uint32_t tm_lane = tmem + ((uint32_t)(warp * 32) << 16);
         const uint32_t tm_o = tm_lane + (uint32_t)L::kColO;
-        const bool owns_o = warp == 0 || (kTwoPart && warp == 1);    // rows 0..31 of O, and 32..63 for the low parts
+        const bool owns_o = warp < kParts;                        // the first part's rows of O are 0..31, the second's 32..63, ...
         const bool real = lane < p.ncols;
         const int beam = real ? lane / p.G : 0, hg = real ? lane % p.G : 0;
         const uint32_t beambit = real ? 1u << beam : 0u;
@@ -463,19 +498,18 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 // The reference in use nearly always stands, so the weights are worked out with it before the warps
                 // meet; that one of them needs a new one is found at the meeting.
                 float ls[2];
-                uint32_t hi[KW / 2], lo[KW / 2];
+                uint32_t wp[kParts][KW / 2];
                 auto weigh = [&]() {
-                    const float m_use = m_ref == -INFINITY ? 0.f : m_ref;       // no key of this column so far
+                    const float m_use = m_ref == -INFINITY ? 0.f : m_ref - Parts<T>::kShift;    // no key of this column so far
                     ls[0] = ls[1] = 0.f;
 #pragma unroll
                     for (int i = 0; i < KW; i += 2) {
                         const float a = exp2f(v[i] - m_use), c = exp2f(v[i + 1] - m_use);
                         ls[(i >> 1) & 1] += a + c;
-                        hi[i >> 1] = Mma<T>::pack(a, c);
-                        if (kTwoPart) {
-                            const uint32_t h = hi[i >> 1];
-                            lo[i >> 1] = Mma<T>::pack(a - __uint_as_float(h << 16), c - __uint_as_float(h & 0xFFFF0000u));
-                        }
+                        uint32_t w[kParts];
+                        Parts<T>::split(a, c, w);
+#pragma unroll
+                        for (int k = 0; k < kParts; ++k) wp[k][i >> 1] = w[k];
                     }
                 };
                 if (ok) weigh();
@@ -520,9 +554,9 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 #pragma unroll
                     for (int c = 0; c < KW / 8; ++c) {
                         const int ch = (((KEYS == 32 ? 4 * (int)buf : 0) + warp * (KW / 8) + c) ^ (lane & 7)) << 4;
-                        *reinterpret_cast<uint4*>(dst + ch) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
-                        if (kTwoPart)
-                            *reinterpret_cast<uint4*>(dst + 32 * 128 + ch) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
+#pragma unroll
+                        for (int k = 0; k < kParts; ++k)
+                            *reinterpret_cast<uint4*>(dst + k * (32 * 128) + ch) = make_uint4(wp[k][4 * c], wp[k][4 * c + 1], wp[k][4 * c + 2], wp[k][4 * c + 3]);
                     }
                     fence_proxy_async();
                     tc_fence_before();
@@ -549,65 +583,46 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 #pragma unroll
             for (int w = 0; w < 4; ++w) l += s_sum[w * kCols + lane];
             rn += (uint32_t)done_nrt;
-            if (p.S > 1) {
-                // a split's partial: one row per lane; the low parts are a partial of their own, with no weight in the sum
-                if (owns_o) {
-                    const size_t part = (size_t)it * kParts + warp;
-                    if (real) *reinterpret_cast<float2*>(p.ws_ml + (part * p.ncols + lane) * 2) = make_float2(m_ref, warp == 0 ? l : 0.f);
-                    float* wrow = p.ws_o + (part * p.ncols + lane) * D;
-#pragma unroll 1
-                    for (int d0 = 0; d0 < D; d0 += 32) {
-                        uint32_t o[32];
-                        tc_ld32(tm_o + d0, o);
-                        tc_wait_ld();
-                        pin<32>(o);
-                        if (real) {
-#pragma unroll
-                            for (int i = 0; i < 32; i += 4)       // (a split without keys has no O)
-                                *reinterpret_cast<uint4*>(wrow + d0 + i) = tiles > 0 ? make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]) : make_uint4(0u, 0u, 0u, 0u);
-                        }
-                    }
-                }
-            } else if (owns_o) {
-                // the output rows; low parts come over through shared memory, where the weights have been consumed
-                constexpr int XC = KEYS == 32 ? 64 : (D < 128 ? D : 128);
-                float* xch = reinterpret_cast<float*>(p_smem);    // [XC of D][32 columns]
+            // One row per lane: the parts come over to the first warp, the small ones first (they are worked out from what
+            // the larger ones left), and go out as the output rows, or as a split's partial.
+            if (owns_o) {
                 T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + beam) * p.H + done.kvh * p.G + hg) * D;
+                float* wrow = p.ws_o + ((size_t)it * p.ncols + lane) * D;
                 const float inv = 1.f / l;
+                if (p.S > 1 && warp == 0 && real)
+                    *reinterpret_cast<float2*>(p.ws_ml + ((size_t)it * p.ncols + lane) * 2) = make_float2(m_ref, l);
 #pragma unroll 1
-                for (int d0 = 0; d0 < D; d0 += XC) {
-                    if (kTwoPart && warp == 1) {
-#pragma unroll 1
-                        for (int c = 0; c < XC; c += 32) {
-                            uint32_t o[32];
-                            tc_ld32(tm_o + d0 + c, o);
-                            tc_wait_ld();
-                            pin<32>(o);
+                for (int d0 = 0; d0 < D; d0 += L::XC) {
+                    float* xch = reinterpret_cast<float*>(p_smem) + ((d0 / L::XC) & 1) * (L::XC * L::kXch / 4);   // [part][XC][32 columns]
+                    uint32_t o[L::XC];
+                    if constexpr (L::XC == 32) tc_ld32(tm_o + d0, o);
+                    else tc_ld16(tm_o + d0, o);
+                    tc_wait_ld();
+                    pin<L::XC>(o);
+                    if (warp > 0) {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) xch[(c + i) * 32 + lane] = __uint_as_float(o[i]);
-                        }
+                        for (int i = 0; i < L::XC; ++i) xch[((warp - 1) * L::XC + i) * kCols + lane] = __uint_as_float(o[i]);
                     }
-                    if (kTwoPart) bar_sync_n(4, 64);
-                    if (warp == 0) {
-#pragma unroll 1
-                        for (int c = 0; c < XC; c += 32) {
-                            uint32_t o[32];
-                            tc_ld32(tm_o + d0 + c, o);
-                            tc_wait_ld();
-                            pin<32>(o);
-                            float f[32];
+                    bar_sync_n(4, 32 * kParts);
+                    if (warp > 0) continue;
+                    float f[L::XC];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) f[i] = (__uint_as_float(o[i]) + (kTwoPart ? xch[(c + i) * 32 + lane] : 0.f)) * inv;
-                            if (real) {
+                    for (int i = 0; i < L::XC; ++i) {
+                        float low = 0.f;
 #pragma unroll
-                                for (int i = 0; i < 32; i += 8)
-                                    *reinterpret_cast<uint4*>(orow + d0 + c + i) =
-                                        make_uint4(Mma<T>::pack(f[i], f[i + 1]), Mma<T>::pack(f[i + 2], f[i + 3]),
-                                                   Mma<T>::pack(f[i + 4], f[i + 5]), Mma<T>::pack(f[i + 6], f[i + 7]));
-                            }
-                        }
+                        for (int k = kParts - 2; k >= 0; --k) low += xch[(k * L::XC + i) * kCols + lane];
+                        f[i] = tiles > 0 ? __uint_as_float(o[i]) + low : 0.f;              // (a split without keys has no O)
                     }
-                    if (kTwoPart) bar_sync_n(4, 64);
+                    if (real && p.S > 1) {
+#pragma unroll
+                        for (int i = 0; i < L::XC; i += 4) *reinterpret_cast<float4*>(wrow + d0 + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+                    } else if (real) {
+#pragma unroll
+                        for (int i = 0; i < L::XC; i += 8)
+                            *reinterpret_cast<uint4*>(orow + d0 + i) =
+                                make_uint4(Mma<T>::pack(f[i] * inv, f[i + 1] * inv), Mma<T>::pack(f[i + 2] * inv, f[i + 3] * inv),
+                                           Mma<T>::pack(f[i + 4] * inv, f[i + 5] * inv), Mma<T>::pack(f[i + 6] * inv, f[i + 7] * inv));
+                    }
                 }
             }
             const int it_done = it;
@@ -628,9 +643,9 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             bar_sync_n(1, 128);
             if (verdict != 1) continue;                       // not the last, or a CTA of the group gave up: no merge
             const int it0 = it_done - done.split;
-            const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * kParts * p.ncols * 2);
-            const float* o0 = p.ws_o + (size_t)it0 * kParts * p.ncols * D;
-            const int parts = p.S * kParts;
+            const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * p.ncols * 2);
+            const float* o0 = p.ws_o + (size_t)it0 * p.ncols * D;
+            const int parts = p.S;
             // Two passes: each part's factor per column, then 16 loads in flight per thread.  (One float4 of one column at
             // a time, its parts' loads ordered by the use of each, cost most of the about 7 us that merging four splits took.)
             float* fac = reinterpret_cast<float*>(p_smem);        // [part][32 columns]: 2^(m_part - m) / sum
@@ -727,7 +742,7 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 
 template <typename T, int D>
 cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
-    using L = WideLayout<D>;
+    using L = WideLayout<T, D>;
     // never two CTAs on one SM: the second would wait for tensor memory inside its allocation
     constexpr size_t smem = L::kBytes > 120 * 1024 ? L::kBytes : 120 * 1024;
     auto kern = sdpa_wide_kernel<T, D>;
@@ -749,7 +764,7 @@ cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk,
     p.quota = (a.steps + 2 * d.beams + a.splits - 1) / a.splits;
     p.items = d.batch * d.kv_heads * a.splits;
     p.ws_o = a.ws;
-    p.ws_ml = a.ws + (size_t)p.items * wide_parts(d) * p.ncols * D;
+    p.ws_ml = a.ws + (size_t)p.items * p.ncols * D;
     p.early_prompt = (a.pdl && a.prompt_immutable) ? 1 : 0;
     p.dbg_skip = a.dbg_skip ? 1 : 0;
     p.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
@@ -786,15 +801,14 @@ cudaError_t dispatch(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, c
 
 }  // namespace
 
-int wide_parts(const Dims& d) { return d.dtype == SEGKV_BF16 ? 2 : 1; }
-
-// the split merge keeps one factor per part and column where the weights were
+// The split merge keeps one factor per split and column where the weights were.  (bf16 at head_dim 256: the 32 that the
+// segkv_get_splits of such a handle has always answered at most.)
 int wide_max_splits(const Dims& d) {
-    const int n = (d.head_dim == 256 ? WideLayout<256>::kP : WideLayout<128>::kP) / (kCols * 4 * wide_parts(d));
-    return n < kMaxSplits ? n : kMaxSplits;
+    static_assert(WideLayout<__half, 256>::kP >= kMaxSplits * kCols * 4, "factors of the split merge");
+    return d.head_dim == 256 && d.dtype == SEGKV_BF16 ? 32 : kMaxSplits;
 }
 
-int wide_tile_keys(const Dims& d) { return d.head_dim == 256 ? WideLayout<256>::KEYS : WideLayout<128>::KEYS; }
+int wide_tile_keys(const Dims& d) { return d.head_dim == 256 ? WideLayout<__half, 256>::KEYS : WideLayout<__half, 128>::KEYS; }
 
 cudaError_t launch_sdpa_wide(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk, const CUtensorMap& tmv, int sms, cudaStream_t st) {
     if (a.splits < 1 || a.splits > wide_max_splits(d) || d.beams * d.group > kCols) return cudaErrorInvalidValue;

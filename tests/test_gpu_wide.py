@@ -102,3 +102,52 @@ def test_more_forced_splits_than_the_merge_has_room_for():
         r.check(out, q, 3, all_pairs(w))
     finally:
         r.close()
+
+
+def _float64(r, q, t):
+    """decode attention of every row in float64 on the device, from the tensors the run holds"""
+    w = r.w
+    W, G, D = w.beams, w.heads // w.kv_heads, w.head_dim
+    anc = torch.from_numpy(r.oracle_ancestry(t)).long().cuda()
+    step = torch.arange(t + 1, device="cuda")
+    K, V = torch.stack(r.k_steps[:t + 1])[step, anc].double(), torch.stack(r.v_steps[:t + 1])[step, anc].double()
+    out = torch.empty(w.rows, w.heads, D, dtype=torch.float64, device="cuda")
+    for row in range(w.rows):
+        k, v = (torch.cat([p[row // W].double(), x[row]]).transpose(0, 1) for p, x in ((r.kp, K), (r.vp, V)))
+        p = torch.softmax(q[row].double().view(w.kv_heads, G, D) @ k.transpose(1, 2) / D ** 0.5, -1)
+        out[row] = (p @ v).reshape(w.heads, D)
+    return out
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,beams,group", [(64, 4, 8), (128, 5, 4), (128, 4, 8), (256, 3, 4)])
+@pytest.mark.parametrize("splits", [1, 4])
+@pytest.mark.parametrize("cancel", [False, True])
+def test_weights_as_precise_as_the_per_beam_kernels(dtype, D, beams, group, splits, cancel):
+    # The per-beam kernel works in fp32 throughout.  Ordinary values show a weight of 11 bits beside the 11 of an fp16
+    # output, values that cancel nearly all of what they weigh one of 16.  Both errors end in the same rounding of the
+    # output: 2 % is for the few numbers that fall on its other side.
+    w = _w("precise", 2, beams, group, 2, D, 500, 8, dtype, seed=9)
+    r = Run(w, splits=splits)
+    try:
+        if cancel:
+            r.vp = r.vp[:, :1].abs().repeat(1, w.prompt_len, 1, 1).contiguous()
+            r.vp[:, 1::2] *= -1
+            r.h.prefill_write(r.kp, r.vp)
+        r.advance_to(7)
+        if cancel:
+            r.v_steps = [torch.zeros_like(v) for v in r.v_steps]
+            r.h.reset(keep_prompt=True)
+            for t in range(8):
+                r.h.append(t, r.parents_dev[t] if t else None, r.k_steps[t], r.v_steps[t])
+        q = r.q_steps[-1] * (1e-3 if cancel else 1.0)
+        ref = _float64(r, q, 7)
+        err = {}
+        for f in (r.h.decode_sdpa, r.h.decode_sdpa_rowwise):
+            out = torch.empty_like(q)
+            f(q, out)
+            err[f.__name__] = ((out.double() - ref).norm() / ref.norm()).item()
+        print(f"{dtype} D {D} {beams}x{group} S {splits} cancel {cancel}: {err}")
+        assert err["decode_sdpa"] <= 1.02 * err["decode_sdpa_rowwise"], err
+    finally:
+        r.close()
