@@ -27,10 +27,15 @@
 //    flight; the gather warps also place the query block;
 //  * splits of a work group meet in the global workspace, the parts of each added up: the last CTA to arrive folds
 //    them (as in the tiled kernel).
+//  * an Inf or a NaN in a value row would reach the columns that do not read the row (their weight there is zero, and
+//    zero times Inf is NaN), and a weight in parts makes a NaN of an Inf.  So the columns of a finished work group
+//    whose output is not finite are worked out again one by one, from the rows that they read (segkv_rowwise.cuh), by
+//    the softmax warps.  Without splits that is done at the end of the CTA's next item, where the warps meet anyhow.
 // Every mbarrier is waited on phase by phase and every wait is bounded; on expiry the kernel flags
 // SEGKV_DEV_WAIT_LIMIT, leaves the output alone and still releases its tensor memory and its tickets.
 #include "segkv_internal.h"
 #include "segkv_ptx.cuh"
+#include "segkv_rowwise.cuh"
 #include "segkv_tc5.cuh"
 
 namespace segkv_impl {
@@ -73,6 +78,7 @@ struct WideParams {
     unsigned long long wait_ns;
     float scale2;
     uint32_t idesc_qk, idesc_pv;
+    rowwise::Args row;             // the same call, for columns that are not finite
 };
 
 // A softmax weight as a sum of 16-bit parts for the tensor cores, with what fp32 has of it: fp16 in two (22 bits), bf16
@@ -125,12 +131,13 @@ struct WideLayout {
     static constexpr int kMax = 2 * 4 * kCols * 4, kSum = 4 * kCols * 4;
     static constexpr int kBars = 3 * SP + 2 * SR + 3 + 6 + 1;    // rings, query, S/P/O x 2, wind-down
     // the small arrays first, then, on a swizzle atom's boundary, weights, rings and the query block
-    static constexpr int kSmall = (kMeta + kMax + kSum + 8 * kBars + 16 + 1023) & ~1023;
+    static constexpr int kSmall = (kMeta + kMax + kSum + 8 * kBars + 32 + 1023) & ~1023;
     static constexpr size_t kBytes = (size_t)kSmall + kP + (SP + SR) * kStage + kQ;
     // the parts of O meet in shared memory, where the weights were, XC of D at a time in two buffers in turn
     static constexpr int kXch = (kParts - 1) * kCols * 4;        // bytes of one of D
     static constexpr int XC = kP >= 64 * kXch ? 32 : 16;
     static_assert(2 * XC * kXch <= kP, "exchange of the parts");
+    static_assert(rowwise::kScratch<D> * 4 <= kP, "columns that are worked out again");
     // tensor memory: two S buffers, O, and the query block (16-bit, two elements per column)
     static constexpr int kColO = 2 * KEYS, kColQ = kColO + D, kColEnd = kColQ + D / 2;
     static constexpr int kTmemCols = kColEnd <= 256 ? 256 : 512;
@@ -139,9 +146,22 @@ struct WideLayout {
     static_assert(kBytes <= 232448, "shared memory");
 };
 
+// The columns `mask` of a finished work group again, each from its own rows; all four softmax warps, the weights' place
+// (s) free.  (Out of line: inlined it cost every launch about 1 us.)
+template <typename T, int D>
+__device__ __noinline__ void redo_columns(const rowwise::Args& a, int slab, uint32_t mask, float* s) {
+    const int b = slab / a.Hkv, kvh = slab - b * a.Hkv;
+    for (; mask; mask &= mask - 1) {
+        const int col = __ffs(mask) - 1;
+        rowwise::attend<T, D>(a, b * a.W + col / a.group, kvh * a.group + col % a.group, threadIdx.x >> 5, threadIdx.x & 31, s,
+                              [] { bar_sync_n(1, 128); });
+        bar_sync_n(1, 128);
+    }
+}
+
 template <typename T, int D>
 __global__ void __launch_bounds__(320, 1)
-sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const WideParams p) {
+sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ WideParams p) {
     using L = WideLayout<T, D>;
     constexpr int KEYS = L::KEYS, KW = L::KW, SP = L::SP, SR = L::SR;
     constexpr int kParts = L::kParts;
@@ -153,6 +173,7 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + L::kBars);
     volatile int* s_flags = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int &s_abort = s_flags[0], &s_ticket = s_flags[1];
+    uint32_t* s_bad = tmem_slot + 3;                              // [2] columns of an item that are not finite: item parity
     uint8_t* p_smem = smem + L::kSmall;                           // two buffers; their A operands reach into the ring behind
     uint8_t* p_ring = p_smem + L::kP;
     uint8_t* r_ring = p_ring + (size_t)SP * L::kStage;
@@ -216,6 +237,7 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             }
             mbar_init(bar_end, 1);
             s_abort = 0;
+            s_bad[0] = s_bad[1] = 0u;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             fence_proxy_async();
         }
@@ -446,6 +468,8 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             rows_of(x, n_b, e0, e1);
             return (e1 - e0 + KEYS - 1) / KEYS;
         };
+        uint32_t items_done = 0;
+        int slab_before = 0;                                      // work group of the item before, without splits
         bool gone = false;                                        // the four warps have agreed to leave: a wait ran out
         int it = blockIdx.x;
         Item x;
@@ -583,12 +607,18 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 #pragma unroll
             for (int w = 0; w < 4; ++w) l += s_sum[w * kCols + lane];
             rn += (uint32_t)done_nrt;
+            if (p.S == 1 && s_bad[(items_done & 1) ^ 1]) {
+                redo_columns<T, D>(p.row, slab_before, s_bad[(items_done & 1) ^ 1], reinterpret_cast<float*>(p_smem));
+                if (tid == 0) s_bad[(items_done & 1) ^ 1] = 0u;
+            }
+            slab_before = done.slab;
             // One row per lane: the parts come over to the first warp, the small ones first (they are worked out from what
             // the larger ones left), and go out as the output rows, or as a split's partial.
             if (owns_o) {
                 T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + beam) * p.H + done.kvh * p.G + hg) * D;
                 float* wrow = p.ws_o + ((size_t)it * p.ncols + lane) * D;
                 const float inv = 1.f / l;
+                bool bad = false;
                 if (p.S > 1 && warp == 0 && real)
                     *reinterpret_cast<float2*>(p.ws_ml + ((size_t)it * p.ncols + lane) * 2) = make_float2(m_ref, l);
 #pragma unroll 1
@@ -618,13 +648,20 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                         for (int i = 0; i < L::XC; i += 4) *reinterpret_cast<float4*>(wrow + d0 + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
                     } else if (real) {
 #pragma unroll
+                        for (int i = 0; i < L::XC; ++i) {
+                            f[i] *= inv;
+                            bad |= !(fabsf(f[i]) < INFINITY);
+                        }
+#pragma unroll
                         for (int i = 0; i < L::XC; i += 8)
-                            *reinterpret_cast<uint4*>(orow + d0 + i) =
-                                make_uint4(Mma<T>::pack(f[i] * inv, f[i + 1] * inv), Mma<T>::pack(f[i + 2] * inv, f[i + 3] * inv),
-                                           Mma<T>::pack(f[i + 4] * inv, f[i + 5] * inv), Mma<T>::pack(f[i + 6] * inv, f[i + 7] * inv));
+                            *reinterpret_cast<uint4*>(orow + d0 + i) = make_uint4(Mma<T>::pack(f[i], f[i + 1]), Mma<T>::pack(f[i + 2], f[i + 3]),
+                                                                                  Mma<T>::pack(f[i + 4], f[i + 5]), Mma<T>::pack(f[i + 6], f[i + 7]));
                     }
                 }
+                const uint32_t mask = __ballot_sync(0xffffffffu, bad);
+                if (p.S == 1 && tid == 0 && mask) s_bad[items_done & 1] = mask;     // read behind the next meeting
             }
+            ++items_done;
             const int it_done = it;
             it = it_next;
             if (p.S == 1) continue;
@@ -704,11 +741,21 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 for (int i = 0; i < NE; ++i) {
                     const int e = e0 + 128 * i, col = e / D4, d = (e % D4) * 4;
                     if (e >= n4) break;
+                    if (!(fabsf(o[i].x) + fabsf(o[i].y) + fabsf(o[i].z) + fabsf(o[i].w) < INFINITY)) atomicOr(&s_bad[0], 1u << col);
                     T* orow = reinterpret_cast<T*>(p.out) + ((size_t)(done.b * p.W + col / p.G) * p.H + done.kvh * p.G + col % p.G) * D + d;
                     *reinterpret_cast<uint2*>(orow) = make_uint2(Mma<T>::pack(o[i].x, o[i].y), Mma<T>::pack(o[i].z, o[i].w));
                 }
             }
             bar_sync_n(1, 128);                                   // the factors' place takes weights again
+            if (const uint32_t mask = s_bad[0]) {
+                redo_columns<T, D>(p.row, done.slab, mask, reinterpret_cast<float*>(p_smem));
+                if (tid == 0) s_bad[0] = 0u;
+                bar_sync_n(1, 128);
+            }
+        }
+        if (!gone && p.S == 1) {                                  // the last item's
+            bar_sync_n(1, 128);
+            if (const uint32_t mask = s_bad[(items_done & 1) ^ 1]) redo_columns<T, D>(p.row, slab_before, mask, reinterpret_cast<float*>(p_smem));
         }
         if (gone) {
             if (tid == 0) {
@@ -766,6 +813,7 @@ cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk,
     p.ws_o = a.ws;
     p.ws_ml = a.ws + (size_t)p.items * p.ncols * D;
     p.early_prompt = (a.pdl && a.prompt_immutable) ? 1 : 0;
+    p.row = rowwise::make_args(d, a);
     p.dbg_skip = a.dbg_skip ? 1 : 0;
     p.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;
     p.scale2 = 1.4426950408889634f / sqrtf((float)D);

@@ -151,3 +151,47 @@ def test_weights_as_precise_as_the_per_beam_kernels(dtype, D, beams, group, spli
         assert err["decode_sdpa"] <= 1.02 * err["decode_sdpa_rowwise"], err
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,beams,group,batch,hkv,splits", [
+    (64, 4, 8, 2, 2, 1), (128, 4, 8, 2, 2, 3), (128, 4, 8, 50, 8, 1), (128, 5, 4, 2, 2, 1), (256, 4, 4, 2, 2, 1),
+    (256, 4, 8, 40, 4, 2)])
+def test_values_that_are_not_finite_stay_with_the_beams_that_read_them(dtype, D, beams, group, batch, hkv, splits):
+    # one beam's value rows hold Inf, -Inf, NaN or numbers whose weighted sum leaves the range; parents keep the beams
+    # apart.  Every column of a group that holds such a row is the per-beam kernel's, bit by bit, the others' as ever
+    w = _w("apart", batch, beams, group, hkv, D, 70, 6, dtype, seed=10)
+    par = np.tile(np.arange(beams, dtype=np.int32), (6, batch))
+    r = Run(w, parents=par, splits=splits)
+    try:
+        r.advance_to(4)
+        q, k, v = wl.make_step(w, 5, "cuda")
+        ref = v.clone()
+        bad = [(b, h) for b in range(0, batch, 3) for h in range(hkv) if (b + h) % 2 == 0]
+        huge = torch.finfo(w.torch_dtype).max
+        for i, (b, h) in enumerate(bad):
+            v[b * beams + 1, h, i % D] = [float("inf"), float("-inf"), float("nan"), huge][i % 4]
+        r.h.append(5, r.parents_dev[5], k, v)
+        out, row = torch.empty_like(q), torch.empty_like(q)
+        r.h.decode_sdpa(q, out)
+        r.h.decode_sdpa_rowwise(q, row)
+        r.h.truncate_last()
+        r.h.append(5, r.parents_dev[5], k, ref)
+        clean = torch.empty_like(q)
+        r.h.decode_sdpa(q, clean)
+        torch.cuda.synchronize()
+        assert r.h.get_error() == 0 and torch.isfinite(clean.float()).all()
+        nonfinite = ~torch.isfinite(row.float())
+        for b in range(batch):
+            for h in range(hkv):
+                a, e, c = (t[b * beams:(b + 1) * beams, h * group:(h + 1) * group] for t in (out, row, clean))
+                hit = (b, h) in bad and bool((~torch.isfinite(e.float())).any())
+                if hit:
+                    assert torch.equal(a.view(torch.int16), e.view(torch.int16)), (b, h)
+                    others = [j for j in range(beams) if j != 1]
+                    assert torch.isfinite(a[others].float()).all()
+                elif (b, h) not in bad:
+                    assert torch.equal(a, c), (b, h)
+        assert bool(nonfinite.any())
+    finally:
+        r.close()
