@@ -422,9 +422,12 @@ bool use_wide(const segkv* h) {
 }
 
 // Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA.  In units of a tile
-// (0.65 us): a round of items costs its tiles plus about two to start and finish an item; meeting in the
-// workspace costs about four (a partial's stores, the arrival, one trip for the factors) plus one per 16 loads of
-// the last CTA's threads.
+// (0.65 us): a round of items costs its tiles (a response tile, which is gathered, twice) plus about two to start and finish an item; meeting in the
+// workspace costs about two, and for every four splits one plus two for each pass of 2048 numbers that the last CTA makes
+// over the partials (fitted to 4 to 64 work groups, prompts of 256 to 16384 in 1 to 64 splits: at most 4 % above the best
+// count, 0.2 % on average).  How many distinct rows the response has is known on the device only: about steps + 2 * beams
+// where beams merge, beams * steps where they stay apart.  The first count decides, the second weighs an eighth: 32 beams
+// that stay apart for 256 steps of 4 work groups, 327 us in one split, get four.
 int wide_splits(const segkv* h) {
     const Dims& d = h->d;
     const int most = wide_max_splits(d) < h->ws_splits ? wide_max_splits(d) : h->ws_splits;
@@ -432,15 +435,16 @@ int wide_splits(const segkv* h) {
     const long long slabs = (long long)d.batch * d.kv_heads;
     const int keys = wide_tile_keys(d);
     const long long ntp = ((h->prompt_len > 0 ? h->prompt_len : 0) + keys - 1) / keys;
-    const long long ntr = (h->steps + 2 * d.beams + keys - 1) / keys;      // estimate, rows are mostly shared
+    const long long ntr = (h->steps + 2 * d.beams + keys - 1) / keys;
+    const long long apart = ((long long)h->steps * d.beams + keys - 1) / keys;
     const long long passes = ((long long)d.beams * d.group * d.head_dim + 2047) / 2048;
     int best = 1;
     long long best_cost = 0;
-    for (int s = 1; s <= most && s <= ntp + ntr; ++s) {
+    for (int s = 1; s <= most && s <= ntp + (ntr > apart ? ntr : apart); ++s) {
         const long long rounds = (slabs * s + h->sm_count - 1) / h->sm_count;
-        const long long merge = s > 1 ? 4 + passes * ((s + 3) / 4) : 0;
-        const long long cost = rounds * ((ntp + s - 1) / s + (ntr + s - 1) / s + 2) + merge;
-        if (s == 1 || cost < best_cost) {
+        const long long merge = s > 1 ? 2 + (2 * passes + 1) * ((s + 3) / 4) : 0;
+        const long long cost = 8 * (rounds * ((ntp + s - 1) / s + 2 * ((ntr + s - 1) / s) + 2) + merge) + rounds * ((apart + s - 1) / s);
+        if (s == 1 || 32 * cost < 31 * best_cost) {               // (more splits for a clear gain only)
             best = s;
             best_cost = cost;
         }

@@ -73,7 +73,7 @@ struct WideParams {
     float* ws_ml;                  // [item][ncols][2] reference maximum (base-2 domain) and sum
     int* tickets;
     int* err_word;
-    int P, steps, S, W, G, H, Hkv, rows, max_steps, ncols, chunk_steps, quota, items;
+    int P, steps, S, W, G, H, Hkv, rows, max_steps, ncols, chunk_steps, items;
     int early_prompt, dbg_skip;
     unsigned long long wait_ns;
     float scale2;
@@ -203,8 +203,9 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     // the distinct rows of an item's request; asked for one item ahead
     auto count_of = [&](int it) { return p.steps > 0 && it < p.items ? p.ucount[it / p.S / p.Hkv] : 0; };
     auto rows_of = [&](const Item& x, int n_b, int& e0, int& e1) {
-        e0 = min(x.split * p.quota, n_b);
-        e1 = x.split == p.S - 1 ? n_b : min((x.split + 1) * p.quota, n_b);
+        const int each = n_b / p.S, left = n_b - each * p.S;      // beams that stay apart have up to beams * steps rows
+        e0 = x.split * each + min(x.split, left);
+        e1 = e0 + each + (x.split < left ? 1 : 0);
     };
     // the K (or V) part of the item's prompt tile k
     auto issue_part = [&](const CUtensorMap* tm, const Item& x, int k, uint32_t dst, uint32_t full) {
@@ -808,7 +809,6 @@ cudaError_t launch_one(const Dims& d, const SdpaArgs& a, const CUtensorMap& tmk,
     p.tickets = a.tickets; p.err_word = a.err_word;
     p.P = a.prompt_len; p.steps = a.steps; p.S = a.splits; p.W = d.beams; p.G = d.group; p.H = d.heads; p.Hkv = d.kv_heads;
     p.rows = d.rows; p.max_steps = d.max_steps; p.ncols = d.beams * d.group;
-    p.quota = (a.steps + 2 * d.beams + a.splits - 1) / a.splits;
     p.items = d.batch * d.kv_heads * a.splits;
     p.ws_o = a.ws;
     p.ws_ml = a.ws + (size_t)p.items * p.ncols * D;

@@ -195,3 +195,31 @@ def test_values_that_are_not_finite_stay_with_the_beams_that_read_them(dtype, D,
         assert bool(nonfinite.any())
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("D,beams", [(64, 32), (128, 32), (256, 16)])
+def test_rows_of_beams_that_stay_apart_are_shared_out_evenly(D, beams):
+    # Beams that never merge have beams * steps distinct rows; a share of the splits that counts on merged beams leaves
+    # nearly all of them to the last one (2.5 times the per-beam kernel's time at 32 beams; evenly shared, half of it).
+    w = _w("shares", 1, beams, 1, 4, D, 128, 256, "f16", seed=11)
+    par = np.tile(np.arange(beams, dtype=np.int32), (256, 1))
+    r = Run(w, parents=par, splits=8)
+    try:
+        r.advance_to(255)
+        q = r.q_steps[-1]
+        out, _ = r.decode(q)
+        r.check(out, q, 255, [(0, 0), (0, 3)])
+        t = {}
+        for f in (r.h.decode_sdpa, r.h.decode_sdpa_rowwise):
+            f(q, out)
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda._sleep(1000000)
+            e[0].record()
+            for _ in range(20):
+                f(q, out)
+            e[1].record()
+            torch.cuda.synchronize()
+            t[f.__name__] = e[0].elapsed_time(e[1])
+        assert t["decode_sdpa"] < t["decode_sdpa_rowwise"], t
+    finally:
+        r.close()
