@@ -428,28 +428,31 @@ bool use_wide(const segkv* h) {
 // count, 0.2 % on average).  How many distinct rows the response has is known on the device only: about steps + 2 * beams
 // where beams merge, beams * steps where they stay apart.  The first count decides, the second weighs an eighth: 32 beams
 // that stay apart for 256 steps of 4 work groups, 327 us in one split, get four.
+// (This runs at every attention call: 32-bit divisions, and no count is looked at whose merge alone costs more than the
+// best so far: 0.06 us where all counts up to 64 in 64-bit divisions took 0.2 to 0.8.)
 int wide_splits(const segkv* h) {
     const Dims& d = h->d;
-    const int most = wide_max_splits(d) < h->ws_splits ? wide_max_splits(d) : h->ws_splits;
-    if (h->splits_forced > 0) return h->splits_forced < most ? h->splits_forced : most;
-    const long long slabs = (long long)d.batch * d.kv_heads;
-    const int keys = wide_tile_keys(d);
-    const long long ntp = ((h->prompt_len > 0 ? h->prompt_len : 0) + keys - 1) / keys;
-    const long long ntr = (h->steps + 2 * d.beams + keys - 1) / keys;
-    const long long apart = ((long long)h->steps * d.beams + keys - 1) / keys;
-    const long long passes = ((long long)d.beams * d.group * d.head_dim + 2047) / 2048;
-    int best = 1;
+    const unsigned most = (unsigned)(wide_max_splits(d) < h->ws_splits ? wide_max_splits(d) : h->ws_splits);
+    if (h->splits_forced > 0) return (unsigned)h->splits_forced < most ? h->splits_forced : (int)most;
+    const unsigned slabs = (unsigned)d.batch * d.kv_heads, keys = wide_tile_keys(d), sms = h->sm_count;
+    const unsigned ntp = ((h->prompt_len > 0 ? h->prompt_len : 0) + keys - 1) / keys;
+    const unsigned ntr = ((unsigned)h->steps + 2 * d.beams + keys - 1) / keys;
+    const unsigned apart = ((unsigned)h->steps * d.beams + keys - 1) / keys;
+    const unsigned passes = ((unsigned)(d.beams * d.group * d.head_dim) + 2047) / 2048;
+    const unsigned last = ntp + (ntr > apart ? ntr : apart);
+    unsigned best = 1;
     long long best_cost = 0;
-    for (int s = 1; s <= most && s <= ntp + (ntr > apart ? ntr : apart); ++s) {
-        const long long rounds = (slabs * s + h->sm_count - 1) / h->sm_count;
+    for (unsigned s = 1; s <= most && s <= last; ++s) {
         const long long merge = s > 1 ? 2 + (2 * passes + 1) * ((s + 3) / 4) : 0;
+        if (s > 1 && 32 * 8 * (merge + 2) >= 31 * best_cost) break;
+        const long long rounds = (slabs * s + sms - 1) / sms;
         const long long cost = 8 * (rounds * ((ntp + s - 1) / s + 2 * ((ntr + s - 1) / s) + 2) + merge) + rounds * ((apart + s - 1) / s);
         if (s == 1 || 32 * cost < 31 * best_cost) {               // (more splits for a clear gain only)
             best = s;
             best_cost = cost;
         }
     }
-    return best;
+    return (int)best;
 }
 
 // Does the separate attention call run in the persistent form?
