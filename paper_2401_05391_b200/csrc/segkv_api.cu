@@ -1057,6 +1057,11 @@ size_t segkv_host_pack_bytes(segkv_t h, size_t* offsets) {
     return off[4] + up(qbytes);
 }
 
+// The last step dropped, if it is `step` and can be: what segkv_truncate_last does.
+static void drop_step(segkv_t h, int step) {
+    if (h->steps == step + 1 && !h->truncated) (void)segkv_truncate_last(h);
+}
+
 int segkv_step_host_packed(segkv_t h, int step, const void* host_in, void* host_out, int has_slopes, void* stream) {
     int rc = segkv_step_host_packed_async(h, step, host_in, host_out, has_slopes, stream);
     if (rc != SEGKV_OK) return rc;
@@ -1118,10 +1123,7 @@ int segkv_layers_step_host(const segkv_t* layers, int n, int step, const void* c
         // a stream being captured (or no streams to be had): everything in order on the caller's stream
         for (int i = 0; i < n; ++i) {
             segkv_t h = layers[i];
-            if (redo && h->steps == step + 1 && !h->truncated) {
-                h->steps -= 1;
-                h->truncated = true;
-            }
+            if (redo) drop_step(h, step);
             const int rc = segkv_step_host_packed_async(h, step, host_in[i], host_out[i], has_slopes, stream);
             if (rc != SEGKV_OK) return rc;
         }
@@ -1182,10 +1184,7 @@ int segkv_layers_step_host(const segkv_t* layers, int n, int step, const void* c
                 SEGKV_CUDA(cudaStreamWaitEvent(st, layers[g0]->ev_in, 0));
                 for (int i = g0; i < g0 + cnt; ++i) {
                     segkv_t h = layers[i];
-                    if (redo && h->steps == step + 1 && !h->truncated) {
-                        h->steps -= 1;
-                        h->truncated = true;
-                    }
+                    if (redo) drop_step(h, step);
                     char* base = gin + (size_t)i * total;
                     const int rc = segkv_decode_step(h, step, step > 0 ? (const int32_t*)(base + off[0]) : nullptr, base + off[2],
                                                      base + off[3], base + off[4], gout + (size_t)i * qbytes,
@@ -1203,10 +1202,7 @@ int segkv_layers_step_host(const segkv_t* layers, int n, int step, const void* c
     }
     for (int i = 0; i < n; ++i) {
         segkv_t h = layers[i];
-        if (redo && h->steps == step + 1 && !h->truncated) {
-            h->steps -= 1;
-            h->truncated = true;
-        }
+        if (redo) drop_step(h, step);
         const Dims& d = h->d;
         size_t off[5];
         const size_t total = segkv_host_pack_bytes(h, off);

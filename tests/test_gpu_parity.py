@@ -638,6 +638,33 @@ def test_layers_step_host_queues_every_layer_in_one_call(one_array, heads, layer
             h.destroy()
 
 
+@pytest.mark.parametrize("layers", [1, 2])
+def test_a_redone_host_step_that_fails_leaves_the_step_dropped(layers):
+    # the step is dropped, then the step itself is refused (a cluster merge of three splits): what attends next sees the
+    # rows of the step before, not the dropped step's
+    w = wl.Workload("dropped", 1, 4, 4, 4, 128, 100, 6, "f16", "uniform", False, 121)
+    rs = [Run(w.scaled(index=121 + i)) for i in range(layers)]
+    try:
+        for r in rs:
+            r.advance_to(5)
+        total, _ = rs[0].h.host_pack_layout()
+        blk = torch.zeros(layers, total, dtype=torch.uint8).pin_memory()
+        out = torch.empty(layers, w.rows, w.heads, w.head_dim, dtype=w.torch_dtype).pin_memory()
+        stack = sk.LayerStack([r.h for r in rs], [blk[i] for i in range(layers)], [out[i] for i in range(layers)])
+        rs[0].h.set_tuning(3, 0, 2)
+        with pytest.raises(sk.SegKVError) as e:
+            stack.step(5, redo=True)
+        assert e.value.code == sk.SEGKV_EINVAL
+        torch.cuda.synchronize()
+        rs[0].h.set_tuning(0, 0, 0)
+        assert rs[0].h.steps == 5
+        got, q = rs[0].decode(rs[0].q_steps[4])
+        rs[0].check(got, q, 4, all_pairs(w))
+    finally:
+        for r in rs:
+            r.close()
+
+
 def test_read_bandwidth_aid():
     buf = torch.zeros(1 << 30, dtype=torch.uint8, device="cuda")
     gbs = sk.read_bandwidth(buf, 5)
