@@ -418,7 +418,7 @@ bool wide_possible(const Dims& d) { return !tiled_supported(d) || (d.head_dim ==
 bool use_wide(const segkv* h) {
     if (!tiled_supported(h->d)) return true;
     return wide_possible(h->d) && h->splits_forced == 0 && h->stages_forced == 0 && h->combine_forced == 0 && h->tile_forced == 0 &&
-           h->overlap && (long long)h->d.batch * h->d.kv_heads * (h->prompt_len > 0 ? h->prompt_len : 0) >= 16384;
+           (long long)h->d.batch * h->d.kv_heads * (h->prompt_len > 0 ? h->prompt_len : 0) >= 16384;
 }
 
 // Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA.  In units of a tile

@@ -223,3 +223,18 @@ def test_rows_of_beams_that_stay_apart_are_shared_out_evenly(D, beams):
         assert t["decode_sdpa"] < t["decode_sdpa_rowwise"], t
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("dtype,beams,group", [("f16", 3, 3), ("bf16", 4, 4)])
+def test_overlap_does_not_choose_the_kernel(dtype, beams, group):
+    # nine to 16 columns at head_dim 128: with dependent launch off the same kernel runs, and every bit is the same
+    w = _w("overlap", 4, beams, group, 8, 128, 600, 6, dtype, alibi=group == 4, seed=12)
+    r = Run(w)
+    try:
+        r.advance_to(5)
+        out, q = r.decode()
+        r.h.set_overlap(False)
+        off, _ = r.decode(q)
+        assert torch.equal(out.view(torch.int16), off.view(torch.int16))
+    finally:
+        r.close()
