@@ -409,16 +409,29 @@ int stream_splits(const segkv* h) {
 // Can the wide kernel (tcgen05, up to 32 query columns) serve this shape at some length?
 bool wide_possible(const Dims& d) { return !tiled_supported(d) || (d.head_dim == 128 && d.beams * d.group > 8); }
 
-// Does it serve this call?  Always where the tiled kernel has no form.  Nine to 16 columns at head_dim 128 run on
-// either: the wide kernel needs a few microseconds more to start, finish and (with an append of its own) fuse
-// nothing, and gets keys through faster.  Measured step, tiled / wide in us, at work groups x prompt = 8 K: 14.1 / 21.2
-// (4 x 2048), 9.8 / 14.0 (16 x 512); at 16 K: 28.8 / 21.8 (4 x 4096), 19.3 / 14.7 (16 x 1024), 18.5 / 14.7 (32 x 512),
-// 21.3 / 11.3 (128 x 128); at 128 K 31 / 21 (128 x 1024).  (At head_dim 64 the tiled kernel stays ahead: 11.6 / 20.8 at
-// 240 x 634.)  A handle whose launch shape has been set by hand keeps the kernel that the setting is for.
+// Does it serve an attention call of its own?  Always where the tiled kernel has no form.  Nine to 16 columns at head_dim
+// 128 run on either.  The wide kernel gets through keys faster, but it keeps one CTA per SM: the tiled one is ahead
+// where the work groups are more than the SMs (append and attention, tiled / wide in us: 35 / 48 with 9 beams, 160 work
+// groups x 512 prompt; 44 / 51 with 16 beams, 512 x 128; 117 / 157 with 16 beams, 320 x 2048, 256 steps) and where there
+// are few keys (14 / 21 at 4 x 2048, 9.8 / 14 at 16 x 512).  In between the wide kernel takes 0.53 to 0.91 of the tiled
+// one's time (8 to 148 work groups, 16384 to 65536 prompt keys, 4 to 16 beams, 4 to 256 steps, merged or apart).  (At
+// head_dim 64 the tiled kernel stays ahead: 11.6 / 20.8 at 240 x 634.)  A handle whose launch shape has been set by hand
+// keeps the kernel that the setting is for.
 bool use_wide(const segkv* h) {
     if (!tiled_supported(h->d)) return true;
     return wide_possible(h->d) && h->splits_forced == 0 && h->stages_forced == 0 && h->combine_forced == 0 && h->tile_forced == 0 &&
+           (long long)h->d.batch * h->d.kv_heads <= h->sm_count &&
            (long long)h->d.batch * h->d.kv_heads * (h->prompt_len > 0 ? h->prompt_len : 0) >= 16384;
+}
+
+// A step of nine to 16 columns that the tiled kernel can fuse: does it, although the wide kernel would serve the
+// attention?  The wide kernel has no fused form, and the append of many beams costs it 3 (9 beams) to 7 us (16).  Fused
+// tiled / wide in us: 20 / 22 (9 beams, 8 work groups x 4096), 22 / 25 (16 beams, 16 x 1024), 21.4 / 23.5 (16 beams, 32 x 512), 24 / 28 (16 beams, 32 x
+// 2048), 25 / 31 (16 beams, 8 x 8192); the other way round 19 / 17 (9 beams, 32 x 512), 19.4 / 18.3 (12 beams, 64 x 512),
+// 22 / 19 (16 beams, 64 x 256).  Five beams lose nothing before a prompt of about 8192 (21 / 23 there), four never.
+bool rather_fused(const segkv* h) {
+    const Dims& d = h->d;
+    return tiled_supported(d) && d.beams > 4 && (long long)d.beams * h->prompt_len >= (d.beams > 12 ? 8192 : d.beams > 8 ? 10240 : 32768);
 }
 
 // Items per work group for the wide kernel, one CTA per SM: the count with the shortest longest CTA.  In units of a tile
@@ -939,7 +952,7 @@ int segkv_decode_step(segkv_t h, int step, const int32_t* beam_parent, const voi
     if (h->prompt_len < 0) return SEGKV_ESTATE;
     if (step != h->steps) return SEGKV_ESTATE;
     if (step >= h->d.max_steps) return SEGKV_ECAPACITY;
-    if (use_wide(h) || h->leader) {
+    if (h->leader || (use_wide(h) && !rather_fused(h))) {
         // the wide kernel has no fused form, and handles that use another handle's tables
         // (nothing to update in the attention kernel): the two separate launches
         int rc = segkv_append(h, step, beam_parent, k_new, v_new, stream);

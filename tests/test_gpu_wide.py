@@ -238,3 +238,25 @@ def test_overlap_does_not_choose_the_kernel(dtype, beams, group):
         assert torch.equal(out.view(torch.int16), off.view(torch.int16))
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("batch,hkv,beams,group,P,launches", [
+    (4, 8, 3, 3, 511, 1),          # too few keys for the wide kernel: the tiled kernel's fused step
+    (4, 8, 3, 3, 512, 2),          # the wide kernel, behind an append of its own
+    (4, 8, 4, 4, 512, 2),
+    (4, 8, 16, 1, 511, 1), (4, 8, 16, 1, 512, 1),      # many beams: fused although the wide kernel could
+    (4, 8, 9, 1, 1137, 2), (4, 8, 9, 1, 1138, 1),
+    (37, 4, 4, 4, 128, 2), (149, 1, 4, 4, 128, 2)])    # at and above one work group per SM (tiled: unsplit, two launches)
+def test_form_of_a_step_with_nine_to_sixteen_columns(batch, hkv, beams, group, P, launches):
+    w = _w("forms", batch, beams, group, hkv, 128, P, 4, "f16", seed=13)
+    r = Run(w)
+    try:
+        for t in range(3):
+            n = r.h.launch_count
+            _, out, q = r.step_fused()
+            assert r.h.launch_count - n == launches
+        r.check(out, q, 2, sampled_pairs(w, 16))
+        again, _ = r.decode(q)                     # and the attention call by itself
+        r.check(again, q, 2, sampled_pairs(w, 16))
+    finally:
+        r.close()
