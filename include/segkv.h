@@ -385,7 +385,8 @@ SEGKV_API int segkv_get_splits(segkv_t h);
  * The same attention as segkv_decode_sdpa computed by the plain per-beam kernel
  * (each beam walks its own rows through the beam-index table, Section 3.3's
  * formulation taken literally; the prompt is re-read per beam).  A
- * cross-check; no other entry point uses it.
+ * cross-check; segkv_decode_sdpa uses it for a few dozen keys where there are
+ * more than 16 query columns per kv head (8 at head_dim 256).
  * Arguments and errors as segkv_decode_sdpa.
  */
 SEGKV_API int segkv_decode_sdpa_rowwise(segkv_t h, const void* q, void* out, const float* alibi_slopes,

@@ -409,7 +409,8 @@ int stream_splits(const segkv* h) {
 // Can the wide kernel (tcgen05, up to 32 query columns) serve this shape at some length?
 bool wide_possible(const Dims& d) { return !tiled_supported(d) || (d.head_dim == 128 && d.beams * d.group > 8); }
 
-// Does it serve an attention call of its own?  Always where the tiled kernel has no form.  Nine to 16 columns at head_dim
+// Does it serve an attention call of its own?  Where the tiled kernel has no form, unless the keys are so few that the
+// per-beam kernel is done before the wide one has started and finished (below).  Nine to 16 columns at head_dim
 // 128 run on either.  The wide kernel gets through keys faster, but it keeps one CTA per SM: the tiled one is ahead
 // where the work groups are more than the SMs (append and attention, tiled / wide in us: 35 / 48 with 9 beams, 160 work
 // groups x 512 prompt; 44 / 51 with 16 beams, 512 x 128; 117 / 157 with 16 beams, 320 x 2048, 256 steps) and where there
@@ -422,6 +423,21 @@ bool use_wide(const segkv* h) {
     return wide_possible(h->d) && h->splits_forced == 0 && h->stages_forced == 0 && h->combine_forced == 0 && h->tile_forced == 0 &&
            (long long)h->d.batch * h->d.kv_heads <= h->sm_count &&
            (long long)h->d.batch * h->d.kv_heads * (h->prompt_len > 0 ? h->prompt_len : 0) >= 16384;
+}
+
+// The per-beam kernel for a few keys: no lists, no tensor memory, no query block, one CTA per row and head.  Append and
+// attention, per-beam / wide in us, at 18, 40 and 72 keys (up to four CTAs an SM): fp16 6.4 / 8.0, 8.3 / 8.0, 11 / 8.0 at
+// head_dim 64, 6.4 / 8.9, 8.3 / 9.0, 10.8 / 9.0 at 128, 6.5 / 10.5, 8.7 / 10.5, 11.4 / 11.1 at 256; bf16 6.4 / 8.4, 8.4 / 8.4
+// at 64, 6.4 / 9.5, 8.3 / 9.6, 10.9 / 9.6 at 128, 6.5 / 12, 8.7 / 12, 11.4 / 12.6 at 256.  With twice the CTAs the lines
+// cross at about two thirds of the keys (7.9 / 10.7, 10.9 / 10.8 at head_dim 256, fp16), with 14 CTAs an SM nowhere.
+bool use_rowwise(const segkv* h) {
+    const Dims& d = h->d;
+    if (tiled_supported(d) || h->splits_forced > 0) return false;
+    const int keys = (h->prompt_len > 0 ? h->prompt_len : 0) + h->steps;
+    const int upto = d.dtype == SEGKV_BF16 ? (d.head_dim == 64 ? 40 : d.head_dim == 128 ? 54 : 80)
+                                           : (d.head_dim == 64 ? 36 : d.head_dim == 128 ? 46 : 64);
+    const long long ctas = (long long)d.rows * d.heads;
+    return ctas <= 8LL * h->sm_count && keys <= (ctas <= 4LL * h->sm_count ? upto : upto * 2 / 3);
 }
 
 // A step of nine to 16 columns that the tiled kernel can fuse: does it, although the wide kernel would serve the
@@ -858,6 +874,14 @@ int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_sl
     if (h->prompt_len < 0) return SEGKV_ESTATE;
     if (h->prompt_len + h->steps <= 0) return SEGKV_ESTATE;
     if (h->leader && h->leader->steps != h->steps) return SEGKV_ESTATE;   // the shared tables describe another step
+    if (use_rowwise(h)) {
+        SdpaArgs a = sdpa_args(h, q, out, alibi_slopes, 1);
+        h->dbg_wait_ns = 0;
+        h->dbg_skip = false;
+        SEGKV_CUDA(launch_sdpa_rowwise(h->d, a, (cudaStream_t)stream));
+        count_launch(h, (cudaStream_t)stream);
+        return SEGKV_OK;
+    }
     {
         int rc = ensure_lists(h, (cudaStream_t)stream);
         if (rc != SEGKV_OK) return rc;
@@ -1329,6 +1353,7 @@ int segkv_set_tuning(segkv_t h, int splits, int stages, int combine) {
 
 int segkv_get_splits(segkv_t h) {
     if (!h) return SEGKV_EINVAL;
+    if (use_rowwise(h)) return 1;
     if (use_wide(h)) return wide_splits(h);
     return choose_tiling(h, false).splits;
 }

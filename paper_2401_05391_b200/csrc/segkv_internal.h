@@ -187,7 +187,8 @@ struct SdpaArgs {
     int32_t* parent_row;
 };
 
-// Plain gather kernel: one CTA per (beam slot, head), fp32 ALU; kept as an in-library cross-check.
+// Plain gather kernel: one CTA per (beam slot, head), fp32 ALU; for a few keys of shapes that the
+// tiled kernel does not cover, and as an in-library cross-check.
 cudaError_t launch_sdpa_rowwise(const Dims& d, const SdpaArgs& a, cudaStream_t st);
 
 // Tiled split-KV kernel (TMA-staged prompt tiles, gathered response rows, tensor-core tiles).

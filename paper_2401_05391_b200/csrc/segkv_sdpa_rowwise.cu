@@ -3,7 +3,8 @@
 // direct transcription of the paper's per-beam formulation (Section 3.3): loop
 // over the prompt rows, then over the index-selected response rows, one online
 // softmax across both (segkv_rowwise.cuh).  It re-reads the prompt once per beam, so it is not the
-// fast path; the library exposes it as a cross-check.
+// fast path: the library uses it for shapes that the tiled kernel does not take while
+// the keys are few, and exposes it as a cross-check.
 #include "segkv_rowwise.cuh"
 
 namespace segkv_impl {

@@ -260,3 +260,41 @@ def test_form_of_a_step_with_nine_to_sixteen_columns(batch, hkv, beams, group, P
         r.check(again, q, 2, sampled_pairs(w, 16))
     finally:
         r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,keys", [(64, (36, 40)), (128, (46, 54)), (256, (64, 80))])
+@pytest.mark.parametrize("batch", [1, 5, 10])
+def test_few_keys_run_on_the_per_beam_kernel(D, keys, dtype, batch):
+    # 32 columns, 4 kv heads: 128, 640 (over four CTAs an SM) and 1280 (over eight) rows and heads; on both sides of the
+    # last key count that the per-beam kernel takes: its bits up to there, the oracle's values always
+    last = keys[dtype == "bf16"] if batch == 1 else keys[dtype == "bf16"] * 2 // 3
+    w = _w("few", batch, 4, 8, 4, D, last - 4, 8, dtype, seed=14)
+    r = Run(w)
+    try:
+        for t in range(6):
+            _, out, q = r.step_fused()
+            ref = torch.empty_like(q)
+            r.h.decode_sdpa_rowwise(q, ref)
+            same = torch.equal(out.view(torch.int16), ref.view(torch.int16))
+            assert same == (batch < 10 and w.prompt_len + t + 1 <= last), (t, same)
+            if t in (3, 4):
+                r.check(out, q, t, sampled_pairs(w, 8))
+    finally:
+        r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,beams,group,P", [(64, 4, 8, 0), (128, 4, 8, 0), (256, 4, 4, 0), (128, 32, 1, 3), (64, 4, 8, 64), (256, 4, 8, 32)])
+def test_wide_kernel_on_a_few_keys(dtype, D, beams, group, P):
+    # a forced split count keeps the wide kernel: no prompt, hardly any keys, a prompt without a step
+    w = _w("smallest", 3, beams, group, 2, D, P, 12, dtype, seed=15)
+    run_workload(w, all_pairs, check_steps=(0, 1, 11), splits=1, every_step_ancestry=False)
+    run_workload(w, all_pairs, check_steps=(11,), splits=2, every_step_ancestry=False)
+    if P:
+        r = Run(w, splits=1)
+        try:
+            out, q = r.decode()
+            r.check(out, q, -1, all_pairs(w))
+        finally:
+            r.close()
