@@ -102,7 +102,7 @@ struct Tc5Layout {
     static constexpr int kRingV = kStagesV * kTileKV;
     static constexpr int kQGroup = kDBoxes * kBoxQ;              // bytes of one group's Q
     static constexpr int kQ = NG * kQGroup;
-    static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 6 * NG;   // K full/empty, V full/empty, per group: S0 S1 P O Qfull Qempty
+    static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 6 * NG + 1;   // K full/empty, V full/empty, per group: S0 S1 P O Qfull Qempty; wind-down
     static constexpr size_t kBytes = 1024 + (size_t)kRingK + kRingV + kQ + 8 * kBars + NG * kRows * 4 + 64;
     // tensor memory: S buffers of KEYS columns first, then one O accumulator of D columns per group
     static constexpr int kColO = NG * NB * KEYS;
@@ -219,6 +219,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t vfull0 = kempty0 + 8 * SK, vempty0 = vfull0 + 8 * SV;
     const uint32_t gbar0 = vempty0 + 8 * SV;                      // group g: + kGB g; S buffer 0, S buffer 1, P, O, Q full, Q empty
     constexpr uint32_t kGB = 48;
+    const uint32_t bar_end = gbar0 + kGB * NG;
     float* s_row = reinterpret_cast<float*>(bars + L::kBars);     // one value per query row, between its two threads
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_row + NG * kRows);
     __shared__ int s_abort;
@@ -279,6 +280,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             mbar_init(gbar0 + kGB * g + 32, 1);
             mbar_init(gbar0 + kGB * g + 40, 1);
         }
+        mbar_init(bar_end, 1);
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -309,7 +311,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         tma_load_4d(dst + cb * kColTile + rb * L::kBoxBytes, tm, cb * 64, kvh,
                                     kt * kKeys + rb * L::kBoxRows, b, full);
             };
-            uint32_t tp = 0;                                       // K/V tiles requested so far (ring position)
+            uint32_t tp = 0, tk = 0;                               // K/V tiles requested so far (ring position); K tiles alone
             uint32_t qi[NG];                                      // items group g has taken part in: Q barrier phases
 #pragma unroll
             for (int g = 0; g < NG; ++g) qi[g] = 0;
@@ -341,12 +343,19 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     ok = mbar_wait(kempty0 + 8 * sk, ((tp / SK) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
                     load_tile(&tm_k, k_ring + (size_t)sk * kTileKV, kt, kvh, b, kfull0 + 8 * sk);
+                    tk = tp + 1;
                     ok = mbar_wait(vempty0 + 8 * sv, ((tp / SV) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
                     load_tile(&tm_v, v_ring + (size_t)sv * kTileKV, kt, kvh, b, vfull0 + 8 * sv);
                 }
             }
             if (!ok) s_abort = 1;
+            // no copy may land after the CTA has gone (all have, unless a wait ran out somewhere)
+            for (uint32_t k = tk > (uint32_t)SK ? tk - SK : 0; k < tk; ++k) (void)mbar_wait(kfull0 + 8 * (k % SK), (k / SK) & 1, p.wait_ns);
+            for (uint32_t k = tp > (uint32_t)SV ? tp - SV : 0; k < tp; ++k) (void)mbar_wait(vfull0 + 8 * (k % SV), (k / SV) & 1, p.wait_ns);
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+                if (qi[g] > 0) (void)mbar_wait(gbar0 + kGB * g + 32, (qi[g] - 1) & 1, p.wait_ns);
         } else if (STORE && lane == 1) {
             // ---- fused prefill: the tiles just read from the caller's K/V also become the prompt segment
             // (paper Section 3.2: the prompt is kept once per request).  Tile kt of a kv head is stored by
@@ -743,9 +752,15 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         }
         if (!ok && lane == 0) s_abort = 1;
     }
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
     if (warp == L::kSoftWarps + 1) {
+        if (s_abort && lane == 0) {
+            // MMAs may still be in flight: let them finish (bounded) before the tensor memory goes back
+            tc_commit(bar_end);
+            (void)mbar_wait(bar_end, 0, p.wait_ns);
+        }
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
         if (lane == 0 && s_abort) atomicOr(p.err_word, SEGKV_DEV_WAIT_LIMIT);
