@@ -245,3 +245,33 @@ def test_prefill_argument_and_state_errors():
     rc = sk.lib().segkv_prefill_sdpa(h._h, None, q.data_ptr(), None, None)
     assert rc == sk.SEGKV_EINVAL
     h.destroy()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,row_groups", [(64, 1), (64, 2), (128, 1), (128, 2), (256, 1)])
+def test_prefill_scores_that_grow_from_tile_to_tile(dtype, D, row_groups):
+    # no bias, keys 4, 10 and 25 times as long from the second, third and fifth tile on: rows whose maximum grows by more
+    # than 2^8 of the reference they use, in full and in diagonal tiles, so that weights worked out in one pass are thrown
+    # away, O is rescaled and the tile done again.  A few keys carry a row's weight then: besides the path's tolerance the
+    # rounding of the weights (2^-9 of each in bf16, 2^-12 in fp16) times the largest value is allowed for.
+    w = wl.Workload("grow", 2, 3, 4, 2, D, 700, 2, dtype, "uniform", False, 140)
+    h = sk.SegKV(w.batch, w.beams, w.heads, w.kv_heads, w.head_dim, w.prompt_len, w.steps, w.torch_dtype)
+    try:
+        h.set_prefill_tuning(row_groups)
+        kp, vp = wl.make_prompt(w, "cuda")
+        for at, by in ((128, 4.0), (256, 2.5), (512, 2.5)):
+            kp[:, at:] *= by
+        q = wl.make_prefill_query(w, "cuda")
+        h.prefill_write(kp, vp)
+        out, fused = h.prefill_sdpa(q, None, None), torch.full_like(q, float("nan"))
+        h.prefill(kp, vp, q, fused, None)
+        torch.cuda.synchronize()
+        assert h.get_error() == 0
+        assert torch.equal(out, fused)
+        rows = sampled_rows(w, 500)
+        ref = oracle.prefill_sdpa(w.dtype, w.batch, w.heads, w.kv_heads, w.head_dim, wl.to_bits(q), wl.to_bits(kp), wl.to_bits(vp), rows=rows)
+        got = np.stack([out[b, i, x].to(torch.float64).cpu().numpy() for b, i, x in rows])
+        err = np.abs(got - ref)
+        assert (err <= ATOL + RTOL * np.abs(ref) + float(vp.abs().max()) * 2.0 ** (-9 if dtype == "bf16" else -12)).all(), err.max()
+    finally:
+        h.destroy()

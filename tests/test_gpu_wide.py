@@ -298,3 +298,82 @@ def test_wide_kernel_on_a_few_keys(dtype, D, beams, group, P):
             r.check(out, q, -1, all_pairs(w))
         finally:
             r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,beams,group", [(64, 4, 8), (128, 3, 4), (256, 3, 4)])
+@pytest.mark.parametrize("splits", [1, 3])
+def test_wide_scores_that_grow_from_tile_to_tile(dtype, D, beams, group, splits):
+    # no bias, longer keys from tile to tile: the reference is renewed and O rescaled behind weights already worked out
+    w = _w("grow", 2, beams, group, 2, D, 400, 9, dtype, seed=16)
+    r = Run(w, splits=splits)
+    try:
+        for at, by in ((64, 4.0), (192, 2.5), (300, 2.5)):
+            r.kp[:, at:] *= by
+        r.h.prefill_write(r.kp, r.vp)
+        r.advance_to(8)
+        out, q = r.decode()
+        r.check(out, q, 8, all_pairs(w))
+        assert r.h.get_error() == 0
+    finally:
+        r.close()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,batch,beams,group,hkv,P,splits", [
+    (64, 3, 4, 8, 4, 130, 0), (128, 2, 4, 8, 4, 700, 0), (128, 40, 4, 8, 4, 90, 0), (128, 4, 4, 4, 8, 600, 0), (256, 3, 3, 4, 2, 300, 4)])
+def test_wide_layers_queued_without_waiting(dtype, D, batch, beams, group, hkv, P, splits):
+    # Three layers stepped in turn, nothing waited for on the host: a launch starts, and asks for its prompt, while the one
+    # before drains.  Against the oracle, and bit by bit against plain stream order, a second run, a captured step that is
+    # replayed, and layers that share one beam-index table.
+    w = _w("queued", batch, beams, group, hkv, D, P, 12, dtype, alibi=group == 8, seed=17)
+    par = wl.make_parents(w)
+    runs = {}
+    try:
+        for name in ("plain", "again", "order", "shared"):
+            rs = runs[name] = [Run(w.scaled(index=170 + i), parents=par, splits=splits) for i in range(3)]
+            if name == "shared":
+                for r in rs[1:]:
+                    r.h.share_index(rs[0].h)
+            for r in rs:
+                r.h.set_overlap(name != "order")
+        steps = [[wl.make_step(r.w, t, "cuda") for r in runs["plain"]] for t in range(w.steps)]
+        torch.cuda.synchronize()
+        outs = {}
+        for name, rs in runs.items():
+            outs[name] = torch.full((w.steps, 3, w.rows, w.heads, D), float("nan"), dtype=w.torch_dtype, device="cuda")
+            torch.cuda.synchronize()
+            for t in range(w.steps):
+                for i, r in enumerate(rs):
+                    q, k, v = steps[t][i]
+                    r.h.decode_step(t, r.parents_dev[t] if t else None, k, v, q, outs[name][t, i], r.slopes)
+            torch.cuda.synchronize()
+            assert all(r.h.get_error() == 0 for r in rs)
+        for name in ("again", "order", "shared"):
+            assert torch.equal(outs[name], outs["plain"]), name
+        rs, last = runs["plain"], w.steps - 1
+        for r, i in ((rs[0], 0), (rs[2], 2)):
+            r.q_steps, r.k_steps, r.v_steps = (list(x) for x in zip(*[steps[t][i] for t in range(w.steps)]))
+            for t in (0, 5, last):
+                r.check(outs["plain"][t, i], r.q_steps[t], t, sampled_pairs(r.w, 8))
+        again = torch.empty_like(outs["plain"][last])
+
+        def redo():
+            for i, r in enumerate(rs):
+                if r.h.steps > last:
+                    r.h.truncate_last()
+                r.h.decode_step(last, r.parents_dev[last], steps[last][i][1], steps[last][i][2], steps[last][i][0], again[i], r.slopes)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            redo()
+        for _ in range(3):
+            again.fill_(float("nan"))
+            g.replay()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(again, outs["plain"][last])
+        assert all(r.h.get_error() == 0 for r in rs)
+    finally:
+        for rs in runs.values():
+            for r in reversed(rs):
+                r.close()
