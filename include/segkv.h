@@ -186,6 +186,9 @@ SEGKV_API int segkv_append(segkv_t h, int step, const int32_t* beam_parent, cons
  * With no step appended the call attends to the prompt only (the paper's
  * "special case" of the kernel).  The call may be repeated; it changes nothing
  * but `out` and the library's own workspace.
+ * A value row that is not finite reaches the beams that read it.  Where there are
+ * at most 16 query columns per kv head (8 at head_dim 256) it can also reach the
+ * request's other beams, whose weight for it is zero (0 * Inf is NaN).
  * Errors: EINVAL, ESTATE (nothing to attend to), ECUDA.
  */
 SEGKV_API int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float* alibi_slopes, void* stream);
@@ -201,7 +204,9 @@ SEGKV_API int segkv_decode_sdpa(segkv_t h, const void* q, void* out, const float
  * Arguments, layouts and errors are those of the two calls.  The library runs
  * the step as the two launches instead where that is the faster form or the only
  * one: shapes with many query columns per kv head (more than 16, or more than 8
- * at head_dim 256 or over long prompts at head_dim 128), handles that share
+ * at head_dim 256; nine to 16 at head_dim 128 where there is at most one
+ * (request, kv head) per SM and batch * kv_heads * prompt is at least 16384,
+ * unless there are so many beams that their append costs more), handles that share
  * another handle's tables, launches whose work groups fill the GPU without being
  * split, and launches whose CTAs would each have many steps' rows or many prompt
  * tiles to go through.  Both forms give the same beam-index tables bit by bit and

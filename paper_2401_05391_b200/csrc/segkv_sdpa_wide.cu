@@ -11,8 +11,9 @@
 //  * S[128 rows, KEYS] = Q.K^T with M = 128: the at most 32 query columns are the rows, REPEATED FOUR TIMES, so
 //    that each of the four softmax warps finds all columns in its own tensor-memory lanes and takes a
 //    quarter of the tile's keys (one column per lane, KEYS/4 keys per thread: no shuffles).  The repeated
-//    rows cost MMA time the tensor pipe has to spare: 8 + 4 MMAs per 32 KB of keys and values, about 900
-//    clocks, against about 1300 clocks for an SM's share of HBM bandwidth;
+//    rows cost MMA time the tensor pipe has to spare: 8 MMAs of 64 keys and 4 of 128 columns per 32 KB of keys
+//    and values, 512 clocks of math in a tile of about 1250, the longer part of which is their issue and the waits
+//    between; an SM's share of HBM bandwidth takes about 1300;
 //  * the four warps agree on a column's maximum through shared memory (one barrier per tile, which also
 //    carries the "a wait ran out" flag, so that all warps leave together) and write the weights P into ONE
 //    shared-memory tile, the A operand of O[128, D] += P.V.  The weights keep what fp32 has of them: they go as the
@@ -24,7 +25,7 @@
 //    the reference in use (sum and weights use the same reference, so the result is exact);
 //  * prompt tiles arrive by TMA in one ring; response tiles are gathered row by row (cp.async into the same
 //    128-byte-swizzled layout) by two groups of two warps, one stage each, so that two gathers are in
-//    flight; the gather warps also place the query block;
+//    flight; the gather warps also stage the query block, which the softmax warps place in tensor memory;
 //  * splits of a work group meet in the global workspace, the parts of each added up: the last CTA to arrive folds
 //    them (as in the tiled kernel).
 //  * an Inf or a NaN in a value row would reach the columns that do not read the row (their weight there is zero, and

@@ -14,25 +14,7 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// D[tmem] (+)= A[smem] . B[smem]
-__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] . B[smem]; A is M x 16 of a 16-bit type, two elements per 32-bit column
-__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc)
-        : "memory");
-}
-// The same for a WHOLE warp that runs converged, with the instruction itself predicated to one lane.  A
+// MMAs and commits are issued by a WHOLE warp that runs converged, with the instruction itself predicated to one lane.  A
 // descriptor that the whole warp computes can live in uniform registers, where the MMA takes it from; one that
 // a single-lane branch computes has to be moved there for every MMA (measured in the wide decode kernel: 60 clocks
 // per MMA issued from a one-lane branch, whatever its shape, against its 32 of math).
@@ -46,6 +28,7 @@ __device__ __forceinline__ void tc_commit_if(uint32_t lead, uint32_t bar) {
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
         "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(lead) : "memory");
 }
+// D[tmem] (+)= A[smem] . B[smem]
 __device__ __forceinline__ void tc_mma_ss_if(uint32_t lead, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
@@ -54,6 +37,7 @@ __device__ __forceinline__ void tc_mma_ss_if(uint32_t lead, uint32_t d_tmem, uin
         ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(lead)
         : "memory");
 }
+// D[tmem] (+)= A[tmem] . B[smem]; A is M x 16 of a 16-bit type, two elements per 32-bit column
 __device__ __forceinline__ void tc_mma_ts_if(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"

@@ -455,7 +455,7 @@ def test_sixteen_query_columns_and_the_rowwise_fallback():
                  check_steps=(0, 7, 19))
     run_workload(wl.Workload("c16b", 1, 16, 2, 2, 64, 70, 20, "bf16", "uniform", False, 25), all_pairs,
                  check_steps=(0, 19))
-    # ... beyond that (here 32 beams) the per-beam kernel serves segkv_decode_sdpa and segkv_decode_step
+    # ... beyond that (here 32 beams) the per-beam kernel serves a few keys, the wide kernel the rest
     w = wl.Workload("w32", 1, 32, 2, 2, 64, 40, 12, "f16", "uniform", False, 26)
     run_workload(w, all_pairs, check_steps=(0, 5, 11))
     run_workload_fused(w, all_pairs, check_steps=(0, 5, 11))

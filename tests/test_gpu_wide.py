@@ -85,8 +85,9 @@ def test_wide_wait_runs_out_and_the_handle_recovers(splits):
 
 @pytest.mark.parametrize("dtype,beams,group", [("f16", 3, 3), ("bf16", 4, 4)])
 def test_nine_to_sixteen_columns_on_both_sides_of_the_dispatch(dtype, beams, group):
-    # head_dim 128: from 16384 prompt keys over all work groups on, these columns run on the wide kernel
-    for P, wide in ((511, False), (512, True)):
+    # head_dim 128: from 16384 prompt keys over all work groups on, these columns run on the wide kernel (which form runs
+    # is asserted by test_form_of_a_step_with_nine_to_sixteen_columns)
+    for P in (511, 512):
         w = _w("nt2", 4, beams, group, 8, 128, P, 20, dtype, alibi=group == 4, seed=6)
         run_workload(w, sampled_pairs, check_steps=(0, 19), every_step_ancestry=False)
         run_workload_fused(w, sampled_pairs, check_steps=(0, 7, 19))
@@ -97,7 +98,7 @@ def test_more_forced_splits_than_the_merge_has_room_for():
     r = Run(w, splits=64)
     try:
         r.advance_to(3)
-        assert r.h.get_splits() == 32                  # two partials (high and low parts) per split
+        assert r.h.get_splits() == 32                  # the most that this shape takes
         out, q = r.decode()
         r.check(out, q, 3, all_pairs(w))
     finally:
