@@ -44,7 +44,7 @@ def build(force: bool = False, verbose: bool = False, timeline: bool = False) ->
     procs = []
     for src in sources():
         obj = os.path.splitext(src)[0] + (".tl.o" if timeline else ".o")
-        cmd = [NVCC, *FLAGS, *(["-DSEGKV_TIMELINE", "-DSEGKV_TC5_TIMELINE=1"] if timeline else []), "-c", src, "-o", obj]
+        cmd = [NVCC, *FLAGS, *(["-DSEGKV_TIMELINE"] if timeline else []), "-c", src, "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))

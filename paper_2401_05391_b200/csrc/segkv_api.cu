@@ -752,6 +752,7 @@ int segkv_prefill_sdpa(segkv_t h, const void* q, void* out, const float* alibi_s
     a.q = q; a.out = out; a.slopes = alibi_slopes; a.err_word = h->err_word;
     a.prompt_len = h->prompt_len; a.tm_k = &h->tm_kp; a.tm_v = &h->tm_vp;
     a.row_groups = h->prefill_groups;
+    a.pdl = h->overlap;
     a.wait_ns = h->dbg_wait_ns;
     a.dbg_skip = h->dbg_skip;
     h->dbg_wait_ns = 0;
@@ -795,6 +796,7 @@ int segkv_prefill(segkv_t h, const void* k, const void* v, const void* q, void* 
     a.q = q; a.out = out; a.slopes = alibi_slopes; a.err_word = h->err_word;
     a.prompt_len = prompt_len; a.tm_k = &h->tm_kp; a.tm_v = &h->tm_vp;
     a.row_groups = h->prefill_groups;
+    a.pdl = h->overlap;
     a.wait_ns = 0;
     a.dbg_skip = false;
     a.plens = nullptr;

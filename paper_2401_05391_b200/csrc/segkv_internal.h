@@ -234,6 +234,7 @@ struct PrefillArgs {
     const CUtensorMap* tm_v_src;
     const CUtensorMap* tm_q;   // over q as [batch][prompt_len][heads][D], box 64 elements x 128 tokens; NULL if unused
     int row_groups;      // 0 = automatic
+    bool pdl;            // launch with programmatic stream serialisation
     unsigned long long wait_ns;   // test aid, as in SdpaArgs
     bool dbg_skip;
 };

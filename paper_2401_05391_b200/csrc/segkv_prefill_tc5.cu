@@ -5,7 +5,10 @@
 //
 //   * one persistent CTA per SM walks a static list of work items (one or two groups of 128
 //     query rows of one (request, head)), longest first; a group's rows are one per TMEM lane and
-//     per TWO softmax threads, which take one half of a tile's keys each;
+//     per TWO softmax threads (four where one group of head_dim 64 or 128 runs), which share a tile's keys;
+//   * an item's keys are gone through from the newest back.  Under an ALiBi bias a row's maximum then stands from its
+//     first tile on; from the oldest forward it grew with every tile, and most of Bloom's heads took two passes over each
+//     and rescaled O.  The two groups of an item also end together, each with a tile that needs no mask;
 //   * Q of each group arrives by TMA (a per-call tensor map over [B, N, H, D]) in the
 //     128-byte-swizzled K-major layout; K and V tiles (128 keys; 64 at head_dim 256) arrive by TMA
 //     in the same layout through separate rings: a K tile is needed one step before the V tile
@@ -18,25 +21,30 @@
 //     takes its A operand from tensor memory.  V is consumed as an MN-major B operand straight from
 //     its row-major tile;
 //   * the softmax threads read S with tcgen05.ld (no shuffles for the row max / sum) and
-//     rescale O in tensor memory only when a row's maximum has grown by more than 2^8 since the
-//     reference it is using (the sum uses the same reference, so the result is exact).  fp16 weights are
-//     worked out with the reference in use in one pass over the scores, and the maximum of that pass decides
-//     whether they stand;
+//     rescale O in tensor memory only when a row's maximum has grown by more than about 2^8 over the
+//     reference it is using (the sum uses the same reference, so the result is exact).  Weights are worked out with the
+//     reference in use in one pass over the scores, 16 keys at a time with the next 16 on their way; what they add up to
+//     decides whether they stand;
 //   * with two groups per CTA each has one S buffer and the tensor cores work for one group
 //     while the other is in its softmax; with one group S is double-buffered so that Q.K^T of
 //     tile j+1 runs under the softmax of tile j.  The tail of one item overlaps the head of the
 //     next (loads, and the first Q.K^T while the previous output is stored).
 //
-// What bounds it (64 requests x 56 heads x 2048 tokens, D 128, fp16: 4.09 ms, 942 TFLOP/s, 0.59 of the cuBLAS burst rate;
-// it was 4.41 ms): a group's chain softmax (1700 clocks a tile of 128 keys, 1024 of them the special-function
-// unit's) -> P.V -> Q.K^T (1024 clocks of MMAs and about 500 of barriers and pipeline), which the
-// other group's overlaps only in part.  Putting a share of the exponentials on the FMA pipes as a polynomial
-// was measured slower (4.42 ms): the issue slots it costs are on the same chain.
+// What bounds it: with thousands of items the power limit (1000 W at 1.5 to 1.65 GHz, where a lone call runs at 1.9), so that a
+// shorter chain buys less than fewer instructions and bytes do; with a few, a group's chain softmax -> P.V -> Q.K^T and
+// the start.  Measured in turn with the form that went from the oldest keys forward, held P back until the row's two
+// threads had met, spilled and was launched behind the whole kernel before (before / now, attention alone): 64 requests x
+// 56 heads x 2048 tokens at D 128 fp16 4620 / 4567 us, bf16 5040 / 4648; 32 x 112 x 1024 bf16 with ALiBi 1704 / 1466, fp16
+// 1825 / 1335; 1 x 32 x 1024 fp16 22.7 / 20.7; D 64, 16 x 64 x 2048, bf16 with ALiBi 1515 / 1053; D 256, 2 x 8 x 2000, bf16 with
+// ALiBi 61.6 / 42.2.  Putting a share of the exponentials on the FMA pipes as a polynomial was measured slower
+// (4.42 against 4.17 ms): the issue slots it costs are on the same chain.
 //
 // Tensor memory (all 512 columns are allocated): S buffers first, then one O accumulator per
 // group.  Every mbarrier is waited on phase by phase (a parity wait cannot tell phases two
 // apart) and every wait is bounded; on expiry the kernel flags SEGKV_DEV_WAIT_LIMIT, skips
 // the output and still releases its tensor memory.
+#include <type_traits>
+
 #include "segkv_internal.h"
 #include "segkv_ptx.cuh"
 #include "segkv_tc5.cuh"
@@ -68,20 +76,10 @@ struct Tc5Params {
 
 template <typename T> struct SplitP { typedef char yes; static constexpr bool value = false; };
 template <> struct SplitP<__nv_bfloat16> { typedef char yes; static constexpr bool value = true; };
-
-#ifdef SEGKV_TC5_TIMELINE
-}  // namespace
-__device__ long long g_tc5_tl[3 * 64 * 8];
-#define TC5_STAMP(role, kt, ev)                                                                   \
-    do {                                                                                          \
-        if ((SEGKV_TC5_TIMELINE != 2 || ((role) == 2 && (ev) == 0)) &&                            \
-            w == 0 && (kt) < 64)                                                                 \
-            g_tc5_tl[((role) * 64 + (kt)) * 8 + (ev)] = clock64();                                \
-    } while (0)
-namespace {
-#else
-#define TC5_STAMP(role, kt, ev) do {} while (0)
-#endif
+// Factor of the weights, as a power of two: fp16 weights are at most 2^8 of the reference times 2^7, which keeps what is
+// far below the maximum above fp16's smallest numbers.
+template <typename T> constexpr float kWeightShift = SplitP<T>::value ? 0.f : 7.f;
+template <typename T> constexpr float kWeightMax = SplitP<T>::value ? 256.f : 32768.f;    // 2^8 of the reference
 
 // Shape of one instantiation: head_dim D (64, 128 or 256), KEYS keys per K/V tile, NG groups of
 // 128 query rows per CTA.  head_dim 256 leaves tensor memory for one group and 64-key tiles only.
@@ -89,8 +87,9 @@ template <int D_, int KEYS_, int NG_>
 struct Tc5Layout {
     static constexpr int D = D_, KEYS = KEYS_, NG = NG_;
     static constexpr int NB = NG == 1 ? 2 : 1;                   // S buffers per group
-    static constexpr int kSoftWarps = 8 * NG;                    // two softmax threads per query row
-    static constexpr int kThreads = 32 * (kSoftWarps + 2);
+    static constexpr int TPR = D == 256 ? 2 : 4 / NG;            // softmax threads per query row
+    static constexpr int kSoftWarps = 4 * TPR * NG;
+    static constexpr int kThreads = 32 * (kSoftWarps + 4);       // and TMA loads, MMAs, TMA stores, one idle (it costs no registers)
     static constexpr int kDBoxes = D / 64;                       // 64-element (128-byte) column blocks of a row
     static constexpr int kBoxRows = D == 256 ? 32 : 64;          // rows of one TMA box of the prompt segment's tensor map
     static constexpr int kBoxBytes = kBoxRows * 128;
@@ -103,25 +102,27 @@ struct Tc5Layout {
     static constexpr int kQGroup = kDBoxes * kBoxQ;              // bytes of one group's Q
     static constexpr int kQ = NG * kQGroup;
     static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 6 * NG + 1;   // K full/empty, V full/empty, per group: S0 S1 P O Qfull Qempty; wind-down
-    static constexpr size_t kBytes = 1024 + (size_t)kRingK + kRingV + kQ + 8 * kBars + NG * kRows * 4 + 64;
+    static constexpr size_t kBytes = (size_t)kRingK + kRingV + kQ + 8 * kBars + NG * TPR * kRows * 4 + 16;
     // tensor memory: S buffers of KEYS columns first, then one O accumulator of D columns per group
     static constexpr int kColO = NG * NB * KEYS;
     static_assert(kColO + NG * D <= kTmemCols, "tensor memory");
     static_assert(kBytes <= 232448, "shared memory");
 };
 
-// Maximum of 32 scores of a row, in log2 units with BIAS (s * scale2 + bias0 + slope2 * i), else raw dot products;
-// MASK: keys above the row (i > lim) do not count.
-template <bool BIAS, bool MASK>
-__device__ __forceinline__ float max32(const uint32_t* sr, float scale2, float slope2, float bias0, int lim) {
-    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+// Maximum of 16 scores of a row, in log2 units with BIAS (s * scale2 + bias0 + slope2 * i), else raw dot products; keys
+// above the row (i > lim) count in `all` only.
+template <bool BIAS>
+__device__ __forceinline__ float max16(const uint32_t* sr, float scale2, float slope2, float bias0, int lim, float& all) {
+    float mx[2] = {-INFINITY, -INFINITY}, ma[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
+    for (int i = 0; i < 16; ++i) {
         float v = __uint_as_float(sr[i]);
         if (BIAS) v = fmaf(v, scale2, fmaf(slope2, (float)i, bias0));
-        mx[i & 3] = fmaxf(mx[i & 3], MASK && i > lim ? -INFINITY : v);
+        else ma[i & 1] = fmaxf(ma[i & 1], v);
+        mx[i & 1] = fmaxf(mx[i & 1], i > lim ? -INFINITY : v);
     }
-    return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+    if (!BIAS) all = fmaxf(all, fmaxf(ma[0], ma[1]));
+    return fmaxf(mx[0], mx[1]);
 }
 
 // bf16 keeps 8 significant bits of a softmax weight.  Where a few keys carry a row's whole weight
@@ -167,20 +168,25 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
     return r;
 }
 
-// Weights of 32 keys of a row from their scores: 2^(s * scale2 + c0 + slope2 * i), c0 = bias minus the row's reference;
-// packed in 16 bits (SPLIT: a second set of 16 words with the low parts), their sum added to ls.  Returns the largest exponent.
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Weights of 16 keys of a row from their scores: 2^(s * scale2 + c0 + slope2 * i), c0 = bias minus the row's reference;
+// packed in 16 bits (SPLIT: a second set of 8 words with the low parts).  Returns their sum.
 template <typename T, bool BIAS, bool MASK, bool SPLIT>
-__device__ __forceinline__ float weigh32(const uint32_t* sr, float scale2, float slope2, float c0, int lim, uint64_t* ls, uint32_t* hi, uint32_t* lo) {
+__device__ __forceinline__ uint64_t weigh16(const uint32_t* sr, float scale2, float slope2, float c0, int lim, uint32_t* hi, uint32_t* lo) {
     const uint64_t sc = f2(scale2, scale2), sl = f2(slope2, slope2), cc = f2(c0, c0);
-    float mx[2] = {-INFINITY, -INFINITY};
+    uint64_t ls[2] = {0ull, 0ull};
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 0; k < 8; ++k) {
         const uint64_t x = f2_fma(f2(__uint_as_float(sr[2 * k]), __uint_as_float(sr[2 * k + 1])), sc,
                                   BIAS ? f2_fma(sl, f2((float)(2 * k), (float)(2 * k + 1)), cc) : cc);
         const float xa = MASK && 2 * k > lim ? -INFINITY : f2_lo(x), xb = MASK && 2 * k + 1 > lim ? -INFINITY : f2_hi(x);
-        asm("max.f32 %0, %0, %1, %2;" : "+f"(mx[k & 1]) : "f"(xa), "f"(xb));
         const float ea = exp2f(xa), eb = exp2f(xb);
-        ls[k & 1] = f2_add(ls[k & 1], f2(ea, eb));
+        ls[k & 1] = k < 2 ? f2(ea, eb) : f2_add(ls[k & 1], f2(ea, eb));
         if (!SPLIT) {
             hi[k] = Mma<T>::pack(ea, eb);
         } else {
@@ -189,7 +195,7 @@ __device__ __forceinline__ float weigh32(const uint32_t* sr, float scale2, float
             lo[k] = Mma<T>::pack(ea - __uint_as_float(b0 & 0xFFFF0000u), eb - __uint_as_float(b1 & 0xFFFF0000u));
         }
     }
-    return fmaxf(mx[0], mx[1]);
+    return f2_add(ls[0], ls[1]);
 }
 
 // One CTA per SM walks a static list of work items (128*NG query rows of one (request, head)),
@@ -205,12 +211,11 @@ __global__ void __launch_bounds__(L::kThreads, 1)
 prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k_seg,
                    const __grid_constant__ CUtensorMap tm_v_seg, const Tc5Params p) {
-    constexpr int NG = L::NG, NB = L::NB, SK = L::kStagesK, SV = L::kStagesV;
+    constexpr int NG = L::NG, NB = L::NB, TPR = L::TPR, SK = L::kStagesK, SV = L::kStagesV;
     constexpr bool STORE = MODE == 1, RAGGED = MODE == 2;
     constexpr bool kSplitP = sizeof(typename SplitP<T>::yes) != 0 && SplitP<T>::value;
     constexpr int kD = L::D, kKeys = L::KEYS, kTileKV = L::kTileKV, kColTile = L::kColTile;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* k_ring = smem;                                       // tile: two halves [128 keys][64 elements]
     uint8_t* v_ring = k_ring + L::kRingK;
     uint8_t* q_smem = v_ring + L::kRingV;                         // per group two halves [128 rows][64 elements]
@@ -220,9 +225,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t gbar0 = vempty0 + 8 * SV;                      // group g: + kGB g; S buffer 0, S buffer 1, P, O, Q full, Q empty
     constexpr uint32_t kGB = 48;
     const uint32_t bar_end = gbar0 + kGB * NG;
-    float* s_row = reinterpret_cast<float*>(bars + L::kBars);     // one value per query row, between its two threads
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_row + NG * kRows);
-    __shared__ int s_abort;
+    float* s_row = reinterpret_cast<float*>(bars + L::kBars);     // [group][thread of the row][row]: one value, for the row's other threads
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_row + NG * TPR * kRows);
+    volatile int& s_abort = *reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nqt = (p.N + kRows * NG - 1) / (kRows * NG);
@@ -275,7 +280,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         for (int g = 0; g < NG; ++g) {
             mbar_init(gbar0 + kGB * g, 1);
             mbar_init(gbar0 + kGB * g + 8, 1);
-            mbar_init(gbar0 + kGB * g + 16, 256);                 // both threads of every row
+            mbar_init(gbar0 + kGB * g + 16, 4 * TPR);             // a lane of each of the group's warps
             mbar_init(gbar0 + kGB * g + 24, 1);
             mbar_init(gbar0 + kGB * g + 32, 1);
             mbar_init(gbar0 + kGB * g + 40, 1);
@@ -294,6 +299,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // Set up while the previous kernel ends: everything it may have written is read from here on.  (The launch of one
+    // prefill behind another took up to 6 us of an idle GPU.)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (warp == L::kSoftWarps) {
         // ------------------------------- TMA producer -------------------------------
@@ -323,10 +332,18 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 const int kvh = h / p.G;
                 int nkt = 0;
 #pragma unroll
-                for (int g = 0; g < NG; ++g) {
-                    const int gt = group_tiles(qt, g, request_len(b));
-                    nkt = max(nkt, gt);
-                    if (gt == 0) continue;
+                for (int g = 0; g < NG; ++g) nkt = max(nkt, group_tiles(qt, g, request_len(b)));
+                auto load_k = [&](int kt) -> bool {
+                    const uint32_t sk = tp % SK;
+                    if (!mbar_wait(kempty0 + 8 * sk, ((tp / SK) & 1) ^ 1, p.wait_ns)) return false;
+                    load_tile(&tm_k, k_ring + (size_t)sk * kTileKV, kt, kvh, b, kfull0 + 8 * sk);
+                    tk = tp + 1;
+                    return true;
+                };
+                if (nkt > 0) ok = load_k(nkt - 1);                // the item's first keys need not wait for its query
+#pragma unroll
+                for (int g = NG - 1; g >= 0; --g) {
+                    if (!ok || group_tiles(qt, g, request_len(b)) == 0) continue;
                     // the group's Q rows (past the prompt: zeros), once its previous Q is no longer read
                     ok = mbar_wait(gbar0 + kGB * g + 40, (qi[g] & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
@@ -338,12 +355,23 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     for (int cb = 0; cb < L::kDBoxes; ++cb)
                         tma_load_4d(dst + cb * kBoxQ, &tm_q, cb * 64, h, (qt * NG + g) * kRows, b, qfull);
                 }
-                for (int kt = 0; kt < nkt && ok; ++kt, ++tp) {
-                    const uint32_t sk = tp % SK, sv = tp % SV;
-                    ok = mbar_wait(kempty0 + 8 * sk, ((tp / SK) & 1) ^ 1, p.wait_ns);
+                // the next item's query into the L2 meanwhile: it is asked for when the group's last scores are done, and
+                // its first ones wait for it
+                const int w2 = j + 1 < p.rounds ? round_item(j + 1) : n_items;
+                if (ok && w2 < n_items) {
+                    const int hb2 = w2 % hb_count;
+#pragma unroll
+                    for (int g = 0; g < NG; ++g) {
+                        const int row = (item_qt(w2) * NG + g) * kRows;
+                        if (row >= p.N) continue;
+#pragma unroll
+                        for (int cb = 0; cb < L::kDBoxes; ++cb) tma_prefetch_4d(&tm_q, cb * 64, hb2 % p.H, row, hb2 / p.H);
+                    }
+                }
+                for (int kt = nkt - 1; kt >= 0 && ok; --kt, ++tp) {
+                    const uint32_t sv = tp % SV;
+                    if (kt < nkt - 1) ok = load_k(kt);
                     if (!ok) break;
-                    load_tile(&tm_k, k_ring + (size_t)sk * kTileKV, kt, kvh, b, kfull0 + 8 * sk);
-                    tk = tp + 1;
                     ok = mbar_wait(vempty0 + 8 * sv, ((tp / SV) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
                     load_tile(&tm_v, v_ring + (size_t)sv * kTileKV, kt, kvh, b, vfull0 + 8 * sv);
@@ -356,7 +384,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
             for (int g = 0; g < NG; ++g)
                 if (qi[g] > 0) (void)mbar_wait(gbar0 + kGB * g + 32, (qi[g] - 1) & 1, p.wait_ns);
-        } else if (STORE && lane == 1) {
+        }
+    } else if (warp == L::kSoftWarps + 2) {
+        if (STORE && lane == 0) {
             // ---- fused prefill: the tiles just read from the caller's K/V also become the prompt segment
             // (paper Section 3.2: the prompt is kept once per request).  Tile kt of a kv head is stored by
             // exactly one item: the first query head of the group, at the query tile whose rows start the
@@ -386,7 +416,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 int nkt = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) nkt = max(nkt, group_tiles(qt, g, request_len(b)));
-                for (int kt = 0; kt < nkt && ok; ++kt, ++tp) {
+                for (int kt = nkt - 1; kt >= 0 && ok; --kt, ++tp) {
                     const bool mine = (h % p.G) == 0 && (kt * kKeys) / (kRows * NG) == qt;
                     const uint32_t sk = tp % SK, sv = tp % SV;
                     ok = mbar_wait(kfull0 + 8 * sk, (tp / SK) & 1, p.wait_ns);
@@ -455,25 +485,25 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     nkt = max(nkt, gt[g]);
                 }
                 if (nkt == 0) continue;                           // the request ends before this item's rows
-                // (each group's query is waited for when its own scores are due: the second group's arrives later, as its
-                // last tile of the item before runs after the first group's)
+                // A group's first scores, from the K tile that holds its diagonal (the second group's: a tile earlier).
+                auto first_qk = [&](int g) -> bool {
+                    if (!wait(gbar0 + kGB * g + 32, qi[g]++ & 1)) return false;   // Q_g landed
+                    tc_fence_after();
+                    issue_qk(g, NB == 2 ? n[g] & 1 : 0u, gt[g] == 1);
+                    return true;
+                };
                 ok = wait_k();
 #pragma unroll
                 for (int g = 0; g < NG; ++g)
-                    if (gt[g] > 0 && ok) {
-                        ok = wait(gbar0 + kGB * g + 32, qi[g]++ & 1);   // Q_g landed
-                        if (ok) issue_qk(g, NB == 2 ? n[g] & 1 : 0u, gt[g] == 1);
-                    }
+                    if (gt[g] == nkt && ok) ok = first_qk(g);
                 if (!ok) break;
                 release_k();
-                for (int kt = 0; kt < nkt && ok; ++kt) {
-                    TC5_STAMP(2, kt, 0);
-                    if (NB == 2 && kt + 1 < nkt) {                // next tile's scores run under this tile's softmax
+                for (int kt = nkt - 1; kt >= 0 && ok; --kt) {     // the newest keys first
+                    if (NB == 2 && kt > 0) {                      // next tile's scores run under this tile's softmax
                         ok = wait_k();
                         if (!ok) break;
 #pragma unroll
-                        for (int g = 0; g < NG; ++g)
-                            if (kt + 1 < gt[g]) issue_qk(g, (n[g] + 1) & 1, kt + 2 == gt[g]);
+                        for (int g = 0; g < NG; ++g) issue_qk(g, (n[g] + 1) & 1, kt == 1);
                         release_k();
                     }
                     const uint64_t vd = dv + (v_lo0 + vst * (uint32_t)(kTileKV >> 4));
@@ -482,58 +512,68 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     bool k_next = false;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
-                        if (kt >= gt[g]) continue;
-                        ok = wait(gbar0 + kGB * g + 16, n[g] & 1);   // P_g written over its S buffer
-                        if (!ok) break;
-                        TC5_STAMP(2, kt, 1 + 3 * g);
-                        tc_fence_after();
-                        const uint32_t p_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + (NB == 2 ? n[g] & 1 : 0u));
-#pragma unroll
-                        for (int kk = 0; kk < kKeys / 16; ++kk)   // O_g += P_g[:, 16 keys] . V[16 keys, :]
-                            tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + (kk >> 1) * 32 + (kk & 1) * 8,
-                                         vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (kt > 0 || kk > 0));
-                        if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, steep)) {
-#pragma unroll
-                            for (int kk = 0; kk < kKeys / 16; ++kk)   // ... and the low parts of the weights that have one
-                                if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, steep))
-                                    tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + (kk >> 1) * 32 + 16 + (kk & 1) * 8,
-                                                 vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
-                        }
-                        tc_commit_if(lead, gbar0 + kGB * g + 24);
-                        ++n[g];
-                        if (NB == 1 && kt + 1 < gt[g]) {          // the group's next scores, behind its P.V in the pipe
+                        if (kt > gt[g]) continue;
+                        if (kt == gt[g]) {                        // its diagonal tile comes next
+                            if (NB == 2 || kt == 0) continue;
                             if (!k_next) {
                                 ok = wait_k();
                                 if (!ok) break;
                                 k_next = true;
                             }
-                            issue_qk(g, 0u, kt + 2 == gt[g]);
+                            ok = first_qk(g);
+                            if (!ok) break;
+                            continue;
+                        }
+                        ok = wait(gbar0 + kGB * g + 16, n[g] & 1);   // P_g written over its S buffer
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t p_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + (NB == 2 ? n[g] & 1 : 0u));
+#pragma unroll
+                        for (int kk = 0; kk < kKeys / 16; ++kk)   // O_g += P_g[:, 16 keys] . V[16 keys, :]
+                            tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16,
+                                         vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (kt + 1 < gt[g] || kk > 0));
+                        if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, steep)) {
+#pragma unroll
+                            for (int kk = 0; kk < kKeys / 16; ++kk)   // ... and the low parts of the weights that have one
+                                if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, steep))
+                                    tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16 + 8,
+                                                 vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
+                        }
+                        tc_commit_if(lead, gbar0 + kGB * g + 24);
+                        ++n[g];
+                        if (NB == 1 && kt > 0) {                  // the group's next scores, behind its P.V in the pipe
+                            if (!k_next) {
+                                ok = wait_k();
+                                if (!ok) break;
+                                k_next = true;
+                            }
+                            issue_qk(g, 0u, kt == 1);
                         }
                     }
                     if (!ok) break;
                     tc_commit_if(lead, vempty0 + 8 * vst);        // stage free once every MMA so far is done
                     if (++vst == SV) { vst = 0; vph ^= 1u; }
-                    if (NB == 1 && kt + 1 < nkt) release_k();
+                    if (NB == 1 && kt > 0) release_k();
                 }
             }
             if (!ok && lane == 0) s_abort = 1;
         }
-    } else {
-        // ------------------------------ softmax warps: two threads per row ------------------------------
-        // Each takes one half of a tile's keys, and at the end of an item one half of the output row.  (One thread per row
+    } else if (warp < L::kSoftWarps) {
+        // ------------------------------ softmax warps: two or four threads per row ------------------------------
+        // Each takes its part of a tile's keys, and at the end of an item its part of the output row.  (One thread per row
         // spent 2200 clocks on a tile of 128 keys, of which 1170 are hidden behind the other group's MMAs: the
-        // chain softmax -> P.V -> next Q.K^T bound the kernel.  Twice the warps hide each other's latencies.)
-        constexpr int KH = kKeys / 2, DH = kD / 2;
-        const int g = warp >> 3, half = (warp >> 2) & 1, r = (warp & 3) * 32 + lane;
-        const int pair = 1 + g * 4 + (warp & 3);                  // barrier of the two warps that share these rows
+        // chain softmax -> P.V -> next Q.K^T bound the kernel.  More warps hide each other's latencies: a lone group's
+        // tile took 1890 clocks with two threads per row.)
+        constexpr int KH = kKeys / TPR, DH = kD / TPR;
+        const int g = warp / (4 * TPR), part = (warp >> 2) % TPR, r = (warp & 3) * 32 + lane;
+        const int rows_bar = 1 + g * 4 + (warp & 3);              // barrier of the warps that share these rows
         const uint32_t bar_s0 = gbar0 + kGB * g, bar_p = bar_s0 + 16, bar_o = bar_s0 + 24;
         const uint32_t tm_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);     // this warp's TMEM lanes
-        const uint32_t tm_o = tm_lane + (uint32_t)(L::kColO + kD * g + DH * half);
-        float* xrow = s_row + g * kRows + r;
-        const bool stamp = lane == 0 && (warp & 7) == 0;
+        const uint32_t tm_o = tm_lane + (uint32_t)(L::kColO + kD * g + DH * part);
+        float* xrow = s_row + g * TPR * kRows + r;                // + kRows x thread of the row
         const size_t qstride = (size_t)p.H * kD;
         uint32_t n = 0;                                           // tiles of this group so far: barrier phases
-        bool ok = true, gone = false;                             // a wait of this thread ran out; the pair of warps has agreed to leave
+        bool ok = true, gone = false;                             // a wait of this thread ran out; the row's warps have agreed to leave
         for (int j = 0; j < p.rounds && !gone; ++j) {
             const int w = round_item(j);
             if (w >= n_items) continue;
@@ -545,124 +585,162 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const float slope2 = slope_nat * 1.4426950408889634f;
             const bool biased = p.slopes != nullptr;
             float m_ref = -INFINITY, l_run = 0.f;
-            for (int kt = 0; kt < my_tiles; ++kt, ++n) {
+            for (int t = 0; t < my_tiles; ++t, ++n) {
+                const int kt = my_tiles - 1 - t;                  // the newest keys first
                 const int buf = NB == 2 ? (int)(n & 1) : 0;
-                const uint32_t tm_s = tm_lane + (uint32_t)(kKeys * (g * NB + buf));
+                const uint32_t tm_s = tm_lane + (uint32_t)(kKeys * (g * NB + buf) + KH * part);
                 if (ok) ok = mbar_wait_hot(bar_s0 + 8 * buf, (NB == 2 ? (n >> 1) : n) & 1, p.wait_ns);
                 ok = __all_sync(0xffffffffu, ok);
-                if (stamp) TC5_STAMP(g, kt, 0);
                 // One tile of the group, from the scores in tensor memory to the weights handed to the MMA thread.
-                // P goes in place of the scores: 32 keys' weights, two to a column, over the first half of those
+                // P goes in place of the scores: 16 keys' weights, two to a column, over the first half of those
                 // keys' columns, low parts (bf16, where the weights go in two parts) over the second half.
-                const int key0 = kt * kKeys + half * KH;
-                const bool diag = key0 + KH - 1 > row0;            // keys that reach past the group's first row
+                const int key0 = kt * kKeys + part * KH;
                 const int lim = row - key0;                        // key index i is visible iff i <= lim
                 const float bias0 = slope2 * (float)(key0 - row);
-                const uint32_t tm_sh = tm_s + KH * half;
                 const bool two = kSplitP && split_p_keys(row0, kt * kKeys, kKeys, slope_nat >= kSplitSlope);
                 float alpha = 1.f;
-                uint64_t ls[2] = {0ull, 0ull};
-                // The reference in use nearly always stands after the first tile: the weights are worked out with it
-                // in one pass over the scores that notes their maximum on the way, and stored when both threads of
-                // the row know that it stands.  (Not under a slope that lifts the maximum by 2^4 and more from tile to
-                // tile; nor in bf16 with two groups, whose two kinds of weights leave no registers for it, 2.61 against
-                // 1.92 ms at 32 x 112 heads x 1024 with ALiBi, or with a bias, 30.2 against 26.7 us at 1 x 32 x 1024.)
-                const bool steady = slope2 * (float)kKeys < 4.f;
-                bool stands = (!kSplitP || (NG == 1 && !biased)) && kt > 0 && !two && steady;
-                if (stands) {
-                    float mx = -INFINITY;
-                    uint32_t pk[KH / 2];
+                uint64_t ls = 0ull;
+                int kept = 0;                                     // keys whose weights are stored
+                // The reference in use nearly always stands behind the diagonal tiles: the weights are worked out and stored
+                // with it in one pass over the scores; 16 keys whose weights add up to more than 2^8 end the pass.  (That they
+                // do is seen from their sum, which is needed anyhow: noting the maximum cost an instruction for every
+                // two scores, and the kernel's large launches run at the power limit.  Not where no key has been visible to a
+                // row so far, nor under a slope that lifts the maximum by 2^4 and more from tile to tile, which towards
+                // older keys is a negative one.)
+                const bool fresh = t == 0 || -slope2 * (float)kKeys >= 4.f || __any_sync(0xffffffffu, m_ref == -INFINITY);
+                bool stands = false;
+                if (!fresh) {
                     if (ok) {
                         tc_fence_after();
+                        const float m_use = m_ref - kWeightShift<T>;
+                        auto pass = [&](auto with_bias, auto in_two) {
+                            constexpr bool BIAS = decltype(with_bias)::value, SPLIT = decltype(in_two)::value;
+                            uint32_t sr[2][16];                   // the next 16 scores are on their way while these are worked on
+                            tc_ld16(tm_s, sr[0]);
 #pragma unroll
-                        for (int c = 0; c < KH; c += 32) {
-                            uint32_t sr[32];
-                            tc_ld32(tm_sh + c, sr);
-                            tc_wait_ld();
-                            pin<32>(sr);
-                            if (c == 0 && stamp) TC5_STAMP(g, kt, 1);
-                            const float c0 = (biased ? bias0 + slope2 * (float)c : 0.f) - m_ref;
-                            if (biased) {
-                                if (diag) mx = fmaxf(mx, weigh32<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
-                                else mx = fmaxf(mx, weigh32<T, true, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
-                            } else {
-                                if (diag) mx = fmaxf(mx, weigh32<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
-                                else mx = fmaxf(mx, weigh32<T, false, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, pk + c / 2, nullptr));
+                            for (int c = 0; c < KH; c += 16) {
+                                uint32_t* cur = sr[(c >> 4) & 1];
+                                tc_wait_ld();
+                                pin<16>(cur);
+                                if (c + 16 < KH) tc_ld16(tm_s + c + 16, sr[((c >> 4) & 1) ^ 1]);
+                                const float c0 = (BIAS ? bias0 + slope2 * (float)c : 0.f) - m_use;
+                                uint32_t hi[8], lo[8];
+                                const uint64_t lp = weigh16<T, BIAS, false, SPLIT>(cur, p.scale2, slope2, c0, 0, hi, lo);
+                                if (__any_sync(0xffffffffu, f2_lo(lp) + f2_hi(lp) > kWeightMax<T>)) break;
+                                ls = f2_add(ls, lp);
+                                tc_st8(tm_s + c, hi);
+                                if (SPLIT) tc_st8(tm_s + c + 8, lo);
+                                kept = c + 16;
                             }
+                            tc_wait_ld();
+                        };
+                        if (kSplitP && two) {
+                            if (biased) pass(std::true_type{}, std::integral_constant<bool, kSplitP>{});
+                            else pass(std::false_type{}, std::integral_constant<bool, kSplitP>{});
+                        } else {
+                            if (biased) pass(std::true_type{}, std::false_type{});
+                            else pass(std::false_type{}, std::false_type{});
                         }
                     }
-                    stands = bar_and(pair, 64, ok && !(mx > 8.f));
-                    if (stands) {
-#pragma unroll
-                        for (int c = 0; c < KH; c += 32) tc_st16(tm_sh + c, pk + c / 2);
-                    }
+                    stands = bar_and(rows_bar, 32 * TPR, ok && kept == KH);
                 }
                 if (!stands) {
-                    // A new reference, if the maximum has grown by more than 2^8: exponentials stay below 2^8 of the
-                    // reference, the sum and O use the same reference, so the result is exact.
-                    float tmax = -INFINITY;
+                    // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4 (those
+                    // that have are below 2^8 of the one in use): the sum and O use the same reference, so the
+                    // result is exact.  Keys beyond the last row of the warp take no part.
+                    float tmax = -INFINITY, tall = -INFINITY;
+                    // A row that sees a few keys of its diagonal tile and many behind it takes the maximum of the whole tile for
+                    // what is to come: the largest weights, just below a power of two, are then rounded best.  (With the
+                    // few keys' maximum the error against 64 bits was up to 1 % larger.)
+                    const bool guess = t == 0 && kt > 0 && !biased;
+                    const int seen = row0 + (warp & 3) * 32 + 32 - key0;       // keys that some row of the warp sees
                     if (ok) {
                         tc_fence_after();
 #pragma unroll 1
-                        for (int c = 0; c < KH; c += 32) {
-                            uint32_t sr[32];
-                            tc_ld32(tm_sh + c, sr);
+                        for (int c = kept; c < KH && (c < seen || guess); c += 16) {
+                            uint32_t sr[16];
+                            tc_ld16(tm_s + c, sr);
                             tc_wait_ld();
-                            pin<32>(sr);
+                            pin<16>(sr);
                             // in log2 units; without a bias the scale is folded into the exponent's FMA
-                            float m;
-                            if (biased) m = diag ? max32<true, true>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c)
-                                                 : max32<true, false>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c);
-                            else m = (diag ? max32<false, true>(sr, p.scale2, slope2, bias0, lim - c)
-                                           : max32<false, false>(sr, p.scale2, slope2, bias0, lim - c)) * p.scale2;
-                            tmax = fmaxf(tmax, m);
+                            tmax = fmaxf(tmax, biased ? max16<true>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c, tall)
+                                                      : max16<false>(sr, p.scale2, slope2, 0.f, lim - c, tall) * p.scale2);
                         }
                     }
-                    bool need = tmax > m_ref + 8.f;
-                    // the two threads of a row compare notes only then (at once where a new reference is expected)
-                    if (kt == 0 || !steady || !bar_and(pair, 64, ok && !need)) {
-                        if (half == 0) *xrow = tmax;
-                        ok = bar_and(pair, 64, ok);
-                        gone = !ok;
-                        if (gone) break;
-                        if (half == 1) {
-                            tmax = fmaxf(tmax, *xrow);
-                            *xrow = tmax;
-                        }
-                        bar_sync_n(pair, 64);
-                        if (half == 0) tmax = *xrow;
-                        need = tmax > m_ref + 8.f;
-                        if (need) {
-                            alpha = exp2f(m_ref - tmax);               // 0 on the first tile
-                            m_ref = tmax;
-                        }
+                    xrow[part * kRows] = tmax;
+                    ok = bar_and(rows_bar, 32 * TPR, ok);
+                    gone = !ok;
+                    if (gone) break;
+#pragma unroll
+                    for (int i = 0; i < TPR; ++i) tmax = fmaxf(tmax, xrow[i * kRows]);
+                    bar_sync_n(rows_bar, 32 * TPR);
+                    if (guess) {
+                        xrow[part * kRows] = tall * p.scale2;
+                        bar_sync_n(rows_bar, 32 * TPR);
+                        tall = xrow[0];
+#pragma unroll
+                        for (int i = 1; i < TPR; ++i) tall = fmaxf(tall, xrow[i * kRows]);
+                        bar_sync_n(rows_bar, 32 * TPR);
+                        tmax = fmaxf(tmax, fminf(tall, tmax + 4.f));
                     }
-                    ls[0] = ls[1] = 0ull;
+                    const bool need = tmax > m_ref + 4.f, rescale = need && m_ref > -INFINITY;   // (O is zero so far, else)
+                    if (need) {
+                        alpha = exp2f(m_ref - tmax);              // 0 on the first keys
+                        m_ref = tmax;
+                    }
+                    // (no visible key of this row so far: its weights are zeros with any reference)
+                    const float m_use = (m_ref == -INFINITY ? 0.f : m_ref) - kWeightShift<T>;
+                    // weights that are stored already, with the reference before
+                    if (kept > 0) tc_wait_st();
+                    ls = f2_mul(ls, f2(alpha, alpha));
 #pragma unroll 1
-                    for (int c = 0; c < KH; c += 32) {
-                        uint32_t sr[32], hi[16], lo[16];
-                        tc_ld32(tm_sh + c, sr);
+                    for (int c = 0; c < kept; c += 16) {
+                        uint32_t u[16];
+                        tc_ld16(tm_s + c, u);
                         tc_wait_ld();
-                        pin<32>(sr);
-                        const float c0 = (biased ? bias0 + slope2 * (float)c : 0.f) - m_ref;
-                        if (kSplitP && two) {
-                            if (biased) (void)weigh32<T, true, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
-                            else (void)weigh32<T, false, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
-                            tc_st16(tm_sh + c + 16, lo);
-                        } else {
-                            if (biased) {
-                                if (diag) (void)weigh32<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
-                                else (void)weigh32<T, true, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                        pin<16>(u);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float2 a = Mma<T>::unpack(u[i]);
+                            if (kSplitP && two) {
+                                const float2 e = Mma<T>::unpack(u[8 + i]);
+                                const float x = (a.x + e.x) * alpha, y = (a.y + e.y) * alpha;
+                                u[i] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+                                u[8 + i] = Mma<T>::pack(x - __uint_as_float(__float_as_uint(x) & 0xFFFF0000u), y - __uint_as_float(__float_as_uint(y) & 0xFFFF0000u));
                             } else {
-                                if (diag) (void)weigh32<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
-                                else (void)weigh32<T, false, false, false>(sr, p.scale2, slope2, c0, lim - c, ls, hi, lo);
+                                u[i] = Mma<T>::pack(a.x * alpha, a.y * alpha);
                             }
                         }
-                        tc_st16(tm_sh + c, hi);
+                        tc_st8(tm_s + c, u);
+                        if (kSplitP && two) tc_st8(tm_s + c + 8, u + 8);
                     }
-                    // O is rescaled, half a row per thread, before this thread hands over its weights (the MMA thread waits for both
-                    // threads'), once P.V of the previous tile is done: after the weights, under which that P.V runs
-                    if (kt > 0 && __any_sync(0xffffffffu, need)) {
+#pragma unroll 1
+                    for (int c = kept; c < KH; c += 16) {
+                        uint32_t sr[16], hi[8], lo[8];
+                        if (c < seen) {
+                            tc_ld16(tm_s + c, sr);
+                            tc_wait_ld();
+                            pin<16>(sr);
+                            const float c0 = (biased ? bias0 + slope2 * (float)c : 0.f) - m_use;
+                            uint64_t lp;
+                            if (kSplitP && two) {
+                                if (biased) lp = weigh16<T, true, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                                else lp = weigh16<T, false, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                            } else {
+                                if (biased) lp = weigh16<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                                else lp = weigh16<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                            }
+                            ls = f2_add(ls, lp);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) hi[i] = lo[i] = 0u;
+                        }
+                        tc_st8(tm_s + c, hi);
+                        if (kSplitP && two) tc_st8(tm_s + c + 8, lo);
+                    }
+                    // O is rescaled, a part of the row per thread, before this thread hands over its weights (the MMA thread waits
+                    // for all of them), once P.V of the previous tile is done: after the weights, under which that P.V runs
+                    if (t > 0 && __any_sync(0xffffffffu, rescale)) {
                         ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
                         ok = __all_sync(0xffffffffu, ok);
                         if (ok) {
@@ -678,63 +756,59 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                                 tc_st16(tm_o + c * 16, orr);
                             }
                         }
-                        if (stamp) TC5_STAMP(g, kt, 3);
                     }
                 }
-                const uint64_t lt = f2_add(ls[0], ls[1]);
-                l_run = l_run * alpha + (f2_lo(lt) + f2_hi(lt));
-                if (stamp) TC5_STAMP(g, kt, 2);
+                l_run = l_run * alpha + (f2_lo(ls) + f2_hi(ls));
                 // With one S buffer these scores were issued behind P.V of the previous tile, which keeps the O and P
                 // barriers at the phases waited for; with two, where a thread could run two phases ahead of the
                 // MMA thread, every phase of the O barrier is waited for in turn.
-                if (NB == 2 && kt > 0 && ok) {
+                if (NB == 2 && t > 0 && ok) {
                     ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
                     ok = __all_sync(0xffffffffu, ok);
                 }
                 tc_wait_st();
                 tc_fence_before();
-                if (ok && !(p.dbg_skip && tid == 0 && n == 0)) mbar_arrive(bar_p);
-                if (stamp) TC5_STAMP(g, kt, 4);
+                __syncwarp();
+                if (lane == 0 && ok && !(p.dbg_skip && tid == 0 && n == 0)) mbar_arrive(bar_p);
             }
             if (gone) break;
             // the item's output: O / l, once the last P.V has landed.  The next item's first P.V
-            // cannot overwrite O before these loads: it waits for this thread's next P arrival.
+            // cannot overwrite O before these loads: it waits for this warp's next P arrival.
             if (ok) ok = mbar_wait_hot(bar_o, (n - 1) & 1, p.wait_ns);
             ok = __all_sync(0xffffffffu, ok);
-            ok = bar_and(pair, 64, ok);
+            xrow[part * kRows] = l_run;
+            ok = bar_and(rows_bar, 32 * TPR, ok);
             gone = !ok;
             if (gone) break;
             tc_fence_after();
-            if (half == 0) *xrow = l_run;
-            bar_sync_n(pair, 64);
-            if (half == 1) {
-                l_run += *xrow;
-                *xrow = l_run;
-            }
-            bar_sync_n(pair, 64);
-            if (half == 0) l_run = *xrow;
-            const float inv = 1.f / l_run;
-            // Four lanes trade 16-byte pieces of their rows, so that a store instruction writes 64 bytes of each of 8 rows
-            // instead of 16 of 32: with one row per lane the stores of an item took 3400 clocks (6500 at head_dim 256).
-            const int len = request_len(b), q4 = lane & 3, rowq = row0 + (r & ~3);
-            T* oq = reinterpret_cast<T*>(p.out) + ((size_t)b * p.N * p.H + h) * kD + (size_t)rowq * qstride + DH * half + q4 * 8;
-#pragma unroll 1
-            for (int c = 0; c < DH / 32; ++c) {
-                uint32_t orr[32];
-                tc_ld32(tm_o + c * 32, orr);
-                tc_wait_ld();
-                pin<32>(orr);
-                uint32_t v[4][4];                                 // [piece][word]
+            l_run = 0.f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < TPR; ++i) l_run += xrow[i * kRows];
+            bar_sync_n(rows_bar, 32 * TPR);
+            const float inv = 1.f / l_run;
+            // NP lanes trade 16-byte pieces of their rows, so that a store instruction writes 64 (32) bytes of each of 8 (16) rows
+            // instead of 16 of 32: with one row per lane the stores of an item took 3400 clocks (6500 at head_dim 256).
+            constexpr int EC = DH < 32 ? DH : 32, NP = EC / 8;    // columns at a time; pieces of a row and lanes that trade
+            const int len = request_len(b), rowq = row0 + (r & ~(NP - 1));
+            T* oq = reinterpret_cast<T*>(p.out) + ((size_t)b * p.N * p.H + h) * kD + (size_t)rowq * qstride + DH * part + (lane & (NP - 1)) * 8;
+#pragma unroll 1
+            for (int c = 0; c < DH / EC; ++c) {
+                uint32_t orr[EC];
+                if constexpr (EC == 32) tc_ld32(tm_o + c * EC, orr);
+                else tc_ld16(tm_o + c * EC, orr);
+                tc_wait_ld();
+                pin<EC>(orr);
+                uint32_t v[NP][4];                                // [piece][word]
+#pragma unroll
+                for (int i = 0; i < NP; ++i)
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
                         v[i][u] = Mma<T>::pack(__uint_as_float(orr[8 * i + 2 * u]) * inv, __uint_as_float(orr[8 * i + 2 * u + 1]) * inv);
 #pragma unroll
-                for (int x = 1; x <= 2; x <<= 1) {                // a 4 x 4 transposition in two exchanges
+                for (int x = 1; x < NP; x <<= 1) {                // an NP x NP transposition, an exchange per bit
                     const bool up = (lane & x) != 0;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < NP; ++i) {
                         if (i & x) continue;
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
@@ -745,9 +819,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     }
                 }
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < NP; ++i)
                     if (rowq + i < len)
-                        *reinterpret_cast<uint4*>(oq + (size_t)i * qstride + c * 32) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                        *reinterpret_cast<uint4*>(oq + (size_t)i * qstride + c * EC) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
             }
         }
         if (!ok && lane == 0) s_abort = 1;
@@ -808,10 +882,19 @@ cudaError_t launch_tc5(const Dims& d, const PrefillArgs& a, Tc5Params p, int sms
     // fused prefill: load through the maps over the caller's arrays, store through the segment's
     const bool store = a.tm_k_src && a.tm_v_src;
     p.store_kv = store ? 1 : 0;
-    if (store) prefill_tc5_kernel<T, L, 1><<<grid, L::kThreads, smem, st>>>(*a.tm_q, *a.tm_k_src, *a.tm_v_src, *a.tm_k, *a.tm_v, p);
-    else if (p.plens) prefill_tc5_kernel<T, L, 2><<<grid, L::kThreads, smem, st>>>(*a.tm_q, *a.tm_k, *a.tm_v, *a.tm_k, *a.tm_v, p);
-    else prefill_tc5_kernel<T, L, 0><<<grid, L::kThreads, smem, st>>>(*a.tm_q, *a.tm_k, *a.tm_v, *a.tm_k, *a.tm_v, p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(L::kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.pdl ? 1 : 0;
+    if (store) return cudaLaunchKernelEx(&cfg, prefill_tc5_kernel<T, L, 1>, *a.tm_q, *a.tm_k_src, *a.tm_v_src, *a.tm_k, *a.tm_v, p);
+    if (p.plens) return cudaLaunchKernelEx(&cfg, prefill_tc5_kernel<T, L, 2>, *a.tm_q, *a.tm_k, *a.tm_v, *a.tm_k, *a.tm_v, p);
+    return cudaLaunchKernelEx(&cfg, prefill_tc5_kernel<T, L, 0>, *a.tm_q, *a.tm_k, *a.tm_v, *a.tm_k, *a.tm_v, p);
 }
 
 template <typename T>
@@ -855,9 +938,3 @@ cudaError_t launch_prefill_tc5(const Dims& d, const PrefillArgs& a, cudaStream_t
 }
 
 }  // namespace segkv_impl
-
-#ifdef SEGKV_TC5_TIMELINE
-extern "C" __attribute__((visibility("default"))) int segkv_debug_tc5_timeline(long long* host) {
-    return cudaMemcpyFromSymbol(host, segkv_impl::g_tc5_tl, sizeof(long long) * 3 * 64 * 8) == cudaSuccess ? 0 : -1;
-}
-#endif
