@@ -29,21 +29,25 @@ int cuda_fail(cudaError_t e, const char* what) {
 // Which of the library's launches came last on each stream.  A kernel launched with programmatic
 // stream serialisation may begin before its predecessor P in the stream has finished, but not
 // before P has passed its own grid-dependency wait, i.e. not before everything older than P is
-// complete.  So data whose producing launch is strictly older than the latest library launch on
-// the same stream may be read by the new kernel from its very first instruction.  (A launch of
-// the caller's own in between only helps: it does not release its dependents early.)
+// complete.  So data whose producing launch is strictly older than P may be read by the new kernel from its
+// very first instruction.  The append kernels let their successors go before that wait: behind one of them
+// only what was complete when IT began counts (launched without programmatic serialisation: everything
+// older; else what was complete for its own predecessor's successor).  (A launch of the caller's own in between
+// only helps: it does not release its dependents early.)
 // ---------------------------------------------------------------------------
 struct StreamLog {
     cudaStream_t st;
     unsigned long long last;      // sequence number of the library's latest launch on st
+    unsigned long long complete;  // launches older than this are complete when the next kernel on st begins
     bool used;
 };
+enum Release { kAfterWait, kAtOnce, kAtOnceSerialised };      // when a launch lets its successor begin
 std::mutex g_log_mu;
 StreamLog g_log[32];
 unsigned long long g_launch_seq = 0;
 
 // Record a launch on `st`; returns its sequence number.
-unsigned long long note_launch(cudaStream_t st) {
+unsigned long long note_launch(cudaStream_t st, Release rel) {
     std::lock_guard<std::mutex> lk(g_log_mu);
     const unsigned long long seq = ++g_launch_seq;
     int slot = -1, oldest = 0;
@@ -53,18 +57,20 @@ unsigned long long note_launch(cudaStream_t st) {
         else if (g_log[i].last < g_log[oldest].last || !g_log[oldest].used) oldest = i;
     }
     if (slot < 0) slot = oldest;          // more than 32 streams: forget the one idle longest
+    if (rel != kAtOnce) g_log[slot].complete = seq;
+    else if (!g_log[slot].used || g_log[slot].st != st) g_log[slot].complete = 0;       // (nothing is known of its predecessor)
     g_log[slot].st = st;
     g_log[slot].last = seq;
     g_log[slot].used = true;
     return seq;
 }
 
-// Is a launch `seq` on stream `st` strictly older than the library's latest launch there?
-bool older_than_latest(cudaStream_t st, cudaStream_t seq_stream, unsigned long long seq) {
+// Is a launch `seq` on stream `st` complete when the next kernel there begins?
+bool complete_for_next(cudaStream_t st, cudaStream_t seq_stream, unsigned long long seq) {
     if (seq == 0 || seq_stream != st) return false;
     std::lock_guard<std::mutex> lk(g_log_mu);
     for (int i = 0; i < 32; ++i)
-        if (g_log[i].used && g_log[i].st == st) return seq < g_log[i].last;
+        if (g_log[i].used && g_log[i].st == st) return seq < g_log[i].complete;
     return false;
 }
 
@@ -166,22 +172,21 @@ int make_kv_source_map(const segkv* h, const void* base, int prompt_len, CUtenso
 }
 
 // Every kernel the library launches is counted on its handle and logged on its stream.
-unsigned long long count_launch(segkv* h, cudaStream_t st) {
+unsigned long long count_launch(segkv* h, cudaStream_t st, Release rel = kAfterWait) {
     h->launches++;
-    return note_launch(st);
+    return note_launch(st, rel);
 }
 
 // The launch just made on `st` wrote the data `m` stands for.
-void mark_written(segkv* h, WriteMark* m, cudaStream_t st) {
-    m->seq = count_launch(h, st);
+void mark_written(segkv* h, WriteMark* m, cudaStream_t st, Release rel = kAfterWait) {
+    m->seq = count_launch(h, st, rel);
     m->stream = st;
 }
 
 // Is the data `m` stands for complete and visible to a kernel launched now on `st`, from that
-// kernel's first instruction on?  Yes if its launch is strictly older than the library's latest
-// launch on the same stream.  The answer depends on the order of the caller's calls alone, never on
+// kernel's first instruction on?  The answer depends on the order of the caller's calls alone, never on
 // how far the GPU has got, so the same program takes the same path every time it runs.
-bool settled(const WriteMark* m, cudaStream_t st) { return older_than_latest(st, m->stream, m->seq); }
+bool settled(const WriteMark* m, cudaStream_t st) { return complete_for_next(st, m->stream, m->seq); }
 
 void free_all(segkv* h) {
     void* ptrs[] = {h->kp, h->vp, h->kr, h->k_chunks_dev, h->parent, h->anc[0], h->anc[1], h->ulist, h->ucount, h->plens,
@@ -501,7 +506,7 @@ int ensure_lists(segkv* h, cudaStream_t st) {
     segkv* x = index_of(h);
     if (x->lists_valid || h->steps == 0) return SEGKV_OK;
     SEGKV_CUDA(launch_rebuild_lists(x->d, h->steps, x->anc[(h->steps - 1) & 1], x->ulist, x->ucount, st));
-    mark_written(h, &x->lists_mark, st);
+    mark_written(h, &x->lists_mark, st, kAtOnceSerialised);
     x->lists_valid = true;
     return SEGKV_OK;
 }
@@ -847,13 +852,15 @@ static int append_impl(segkv_t h, int step, const int32_t* beam_parent, const vo
         int rc = ensure_chunk(h, step, (cudaStream_t)stream);
         if (rc != SEGKV_OK) return rc;
     }
+    const bool pdl = h->overlap && step > 0;
+    const Release rel = pdl ? kAtOnce : kAtOnceSerialised;
     if (h->leader) {
         // the tables of this step have been made by the leader's call: only the K/V rows are stored
         if (h->leader->steps != step + 1 || h->leader->truncated) return SEGKV_ESTATE;
         SEGKV_CUDA(launch_append(h->d, step, nullptr, k_new, v_new, k_slab_of(h, step),
                                  k_slab_of(h, step) + vdelta_of(h), nullptr, nullptr, nullptr, nullptr, nullptr,
-                                 h->err_word, h->sm_count, h->overlap && step > 0, (cudaStream_t)stream, rope, false));
-        mark_written(h, &h->rows_mark, (cudaStream_t)stream);
+                                 h->err_word, h->sm_count, pdl, (cudaStream_t)stream, rope, false));
+        mark_written(h, &h->rows_mark, (cudaStream_t)stream, rel);
         h->steps = step + 1;
         h->truncated = false;
         return SEGKV_OK;
@@ -861,8 +868,8 @@ static int append_impl(segkv_t h, int step, const int32_t* beam_parent, const vo
     SEGKV_CUDA(launch_append(h->d, step, beam_parent, k_new, v_new, k_slab_of(h, step),
                              k_slab_of(h, step) + vdelta_of(h), h->parent,
                              h->anc[(step + 1) & 1], h->anc[step & 1], h->ulist, h->ucount, h->err_word,
-                             h->sm_count, h->overlap && step > 0, (cudaStream_t)stream, rope));
-    mark_written(h, &h->rows_mark, (cudaStream_t)stream);
+                             h->sm_count, pdl, (cudaStream_t)stream, rope));
+    mark_written(h, &h->rows_mark, (cudaStream_t)stream, rel);
     h->lists_mark = h->rows_mark;                  // the same launch made the lists
     h->steps = step + 1;
     h->truncated = false;

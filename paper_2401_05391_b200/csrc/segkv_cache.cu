@@ -186,10 +186,12 @@ append_kernel(int B, int W, int rows, int max_steps, int step, const int32_t* __
               const int32_t* __restrict__ anc_prev, int32_t* __restrict__ anc_cur, URow* __restrict__ ulist,
               int32_t* __restrict__ ucount, int* __restrict__ err_word, int rebuild, const RopeArgs rope) {
     // Programmatic dependent launch: this kernel touches nothing until the previous kernel of
-    // the stream has completed, and only then lets the next one start its prologue (so a kernel
-    // that starts early always finds everything older than its predecessor complete).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // the stream has completed, but lets the next one, the attention that follows it, start its prologue
+    // at once: its CTAs move in where those of the attention before this append end, and fetch their
+    // prompt tiles under the end of that launch and under this one.  (What a kernel behind this one may read
+    // ahead of its own wait is counted by the host accordingly: see StreamLog.)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if ((int)blockIdx.x >= B) {
         // ---- copy blocks -------------------------------------------------
         const long long nb = gridDim.x - B;
