@@ -13,6 +13,8 @@ LIB = os.path.join(PKG, "libsegkv.so")
 # the same library with per-CTA time stamps compiled in (read by paper_2401_05391_b200/timeline.py);
 # never loaded by the binding, the tests or the benchmark
 LIB_TIMELINE = os.path.join(PKG, "libsegkv_timeline.so")
+# the binding's calls of the decode loop (a CPython extension module over torch's tensor objects)
+LIB_HOT = os.path.join(PKG, "segkv_hot.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = [
@@ -34,10 +36,31 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_hot(force: bool = False) -> str:
+    """Compile csrc/segkv_hot.cpp into the extension module segkv_hot.so (no-op when up to date)."""
+    src = os.path.join(CSRC, "segkv_hot.cpp")
+    if not force and os.path.exists(LIB_HOT) and os.path.getmtime(LIB_HOT) >= os.path.getmtime(src):
+        return LIB_HOT
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = LIB_HOT + f".{os.getpid()}.tmp"
+    subprocess.check_call([
+        os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+        "-I", os.path.join(root, "include"), "-I", sysconfig.get_paths()["include"],
+        "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), src, "-o", tmp,
+        "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, LIB_HOT)
+    return LIB_HOT
+
+
 def build(force: bool = False, verbose: bool = False, timeline: bool = False) -> str:
     """Compile every .cu under csrc/ into libsegkv.so (no-op when up to date).  `timeline` builds
     the instrumented copy libsegkv_timeline.so instead."""
     lib = LIB_TIMELINE if timeline else LIB
+    build_hot(force)
     if not (force or _stale(lib)):
         return lib
     objs = []

@@ -2,6 +2,8 @@
 
 Argument marshalling only: every step of the decode path runs in the library's
 CUDA kernels.  PyTorch appears only as the owner of device memory and streams.
+The calls of the decode loop check their tensors in the extension module ``segkv_hot`` (``csrc/segkv_hot.cpp``); what it does
+not take as it is goes through the checks here.
 The module-level functions carry the C names; :class:`SegKV` wraps a handle.
 There is no fallback: if ``libsegkv.so`` has not been built the import of the
 library fails with an error that says how to build it.
@@ -9,6 +11,7 @@ library fails with an error that says how to build it.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -69,6 +72,19 @@ SIGNATURES = {
 }
 
 _lib = None
+HOT_PATH = os.path.join(_PKG, "segkv_hot.so")
+_hot = None
+
+
+def _hot_module():
+    """The extension module of the decode loop's calls (once).  Raises if it has not been built."""
+    global _hot
+    if _hot is None:
+        if not os.path.exists(HOT_PATH):
+            raise ImportError(f"{HOT_PATH} is missing: build it with `python -m paper_2401_05391_b200.build`")
+        spec = importlib.util.spec_from_file_location("segkv_hot", HOT_PATH)
+        _hot = importlib.util.module_from_spec(spec)
+    return _hot
 
 
 def lib() -> ctypes.CDLL:
@@ -193,12 +209,16 @@ class SegKV:
         else:
             _check(lib().segkv_create(ctypes.byref(self._h), batch, beams, heads, kv_heads, head_dim,
                                       max_prompt, max_steps, code), "segkv_create")
+        L = lib()
+        self._hot = _hot_module().Hot(self._h.value, self.rows, heads, kv_heads, head_dim, dtype is torch.bfloat16, tuple(
+            ctypes.cast(f, ctypes.c_void_p).value for f in (L.segkv_decode_step, L.segkv_append, L.segkv_decode_sdpa,
+                                                            L.segkv_truncate_last, L.segkv_steps)))
 
     # ------------------------------------------------------------ life cycle
     def destroy(self) -> None:
         if getattr(self, "_h", None) is not None and self._h:
             _check(lib().segkv_destroy(self._h), "segkv_destroy")     # refused while other handles follow this one
-            self._h = None
+            self._h = self._hot = None
 
     def __del__(self):
         try:
@@ -256,6 +276,11 @@ class SegKV:
 
     def append(self, step: int, beam_parent: Optional[torch.Tensor], k_new: torch.Tensor, v_new: torch.Tensor,
                stream=None) -> None:
+        code = self._hot.append(step, beam_parent, k_new, v_new) if stream is None and self._hot is not None else None
+        if code == 0:
+            return
+        if code is not None:
+            _check(code, "segkv_append")
         dt = self.dtype
         code = lib().segkv_append(self._h, step, _dev(beam_parent, self._parent_shape, torch.int32, "beam_parent"),
                                   _dev(k_new, self._kv_shape, dt, "k_new"), _dev(v_new, self._kv_shape, dt, "v_new"),
@@ -283,6 +308,11 @@ class SegKV:
                     alibi_slopes: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         if out is None:
             out = torch.empty(self._q_shape, dtype=self.dtype, device=q.device)
+        code = self._hot.decode_sdpa(q, out, alibi_slopes) if stream is None and self._hot is not None else None
+        if code == 0:
+            return out
+        if code is not None:
+            _check(code, "segkv_decode_sdpa")
         dt = self.dtype
         code = lib().segkv_decode_sdpa(self._h, _dev(q, self._q_shape, dt, "q"), _dev(out, self._q_shape, dt, "out"),
                                        _dev(alibi_slopes, self._slopes_shape, torch.float32, "alibi_slopes"),
@@ -296,6 +326,11 @@ class SegKV:
                     alibi_slopes: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         if out is None:
             out = torch.empty(self._q_shape, dtype=self.dtype, device=q.device)
+        code = self._hot.decode_step(step, beam_parent, k_new, v_new, q, out, alibi_slopes) if stream is None and self._hot is not None else None
+        if code == 0:
+            return out
+        if code is not None:
+            _check(code, "segkv_decode_step")
         dt, kv, qs = self.dtype, self._kv_shape, self._q_shape
         code = lib().segkv_decode_step(self._h, step, _dev(beam_parent, self._parent_shape, torch.int32, "beam_parent"),
                                        _dev(k_new, kv, dt, "k_new"), _dev(v_new, kv, dt, "v_new"),
@@ -360,13 +395,13 @@ class SegKV:
         _check(lib().segkv_reset(self._h, int(keep_prompt)), "segkv_reset")
 
     def truncate_last(self) -> None:
-        code = lib().segkv_truncate_last(self._h)
+        code = self._hot.truncate_last() if self._hot is not None else lib().segkv_truncate_last(self._h)
         if code:
             _check(code, "segkv_truncate_last")
 
     @property
     def steps(self) -> int:
-        return lib().segkv_steps(self._h)
+        return self._hot.steps() if self._hot is not None else lib().segkv_steps(self._h)
 
     @property
     def prompt_len(self) -> int:
