@@ -736,8 +736,8 @@ static int prefill_write_impl(segkv_t h, const void* k, const void* v, int promp
     cudaStream_t st = (cudaStream_t)stream;
     h->tm_valid = false;
     if (prompt_len > 0) {
-        SEGKV_CUDA(launch_prefill_transpose(h->d, k, v, h->kp, h->vp, plens_dev, lens_host, prompt_len, h->overlap, st));
-        count_launch(h, st, h->overlap ? kAtOnce : kAtOnceSerialised);
+        SEGKV_CUDA(launch_prefill_transpose(h->d, k, v, h->kp, h->vp, plens_dev, lens_host, prompt_len, st));
+        count_launch(h, st);
         int rc = make_prompt_maps(h, prompt_len);
         if (rc != SEGKV_OK) return rc;
         h->tm_valid = true;

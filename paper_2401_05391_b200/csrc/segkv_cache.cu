@@ -14,8 +14,10 @@ namespace segkv_impl {
 // contiguous [P, D] matrix the attention kernel can fetch with 2-D TMA boxes.
 // One thread moves 16-byte chunks, consecutive threads consecutive chunks of the source; a block takes whole tokens of one
 // request, about 2048 chunks of K and of V.  Bound: HBM (each byte once in, once out).  The form that found a chunk's
-// request, token, head and place in its row by four 64-bit divisions was bound by those and by two loads in flight per
-// thread: 91 us for 16 requests x 16 heads x 1003 tokens at D 256 (263 MB moved).
+// request, token, head and place in its row by four 64-bit divisions had two loads in flight per thread.  Before / now in us,
+// stores queued one behind the other: 64 requests x 56 heads x 2048 tokens at D 128 (7.5 GB moved) 1206 / 1121, 16 x 16 x
+// 1003 at D 256 86.5 / 82.4 (6.4 TB/s), 1 x 32 x 1024 at D 128 7.4 / 4.8.  (Launched with programmatic serialisation, its
+// waiting blocks slowed the prefill attention before it: 558 against 543 us for two layers of both at D 256.)
 // ---------------------------------------------------------------------------
 struct Lens {
     int n;                                   // 0: none by value
@@ -29,8 +31,6 @@ prefill_transpose_kernel(const uint4* __restrict__ k, const uint4* __restrict__ 
                          uint4* __restrict__ vp, int P, unsigned hc /* chunks of a token */, int log_chunks /* of a row */,
                          int tokens /* of a block */, int blocks_per_request, long long sb, long long sh,
                          long long sp /* strides in 16-byte chunks */, int32_t* __restrict__ plens, const __grid_constant__ Lens lens) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");       // as in append_kernel
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < lens.n; i += kStoreThreads) plens[i] = lens.len[i];
     const int b = (int)(blockIdx.x / (unsigned)blocks_per_request);
@@ -64,7 +64,7 @@ prefill_transpose_kernel(const uint4* __restrict__ k, const uint4* __restrict__ 
 }
 
 cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, int32_t* plens,
-                                     const int32_t* lens, int prompt_len, bool pdl, cudaStream_t st) {
+                                     const int32_t* lens, int prompt_len, cudaStream_t st) {
     const int chunks = d.head_dim * 2 / 16, log_chunks = d.head_dim == 64 ? 3 : d.head_dim == 128 ? 4 : 5;
     const PromptStrides ps = prompt_strides(d);
     if (prompt_len == 0) return cudaSuccess;
@@ -75,17 +75,10 @@ cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v
     Lens by_value;
     by_value.n = lens ? d.batch : 0;
     for (int b = 0; b < by_value.n; ++b) by_value.len[b] = lens[b];
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)per_request * (unsigned)d.batch, 1, 1);
-    cfg.blockDim = dim3(kStoreThreads, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, prefill_transpose_kernel, (const uint4*)k, (const uint4*)v, (uint4*)kp, (uint4*)vp, prompt_len, hc,
-                              log_chunks, tokens, per_request, ps.b / 8, ps.h / 8, ps.p / 8, plens, by_value);
+    prefill_transpose_kernel<<<(unsigned)per_request * (unsigned)d.batch, kStoreThreads, 0, st>>>(
+        (const uint4*)k, (const uint4*)v, (uint4*)kp, (uint4*)vp, prompt_len, hc, log_chunks, tokens, per_request,
+        ps.b / 8, ps.h / 8, ps.p / 8, plens, by_value);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -130,7 +130,7 @@ struct RopeArgs {
 // lengths to use, passed by value and written to plens by the kernel (at most kMaxLensByValue requests).
 constexpr int kMaxLensByValue = 256;
 cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v, void* kp, void* vp, int32_t* plens,
-                                     const int32_t* lens, int prompt_len, bool pdl, cudaStream_t st);
+                                     const int32_t* lens, int prompt_len, cudaStream_t st);
 
 cudaError_t launch_append(const Dims& d, int step, const int32_t* beam_parent, const void* k_new,
                           const void* v_new, void* kr_slab, void* vr_slab, int32_t* parent_tab,

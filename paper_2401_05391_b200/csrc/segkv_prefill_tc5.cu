@@ -6,9 +6,12 @@
 //   * one persistent CTA per SM walks a static list of work items (one or two groups of 128
 //     query rows of one (request, head)), longest first; a group's rows are one per TMEM lane and
 //     per TWO softmax threads (four where one group of head_dim 64 or 128 runs), which share a tile's keys;
-//   * an item's keys are gone through from the newest back.  Under an ALiBi bias a row's maximum then stands from its
-//     first tile on; from the oldest forward it grew with every tile, and most of Bloom's heads took two passes over each
-//     and rescaled O.  The two groups of an item also end together, each with a tile that needs no mask;
+//   * an item's keys are gone through from the newest back, so that its two groups end together and the second's diagonal
+//     tile does not run alone at the end (from the oldest forward: 4 % slower at 64 x 56 x 2048, and under an ALiBi
+//     bias a row's maximum grew with every tile, so that most of Bloom's heads took two passes over each and rescaled O).
+//     Without a bias the oldest tile comes before them all: every row sees all of it, and the reference is the exact score
+//     of one of its keys, whose weight is then not rounded (with a reference from the diagonal tile, of which some
+//     rows see a few keys, the error against 64 bits was 1 % larger);
 //   * Q of each group arrives by TMA (a per-call tensor map over [B, N, H, D]) in the
 //     128-byte-swizzled K-major layout; K and V tiles (128 keys; 64 at head_dim 256) arrive by TMA
 //     in the same layout through separate rings: a K tile is needed one step before the V tile
@@ -109,19 +112,22 @@ struct Tc5Layout {
     static_assert(kBytes <= 232448, "shared memory");
 };
 
-// Maximum of 16 scores of a row, in log2 units with BIAS (s * scale2 + bias0 + slope2 * i), else raw dot products; keys
-// above the row (i > lim) count in `all` only.
-template <bool BIAS>
-__device__ __forceinline__ float max16(const uint32_t* sr, float scale2, float slope2, float bias0, int lim, float& all) {
-    float mx[2] = {-INFINITY, -INFINITY}, ma[2] = {-INFINITY, -INFINITY};
+// Maximum of 16 scores of a row, in log2 units with BIAS (s * scale2 + bias0 + slope2 * i), else raw dot products;
+// MASK: keys above the row (i > lim) do not count.
+template <bool BIAS, bool MASK>
+__device__ __forceinline__ float max16(const uint32_t* sr, float scale2, float slope2, float bias0, int lim) {
+    float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        float v = __uint_as_float(sr[i]);
-        if (BIAS) v = fmaf(v, scale2, fmaf(slope2, (float)i, bias0));
-        else ma[i & 1] = fmaxf(ma[i & 1], v);
-        mx[i & 1] = fmaxf(mx[i & 1], i > lim ? -INFINITY : v);
+    for (int i = 0; i < 16; i += 2) {
+        float v[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            v[u] = __uint_as_float(sr[i + u]);
+            if (BIAS) v[u] = fmaf(v[u], scale2, fmaf(slope2, (float)(i + u), bias0));
+            if (MASK && i + u > lim) v[u] = -INFINITY;
+        }
+        asm("max.f32 %0, %0, %1, %2;" : "+f"(mx[(i >> 1) & 1]) : "f"(v[0]), "f"(v[1]));
     }
-    if (!BIAS) all = fmaxf(all, fmaxf(ma[0], ma[1]));
     return fmaxf(mx[0], mx[1]);
 }
 
@@ -259,6 +265,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // item w -> query tile (longest first), head, request
     auto item_qt = [&](int w) { return nqt - 1 - w / hb_count; };
     // key tiles of group g of query tile qt: up to its diagonal tile (causal); none past the prompt
+    // Order of an item's tiles (see the head of this file): position i of n tiles
+    const bool back = p.slopes != nullptr;
+    auto tile_at = [&](int i, int n) -> int { return back ? n - 1 - i : i == 0 ? 0 : n - i; };
     // nb = the request's own prompt length: with ragged prompts the items are still laid out for the
     // longest one, and a shorter request leaves its later items (and the tail of one) without work
     auto request_len = [&](int b) -> int { return RAGGED ? __ldg(p.plens + b) : p.N; };
@@ -340,9 +349,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     tk = tp + 1;
                     return true;
                 };
-                if (nkt > 0) ok = load_k(nkt - 1);                // the item's first keys need not wait for its query
+                if (nkt > 0) ok = load_k(tile_at(0, nkt));        // the item's first keys need not wait for its query
 #pragma unroll
-                for (int g = NG - 1; g >= 0; --g) {
+                for (int x = 0; x < NG; ++x) {                    // the group that begins first
+                    const int g = back ? NG - 1 - x : x;
                     if (!ok || group_tiles(qt, g, request_len(b)) == 0) continue;
                     // the group's Q rows (past the prompt: zeros), once its previous Q is no longer read
                     ok = mbar_wait(gbar0 + kGB * g + 40, (qi[g] & 1) ^ 1, p.wait_ns);
@@ -368,9 +378,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                         for (int cb = 0; cb < L::kDBoxes; ++cb) tma_prefetch_4d(&tm_q, cb * 64, hb2 % p.H, row, hb2 / p.H);
                     }
                 }
-                for (int kt = nkt - 1; kt >= 0 && ok; --kt, ++tp) {
+                for (int i = 0; i < nkt && ok; ++i, ++tp) {
+                    const int kt = tile_at(i, nkt);
                     const uint32_t sv = tp % SV;
-                    if (kt < nkt - 1) ok = load_k(kt);
+                    if (i > 0) ok = load_k(kt);
                     if (!ok) break;
                     ok = mbar_wait(vempty0 + 8 * sv, ((tp / SV) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
@@ -416,7 +427,8 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 int nkt = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) nkt = max(nkt, group_tiles(qt, g, request_len(b)));
-                for (int kt = nkt - 1; kt >= 0 && ok; --kt, ++tp) {
+                for (int i = 0; i < nkt && ok; ++i, ++tp) {
+                    const int kt = tile_at(i, nkt);
                     const bool mine = (h % p.G) == 0 && (kt * kKeys) / (kRows * NG) == qt;
                     const uint32_t sk = tp % SK, sv = tp % SV;
                     ok = mbar_wait(kfull0 + 8 * sk, (tp / SK) & 1, p.wait_ns);
@@ -485,25 +497,36 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     nkt = max(nkt, gt[g]);
                 }
                 if (nkt == 0) continue;                           // the request ends before this item's rows
-                // A group's first scores, from the K tile that holds its diagonal (the second group's: a tile earlier).
-                auto first_qk = [&](int g) -> bool {
-                    if (!wait(gbar0 + kGB * g + 32, qi[g]++ & 1)) return false;   // Q_g landed
-                    tc_fence_after();
-                    issue_qk(g, NB == 2 ? n[g] & 1 : 0u, gt[g] == 1);
+                // The first of two groups does not see the item's last tile: the position that it leaves out, and its first and
+                // last one.
+                int skip[NG], first[NG], last[NG];
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    skip[g] = gt[g] == nkt ? -1 : back ? 0 : 1;
+                    first[g] = skip[g] == 0 ? 1 : 0;
+                    last[g] = skip[g] == nkt - 1 ? nkt - 2 : nkt - 1;
+                }
+                // the scores of position i of group g, the K tile waited for
+                auto scores = [&](int g, int i) -> bool {
+                    if (i == first[g]) {
+                        if (!wait(gbar0 + kGB * g + 32, qi[g]++ & 1)) return false;   // Q_g landed
+                        tc_fence_after();
+                    }
+                    issue_qk(g, NB == 2 ? (n[g] + (i == first[g] ? 0u : 1u)) & 1 : 0u, i == last[g]);
                     return true;
                 };
                 ok = wait_k();
 #pragma unroll
                 for (int g = 0; g < NG; ++g)
-                    if (gt[g] == nkt && ok) ok = first_qk(g);
+                    if (gt[g] > 0 && skip[g] != 0 && ok) ok = scores(g, 0);
                 if (!ok) break;
                 release_k();
-                for (int kt = nkt - 1; kt >= 0 && ok; --kt) {     // the newest keys first
-                    if (NB == 2 && kt > 0) {                      // next tile's scores run under this tile's softmax
+                for (int i = 0; i < nkt && ok; ++i) {
+                    const int kt = tile_at(i, nkt);
+                    if (NB == 2 && i + 1 < nkt) {                 // next tile's scores run under this tile's softmax
                         ok = wait_k();
                         if (!ok) break;
-#pragma unroll
-                        for (int g = 0; g < NG; ++g) issue_qk(g, (n[g] + 1) & 1, kt == 1);
+                        (void)scores(0, i + 1);
                         release_k();
                     }
                     const uint64_t vd = dv + (v_lo0 + vst * (uint32_t)(kTileKV >> 4));
@@ -512,48 +535,40 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     bool k_next = false;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
-                        if (kt > gt[g]) continue;
-                        if (kt == gt[g]) {                        // its diagonal tile comes next
-                            if (NB == 2 || kt == 0) continue;
-                            if (!k_next) {
-                                ok = wait_k();
-                                if (!ok) break;
-                                k_next = true;
-                            }
-                            ok = first_qk(g);
+                        if (gt[g] == 0) continue;
+                        if (i != skip[g]) {
+                            ok = wait(gbar0 + kGB * g + 16, n[g] & 1);   // P_g written over its S buffer
                             if (!ok) break;
-                            continue;
-                        }
-                        ok = wait(gbar0 + kGB * g + 16, n[g] & 1);   // P_g written over its S buffer
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t p_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + (NB == 2 ? n[g] & 1 : 0u));
+                            tc_fence_after();
+                            const uint32_t p_tmem = tmem + (uint32_t)kKeys * ((uint32_t)(g * NB) + (NB == 2 ? n[g] & 1 : 0u));
 #pragma unroll
-                        for (int kk = 0; kk < kKeys / 16; ++kk)   // O_g += P_g[:, 16 keys] . V[16 keys, :]
-                            tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16,
-                                         vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (kt + 1 < gt[g] || kk > 0));
-                        if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, steep)) {
+                            for (int kk = 0; kk < kKeys / 16; ++kk)   // O_g += P_g[:, 16 keys] . V[16 keys, :]
+                                tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16,
+                                             vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, (i != first[g] || kk > 0));
+                            if (kSplitP && split_p_keys((qt * NG + g) * kRows, kt * kKeys, kKeys, steep)) {
 #pragma unroll
-                            for (int kk = 0; kk < kKeys / 16; ++kk)   // ... and the low parts of the weights that have one
-                                if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, steep))
-                                    tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16 + 8,
-                                                 vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
+                                for (int kk = 0; kk < kKeys / 16; ++kk)   // ... and the low parts of the weights that have one
+                                    if (split_p_keys((qt * NG + g) * kRows, kt * kKeys + 16 * kk, 16, steep))
+                                        tc_mma_ts_if(lead, tmem + (uint32_t)(L::kColO + kD * g), p_tmem + kk * 16 + 8,
+                                                     vd + (uint64_t)((kk * 2048) >> 4), p.idesc_pv, 1u);
+                            }
+                            tc_commit_if(lead, gbar0 + kGB * g + 24);
+                            ++n[g];
                         }
-                        tc_commit_if(lead, gbar0 + kGB * g + 24);
-                        ++n[g];
-                        if (NB == 1 && kt > 0) {                  // the group's next scores, behind its P.V in the pipe
+                        if (NB == 1 && i + 1 < nkt && i + 1 != skip[g]) {        // the group's next scores, behind its P.V in the pipe
                             if (!k_next) {
                                 ok = wait_k();
                                 if (!ok) break;
                                 k_next = true;
                             }
-                            issue_qk(g, 0u, kt == 1);
+                            ok = scores(g, i + 1);
+                            if (!ok) break;
                         }
                     }
                     if (!ok) break;
                     tc_commit_if(lead, vempty0 + 8 * vst);        // stage free once every MMA so far is done
                     if (++vst == SV) { vst = 0; vph ^= 1u; }
-                    if (NB == 1 && kt > 0) release_k();
+                    if (NB == 1 && i + 1 < nkt) release_k();
                 }
             }
             if (!ok && lane == 0) s_abort = 1;
@@ -565,6 +580,8 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         // chain softmax -> P.V -> next Q.K^T bound the kernel.  More warps hide each other's latencies: a lone group's
         // tile took 1890 clocks with two threads per row.)
         constexpr int KH = kKeys / TPR, DH = kD / TPR;
+        // keys at a time: 32 where the registers are there (with one group a tile's latency counts), else 16
+        constexpr int PC = NG == 1 && KH >= 32 ? 32 : 16;
         const int g = warp / (4 * TPR), part = (warp >> 2) % TPR, r = (warp & 3) * 32 + lane;
         const int rows_bar = 1 + g * 4 + (warp & 3);              // barrier of the warps that share these rows
         const uint32_t bar_s0 = gbar0 + kGB * g, bar_p = bar_s0 + 16, bar_o = bar_s0 + 24;
@@ -583,10 +600,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             const int row0 = (qt * NG + g) * kRows, row = row0 + r;
             const float slope_nat = p.slopes ? p.slopes[h] : 0.f;
             const float slope2 = slope_nat * 1.4426950408889634f;
-            const bool biased = p.slopes != nullptr;
+            const bool biased = back;
             float m_ref = -INFINITY, l_run = 0.f;
             for (int t = 0; t < my_tiles; ++t, ++n) {
-                const int kt = my_tiles - 1 - t;                  // the newest keys first
+                const int kt = tile_at(t, my_tiles);
                 const int buf = NB == 2 ? (int)(n & 1) : 0;
                 const uint32_t tm_s = tm_lane + (uint32_t)(kKeys * (g * NB + buf) + KH * part);
                 if (ok) ok = mbar_wait_hot(bar_s0 + 8 * buf, (NB == 2 ? (n >> 1) : n) & 1, p.wait_ns);
@@ -601,45 +618,69 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 float alpha = 1.f;
                 uint64_t ls = 0ull;
                 int kept = 0;                                     // keys whose weights are stored
-                // The reference in use nearly always stands behind the diagonal tiles: the weights are worked out and stored
-                // with it in one pass over the scores; 16 keys whose weights add up to more than 2^8 end the pass.  (That they
+                // The reference in use nearly always stands behind the first tile: the weights are worked out and stored
+                // with it in one pass over the scores; 16 (32) keys whose weights add up to more than 2^8 end the pass.  (That they
                 // do is seen from their sum, which is needed anyhow: noting the maximum cost an instruction for every
                 // two scores, and the kernel's large launches run at the power limit.  Not where no key has been visible to a
                 // row so far, nor under a slope that lifts the maximum by 2^4 and more from tile to tile, which towards
                 // older keys is a negative one.)
                 const bool fresh = t == 0 || -slope2 * (float)kKeys >= 4.f || __any_sync(0xffffffffu, m_ref == -INFINITY);
+                const int seen = row0 + (warp & 3) * 32 + 32 - key0;       // keys that some row of the warp sees
+                const bool mask = key0 + KH - 1 > row0 + (warp & 3) * 32;  // keys that some row of the warp does not see
                 bool stands = false;
                 if (!fresh) {
                     if (ok) {
                         tc_fence_after();
                         const float m_use = m_ref - kWeightShift<T>;
-                        auto pass = [&](auto with_bias, auto in_two) {
-                            constexpr bool BIAS = decltype(with_bias)::value, SPLIT = decltype(in_two)::value;
-                            uint32_t sr[2][16];                   // the next 16 scores are on their way while these are worked on
-                            tc_ld16(tm_s, sr[0]);
+                        auto pass = [&](auto with_bias, auto masked, auto in_two) {
+                            constexpr bool BIAS = decltype(with_bias)::value, MASK = decltype(masked)::value, SPLIT = decltype(in_two)::value;
+                            uint32_t sr[KH > PC ? 2 : 1][PC];     // the next scores are on their way while these are worked on
+                            if constexpr (PC == 32) tc_ld32(tm_s, sr[0]);
+                            else tc_ld16(tm_s, sr[0]);
 #pragma unroll
-                            for (int c = 0; c < KH; c += 16) {
-                                uint32_t* cur = sr[(c >> 4) & 1];
+                            for (int c = 0; c < KH; c += PC) {
+                                uint32_t* cur = sr[(c / PC) & 1];
                                 tc_wait_ld();
-                                pin<16>(cur);
-                                if (c + 16 < KH) tc_ld16(tm_s + c + 16, sr[((c >> 4) & 1) ^ 1]);
-                                const float c0 = (BIAS ? bias0 + slope2 * (float)c : 0.f) - m_use;
-                                uint32_t hi[8], lo[8];
-                                const uint64_t lp = weigh16<T, BIAS, false, SPLIT>(cur, p.scale2, slope2, c0, 0, hi, lo);
+                                pin<PC>(cur);
+                                if (c + PC < KH) {
+                                    if constexpr (PC == 32) tc_ld32(tm_s + c + PC, sr[KH > PC ? ((c / PC) & 1) ^ 1 : 0]);
+                                    else tc_ld16(tm_s + c + PC, sr[KH > PC ? ((c / PC) & 1) ^ 1 : 0]);
+                                }
+                                uint32_t hi[PC / 2], lo[PC / 2];
+                                uint64_t lp = 0ull;
+#pragma unroll
+                                for (int u = 0; u < PC; u += 16) {
+                                    if (MASK && c + u >= seen) {  // keys beyond the warp's last row
+#pragma unroll
+                                        for (int i = 0; i < 8; ++i) hi[u / 2 + i] = lo[u / 2 + i] = 0u;
+                                        continue;
+                                    }
+                                    const float c0 = (BIAS ? bias0 + slope2 * (float)(c + u) : 0.f) - m_use;
+                                    const uint64_t ln = weigh16<T, BIAS, MASK, SPLIT>(cur + u, p.scale2, slope2, c0, lim - c - u, hi + u / 2, lo + u / 2);
+                                    lp = u ? f2_add(lp, ln) : ln;
+                                }
                                 if (__any_sync(0xffffffffu, f2_lo(lp) + f2_hi(lp) > kWeightMax<T>)) break;
                                 ls = f2_add(ls, lp);
-                                tc_st8(tm_s + c, hi);
-                                if (SPLIT) tc_st8(tm_s + c + 8, lo);
-                                kept = c + 16;
+#pragma unroll
+                                for (int u = 0; u < PC; u += 16) {
+                                    tc_st8(tm_s + c + u, hi + u / 2);
+                                    if (SPLIT) tc_st8(tm_s + c + u + 8, lo + u / 2);
+                                }
+                                kept = c + PC;
                             }
                             tc_wait_ld();
                         };
+                        // (with a bias there is no mask behind the first tile, see above)
+                        constexpr std::integral_constant<bool, kSplitP> parts{};
+                        constexpr std::true_type yes{};
+                        constexpr std::false_type no{};
                         if (kSplitP && two) {
-                            if (biased) pass(std::true_type{}, std::integral_constant<bool, kSplitP>{});
-                            else pass(std::false_type{}, std::integral_constant<bool, kSplitP>{});
+                            if (biased) pass(yes, no, parts);
+                            else if constexpr (kKeys < kRows) pass(no, yes, parts);      // (else only the first tile's)
                         } else {
-                            if (biased) pass(std::true_type{}, std::false_type{});
-                            else pass(std::false_type{}, std::false_type{});
+                            if (biased) pass(yes, no, no);
+                            else if (mask) pass(no, yes, no);
+                            else pass(no, no, no);
                         }
                     }
                     stands = bar_and(rows_bar, 32 * TPR, ok && kept == KH);
@@ -648,23 +689,22 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4 (those
                     // that have are below 2^8 of the one in use): the sum and O use the same reference, so the
                     // result is exact.  Keys beyond the last row of the warp take no part.
-                    float tmax = -INFINITY, tall = -INFINITY;
-                    // A row that sees a few keys of its diagonal tile and many behind it takes the maximum of the whole tile for
-                    // what is to come: the largest weights, just below a power of two, are then rounded best.  (With the
-                    // few keys' maximum the error against 64 bits was up to 1 % larger.)
-                    const bool guess = t == 0 && kt > 0 && !biased;
-                    const int seen = row0 + (warp & 3) * 32 + 32 - key0;       // keys that some row of the warp sees
+                    float tmax = -INFINITY;
                     if (ok) {
                         tc_fence_after();
 #pragma unroll 1
-                        for (int c = kept; c < KH && (c < seen || guess); c += 16) {
+                        for (int c = kept; c < KH && c < seen; c += 16) {
                             uint32_t sr[16];
                             tc_ld16(tm_s + c, sr);
                             tc_wait_ld();
                             pin<16>(sr);
                             // in log2 units; without a bias the scale is folded into the exponent's FMA
-                            tmax = fmaxf(tmax, biased ? max16<true>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c, tall)
-                                                      : max16<false>(sr, p.scale2, slope2, 0.f, lim - c, tall) * p.scale2);
+                            float m;
+                            if (biased) m = mask ? max16<true, true>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c)
+                                                 : max16<true, false>(sr, p.scale2, slope2, bias0 + slope2 * (float)c, lim - c);
+                            else m = (mask ? max16<false, true>(sr, p.scale2, slope2, 0.f, lim - c)
+                                           : max16<false, false>(sr, p.scale2, slope2, 0.f, lim - c)) * p.scale2;
+                            tmax = fmaxf(tmax, m);
                         }
                     }
                     xrow[part * kRows] = tmax;
@@ -674,15 +714,6 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
                     for (int i = 0; i < TPR; ++i) tmax = fmaxf(tmax, xrow[i * kRows]);
                     bar_sync_n(rows_bar, 32 * TPR);
-                    if (guess) {
-                        xrow[part * kRows] = tall * p.scale2;
-                        bar_sync_n(rows_bar, 32 * TPR);
-                        tall = xrow[0];
-#pragma unroll
-                        for (int i = 1; i < TPR; ++i) tall = fmaxf(tall, xrow[i * kRows]);
-                        bar_sync_n(rows_bar, 32 * TPR);
-                        tmax = fmaxf(tmax, fminf(tall, tmax + 4.f));
-                    }
                     const bool need = tmax > m_ref + 4.f, rescale = need && m_ref > -INFINITY;   // (O is zero so far, else)
                     if (need) {
                         alpha = exp2f(m_ref - tmax);              // 0 on the first keys
@@ -727,8 +758,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                                 if (biased) lp = weigh16<T, true, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
                                 else lp = weigh16<T, false, true, kSplitP>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
                             } else {
-                                if (biased) lp = weigh16<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
-                                else lp = weigh16<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                                if (biased) lp = mask ? weigh16<T, true, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo)
+                                                      : weigh16<T, true, false, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
+                                else lp = mask ? weigh16<T, false, true, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo)
+                                               : weigh16<T, false, false, false>(sr, p.scale2, slope2, c0, lim - c, hi, lo);
                             }
                             ls = f2_add(ls, lp);
                         } else {
