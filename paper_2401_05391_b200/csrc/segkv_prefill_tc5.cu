@@ -342,14 +342,6 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 int nkt = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) nkt = max(nkt, group_tiles(qt, g, request_len(b)));
-                auto load_k = [&](int kt) -> bool {
-                    const uint32_t sk = tp % SK;
-                    if (!mbar_wait(kempty0 + 8 * sk, ((tp / SK) & 1) ^ 1, p.wait_ns)) return false;
-                    load_tile(&tm_k, k_ring + (size_t)sk * kTileKV, kt, kvh, b, kfull0 + 8 * sk);
-                    tk = tp + 1;
-                    return true;
-                };
-                if (nkt > 0) ok = load_k(tile_at(0, nkt));        // the item's first keys need not wait for its query
 #pragma unroll
                 for (int x = 0; x < NG; ++x) {                    // the group that begins first
                     const int g = back ? NG - 1 - x : x;
@@ -365,24 +357,13 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     for (int cb = 0; cb < L::kDBoxes; ++cb)
                         tma_load_4d(dst + cb * kBoxQ, &tm_q, cb * 64, h, (qt * NG + g) * kRows, b, qfull);
                 }
-                // the next item's query into the L2 meanwhile: it is asked for when the group's last scores are done, and
-                // its first ones wait for it
-                const int w2 = j + 1 < p.rounds ? round_item(j + 1) : n_items;
-                if (ok && w2 < n_items) {
-                    const int hb2 = w2 % hb_count;
-#pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        const int row = (item_qt(w2) * NG + g) * kRows;
-                        if (row >= p.N) continue;
-#pragma unroll
-                        for (int cb = 0; cb < L::kDBoxes; ++cb) tma_prefetch_4d(&tm_q, cb * 64, hb2 % p.H, row, hb2 / p.H);
-                    }
-                }
                 for (int i = 0; i < nkt && ok; ++i, ++tp) {
                     const int kt = tile_at(i, nkt);
-                    const uint32_t sv = tp % SV;
-                    if (i > 0) ok = load_k(kt);
+                    const uint32_t sk = tp % SK, sv = tp % SV;
+                    ok = mbar_wait(kempty0 + 8 * sk, ((tp / SK) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
+                    load_tile(&tm_k, k_ring + (size_t)sk * kTileKV, kt, kvh, b, kfull0 + 8 * sk);
+                    tk = tp + 1;
                     ok = mbar_wait(vempty0 + 8 * sv, ((tp / SV) & 1) ^ 1, p.wait_ns);
                     if (!ok) break;
                     load_tile(&tm_v, v_ring + (size_t)sv * kTileKV, kt, kvh, b, vfull0 + 8 * sv);
