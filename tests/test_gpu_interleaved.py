@@ -83,3 +83,28 @@ def test_fused_steps_over_three_layers(dtype, D, B, W, steps, tile, splits, comb
     finally:
         for r in ls + [ref]:
             r.close()
+
+
+@pytest.mark.parametrize("B,heads,kv_heads,P", [(2, 8, 4, 200), (5, 64, 64, 300), (2, 32, 4, 512)])
+def test_appends_in_a_row_and_attention_behind_them(B, heads, kv_heads, P):
+    # Appends let their successors go at once, so behind several of them only what was complete before the first may be read
+    # ahead: the small form, more work groups than SMs and the wide kernel, against the same calls with a wait after each.
+    w = wl.Workload("chain", B, 4, heads, kv_heads, 128, P, 24, "f16", "uniform", False, 310)
+    ls, refs = layers_of(w, 3), layers_of(w, 3)
+    try:
+        for t in range(w.steps):
+            for r in ls:
+                r.append_next()
+            outs = [r.decode()[0] for r in (ls if t % 2 else ls[::-1])]
+            for r in refs:
+                r.append_next()
+                torch.cuda.synchronize()
+            for r, out in zip(refs if t % 2 else refs[::-1], outs):
+                ref = r.decode()[0]
+                torch.cuda.synchronize()
+                assert torch.equal(out.view(torch.int16), ref.view(torch.int16)), f"step {t}"
+        for r in ls + refs:
+            assert r.h.get_error() == 0
+    finally:
+        for r in ls + refs:
+            r.close()

@@ -275,3 +275,60 @@ def test_prefill_scores_that_grow_from_tile_to_tile(dtype, D, row_groups):
         assert (err <= ATOL + RTOL * np.abs(ref) + float(vp.abs().max()) * 2.0 ** (-9 if dtype == "bf16" else -12)).all(), err.max()
     finally:
         h.destroy()
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,row_groups", [(64, 1), (64, 2), (128, 1), (128, 2), (256, 1)])
+def test_prefill_references_that_fall_in_the_middle_of_a_tile(dtype, D, row_groups):
+    # Single keys eight times as long at places that end a tile's one pass behind its first, second and last pieces of 16
+    # keys (what is stored by then is scaled), at prompts that end in every part of a pair of row groups; and, in the
+    # second half of the heads, slopes that favour OLDER keys, so that going back through the keys the maximum grows.  The
+    # rounding of the weights is allowed for as above.
+    for P in (129, 257, 390, 515):
+        w = wl.Workload("spike", 1, 2, 4, 2, D, P, 2, dtype, "uniform", True, 150 + P)
+        h = sk.SegKV(w.batch, w.beams, w.heads, w.kv_heads, w.head_dim, w.prompt_len, w.steps, w.torch_dtype)
+        try:
+            h.set_prefill_tuning(row_groups)
+            kp, vp = wl.make_prompt(w, "cuda")
+            for at in (20, 135, 128 + 40, 256 + 17, 256 + 63, 384 + 1, 512):
+                kp[:, at:at + 1] *= 8.0
+            q = wl.make_prefill_query(w, "cuda")
+            for slopes in (None, torch.tensor([0.25, 0.01, -0.02, -0.25], device="cuda")):
+                out, fused = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+                h.prefill_write(kp, vp)
+                h.prefill_sdpa(q, out, slopes)
+                h.prefill(kp, vp, q, fused, slopes)
+                torch.cuda.synchronize()
+                assert h.get_error() == 0
+                assert torch.equal(out, fused)
+                rows = all_rows(w)[::3]
+                ref = oracle.prefill_sdpa(w.dtype, w.batch, w.heads, w.kv_heads, w.head_dim, wl.to_bits(q), wl.to_bits(kp),
+                                          wl.to_bits(vp), slopes=None if slopes is None else slopes.cpu().numpy(), rows=rows)
+                got = np.stack([out[b, i, x].to(torch.float64).cpu().numpy() for b, i, x in rows])
+                err = np.abs(got - ref)
+                assert (err <= ATOL + RTOL * np.abs(ref) + float(vp.abs().max()) * 2.0 ** (-9 if dtype == "bf16" else -12)).all(), err.max()
+        finally:
+            h.destroy()
+
+
+@pytest.mark.parametrize("D,kv_heads,P", [(64, 1, 1), (64, 3, 700), (128, 5, 77), (256, 7, 130), (256, 80, 3)])
+def test_prompt_store_of_odd_shapes(D, kv_heads, P):
+    # blocks of whole tokens: one head, odd heads, tokens that do not divide a block's, a token larger than a block; the fused
+    # prefill, whose tiles go through the tensor maps, leaves the same segment
+    w = wl.Workload("store", 3, 2, kv_heads, kv_heads, D, P, 2, "f16", "uniform", False, 160)
+    outs = []
+    for fused in (False, True):
+        h = sk.SegKV(w.batch, w.beams, w.heads, w.kv_heads, w.head_dim, w.prompt_len, w.steps, w.torch_dtype)
+        kp, vp = wl.make_prompt(w, "cuda")
+        qp = wl.make_prefill_query(w, "cuda")
+        q, k, v = wl.make_step(w, 0, "cuda")
+        if fused:
+            h.prefill(kp, vp, qp)
+        else:
+            h.prefill_write(kp, vp)
+        h.append(0, None, k, v)
+        outs.append(h.decode_sdpa(q))
+        torch.cuda.synchronize()
+        assert h.get_error() == 0
+        h.destroy()
+    assert torch.equal(outs[0], outs[1])
