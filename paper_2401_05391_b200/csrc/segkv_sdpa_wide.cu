@@ -685,6 +685,15 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             const float2* ml0 = reinterpret_cast<const float2*>(p.ws_ml + (size_t)it0 * p.ncols * 2);
             const float* o0 = p.ws_o + (size_t)it0 * p.ncols * D;
             const int parts = p.S;
+            // A CTA without further items has its prompt ring free (all tiles in it have been used): if they fit, all partials are
+            // on their way there at once while the factors are worked out.  (Merging four splits of 32 columns at D 128, 64 KB,
+            // by 16 loads per thread at a time took 4.6 us, by 8 6.4: the loads' latency.)
+            constexpr int D4 = D / 4, NE = 4;
+            const int n4 = p.ncols * D4;
+            const bool landed = it >= p.items && (size_t)parts * n4 * 16 <= (size_t)SP * L::kStage;
+            const float4* land = reinterpret_cast<const float4*>(p_ring);
+            if (landed)
+                for (int i = tid; i < parts * n4; i += 128) cp_async_16(p_ring_u + 16 * i, reinterpret_cast<const float4*>(o0) + i);
             // Two passes: each part's factor per column, then 16 loads in flight per thread.  (One float4 of one column at
             // a time, its parts' loads ordered by the use of each, cost most of the about 7 us that merging four splits took.)
             float* fac = reinterpret_cast<float*>(p_smem);        // [part][32 columns]: 2^(m_part - m) / sum
@@ -714,15 +723,23 @@ sdpa_wide_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                     fac[u * kCols + lane] = m == -INFINITY ? 0.f : exp2f(m - mm) * inv;
                 }
             }
+            if (landed) cp_async_wait_all();
             bar_sync_n(1, 128);
-            constexpr int D4 = D / 4, NE = 4;
-            const int n4 = p.ncols * D4;
             for (int e0 = tid; e0 < n4; e0 += 128 * NE) {
                 float4 o[NE];
 #pragma unroll
                 for (int i = 0; i < NE; ++i) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-                for (int s0 = 0; s0 < parts; s0 += 4) {
+                for (int s0 = 0; s0 < parts && landed; ++s0)
+#pragma unroll
+                    for (int i = 0; i < NE; ++i) {
+                        const int e = min(e0 + 128 * i, n4 - 1);
+                        const float4 w = land[s0 * n4 + e];
+                        const float f = fac[s0 * kCols + e / D4];
+                        o[i].x += w.x * f; o[i].y += w.y * f; o[i].z += w.z * f; o[i].w += w.w * f;
+                    }
+#pragma unroll 1
+                for (int s0 = 0; s0 < parts && !landed; s0 += 4) {
                     float4 w[NE][4];
 #pragma unroll
                     for (int i = 0; i < NE; ++i)
