@@ -20,7 +20,7 @@
 //   * one warp, converged, issues one lane's MMAs: S = Q.K^T (M 128, N = keys of a tile, K-steps of 16)
 //     into a TMEM buffer and O += P.V (M 128, N = head_dim) into a TMEM accumulator.  P never
 //     touches shared memory: the softmax threads write it, rounded to the 16-bit type, over
-//     the scores it came from (32 keys' weights over the first half of their columns), and the MMA
+//     the scores it came from (16 keys' weights over the first half of their columns), and the MMA
 //     takes its A operand from tensor memory.  V is consumed as an MN-major B operand straight from
 //     its row-major tile;
 //   * the softmax threads read S with tcgen05.ld (no shuffles for the row max / sum) and
@@ -35,12 +35,13 @@
 //
 // What bounds it: with thousands of items the power limit (1000 W at 1.5 to 1.65 GHz, where a lone call runs at 1.9), so that a
 // shorter chain buys less than fewer instructions and bytes do; with a few, a group's chain softmax -> P.V -> Q.K^T and
-// the start.  Measured in turn with the form that went from the oldest keys forward, held P back until the row's two
-// threads had met, spilled and was launched behind the whole kernel before (before / now, attention alone): 64 requests x
-// 56 heads x 2048 tokens at D 128 fp16 4620 / 4567 us, bf16 5040 / 4648; 32 x 112 x 1024 bf16 with ALiBi 1704 / 1466, fp16
-// 1825 / 1335; 1 x 32 x 1024 fp16 22.7 / 20.7; D 64, 16 x 64 x 2048, bf16 with ALiBi 1515 / 1053; D 256, 2 x 8 x 2000, bf16 with
-// ALiBi 61.6 / 42.2.  Putting a share of the exponentials on the FMA pipes as a polynomial was measured slower
-// (4.42 against 4.17 ms): the issue slots it costs are on the same chain.
+// the start.  Measured in turn with the form that went from the oldest keys forward throughout, held P back until the row's two
+// threads had met, spilled and was launched behind the whole kernel before (before / now in us, attention alone): with ALiBi
+// 32 x 112 heads x 1024 at D 128 bf16 1922 / 1607 (fp16 1825 / 1335), D 64, 16 x 64 x 2048, bf16 1515 / 1053, D 256, 2 x 8 x 2000, bf16
+// 61.6 / 42.1; without 64 x 56 x 2048 at D 128 fp16 4810 / 4789, bf16 5118 / 4787, 1 x 32 x 1024 20.6 / 18.9, 4 x 40 x 700 49.3 / 44.6,
+// D 64, 16 x 64 x 2048, 992 / 978, D 256, 16 x 16 x 1003, 182 / 185 (with the store fused 228 / 225).  Putting a share of the
+// exponentials on the FMA pipes as a polynomial was measured slower (4.42 against 4.17 ms): the issue slots it costs are on
+// the same chain.
 //
 // Tensor memory (all 512 columns are allocated): S buffers first, then one O accumulator per
 // group.  Every mbarrier is waited on phase by phase (a parity wait cannot tell phases two
