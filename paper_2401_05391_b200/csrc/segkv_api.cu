@@ -3,7 +3,6 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <mutex>
 #include <new>
 
 #include "segkv_internal.h"
@@ -25,53 +24,12 @@ int cuda_fail(cudaError_t e, const char* what) {
         if (e__ != cudaSuccess) return cuda_fail(e__, #call); \
     } while (0)
 
-// ---------------------------------------------------------------------------
-// Which of the library's launches came last on each stream.  A kernel launched with programmatic
-// stream serialisation may begin before its predecessor P in the stream has finished, but not
-// before P has passed its own grid-dependency wait, i.e. not before everything older than P is
-// complete.  So data whose producing launch is strictly older than P may be read by the new kernel from its
-// very first instruction.  The append kernels let their successors go before that wait: behind one of them
-// only what was complete when IT began counts (launched without programmatic serialisation: everything
-// older; else what was complete for its own predecessor's successor).  (A launch of the caller's own in between
-// only helps: it does not release its dependents early.)
-// ---------------------------------------------------------------------------
-struct StreamLog {
-    cudaStream_t st;
-    unsigned long long last;      // sequence number of the library's latest launch on st
-    unsigned long long complete;  // launches older than this are complete when the next kernel on st begins
-    bool used;
-};
-enum Release { kAfterWait, kAtOnce, kAtOnceSerialised };      // when a launch lets its successor begin
-std::mutex g_log_mu;
-StreamLog g_log[32];
-unsigned long long g_launch_seq = 0;
+StreamLog g_log;
 
-// Record a launch on `st`; returns its sequence number.
-unsigned long long note_launch(cudaStream_t st, Release rel) {
-    std::lock_guard<std::mutex> lk(g_log_mu);
-    const unsigned long long seq = ++g_launch_seq;
-    int slot = -1, oldest = 0;
-    for (int i = 0; i < 32; ++i) {
-        if (g_log[i].used && g_log[i].st == st) { slot = i; break; }
-        if (!g_log[i].used) { if (slot < 0) slot = i; }
-        else if (g_log[i].last < g_log[oldest].last || !g_log[oldest].used) oldest = i;
-    }
-    if (slot < 0) slot = oldest;          // more than 32 streams: forget the one idle longest
-    if (rel != kAtOnce) g_log[slot].complete = seq;
-    else if (!g_log[slot].used || g_log[slot].st != st) g_log[slot].complete = 0;       // (nothing is known of its predecessor)
-    g_log[slot].st = st;
-    g_log[slot].last = seq;
-    g_log[slot].used = true;
-    return seq;
-}
-
-// Is a launch `seq` on stream `st` complete when the next kernel there begins?
-bool complete_for_next(cudaStream_t st, cudaStream_t seq_stream, unsigned long long seq) {
-    if (seq == 0 || seq_stream != st) return false;
-    std::lock_guard<std::mutex> lk(g_log_mu);
-    for (int i = 0; i < 32; ++i)
-        if (g_log[i].used && g_log[i].st == st) return seq < g_log[i].complete;
-    return false;
+// The stream of a launch for handle h.
+StreamKey stream_key(const segkv* h, cudaStream_t st) {
+    static thread_local char own;
+    return {h->device, st, st == cudaStreamPerThread ? &own : nullptr};
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -174,19 +132,19 @@ int make_kv_source_map(const segkv* h, const void* base, int prompt_len, CUtenso
 // Every kernel the library launches is counted on its handle and logged on its stream.
 unsigned long long count_launch(segkv* h, cudaStream_t st, Release rel = kAfterWait) {
     h->launches++;
-    return note_launch(st, rel);
+    return g_log.note(stream_key(h, st), rel);
 }
 
 // The launch just made on `st` wrote the data `m` stands for.
 void mark_written(segkv* h, WriteMark* m, cudaStream_t st, Release rel = kAfterWait) {
     m->seq = count_launch(h, st, rel);
-    m->stream = st;
+    m->at = stream_key(h, st);
 }
 
 // Is the data `m` stands for complete and visible to a kernel launched now on `st`, from that
 // kernel's first instruction on?  The answer depends on the order of the caller's calls alone, never on
 // how far the GPU has got, so the same program takes the same path every time it runs.
-bool settled(const WriteMark* m, cudaStream_t st) { return complete_for_next(st, m->stream, m->seq); }
+bool settled(const segkv* h, const WriteMark* m, cudaStream_t st) { return g_log.complete_for_next(stream_key(h, st), *m); }
 
 void free_all(segkv* h) {
     void* ptrs[] = {h->kp, h->vp, h->kr, h->k_chunks_dev, h->parent, h->anc[0], h->anc[1], h->ulist, h->ucount, h->plens,
@@ -513,12 +471,13 @@ int ensure_lists(segkv* h, cudaStream_t st) {
 
 // May the next attention launch on `st` read the handle's response rows (and, for the separate
 // form, the distinct-row lists) before its grid-dependency wait?  Only if the launches that wrote
-// them are strictly older than the library's latest launch on the same stream.
+// them are complete when a kernel begins behind the library's latest launch on the same stream (StreamLog; to be older
+// than that launch is not enough: behind two appends the first one's rows are, and may still be on their way).
 bool rows_settled(const segkv* h, cudaStream_t st, bool lists_too) {
     if (!h->overlap || h->steps == 0) return false;
-    if (!settled(&h->rows_mark, st)) return false;
+    if (!settled(h, &h->rows_mark, st)) return false;
     if (!lists_too) return true;
-    return settled(&index_of(h)->lists_mark, st);
+    return settled(h, &index_of(h)->lists_mark, st);
 }
 
 // May an attention launch start before its predecessor in the stream has finished?  Not before the first step: the

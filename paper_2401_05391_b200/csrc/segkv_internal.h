@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "segkv.h"
+#include "segkv_stream_log.h"
 
 namespace segkv_impl {
 
@@ -20,12 +21,6 @@ constexpr int kMaxTiledBeams = 16;  // beams the tiled kernel handles (16 query 
 struct URow {
     int32_t row;
     uint32_t mask;
-};
-
-// Where and when data was last written: the stream and the per-process sequence number of the launch.
-struct WriteMark {
-    cudaStream_t stream;
-    unsigned long long seq;       // 0: never written
 };
 
 struct Dims {
