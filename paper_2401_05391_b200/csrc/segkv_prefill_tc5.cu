@@ -270,8 +270,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const bool back = p.slopes != nullptr;
     auto tile_at = [&](int i, int n) -> int { return back ? n - 1 - i : i == 0 ? 0 : n - i; };
     // nb = the request's own prompt length: with ragged prompts the items are still laid out for the
-    // longest one, and a shorter request leaves its later items (and the tail of one) without work
-    auto request_len = [&](int b) -> int { return RAGGED ? __ldg(p.plens + b) : p.N; };
+    // longest one, and a shorter request leaves its later items (and the tail of one) without work.  (Lengths and slopes are read
+    // by plain loads: the kernel before may write them, and a read-only load need not stay behind the wait for it below.)
+    auto request_len = [&](int b) -> int { return RAGGED ? p.plens[b] : p.N; };
     auto group_tiles = [&](int qt, int g, int nb) -> int {
         const int base = (qt * NG + g) * kRows;
         return base < nb ? min((nb + kKeys - 1) / kKeys, (base + kRows - 1) / kKeys + 1) : 0;
@@ -471,7 +472,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 if (w >= n_items) continue;
                 const int qt = item_qt(w), nb = RAGGED ? (int)__reduce_max_sync(0xffffffffu, (unsigned)request_len((w % hb_count) / p.H)) : p.N;
                 // is the head's slope one of those whose weights go in two parts next to the diagonal?
-                const bool steep = kSplitP && p.slopes && __any_sync(0xffffffffu, __ldg(p.slopes + (w % hb_count) % p.H) >= kSplitSlope);
+                const bool steep = kSplitP && p.slopes && __any_sync(0xffffffffu, p.slopes[(w % hb_count) % p.H] >= kSplitSlope);
                 int gt[NG], nkt = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
@@ -604,9 +605,9 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // with it in one pass over the scores; 16 (32) keys whose weights add up to more than 2^8 end the pass.  (That they
                 // do is seen from their sum, which is needed anyhow: noting the maximum cost an instruction for every
                 // two scores, and the kernel's large launches run at the power limit.  Not where no key has been visible to a
-                // row so far, nor under a slope that lifts the maximum by 2^4 and more from tile to tile, which towards
-                // older keys is a negative one.)
-                const bool fresh = t == 0 || -slope2 * (float)kKeys >= 4.f || __any_sync(0xffffffffu, m_ref == -INFINITY);
+                // row so far, nor under a negative slope, whose maximum grows from tile to tile towards the oldest key: there the
+                // reference follows it exactly, so that the weight of the key that counts most is not rounded.)
+                const bool fresh = t == 0 || slope2 < 0.f || __any_sync(0xffffffffu, m_ref == -INFINITY);
                 const int seen = row0 + (warp & 3) * 32 + 32 - key0;       // keys that some row of the warp sees
                 const bool mask = key0 + KH - 1 > row0 + (warp & 3) * 32;  // keys that some row of the warp does not see
                 bool stands = false;
@@ -668,7 +669,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     stands = bar_and(rows_bar, 32 * TPR, ok && kept == KH);
                 }
                 if (!stands) {
-                    // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4 (those
+                    // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4 or at all (those
                     // that have are below 2^8 of the one in use): the sum and O use the same reference, so the
                     // result is exact.  Keys beyond the last row of the warp take no part.
                     float tmax = -INFINITY;
@@ -696,7 +697,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
                     for (int i = 0; i < TPR; ++i) tmax = fmaxf(tmax, xrow[i * kRows]);
                     bar_sync_n(rows_bar, 32 * TPR);
-                    const bool need = tmax > m_ref + 4.f, rescale = need && m_ref > -INFINITY;   // (O is zero so far, else)
+                    const bool need = tmax > m_ref + (slope2 < 0.f ? 0.f : 4.f), rescale = need && m_ref > -INFINITY;   // (O is zero so far, else)
                     if (need) {
                         alpha = exp2f(m_ref - tmax);              // 0 on the first keys
                         m_ref = tmax;

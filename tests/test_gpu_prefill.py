@@ -332,3 +332,35 @@ def test_prompt_store_of_odd_shapes(D, kv_heads, P):
         assert h.get_error() == 0
         h.destroy()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,row_groups", [(64, 1), (64, 2), (128, 1), (128, 2), (256, 1)])
+def test_prefill_under_negative_slopes_keeps_the_largest_weight_exact(dtype, D, row_groups):
+    # Slopes that favour OLDER keys: keys of zeros, so that the weights are the bias alone and the oldest key's is the largest, and
+    # values of zeros but the oldest key's ones.  The output is that key's weight over their sum, rounded once if the weight is exact;
+    # a reference left up to 2^4 behind rounds the weight too, which moves about every third output by a unit in the last place.
+    # The exponents' fp32 error (2^-24 of a bias of up to 22 in log2 units, times ln 2: 1e-6) can move a result that lies as near
+    # to a rounding boundary: one in 2^9 (bf16: 2^12) is allowed for, twice over.
+    P = 515
+    slopes = torch.tensor([-0.01, -0.015, -0.02, -0.03], dtype=torch.float32)
+    w = wl.Workload("neg", 1, 2, 4, 2, D, P, 2, dtype, "uniform", True, 170)
+    h = sk.SegKV(w.batch, w.beams, w.heads, w.kv_heads, w.head_dim, w.prompt_len, w.steps, w.torch_dtype)
+    try:
+        h.set_prefill_tuning(row_groups)
+        kp, vp = (torch.zeros_like(x) for x in wl.make_prompt(w, "cuda"))
+        vp[:, 0] = 1
+        q = wl.make_prefill_query(w, "cuda")
+        h.prefill_write(kp, vp)
+        out = h.prefill_sdpa(q, None, slopes.cuda())
+        torch.cuda.synchronize()
+        assert h.get_error() == 0
+        i = torch.arange(P, dtype=torch.float64)
+        s = slopes.to(torch.float64)
+        weights = torch.exp(s[:, None] * i)                       # of a key i places behind the oldest, [heads, P]
+        exact = 1.0 / weights.cumsum(1)                           # of row x: all keys up to x
+        got = out[0].permute(1, 0, 2).cpu()                       # [heads, P, D]
+        off = got != exact.to(w.torch_dtype)[:, :, None]
+        assert off.double().mean() <= 2.0 ** (-11 if dtype == "bf16" else -8), off.double().mean()
+    finally:
+        h.destroy()
