@@ -857,6 +857,29 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
 }
 
+// Are a launch's items dealt in pairs of query tiles of one (request, head) (round_item)?  What that gains is K and V found in the
+// L2 by the other query tiles instead of read from HBM again: nothing where all of them stay there anyhow, little where a tile's
+// arithmetic hides the reads.  What it costs is balance: the middle one of an odd number of query tiles has a CTA to itself, and
+// whole rounds of bpw (request, head)s are dealt.  `share` is the busiest CTA's work in hundredths of the mean.  Pairs against
+// longest-first, times of the attention alone in us: head_dim 128, 3 query tiles 16 x 56 x 768 294 / 235, 11 x 96 x 549 291 / 215; 5, 20 x 56 x
+// 1280 740 / 690; 4, 32 x 56 x 1024 751 / 741; 8, 8 x 56 x 2048 606 / 643; 16, 6 x 56 x 4096 1548 / 1731; two query heads per kv head 8, 8 x 56 x
+// 2048 592 / 598, four (117 MB of K and V) 587 / 576.  head_dim 256 (128-row items), 4, 16 x 32 x 500 150 / 166; 5, 125 x 16 x 640 913 / 864; 7, 16 x 16 x
+// 900 207 / 251; 8, 16 x 16 x 1003 220 / 265; 32, 20 x 16 x 4096 3120 / 3916; eight query heads per kv head, 9, 16 x 56 x 1100 907 / 844, 16, 8 x 56 x
+// 2048 1193 / 1236.  head_dim 64, 2, 36 x 56 x 500 213 / 205; 6, 15 x 56 x 1500 513 / 505; 8, 8 x 56 x 2048 (share 107) 458 / 453, 12 x 40 x 2048 with
+// the store (share 100) 467 / 502; 12, 6 x 56 x 3072 684 / 719.  bf16 with ALiBi: head_dim 64
+// 6 x 56 x 4096 1312 / 1265, 128 32 x 56 x 1024 837 / 840, 8 x 56 x 2048 640 / 660, 4 x 56 x 4000 1059 / 1137, 256 8 x 32 x 1024 211 / 248.
+bool deal_in_pairs(const Dims& d, int prompt_len, bool biased, int nqt, int bpw, int sms) {
+    const long hb = (long)d.heads * d.batch;
+    const long share = 200L * sms * ((hb + bpw - 1) / bpw) / (hb * nqt);
+    const bool in_l2 = 4LL * d.batch * d.kv_heads * prompt_len * d.head_dim < 150000000LL;      // (126 MB of it)
+    const bool two_part = d.dtype == SEGKV_BF16 && biased;        // more work next to the diagonal
+    switch (d.head_dim) {
+        case 64: return nqt >= 4 && !in_l2 && !two_part && share <= (nqt >= 8 ? 104 : 102);
+        case 128: return !in_l2 && (nqt >= 6 ? share <= 115 : !two_part && share <= 104);
+        default: return share <= (in_l2 || nqt < 4 ? 104 : 120);
+    }
+}
+
 template <typename T, typename L>
 cudaError_t launch_tc5(const Dims& d, const PrefillArgs& a, Tc5Params p, int sms, cudaStream_t st) {
     constexpr int NG = L::NG;
@@ -889,10 +912,7 @@ cudaError_t launch_tc5(const Dims& d, const PrefillArgs& a, Tc5Params p, int sms
         const int nqt = (a.prompt_len + kRows * NG - 1) / (kRows * NG), ppb = (nqt + 1) / 2;
         const long hb_count = (long)d.heads * d.batch;
         const int bpw = ppb <= sms ? sms / ppb : 0;
-        // (not for bf16 with ALiBi, where the two-part weights make the tiles next to the diagonal the
-        // expensive ones: measured 20 % slower this way at the Bloom shape, 4 % at twice its prompt)
-        const bool two_part_alibi = d.dtype == SEGKV_BF16 && p.slopes != nullptr;
-        p.paired = (grid == (unsigned)sms && bpw > 0 && hb_count >= 4L * bpw && !two_part_alibi) ? 1 : 0;
+        p.paired = (grid == (unsigned)sms && bpw > 0 && hb_count >= 4L * bpw && deal_in_pairs(d, a.prompt_len, p.slopes != nullptr, nqt, bpw, sms)) ? 1 : 0;
         p.rounds = p.paired ? 2 * (int)((hb_count + bpw - 1) / bpw) : (int)((items + grid - 1) / grid);
     }
     // fused prefill: load through the maps over the caller's arrays, store through the segment's

@@ -364,3 +364,35 @@ def test_prefill_under_negative_slopes_keeps_the_largest_weight_exact(dtype, D, 
         assert off.double().mean() <= 2.0 ** (-11 if dtype == "bf16" else -8), off.double().mean()
     finally:
         h.destroy()
+
+
+@pytest.mark.parametrize("D,B,heads,kv_heads,P,dtype,alibi", [
+    (128, 8, 30, 30, 1300, "bf16", True), (128, 8, 30, 30, 1300, "f16", False), (128, 11, 32, 32, 549, "bf16", False), (256, 16, 37, 37, 500, "bf16", True),
+    (256, 16, 37, 37, 500, "f16", True), (256, 6, 56, 28, 900, "bf16", False), (64, 9, 29, 29, 2400, "f16", False), (64, 9, 29, 29, 2400, "bf16", True),
+    (256, 40, 16, 16, 130, "f16", False), (128, 40, 16, 16, 100, "bf16", True)])
+def test_prefill_dealing_does_not_change_an_output(D, B, heads, kv_heads, P, dtype, alibi):
+    # on both sides of the rule that deals items in pairs: many requests at once against one at a time (too few for pairs)
+    w = wl.Workload("deal", B, 2, heads, kv_heads, D, P, 2, dtype, "uniform", alibi, 180)
+    one = wl.Workload("deal", 1, 2, heads, kv_heads, D, P, 2, dtype, "uniform", alibi, 180)
+    slopes = wl.alibi_slopes(heads).cuda() if alibi else None
+    h, h1 = (sk.SegKV(x.batch, x.beams, x.heads, x.kv_heads, x.head_dim, x.prompt_len, x.steps, x.torch_dtype) for x in (w, one))
+    try:
+        kp, vp = wl.make_prompt(w, "cuda")
+        q = wl.make_prefill_query(w, "cuda")
+        out, fused, ragged = (torch.full_like(q, float("nan")) for _ in range(3))
+        h.prefill(kp, vp, q, fused, slopes)
+        h.prefill_sdpa(q, out, slopes)
+        lens = [P - (37 * b) % (P // 2) for b in range(B)]
+        lens[B // 2] = P
+        h.prefill_write_ragged(kp, vp, lens)
+        h.prefill_sdpa(q, ragged, slopes)
+        h1.set_prefill_tuning(1 if D == 256 else 2)
+        for b in range(B):
+            ref = torch.empty_like(q[b:b + 1])
+            h1.prefill(kp[b:b + 1], vp[b:b + 1], q[b:b + 1], ref, slopes)
+            assert torch.equal(out[b:b + 1], ref) and torch.equal(fused[b:b + 1], ref)
+            assert torch.equal(ragged[b, :lens[b]], ref[0, :lens[b]])
+        assert h.get_error() == 0 and h1.get_error() == 0
+    finally:
+        h.destroy()
+        h1.destroy()
