@@ -13,8 +13,6 @@ LIB = os.path.join(PKG, "libsegkv.so")
 # the same library with per-CTA time stamps compiled in (read by paper_2401_05391_b200/timeline.py);
 # never loaded by the binding, the tests or the benchmark
 LIB_TIMELINE = os.path.join(PKG, "libsegkv_timeline.so")
-# the binding's calls of the decode loop (a CPython extension module over torch's tensor objects)
-LIB_HOT = os.path.join(PKG, "segkv_hot.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = [
@@ -36,31 +34,50 @@ def _stale(lib: str = LIB) -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
-def build_hot(force: bool = False) -> str:
-    """Compile csrc/segkv_hot.cpp into the extension module segkv_hot.so (no-op when up to date)."""
-    src = os.path.join(CSRC, "segkv_hot.cpp")
-    if not force and os.path.exists(LIB_HOT) and os.path.getmtime(LIB_HOT) >= os.path.getmtime(src):
-        return LIB_HOT
+def hot_path() -> str:
+    """Where the binding's extension module (csrc/segkv_hot.cpp) belongs for the torch and the Python that run here: it reads
+    torch's C++ objects, so each version of either has a file of its own and never loads another's."""
     import sysconfig
 
     import torch
+    return os.path.join(PKG, f"segkv_hot.torch-{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
+def build_hot(force: bool = False) -> str:
+    """Compile csrc/segkv_hot.cpp into the extension module at hot_path() (no-op when up to date)."""
+    import sysconfig
+
+    import torch
+    src, out = os.path.join(CSRC, "segkv_hot.cpp"), hot_path()
+    if not force and os.path.exists(out) and os.path.getmtime(out) >= os.path.getmtime(src):
+        return out
     root = os.path.dirname(torch.__file__)
-    tmp = LIB_HOT + f".{os.getpid()}.tmp"
+    tmp = out + f".{os.getpid()}.tmp"
     subprocess.check_call([
         os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
         f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
         "-I", os.path.join(root, "include"), "-I", sysconfig.get_paths()["include"],
         "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), src, "-o", tmp,
         "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
-    os.replace(tmp, LIB_HOT)
-    return LIB_HOT
+    os.replace(tmp, out)
+    return out
 
 
 def build(force: bool = False, verbose: bool = False, timeline: bool = False) -> str:
-    """Compile every .cu under csrc/ into libsegkv.so (no-op when up to date).  `timeline` builds
-    the instrumented copy libsegkv_timeline.so instead."""
-    lib = LIB_TIMELINE if timeline else LIB
-    build_hot(force)
+    """Compile every .cu under csrc/ into libsegkv.so (no-op when up to date), then the binding's extension module where torch and a
+    C++ compiler allow it (the library needs neither, and the binding runs without it).  `timeline` builds the
+    instrumented copy libsegkv_timeline.so instead."""
+    if timeline:
+        return _build_lib(LIB_TIMELINE, force, verbose, timeline)
+    lib = _build_lib(LIB, force, verbose)
+    try:
+        build_hot(force)
+    except (ImportError, OSError, subprocess.CalledProcessError) as e:
+        sys.stderr.write(f"the decode loop's extension module was not built ({e}): its calls go through ctypes\n")
+    return lib
+
+
+def _build_lib(lib: str, force: bool, verbose: bool, timeline: bool = False) -> str:
     if not (force or _stale(lib)):
         return lib
     objs = []

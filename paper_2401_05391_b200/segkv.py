@@ -2,8 +2,8 @@
 
 Argument marshalling only: every step of the decode path runs in the library's
 CUDA kernels.  PyTorch appears only as the owner of device memory and streams.
-The calls of the decode loop check their tensors in the extension module ``segkv_hot`` (``csrc/segkv_hot.cpp``); what it does
-not take as it is goes through the checks here.
+The calls of the decode loop check their tensors in the extension module ``segkv_hot`` (``csrc/segkv_hot.cpp``) where it has been
+built for this torch; what it does not take as it is, and everything without it, goes through the checks here.
 The module-level functions carry the C names; :class:`SegKV` wraps a handle.
 There is no fallback: if ``libsegkv.so`` has not been built the import of the
 library fails with an error that says how to build it.
@@ -17,6 +17,8 @@ from typing import Optional
 
 import numpy as np
 import torch
+
+from .build import hot_path
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libsegkv.so")
@@ -72,18 +74,17 @@ SIGNATURES = {
 }
 
 _lib = None
-HOT_PATH = os.path.join(_PKG, "segkv_hot.so")
 _hot = None
 
 
 def _hot_module():
-    """The extension module of the decode loop's calls (once).  Raises if it has not been built."""
+    """The extension module of the decode loop's calls (once), or None if it has not been built for this torch and Python."""
     global _hot
     if _hot is None:
-        if not os.path.exists(HOT_PATH):
-            raise ImportError(f"{HOT_PATH} is missing: build it with `python -m paper_2401_05391_b200.build`")
-        spec = importlib.util.spec_from_file_location("segkv_hot", HOT_PATH)
-        _hot = importlib.util.module_from_spec(spec)
+        path = hot_path()
+        if not os.path.exists(path):
+            return None
+        _hot = importlib.util.module_from_spec(importlib.util.spec_from_file_location("segkv_hot", path))
     return _hot
 
 
@@ -209,8 +210,8 @@ class SegKV:
         else:
             _check(lib().segkv_create(ctypes.byref(self._h), batch, beams, heads, kv_heads, head_dim,
                                       max_prompt, max_steps, code), "segkv_create")
-        L = lib()
-        self._hot = _hot_module().Hot(self._h.value, self.rows, heads, kv_heads, head_dim, dtype is torch.bfloat16, tuple(
+        L, hot = lib(), _hot_module()
+        self._hot = None if hot is None else hot.Hot(self._h.value, self.rows, heads, kv_heads, head_dim, dtype is torch.bfloat16, tuple(
             ctypes.cast(f, ctypes.c_void_p).value for f in (L.segkv_decode_step, L.segkv_append, L.segkv_decode_sdpa,
                                                             L.segkv_truncate_last, L.segkv_steps)))
 
