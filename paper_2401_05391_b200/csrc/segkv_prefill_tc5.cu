@@ -669,7 +669,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     stands = bar_and(rows_bar, 32 * TPR, ok && kept == KH);
                 }
                 if (!stands) {
-                    // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4 or at all (those
+                    // A new reference, where the maximum of the keys that have no weights yet has grown by more than 2^4, or at all under a negative slope (those
                     // that have are below 2^8 of the one in use): the sum and O use the same reference, so the
                     // result is exact.  Keys beyond the last row of the warp take no part.
                     float tmax = -INFINITY;
@@ -696,11 +696,18 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     if (gone) break;
 #pragma unroll
                     for (int i = 0; i < TPR; ++i) tmax = fmaxf(tmax, xrow[i * kRows]);
-                    bar_sync_n(rows_bar, 32 * TPR);
+                    const bool none = bar_and(rows_bar, 32 * TPR, kept == 0);
                     const bool need = tmax > m_ref + (slope2 < 0.f ? 0.f : 4.f), rescale = need && m_ref > -INFINITY;   // (O is zero so far, else)
-                    if (need) {
+                    if (need && none) {
                         alpha = exp2f(m_ref - tmax);              // 0 on the first keys
                         m_ref = tmax;
+                    } else if (need) {
+                        // Some of the rows' weights are stored: a whole number of powers of two further up, so that they move by
+                        // their exponents alone and none is rounded a second time (read back, scaled by 2^(m_ref - tmax) and
+                        // rounded again their error was half as large again).
+                        const float up = ceilf(tmax - m_ref);
+                        alpha = up < 127.f ? __uint_as_float((uint32_t)(127 - (int)up) << 23) : 0.f;
+                        m_ref += up;
                     }
                     // (no visible key of this row so far: its weights are zeros with any reference)
                     const float m_use = (m_ref == -INFINITY ? 0.f : m_ref) - kWeightShift<T>;
@@ -716,13 +723,10 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const float2 a = Mma<T>::unpack(u[i]);
+                            u[i] = Mma<T>::pack(a.x * alpha, a.y * alpha);
                             if (kSplitP && two) {
                                 const float2 e = Mma<T>::unpack(u[8 + i]);
-                                const float x = (a.x + e.x) * alpha, y = (a.y + e.y) * alpha;
-                                u[i] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
-                                u[8 + i] = Mma<T>::pack(x - __uint_as_float(__float_as_uint(x) & 0xFFFF0000u), y - __uint_as_float(__float_as_uint(y) & 0xFFFF0000u));
-                            } else {
-                                u[i] = Mma<T>::pack(a.x * alpha, a.y * alpha);
+                                u[8 + i] = Mma<T>::pack(e.x * alpha, e.y * alpha);
                             }
                         }
                         tc_st8(tm_s + c, u);

@@ -311,6 +311,44 @@ def test_prefill_references_that_fall_in_the_middle_of_a_tile(dtype, D, row_grou
             h.destroy()
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("D,row_groups", [(64, 1), (64, 2), (128, 1), (128, 2), (256, 1)])
+def test_prefill_rounds_no_weight_twice(dtype, D, row_groups):
+    # Scores of 0 but in the third tile: weights of 2^-3 to 2^2 at keys 320 to 351, and behind them a key 2^9 to 2^11 times the
+    # reference, which ends the tile's pass when those are stored.  Each of them is read off by an output element of its own.  Its
+    # error is the rounding of the weight and that of the output: rounding to p bits is uniform within half a unit, 2^(1-p) of the
+    # number's power of two, so with mantissas spread evenly over their logarithm its mean square is
+    # r2 = 4^(1-p) / 12 * 3 / (8 ln 2), and the two together make 2 r2; a weight that is rounded again makes 3.
+    H, P, keys = 8, 640, range(320, 352)
+    w = wl.Workload("once", 1, 2, H, H, D, P, 2, dtype, "uniform", False, 160)
+    g = torch.Generator().manual_seed(161)
+    u = lambda *n: torch.rand(*n, generator=g, dtype=torch.float64)
+    unit = np.log(2.0) * np.sqrt(D)                               # of q . k for a factor of two
+    q, k, v = (torch.zeros(1, P, H, D, dtype=torch.float64) for _ in range(3))
+    q[0, :, :, 0] = 1 + 0.25 * u(P, H)
+    k[0, keys.start:keys.stop, :, 0] = (-2.4 + 4 * u(len(keys), H)) * unit
+    k[0, 383, :, 0] = (9 + 0.2 * u(H)) * unit
+    for i, j in enumerate(keys):
+        v[0, j, :, i] = 64                                        # (keeps the outputs among the normal numbers)
+    q, k, v = (x.to(w.torch_dtype) for x in (q, k, v))
+    h = sk.SegKV(w.batch, w.beams, w.heads, w.kv_heads, w.head_dim, w.prompt_len, w.steps, w.torch_dtype)
+    try:
+        h.set_prefill_tuning(row_groups)
+        h.prefill_write(k.cuda(), v.cuda())
+        out = h.prefill_sdpa(q.cuda())
+        torch.cuda.synchronize()
+        assert h.get_error() == 0
+        got = out[0, 512:, :, :len(keys)].double().cpu()          # [row, head, key]
+        s = q[0, 512:, :, None, 0].double() * k[0, :, :, 0].double().T[None] / np.sqrt(D)      # [row, head, all keys]
+        e = torch.exp(s) * (torch.arange(P)[None, None] <= torch.arange(512, P)[:, None, None])
+        ref = 64 * e[:, :, keys.start:keys.stop] / e.sum(2, keepdim=True)
+        r2 = 4.0 ** -(7 if dtype == "bf16" else 10) / 12 * 3 / (8 * np.log(2.0))
+        mean = ((got / ref - 1) ** 2).mean().item()
+        assert mean <= 2.4 * r2, mean / r2
+    finally:
+        h.destroy()
+
+
 @pytest.mark.parametrize("D,kv_heads,P", [(64, 1, 1), (64, 3, 700), (128, 5, 77), (256, 7, 130), (256, 80, 3)])
 def test_prompt_store_of_odd_shapes(D, kv_heads, P):
     # blocks of whole tokens: one head, odd heads, tokens that do not divide a block's, a token larger than a block; the fused
