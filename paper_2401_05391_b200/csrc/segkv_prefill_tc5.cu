@@ -64,14 +64,12 @@ constexpr int kBoxQ = kRows * 128;           // 64 head-dim elements of a group'
 constexpr int kTmemCols = 512;
 
 struct Tc5Params {
-    const void* q;
     void* out;
     const float* slopes;
     int* err_word;
     const int32_t* plens;    // per-request prompt lengths (rows and keys past them are skipped), or NULL
-    int N, H, Hkv, G, B, snake;
+    int N, H, G, B, snake;
     int paired, rounds;      // item order: see round_item; rounds = items a CTA walks through (some may be empty)
-    int store_kv;            // 1: every K/V tile is also written to the prompt segment, by the item that owns it
     float scale2;
     uint32_t idesc_qk, idesc_pv;
     int dbg_skip;            // test aid: one softmax thread leaves out one barrier arrival, so that a wait runs out
@@ -921,7 +919,6 @@ cudaError_t launch_tc5(const Dims& d, const PrefillArgs& a, Tc5Params p, int sms
     }
     // fused prefill: load through the maps over the caller's arrays, store through the segment's
     const bool store = a.tm_k_src && a.tm_v_src;
-    p.store_kv = store ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(L::kThreads, 1, 1);
@@ -962,9 +959,9 @@ bool prefill_tc5_supported(const Dims& d) { return d.head_dim == 64 || d.head_di
 cudaError_t launch_prefill_tc5(const Dims& d, const PrefillArgs& a, cudaStream_t st) {
     if (!prefill_tc5_supported(d) || !a.tm_q) return cudaErrorInvalidValue;
     Tc5Params p;
-    p.q = a.q; p.out = a.out; p.slopes = a.slopes; p.err_word = a.err_word;
+    p.out = a.out; p.slopes = a.slopes; p.err_word = a.err_word;
     p.plens = a.plens;
-    p.N = a.prompt_len; p.H = d.heads; p.Hkv = d.kv_heads; p.G = d.group; p.B = d.batch;
+    p.N = a.prompt_len; p.H = d.heads; p.G = d.group; p.B = d.batch;
     p.scale2 = 0.f; p.idesc_qk = p.idesc_pv = 0; p.snake = 0; p.paired = 0; p.rounds = 0;
     p.dbg_skip = a.dbg_skip ? 1 : 0;
     p.wait_ns = a.wait_ns ? a.wait_ns : kWaitLimitNs;

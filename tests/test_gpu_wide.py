@@ -383,7 +383,7 @@ def test_wide_layers_queued_without_waiting(dtype, D, batch, beams, group, hkv, 
 # the partials of a work group land in the prompt ring (128 KB) at once where they fit and the CTA has no further items: the
 # largest counts that fit, one more, columns that do not fill the padding, and CTAs with and without further items
 @pytest.mark.parametrize("D,beams,group,B,kv_heads,splits", [
-    (128, 4, 8, 1, 2, 8), (128, 4, 8, 1, 2, 9), (128, 3, 6, 1, 1, 40), (64, 4, 8, 1, 2, 16), (64, 4, 8, 1, 2, 17),
+    (128, 4, 8, 1, 2, 8), (128, 4, 8, 1, 2, 9), (128, 3, 6, 1, 1, 14), (128, 3, 6, 1, 1, 15), (128, 3, 6, 1, 1, 40), (64, 4, 8, 1, 2, 16), (64, 4, 8, 1, 2, 17),
     (256, 4, 8, 1, 1, 4), (256, 4, 8, 1, 1, 5), (128, 4, 8, 20, 4, 3)])
 def test_split_merge_in_the_prompt_ring(D, beams, group, B, kv_heads, splits):
     w = wl.Workload("land", B, beams, kv_heads * group, kv_heads, D, 700, 4, "f16", "uniform", False, 620 + splits)
