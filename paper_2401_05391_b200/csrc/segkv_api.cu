@@ -417,7 +417,8 @@ bool rather_fused(const segkv* h) {
 // (0.65 us): a round of items costs its tiles (a response tile, which is gathered, twice) plus about two to start and finish an item; meeting in the
 // workspace costs about two, and for every four splits one plus two for each pass of 2048 numbers that the last CTA makes
 // over the partials (fitted to 4 to 64 work groups, prompts of 256 to 16384 in 1 to 64 splits: at most 4 % above the best
-// count, 0.2 % on average).  How many distinct rows the response has is known on the device only: about steps + 2 * beams
+// count, 0.2 % on average; the fit is to partials that go through the workspace: where they land in the merging CTA's ring at
+// once, four splits meet in about 2 us instead of 4.6, so that the count errs towards few splits there).  How many distinct rows the response has is known on the device only: about steps + 2 * beams
 // where beams merge, beams * steps where they stay apart.  The first count decides, the second weighs an eighth: 32 beams
 // that stay apart for 256 steps of 4 work groups, 327 us in one split, get four.
 // (This runs at every attention call: 32-bit divisions, and no count is looked at whose merge alone costs more than the
@@ -800,6 +801,23 @@ int segkv_append_rope(segkv_t h, int step, const int32_t* beam_parent, const voi
     return append_impl(h, step, beam_parent, k_new, v_new, &r, stream);
 }
 
+// Does an append let the attention behind it begin at once, or when the kernel before is complete?  At once that attention sets
+// up on the SMs of the attention before, which slows a short launch down as a whole; a long one, or one whose requests end at
+// different times, has SMs to spare at its end.  Append and attention of a layer, eight layers on a stream, us, after the wait /
+// at once.  From 100 MB of prompt on: 6 x 40 x 1237 keys D 128 32.2 / 31.9, 12 x 40 x 2000 80.7 / 79.6, 16 x 16 x 1024 D 256
+// 51.8 / 50.7, 32 x 16 x 300 D 256 37.4 / 36.4, 40 x 20 x 825 D 64 39.9 / 39.2, 2 x 112 x 1024 and 5 x 40 x 2000 level.
+// Below: 1 x 32 x 1024 D 128 9.8 / 10.3, 1 x 16 x 300 D 64 6.7 / 7.2, 10 x 32 x 500 22.8 / 23.4, 20 x 20 x 400 D 64 with five beams
+// 14.3 / 15.2, 13 x 21 x 825 D 64 16.3 / 17.1, 3 x 40 x 900 with eight beams 20.1 / 21.4.  Lengths between a quarter and the whole
+// of the longest: 2 x 40 x 1237 16.6 / 16.0, 21 x 13 x 825 D 64 15.8 / 14.8, five beams 20 x 20 x 400 D 64 14.2 / 13.9 (but 10 x 32 x
+// 500 21.2 / 22.1); with eight query columns and more 3 x 40 x 900 20.2 / 21.3.  More than 16 columns, in the wide kernel, whose
+// tiles take longer than their loads: 8 x 4 x 2048 with 32, four layers a step, 22.6 / 21.6 (16: 4 x 8 x 1024 16.6 / 16.9).
+bool append_at_once(const segkv* h) {
+    const Dims& d = h->d;
+    if (4LL * d.batch * d.kv_heads * h->prompt_len * d.head_dim >= 100000000LL) return true;
+    const int columns = d.beams * d.group;
+    return columns > 16 || (h->ragged && columns < 8);
+}
+
 static int append_impl(segkv_t h, int step, const int32_t* beam_parent, const void* k_new, const void* v_new,
                        const RopeArgs* rope, void* stream) {
     if (!h || step < 0 || !k_new || !v_new || !aligned16(k_new) || !aligned16(v_new)) return SEGKV_EINVAL;
@@ -812,13 +830,14 @@ static int append_impl(segkv_t h, int step, const int32_t* beam_parent, const vo
         if (rc != SEGKV_OK) return rc;
     }
     const bool pdl = h->overlap && step > 0;
-    const Release rel = pdl ? kAtOnce : kAtOnceSerialised;
+    const bool at_once = append_at_once(h);
+    const Release rel = !at_once ? kAfterWait : pdl ? kAtOnce : kAtOnceSerialised;
     if (h->leader) {
         // the tables of this step have been made by the leader's call: only the K/V rows are stored
         if (h->leader->steps != step + 1 || h->leader->truncated) return SEGKV_ESTATE;
         SEGKV_CUDA(launch_append(h->d, step, nullptr, k_new, v_new, k_slab_of(h, step),
                                  k_slab_of(h, step) + vdelta_of(h), nullptr, nullptr, nullptr, nullptr, nullptr,
-                                 h->err_word, h->sm_count, pdl, (cudaStream_t)stream, rope, false));
+                                 h->err_word, h->sm_count, pdl, at_once, (cudaStream_t)stream, rope, false));
         mark_written(h, &h->rows_mark, (cudaStream_t)stream, rel);
         h->steps = step + 1;
         h->truncated = false;
@@ -827,7 +846,7 @@ static int append_impl(segkv_t h, int step, const int32_t* beam_parent, const vo
     SEGKV_CUDA(launch_append(h->d, step, beam_parent, k_new, v_new, k_slab_of(h, step),
                              k_slab_of(h, step) + vdelta_of(h), h->parent,
                              h->anc[(step + 1) & 1], h->anc[step & 1], h->ulist, h->ucount, h->err_word,
-                             h->sm_count, pdl, (cudaStream_t)stream, rope));
+                             h->sm_count, pdl, at_once, (cudaStream_t)stream, rope));
     mark_written(h, &h->rows_mark, (cudaStream_t)stream, rel);
     h->lists_mark = h->rows_mark;                  // the same launch made the lists
     h->steps = step + 1;

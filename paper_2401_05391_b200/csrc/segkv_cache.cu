@@ -202,14 +202,15 @@ append_kernel(int B, int W, int rows, int max_steps, int step, const int32_t* __
               const uint4* __restrict__ k_new, const uint4* __restrict__ v_new, uint4* __restrict__ kr_slab,
               uint4* __restrict__ vr_slab, long long slab_chunks, int32_t* __restrict__ parent_row,
               const int32_t* __restrict__ anc_prev, int32_t* __restrict__ anc_cur, URow* __restrict__ ulist,
-              int32_t* __restrict__ ucount, int* __restrict__ err_word, int rebuild, const RopeArgs rope) {
-    // Programmatic dependent launch: this kernel touches nothing until the previous kernel of
-    // the stream has completed, but lets the next one, the attention that follows it, start its prologue
-    // at once: its CTAs move in where those of the attention before this append end, and fetch their
-    // prompt tiles under the end of that launch and under this one.  (What a kernel behind this one may read
-    // ahead of its own wait is counted by the host accordingly: see StreamLog.)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+              int32_t* __restrict__ ucount, int* __restrict__ err_word, int rebuild, int at_once, const RopeArgs rope) {
+    // Programmatic dependent launch: this kernel touches nothing until the previous kernel of the stream has completed.  The next
+    // one, the attention that follows it, may start its prologue at once where `at_once` says so: its CTAs move in where those of
+    // the attention before this append end, and fetch their prompt tiles under the end of that launch and under this one; else
+    // under this one only.  (See append_at_once for the choice; what a kernel behind this one may read ahead of its own wait is
+    // counted by the host accordingly: see StreamLog.)
+    if (at_once) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!at_once) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if ((int)blockIdx.x >= B) {
         // ---- copy blocks -------------------------------------------------
         const long long nb = gridDim.x - B;
@@ -313,7 +314,7 @@ append_kernel(int B, int W, int rows, int max_steps, int step, const int32_t* __
 cudaError_t launch_append(const Dims& d, int step, const int32_t* beam_parent, const void* k_new,
                           const void* v_new, void* kr_slab_v, void* vr_slab_v, int32_t* parent_tab,
                           const int32_t* anc_prev, int32_t* anc_cur, URow* ulist, int32_t* ucount,
-                          int* err_word, int sm_count, bool pdl, cudaStream_t st, const RopeArgs* rope, bool tables) {
+                          int* err_word, int sm_count, bool pdl, bool at_once, cudaStream_t st, const RopeArgs* rope, bool tables) {
     const long long slab_elems = (long long)d.rows * d.kv_heads * d.head_dim;
     const long long slab_chunks = slab_elems * 2 / 16;
     long long copy_blocks = (slab_chunks + kBtThreads * 4 - 1) / (kBtThreads * 4);
@@ -338,7 +339,7 @@ cudaError_t launch_append(const Dims& d, int step, const int32_t* beam_parent, c
     return cudaLaunchKernelEx(&cfg, append_kernel, table_blocks, d.beams, d.rows, d.max_steps, step, bp,
                               (const uint4*)k_new, (const uint4*)v_new, kr_slab, vr_slab, slab_chunks,
                               tables ? parent_tab + (size_t)step * d.rows : (int32_t*)nullptr, anc_prev, anc_cur, ulist,
-                              ucount, err_word, 0,
+                              ucount, err_word, 0, at_once ? 1 : 0,
                               rope ? *rope : RopeArgs{});
 }
 
@@ -349,7 +350,7 @@ cudaError_t launch_rebuild_lists(const Dims& d, int steps, const int32_t* anc_cu
     if (steps <= 0) return cudaSuccess;
     append_kernel<<<(unsigned)d.batch, kBtThreads, 0, st>>>(
         d.batch, d.beams, d.rows, d.max_steps, steps - 1, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr,
-        nullptr, const_cast<int32_t*>(anc_cur), ulist, ucount, nullptr, 1, RopeArgs{});
+        nullptr, const_cast<int32_t*>(anc_cur), ulist, ucount, nullptr, 1, 1, RopeArgs{});
     return cudaGetLastError();
 }
 

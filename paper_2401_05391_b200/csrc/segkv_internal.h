@@ -130,7 +130,7 @@ cudaError_t launch_prefill_transpose(const Dims& d, const void* k, const void* v
 cudaError_t launch_append(const Dims& d, int step, const int32_t* beam_parent, const void* k_new,
                           const void* v_new, void* kr_slab, void* vr_slab, int32_t* parent_tab,
                           const int32_t* anc_prev, int32_t* anc_cur, URow* ulist, int32_t* ucount,
-                          int* err_word, int sm_count, bool pdl, cudaStream_t st, const RopeArgs* rope = nullptr,
+                          int* err_word, int sm_count, bool pdl, bool at_once, cudaStream_t st, const RopeArgs* rope = nullptr,
                           bool tables = true);
 // A read-only pass over `bytes` of device memory (16-byte loads); sink: 64 words of device memory.
 cudaError_t launch_read_stream(const void* src, size_t bytes, unsigned* sink, int sm_count, cudaStream_t st);

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2401_05391_b200 import segkv as sk
 from paper_2401_05391_b200 import workloads as wl
 
 from _harness import Run, all_pairs, sampled_pairs
@@ -108,3 +109,42 @@ def test_appends_in_a_row_and_attention_behind_them(B, heads, kv_heads, P):
     finally:
         for r in ls + refs:
             r.close()
+
+
+@pytest.mark.parametrize("D,B,W,heads,kv_heads,P,ragged", [
+    (64, 3, 4, 8, 8, 300, False), (64, 3, 4, 8, 8, 300, True), (64, 3, 8, 8, 8, 300, True), (128, 5, 4, 8, 4, 300, True),
+    (128, 6, 4, 40, 40, 813, False), (128, 6, 4, 40, 40, 814, False)])          # 99.9 and 100.02 MB of prompt
+def test_appends_that_release_at_once_and_after_their_wait(D, B, W, heads, kv_heads, P, ragged):
+    # three layers' appends in a row, then their attentions, and layer by layer: the bits of calls that are each waited for
+    w = wl.Workload("rel", B, W, heads, kv_heads, D, P, 4, "f16", "uniform", False, 340)
+    par = torch.from_numpy(wl.make_parents(w)).cuda()
+    kp, vp = wl.make_prompt(w, "cuda")
+    steps = [[wl.make_step(w.scaled(index=w.index + 11 * i), t, "cuda") for i in range(3)] for t in range(w.steps)]
+    outs = {}
+    for mode in ("plain", "rows", "layers"):
+        hs = [sk.SegKV(B, W, heads, kv_heads, D, P, w.steps, w.torch_dtype) for _ in range(3)]
+        outs[mode] = []
+        for h in hs:
+            if ragged:
+                h.prefill_write_ragged(kp, vp, [P - (61 * b) % (P // 2) for b in range(B)])
+            else:
+                h.prefill_write(kp, vp)
+        for t in range(w.steps):
+            if mode == "rows":
+                for h, (q, k, v) in zip(hs, steps[t]):
+                    h.append(t, par[t] if t else None, k, v)
+                outs[mode] += [h.decode_sdpa(q) for h, (q, k, v) in zip(hs, steps[t])]
+            else:
+                for h, (q, k, v) in zip(hs, steps[t]):
+                    h.append(t, par[t] if t else None, k, v)
+                    if mode == "plain":
+                        torch.cuda.synchronize()
+                    outs[mode].append(h.decode_sdpa(q))
+                    if mode == "plain":
+                        torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert all(h.get_error() == 0 for h in hs)
+        for h in hs:
+            h.destroy()
+    for x, y, z in zip(*(outs[m] for m in ("plain", "rows", "layers"))):
+        assert torch.equal(x, y) and torch.equal(x, z)
