@@ -33,9 +33,9 @@
 //     tile j+1 runs under the softmax of tile j.  The tail of one item overlaps the head of the
 //     next (loads, and the first Q.K^T while the previous output is stored).
 //
-// What bounds it: with thousands of items the power limit (1000 W at 1.5 to 1.65 GHz, where a lone call runs at 1.9), so that a
-// shorter chain buys less than fewer instructions and bytes do; with a few, a group's chain softmax -> P.V -> Q.K^T and
-// the start.  Measured in turn with the form that went from the oldest keys forward throughout, held P back until the row's two
+// What bounds it: a group's chain softmax -> P.V -> Q.K^T (1024 clocks of MMAs and as many of exponentials a tile), which two
+// groups overlap in part, and the issue slots of the softmax; with a few items the start as well.  (Large launches run at 1.5 to
+// 1.65 GHz where a lone call runs at 1.9, so compare queued times with queued ones: these are.)  Measured in turn with the form that went from the oldest keys forward throughout, held P back until the row's two
 // threads had met, spilled and was launched behind the whole kernel before (before / now in us, attention alone): with ALiBi
 // 32 x 112 heads x 1024 at D 128 bf16 1922 / 1607 (fp16 1825 / 1335), D 64, 16 x 64 x 2048, bf16 1515 / 1053, D 256, 2 x 8 x 2000, bf16
 // 61.6 / 42.1; without 64 x 56 x 2048 at D 128 fp16 4810 / 4789, bf16 5118 / 4787, 1 x 32 x 1024 20.6 / 18.9, 4 x 40 x 700 49.3 / 44.6,
@@ -602,7 +602,7 @@ prefill_tc5_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 // The reference in use nearly always stands behind the first tile: the weights are worked out and stored
                 // with it in one pass over the scores; 16 (32) keys whose weights add up to more than 2^8 end the pass.  (That they
                 // do is seen from their sum, which is needed anyhow: noting the maximum cost an instruction for every
-                // two scores, and the kernel's large launches run at the power limit.  Not where no key has been visible to a
+                // two scores, on the chain that sets the pace.  Not where no key has been visible to a
                 // row so far, nor under a negative slope, whose maximum grows from tile to tile towards the oldest key: there the
                 // reference follows it exactly, so that the weight of the key that counts most is not rounded.)
                 const bool fresh = t == 0 || slope2 < 0.f || __any_sync(0xffffffffu, m_ref == -INFINITY);
